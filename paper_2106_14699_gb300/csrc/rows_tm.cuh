@@ -270,10 +270,17 @@ k_pair_rows_tm(const cpx<float>* __restrict__ Y, Geom g, Tw<float> tw, double* _
             cpx<float> v[M];
             if constexpr (R == 1 && M == 32 && C::STAGE_BYTES >= M * M * 8) {
                 // the staged row is consumed by the loads: its buffer takes the one-pass
-                // complex transpose (the next copy into it is issued after the transform)
+                // complex transpose (the next copy into it is issued after the transform).
+                // A team without a pair in this round must leave the buffer alone: the copy
+                // of its next row's pair may already be in flight into it.
+                if (act) {
 #pragma unroll
-                for (int i = 0; i < M; ++i) v[i] = load(j + M * i);
-                team_fft_core<M, +1, false, true, 3>(v, j, const_cast<cpx<float>*>(stage), tw_sq);
+                    for (int i = 0; i < M; ++i) v[i] = load(j + M * i);
+                    team_fft_core<M, +1, false, true, 3>(v, j, const_cast<cpx<float>*>(stage), tw_sq);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < M; ++i) v[i] = {0.f, 0.f};
+                }
             } else {
                 team_fft<M, R, +1, false, C::ONCE, false, 3>(v, r, j, load, region + r * grp_scratch_bytes<float, M>(),
                                                                  tw_sq, tw_pre);

@@ -120,6 +120,22 @@ def test_wide_rows_tmem_path(cm, shape, K, monkeypatch):
     assert np.array_equal(g2["n"], g["n"]) and np.array_equal(g2["mi"], g["mi"])
 
 
+@pytest.mark.parametrize("W,Q", [(450, 512), (900, 1024), (1100, 2048)])
+@pytest.mark.parametrize("K", [(9, 3), (5, 5)], ids=lambda x: "x".join(map(str, x)))
+def test_wide_rows_tmem_partial_rounds(cm, W, Q, K):
+    """Label pairs that do not fill the last round of 16 teams, with more output rows than
+    resident blocks: the teams without a pair in that round already hold the copy of their
+    next row's pair in flight.  N and MI over the whole map against the oracle."""
+    rng = np.random.default_rng(W + K[0])
+    A, MA, B, MB = _rand(rng, 170, W, 160, 40, *K)
+    assert 3 * Q // 4 < W + 39 <= Q or Q == 2048 and 1024 < W + 39
+    g = run_gpu(cm, A, MA, B, MB, K[0], K[1], cm.FP32, counts=False, gamma=0.5)
+    assert g["status"][0] == "OK", g["status"]
+    ref = oracle.cmif(A, MA, B, MB, K[0], K[1])
+    np.testing.assert_array_equal(g["n"], ref["n"])
+    assert float(np.abs(g["mi"] - ref["mi"]).max()) <= MI_TOL
+
+
 @pytest.mark.parametrize("shape,K", WIDE[:3], ids=lambda x: "x".join(map(str, x)))
 def test_wide_rows_tmem_auto(cm, shape, K, monkeypatch):
     """CMIF_AUTO at the Tensor-Memory widths: the row kernel's AUTO form (exact
