@@ -146,7 +146,7 @@ cmif_status choose_rows(cmif_plan p, Workspace<T>& w) {
     if (sizeof(T) == 4 && !(no_tm && no_tm[0] == '1')) {
         const int cols = rows_tm_cols(g.Q, g.KB);
         if (cols > 0) {
-            e = rows_tm_max_blocks_per_sm(g.Q, &bps);
+            e = rows_tm_max_blocks_per_sm(g.Q, cols, &bps);
             if (e != cudaSuccess) return from_cuda(e);
             if (bps >= 1) w.args.tm_cols = cols;
         }
@@ -200,7 +200,7 @@ size_t workspace_bytes(const Geom& g, const Workspace<T>& w) {
     off = align_up(off + (size_t)g.KB * g.DB * g.HB * g.Qs * cs, 256);  // T1B
     off = align_up(off + (size_t)g.KA * g.DA * g.Qh * g.P * cs, 256);   // FA
     off = align_up(off + (size_t)g.KB * g.DB * g.Qh * g.P * cs, 256);   // FB
-    off = align_up(off + (size_t)(w.ypairs > 0 ? w.ypairs : g.KA * g.KB) * g.R * g.Qs * cs, 256);  // Y
+    off = align_up(off + (size_t)(w.ypairs > 0 ? w.ypairs : g.KA * g.KB) * y_rows<T>(g.R) * g.Ys * cs, 256);  // Y
     off = align_up(off + (w.cb_smem ? 0 : (size_t)w.rows_grid * g.KB * g.Q * sizeof(float)), 256);  // CB
     off = align_up(off + sizeof(int), 256);  // work counter
     if (w.rows_grid_w > 0) {
@@ -220,7 +220,7 @@ void carve_workspace(const Geom& g, Workspace<T>& w, char* base) {
     w.args.FA = (cpx<T>*)(base + off); off = align_up(off + (size_t)g.KA * g.DA * g.Qh * g.P * cs, 256);
     w.args.FB = (cpx<T>*)(base + off); off = align_up(off + (size_t)g.KB * g.DB * g.Qh * g.P * cs, 256);
     w.args.Y = (cpx<T>*)(base + off);
-    off = align_up(off + (size_t)(w.ypairs > 0 ? w.ypairs : g.KA * g.KB) * g.R * g.Qs * cs, 256);
+    off = align_up(off + (size_t)(w.ypairs > 0 ? w.ypairs : g.KA * g.KB) * y_rows<T>(g.R) * g.Ys * cs, 256);
     w.args.cb_global = w.cb_smem ? nullptr : (float*)(base + off);
     off = align_up(off + (w.cb_smem ? 0 : (size_t)w.rows_grid * g.KB * g.Q * sizeof(float)), 256);
     w.args.work_ctr = (int*)(base + off);
@@ -497,6 +497,7 @@ cmif_status plan_init(cmif_plan p, int H_A, int W_A, int H_B, int W_B, int K_A, 
     if (g.P > 4096 || g.Q > 4096) return CMIF_ERR_UNSUPPORTED;
     g.Qh = g.Q / 2 + 1;
     g.Qs = (int)align_up((size_t)g.Qh, 4);
+    g.Ys = g.Q / 2;
     g.r0 = 0; g.r1 = g.R; g.c0 = 0; g.c1 = g.C;
     cudaError_t e = cudaGetDevice(&p->device);
     if (e != cudaSuccess) return CMIF_ERR_CUDA;
@@ -508,7 +509,7 @@ cmif_status plan_init(cmif_plan p, int H_A, int W_A, int H_B, int W_B, int K_A, 
     if ((flags & CMIF_FLAG_BATCH_ANGLES) && !volume && prec == CMIF_FP32) {
         // as many angles per launch as 40% of the free device memory holds (at most 64)
         const size_t per_unit = (size_t)K_B * H_B * g.Qs * 8 + (size_t)K_B * g.Qh * g.P * 8 +
-                                (size_t)K_A * K_B * g.R * g.Qs * 8 + (size_t)g.R * g.C * 12 + (size_t)H_B * W_B * 5;
+                                (size_t)K_A * K_B * y_rows<float>(g.R) * g.Ys * 8 + (size_t)g.R * g.C * 12 + (size_t)H_B * W_B * 5;
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return CMIF_ERR_CUDA;
         long long u = (long long)(0.4 * (double)fr / (double)per_unit);
@@ -550,7 +551,7 @@ cmif_status plan_init(cmif_plan p, int H_A, int W_A, int H_B, int W_B, int K_A, 
         // of listed pairs at a time (a few GB at most), and the exact counts of at
         // most `cap` listed pairs
         const int npairs = K_A * K_B;
-        const size_t per_pair = (size_t)g.R * g.Qs * (p->tier2 == CMIF_FP64 ? sizeof(cpx<double>) : sizeof(cpx<df32>));
+        const size_t per_pair = (size_t)g.R * g.Ys * (p->tier2 == CMIF_FP64 ? sizeof(cpx<double>) : sizeof(cpx<df32>));
         const size_t budget = 4ull << 30;
         p->esc.chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)npairs, budget / per_pair));
         p->esc.cap = std::min(npairs, 128);

@@ -4,11 +4,10 @@
 // in the frequency domain with FFTs (Sec. 3.5, Eq. maincomplexity).  These
 // are the transforms, written for sm_103a:
 //
-//  * dft_reg<M>     : an M-point DFT (M = 2..32) held in one thread's
-//                     registers, radix-2 decimation in frequency, twiddles
-//                     folded to compile-time constants (optionally in the
-//                     radix-2^2 order, fewer general rotations).  Output in
-//                     bit-reversed register order.
+//  * dft_reg<M>     : an M-point DFT held in one thread's registers, radix-2
+//                     decimation in frequency, twiddles folded to compile-time
+//                     constants.  Output in bit-reversed register order.  FP32
+//                     DFTs of 8 and more points are the packed ones of fft_pk.cuh.
 //  * team_fft<M,R>  : a length N = R*M*M DFT done by a "team" of R groups of
 //                     M lanes (M points per lane).  The four-step split
 //                     N' = M*M needs a single shared-memory transpose (XOR
@@ -100,73 +99,25 @@ __device__ __forceinline__ cpx<T> twc(cpx<T> d, int k) {
 
 // In-register M-point DFT, natural order in, bit-reversed order out:
 // after the call v[brev(k, M)] = sum_n v_in[n] e^{DIR 2 pi i n k / M}.
-// PACK = false keeps the butterflies' adds in scalar form (the +-i twiddles then
-// stay free operand negations), for kernels where that issues fewer instructions.
-template <int M, int DIR, bool PACK, typename T>
-__device__ __forceinline__ void dft_reg_r22(cpx<T> (&v)[M]) {
-    // Radix-2^2 ordering of the radix-2 network: the stages go in pairs; on the first
-    // stage of a pair a lower output keeps only the quarter-turn part of its twiddle
-    // (a free swap / negation) and defers the rest, which is the same for the two
-    // inputs of its next butterfly and so moves past it; the second stage applies
-    // everything pending.  N = 32: 28 general rotations instead of 34 (16: 8 vs 10).
-    // pend[i]: rotation still owed by v[i], in units of 2 pi / 32 (all compile-time).
-    int pend[M];
-#pragma unroll
-    for (int i = 0; i < M; ++i) pend[i] = 0;
-#pragma unroll
-    for (int span = M / 2, stage = 0; span >= 1; span >>= 1, ++stage) {
-        const bool first = (stage % 2 == 0) && span >= 2;
-#pragma unroll
-        for (int start = 0; start < M; start += 2 * span) {
-#pragma unroll
-            for (int j = 0; j < span; ++j) {
-                const cpx<T> a = v[start + j], b = v[start + j + span];
-                if constexpr (PACK) {
-                    v[start + j] = a + b;
-                    v[start + j + span] = a - b;
-                } else {
-                    v[start + j] = cpx<T>{a.x + b.x, a.y + b.y};
-                    v[start + j + span] = cpx<T>{a.x - b.x, a.y - b.y};
-                }
-                pend[start + j + span] = (pend[start + j] + j * (32 / (2 * span))) & 31;
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            const int e = pend[i];
-            const int q = first ? (e & ~7) : e;
-            if (q) v[i] = twc<32, DIR>(v[i], q);
-            pend[i] = e - q;
-        }
-    }
-}
-
-template <int M, int DIR, bool PACK = true, bool R22 = false, typename T>
+template <int M, int DIR, typename T>
 __device__ __forceinline__ void dft_reg(cpx<T> (&v)[M]) {
-    if constexpr (R22) {
-        dft_reg_r22<M, DIR, PACK>(v);
-        return;
-    }
 #pragma unroll
     for (int span = M / 2; span >= 1; span >>= 1) {
 #pragma unroll
         for (int start = 0; start < M; start += 2 * span) {
 #pragma unroll
             for (int j = 0; j < span; ++j) {
-                cpx<T> a = v[start + j], b = v[start + j + span];
-                if constexpr (PACK) {
-                    v[start + j] = a + b;
-                    v[start + j + span] = twc<M, DIR>(a - b, j * (M / (2 * span)));
-                } else {
-                    v[start + j] = cpx<T>{a.x + b.x, a.y + b.y};
-                    v[start + j + span] = twc<M, DIR>(cpx<T>{a.x - b.x, a.y - b.y}, j * (M / (2 * span)));
-                }
+                const cpx<T> a = v[start + j], b = v[start + j + span];
+                v[start + j] = a + b;
+                v[start + j + span] = twc<M, DIR>(a - b, j * (M / (2 * span)));
             }
         }
     }
 }
 
 }  // namespace cmif
+
+#include "fft_pk.cuh"
 
 namespace cmif {
 
@@ -231,7 +182,9 @@ __host__ __device__ constexpr int max_m() { return sizeof(T) == 4 ? 32 : 16; }  
 
 // Twiddle tables in device memory, filled once per device from FP64 values.
 //   n[l][k]         = e^{-2 pi i k / 2^l},           k < 2^l
-//   sq[l][k1*M + j] = e^{-2 pi i j k1 / (M*M)},       M = 2^l, j, k1 < M
+//   sq[l][k1*M + j] = e^{-2 pi i j k1 / (M*M)},       M = 2^l, j, k1 < M; FP32, M >= 8: as float4
+//                     entries k*M + j, k < M/2, with rows k and k + M/2 side by side
+//                     (cos, cos', sin, sin')
 //   n3[l][k]        = e^{-2 pi i k / (3 2^l)},       k < 3 2^l
 template <typename T>
 struct Tw {
@@ -286,112 +239,140 @@ __host__ __device__ constexpr int team_scratch_bytes() {
 // Every lane of every warp taking part must call this (it uses __syncwarp).
 // The four-step core on values already in registers: v[i] = y[j + M*i] for the
 // group's M*M-point sequence y.  Result: v[brev(k2, M)] = Y[j + M*k2].
-// R22: bit 0 / bit 1 put the first / second register DFT in the radix-2^2 order.
-template <int M, int DIR, bool PACK = true, bool WIDE = false, int R22 = 0, typename T>
-__device__ __forceinline__ void team_fft_core(cpx<T> (&v)[M], int j, void* sm, const cpx<T>* __restrict__ twq) {
-    dft_reg<M, DIR, PACK, (R22 & 1) != 0>(v);  // v[brev(k1)] = A[j][k1]
+//
+// FP32, M >= 8: packed DFTs (fft_pk.cuh).  The transpose holds the real and the imaginary
+// parts in planes of M rows by M floats (WIDE: both planes at once, a group scratch of M*M
+// complex; else one after the other).  A row's M/4 blocks of 4 floats are XOR-permuted by
+// the row, so that 8 lanes reading 8 rows hit 8 different 16-byte bank groups; the writes
+// of one row are a permutation of it.  Groups narrower than a warp sit in different banks
+// (their padding, or WIDE: each group permutes its rows by its place in the warp).
+template <int M>
+__device__ __forceinline__ int tr_swz(int row) {  // the row's XOR of its block index
+    return M == 32 ? row & 7 : M == 16 ? (row >> 1) & 3 : (row >> 2) & 1;
+}
+// Position pairs: on entry re[m] = (y[j + M 2m].re, y[j + M (2m + 1)].re); on exit re[k] =
+// (Y[j + M k].re, Y[j + M (k + M/2)].re); im likewise.
+template <int M, int DIR, bool WIDE>
+__device__ __forceinline__ void team_core_pk(float2 (&re)[M / 2], float2 (&im)[M / 2], int j, float* sf,
+                                             const float4* __restrict__ twp) {
+    constexpr int H = M / 2, NB = M / 4;
+    dft_pk<M, DIR>(re, im);
 #pragma unroll
-    for (int k1 = 1; k1 < M; ++k1) v[brev(k1, M)] = cmul(v[brev(k1, M)], twl<DIR>(twq, k1 * M + j));
-    if constexpr (WIDE) {
-        // WIDE (FP32, M = 16 or 32, a group scratch of M*M complex): one pass of complex
-        // values.  Row k1 holds M/2 blocks of two complex; element (k1, col) sits in
-        // block (col / 2) ^ (k1 % 8).  A row write by the 32 lanes is a permutation of
-        // the row; the 16-byte row reads of 8 lanes (rows j .. j + 7) hit 8 different
-        // 16-byte bank groups: conflict-free.
-        static_assert(sizeof(T) == 4 && (M == 32 || M == 16), "wide transpose: FP32, 16- or 32-lane groups");
-        float2* sc = reinterpret_cast<float2*>(sm);
-        __syncwarp();
-#pragma unroll
-        for (int k1 = 0; k1 < M; ++k1) {
-            const cpx<T> z = v[brev(k1, M)];
-            sc[k1 * M + ((((j >> 1) ^ (k1 & 7)) << 1) | (j & 1))] = make_float2(z.x, z.y);
+    for (int k = 0; k < H; ++k) {
+        const float4 w = twp[k * M + j];  // rows k and k + H: (cos, cos', sin, sin'), forward sign
+        const float2 c = make_float2(w.x, w.y), s = make_float2(w.z, w.w), a = re[k], b = im[k];
+        if (DIR > 0) {
+            re[k] = __ffma2_rn(b, s, __fmul2_rn(a, c));
+            im[k] = __fmul2_rn(b, c);
+            im[k] = make_float2(fmaf(-a.x, s.x, im[k].x), fmaf(-a.y, s.y, im[k].y));
+        } else {
+            re[k] = __fmul2_rn(a, c);
+            re[k] = make_float2(fmaf(-b.x, s.x, re[k].x), fmaf(-b.y, s.y, re[k].y));
+            im[k] = __ffma2_rn(a, s, __fmul2_rn(b, c));
         }
-        __syncwarp();
+    }
+    const int gx = WIDE && M < 32 ? (threadIdx.x / M) & (32 / M - 1) : 0;  // the group's place in its warp
+    // byte offsets: rows sharing a block permutation x differ by whole multiples of the row
+    // length, so one address per x serves all of them
+    char* const base = reinterpret_cast<char*>(sf);
+    auto put = [&](auto store) {
 #pragma unroll
-        for (int b = 0; b < M / 2; ++b) {
-            const float4 q = *reinterpret_cast<const float4*>(sc + j * M + ((b ^ (j & 7)) << 1));
-            v[2 * b] = {q.x, q.y};
-            v[2 * b + 1] = {q.z, q.w};
-        }
-        __syncwarp();
-    } else if constexpr (sizeof(T) == 4 && M == 32) {
-        // Rows of 32 floats in 8 blocks of 4; element (row, col) sits in block
-        // (col/4) ^ (row % 8).  Column writes (one float per lane) are a
-        // permutation of the row's 32 banks; row reads take 16-byte loads and the
-        // 8 lanes of each 16-byte phase hit 8 different blocks: conflict-free.
-        float* sf = reinterpret_cast<float*>(sm);
-        const int jb = j >> 2, jl = j & 3;
+        for (int x = 0; x < NB; ++x) {
+            char* const p = base + ((j << 2) ^ (x << 4));
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            __syncwarp();
-#pragma unroll
-            for (int k1 = 0; k1 < M; ++k1)
-                sf[k1 * M + (((jb ^ k1) & 7) << 2) + jl] = half ? v[brev(k1, M)].y : v[brev(k1, M)].x;
-            __syncwarp();
-#pragma unroll
-            for (int b4 = 0; b4 < 8; ++b4) {
-                const float4 q = *reinterpret_cast<const float4*>(sf + j * M + (((b4 ^ j) & 7) << 2));
-                if (half) { v[4 * b4].y = q.x; v[4 * b4 + 1].y = q.y; v[4 * b4 + 2].y = q.z; v[4 * b4 + 3].y = q.w; }
-                else      { v[4 * b4].x = q.x; v[4 * b4 + 1].x = q.y; v[4 * b4 + 2].x = q.z; v[4 * b4 + 3].x = q.w; }
+            for (int row = 0; row < M; ++row) {
+                if (tr_swz<M>(row) != x) continue;
+                char* const q = WIDE && M < 32 ? p + ((row ^ gx) * M * 4) : p + row * M * 4;
+                store(q, row);
             }
         }
-        __syncwarp();
-    } else if constexpr (sizeof(T) == 4) {
-        float* sf = reinterpret_cast<float*>(sm);
-        __syncwarp();
+    };
+    auto get = [&](int off, float2(&d)[H]) {
+        const char* const rb = base + off + (j ^ gx) * M * 4;
 #pragma unroll
-        for (int k1 = 0; k1 < M; ++k1) sf[k1 * M + (j ^ k1)] = v[brev(k1, M)].x;
+        for (int b = 0; b < NB; ++b) {
+            const float4 q = *reinterpret_cast<const float4*>(rb + ((b ^ tr_swz<M>(j)) << 4));
+            d[2 * b] = make_float2(q.x, q.y);
+            d[2 * b + 1] = make_float2(q.z, q.w);
+        }
+    };
+    auto val = [&](const float2(&d)[H], int row) { return row < H ? d[row].x : d[row - H].y; };
+    __syncwarp();
+    if constexpr (WIDE) {
+        put([&](char* q, int row) {
+            *reinterpret_cast<float*>(q) = val(re, row);
+            *reinterpret_cast<float*>(q + M * M * 4) = val(im, row);
+        });
         __syncwarp();
-#pragma unroll
-        for (int n2 = 0; n2 < M; ++n2) v[n2].x = sf[j * M + (n2 ^ j)];
-        __syncwarp();
-#pragma unroll
-        for (int k1 = 0; k1 < M; ++k1) sf[k1 * M + (j ^ k1)] = v[brev(k1, M)].y;
-        __syncwarp();
-#pragma unroll
-        for (int n2 = 0; n2 < M; ++n2) v[n2].y = sf[j * M + (n2 ^ j)];
-        __syncwarp();
+        get(0, re);
+        get(M * M * 4, im);
     } else {
-        cpx<T>* sc = reinterpret_cast<cpx<T>*>(sm);
+        put([&](char* q, int row) { *reinterpret_cast<float*>(q) = val(re, row); });
         __syncwarp();
-#pragma unroll
-        for (int k1 = 0; k1 < M; ++k1) sc[k1 * M + (j ^ k1)] = v[brev(k1, M)];
+        get(0, re);
         __syncwarp();
-#pragma unroll
-        for (int n2 = 0; n2 < M; ++n2) v[n2] = sc[j * M + (n2 ^ j)];
+        put([&](char* q, int row) { *reinterpret_cast<float*>(q) = val(im, row); });
         __syncwarp();
+        get(0, im);
     }
-    dft_reg<M, DIR, PACK, (R22 & 2) != 0>(v);  // v[brev(k2)] = X_r[j + M k2]
+    __syncwarp();
+    dft_pk<M, DIR>(re, im);
 }
 
-template <int M, int R, int DIR, bool PACK = true, bool ONCE = false, bool WIDE = false, int R22 = 0,
-          typename T, typename Load>
+template <int M, int DIR, bool WIDE = false, typename T>
+__device__ __forceinline__ void team_fft_core(cpx<T> (&v)[M], int j, void* sm, const cpx<T>* __restrict__ twq) {
+    if constexpr (sizeof(T) == 4 && M >= 8) {
+        constexpr int H = M / 2;
+        float2 re[H], im[H];
+#pragma unroll
+        for (int m = 0; m < H; ++m) {
+            re[m] = make_float2(v[2 * m].x, v[2 * m + 1].x);
+            im[m] = make_float2(v[2 * m].y, v[2 * m + 1].y);
+        }
+        team_core_pk<M, DIR, WIDE>(re, im, j, reinterpret_cast<float*>(sm), reinterpret_cast<const float4*>(twq));
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+            v[brev(k, M)] = {re[k].x, im[k].x};
+            v[brev(k + H, M)] = {re[k].y, im[k].y};
+        }
+    } else {
+        dft_reg<M, DIR>(v);  // v[brev(k1)] = A[j][k1]
+#pragma unroll
+        for (int k1 = 1; k1 < M; ++k1) v[brev(k1, M)] = cmul(v[brev(k1, M)], twl<DIR>(twq, k1 * M + j));
+        if constexpr (sizeof(T) == 4) {
+            float* sf = reinterpret_cast<float*>(sm);
+            __syncwarp();
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) sf[k1 * M + (j ^ k1)] = v[brev(k1, M)].x;
+            __syncwarp();
+#pragma unroll
+            for (int n2 = 0; n2 < M; ++n2) v[n2].x = sf[j * M + (n2 ^ j)];
+            __syncwarp();
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) sf[k1 * M + (j ^ k1)] = v[brev(k1, M)].y;
+            __syncwarp();
+#pragma unroll
+            for (int n2 = 0; n2 < M; ++n2) v[n2].y = sf[j * M + (n2 ^ j)];
+            __syncwarp();
+        } else {
+            cpx<T>* sc = reinterpret_cast<cpx<T>*>(sm);
+            __syncwarp();
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) sc[k1 * M + (j ^ k1)] = v[brev(k1, M)];
+            __syncwarp();
+#pragma unroll
+            for (int n2 = 0; n2 < M; ++n2) v[n2] = sc[j * M + (n2 ^ j)];
+            __syncwarp();
+        }
+        dft_reg<M, DIR>(v);  // v[brev(k2)] = X_r[j + M k2]
+    }
+}
+
+template <int M, int R, int DIR, typename T, typename Load>
 __device__ __forceinline__ void team_fft(cpx<T> (&v)[M], int r, int j, Load&& load, void* sm,
                                          const cpx<T>* __restrict__ twq, const cpx<T>* __restrict__ twn) {
-    // WIDE: the groups' scratch are M*M complex each (one-pass complex transposes);
-    // sm is then this group's slice at r * M*M complex from the team's base
-    // ONCE (R = 2, teams of one warp): the radix-2 step loads every input once and
-    // passes the groups' halves through the team's buffer (2 M^2 complex values in
-    // front of the groups' scratch), instead of each group loading all inputs.
     constexpr int NQ = M * M;
-    if constexpr (ONCE) {
-        static_assert(R == 2 && R * M == 32, "load-once radix-2 step: one-warp teams");
-        constexpr int H2 = M / 2;
-        constexpr int GS = WIDE ? M * M * (int)sizeof(cpx<T>) : grp_scratch_bytes<T, M>();
-        cpx<T>* xs = reinterpret_cast<cpx<T>*>(reinterpret_cast<char*>(sm) - r * GS);
-        __syncwarp();  // earlier users of the team's scratch are done
-#pragma unroll
-        for (int t = 0; t < H2; ++t) {
-            const int m = j + M * (r * H2 + t);  // the lanes of both groups cover m < NQ once
-            const cpx<T> x0 = load(m), x1 = load(m + NQ);
-            xs[m] = x0 + x1;
-            xs[NQ + m] = cmul(x0 - x1, twl<DIR>(twn, m));
-        }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < M; ++i) v[i] = xs[r * NQ + j + M * i];
-        __syncwarp();  // the groups' transposes below reuse this buffer
-    } else if constexpr (R > 2 && !is_pow2(R)) {
+    if constexpr (R > 2 && !is_pow2(R)) {
         // Radix-R decimation in frequency (R = 3, 6) with every input loaded once: the
         // team's lanes l = r M + j take the points m = l + TEAM t, form the R-point DFT
         // of x[m + s NQ], s < R, twiddle frequency q by w_N^{m q} and hand it to group q
@@ -433,7 +414,7 @@ __device__ __forceinline__ void team_fft(cpx<T> (&v)[M], int r, int j, Load&& lo
             cpx<T> u[R];
 #pragma unroll
             for (int s2 = 0; s2 < R; ++s2) u[s2] = load(m + s2 * NQ);
-            dft_reg<R, DIR, PACK>(u);  // u[brev(q)] = sum_s x[m + s NQ] w_R^{s q}
+            dft_reg<R, DIR>(u);  // u[brev(q)] = sum_s x[m + s NQ] w_R^{s q}
 #pragma unroll
             for (int q = 0; q < R; ++q) {
                 const cpx<T> y = u[brev(q, R)];
@@ -458,7 +439,7 @@ __device__ __forceinline__ void team_fft(cpx<T> (&v)[M], int r, int j, Load&& lo
             }
         }
     }
-    team_fft_core<M, DIR, PACK, WIDE, R22>(v, j, sm, twq);
+    team_fft_core<M, DIR>(v, j, sm, twq);
 }
 
 }  // namespace cmif

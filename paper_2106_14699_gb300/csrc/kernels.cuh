@@ -5,9 +5,10 @@
 //                half spectra of both planes.  Also checks labels in range.
 //   fwd_cols   : column FFT of length P -> 2-D half spectra F[plane][kx][ky].
 //   pair_cols  : for every label pair (a, b): conj(F[L_a A]) * F[L_b B] (the
-//                correlation theorem for Eq. cc), inverse column FFT -> Y.
-//   pair_rows  : inverse row FFT (complex-to-real, length Q) of every pair's
-//                Y row, rounded to integer joint counts C_AB^{a,b}(chi)
+//                correlation theorem for Eq. cc), inverse column FFT, and the
+//                Hermitian step of the complex-to-real row transform -> Y.
+//   pair_rows  : inverse row FFT (complex, length Q/2, giving Q reals) of every
+//                pair's Y row, rounded to integer joint counts C_AB^{a,b}(chi)
 //                (Eq. correlationjointhisto; rounding per Sec. 3.2), fused
 //                with the per-shift entropy reduction: the marginals
 //                C_A^a = sum_b C_AB^{a,b}, C_B^b = sum_a C_AB^{a,b} and
@@ -32,20 +33,39 @@ namespace cmif {
 // MUFU lg2 approximation; the rounding to the 2^-F grid adds at most 2^-(F+1).
 // The largest |L(c) 2^-F - log2 c| over every count the epilogue can meet is
 // measured exhaustively through cmif_entropy_terms (include/cmif.h).
-__device__ __forceinline__ long long clog2c_fixed(float c) {
+//
+// The sums take c * (L(c) + kTermBias): the bias drops out of every result, because
+// each of the joint, A- and B-marginal counts of a shift sums to N (so MI and NMI
+// combine the four sums with the biases N - N - N + N = 0), and leaving it in saves an
+// add per count.  c = 0 gives 0 whatever L is (Sec. 3.2: 0 log 0 = 0).  The term is one
+// fixed function of c, so equal counts cancel exactly between joint and marginal sums.
+constexpr int kTermBias = 0x4B000000;
+// log2 of a mantissa in [1, 2): no denormals, so the flush-to-zero form (the default one
+// carries a rescaling of denormal inputs, three more instructions per count)
+__device__ __forceinline__ float lg2_mantissa(float m) {
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(m));
+    return r;
+}
+__device__ __forceinline__ long long clog2c_biased(float c) {
     const int ci = __float_as_int(c + 8388608.0f) - 0x4B000000;
-    const int bits = __float_as_int(c);
-    const float lm = __log2f(__int_as_float((bits & 0x7FFFFF) | 0x3F800000));
+    const int bits = __float_as_int(c), mb = (bits & 0x7FFFFF) | 0x3F800000;
     // 2^23 + log2(m) 2^23 lies in [2^23, 2^24], where floats are spaced 1 apart and
     // their bit patterns grow by 1 per unit: the FMA rounds log2(m) 2^23 to the
-    // nearest integer and the bits give it back (no float-to-integer conversion).
-    // bits & 0x7F800000 = (e + 127) 2^23.  c = 0: ci = 0, so the term is 0 (Sec. 3.2:
-    // 0 log 0 = 0) whatever L is.  c = 1: m = 1 and e = 0, so L = 0.  T stays one
-    // fixed function of c, so equal counts still cancel exactly between joint and
-    // marginal sums.
-    const int t = __float_as_int(fmaf(lm, 8388608.0f, 8388608.0f));
-    const int L = ((bits & 0x7F800000) - 0x3F800000) + (t - 0x4B000000);  // e 2^23 + round(log2(m) 2^23)
-    return (long long)ci * (long long)L;
+    // nearest integer and the bits hold it above 0x4B000000 (= kTermBias; no
+    // float-to-integer conversion).  bits - mb = e 2^23.
+    const int t = __float_as_int(fmaf(lg2_mantissa(__int_as_float(mb)), 8388608.0f, 8388608.0f));
+    return (long long)ci * (long long)(bits - mb + t);
+}
+// Two counts at once: the float adds and the FMA as two-lane instructions.
+__device__ __forceinline__ void clog2c_biased2(float2 c, long long& t0, long long& t1) {
+    const float2 b = __fadd2_rn(c, make_float2(8388608.0f, 8388608.0f));
+    const int x0 = __float_as_int(c.x), x1 = __float_as_int(c.y);
+    const int m0 = (x0 & 0x7FFFFF) | 0x3F800000, m1 = (x1 & 0x7FFFFF) | 0x3F800000;
+    const float2 l = make_float2(lg2_mantissa(__int_as_float(m0)), lg2_mantissa(__int_as_float(m1)));
+    const float2 t = __ffma2_rn(l, make_float2(8388608.0f, 8388608.0f), make_float2(8388608.0f, 8388608.0f));
+    t0 = (long long)(__float_as_int(b.x) - 0x4B000000) * (long long)(x0 - m0 + __float_as_int(t.x));
+    t1 = (long long)(__float_as_int(b.y) - 0x4B000000) * (long long)(x1 - m1 + __float_as_int(t.y));
 }
 
 // Nearest integer of |v| < 2^22 with two FP32 adds (the 1.5 * 2^23 shift
@@ -53,11 +73,11 @@ __device__ __forceinline__ long long clog2c_fixed(float c) {
 __device__ __forceinline__ float round_fp32(float v) { return (v + 12582912.0f) - 12582912.0f; }
 
 // MI(chi) = (S + N log2 N) / N, where S = sum_joint c log2 c - sum_A - sum_B and
-// every c log2 c term (N log2 N included) comes from clog2c_fixed, so that MI is
+// every c log2 c term (N log2 N included) comes from clog2c_biased, so that MI is
 // exactly 0 whenever the entropies cancel exactly (e.g. a single label).
 __device__ __forceinline__ double mi_finish(long long S, int N) {
     if (N <= 0) return 0.0;  // 0/0 = 0: no overlap, no information (Sec. 3.2)
-    const long long Sp = S + clog2c_fixed((float)N);
+    const long long Sp = S + clog2c_biased((float)N);
     const float sh = (float)Sp;
     const long long rem = Sp - (long long)sh;
     const float sl = (float)rem;
@@ -75,7 +95,7 @@ __device__ __forceinline__ double mi_finish(long long S, int N) {
 // H_AB = (T(N) - SJ) / N.  0 when N = 0 or H_AB = 0 (0/0 = 0, Sec. 3.2).
 __device__ __forceinline__ double nmi_finish(long long SJ, long long SM, int N) {
     if (N <= 0) return 0.0;
-    const long long TN = clog2c_fixed((float)N);
+    const long long TN = clog2c_biased((float)N);
     const long long den = TN - SJ;
     if (den == 0) return 0.0;
     return (double)(2 * TN - SM) / (double)den;
@@ -272,6 +292,16 @@ struct ColCfg {
     static constexpr size_t smem(int H) { return SCR + (size_t)H * TPB * sizeof(cpx<T>); }
 };
 
+// FP32 groups of 8 lanes and more keep the spectra in the order the packed DFTs take them:
+// samples i = 4q .. 4q + 3 of lane j as 8 floats (re, re', im, im' of 4q, 4q + 1, then of
+// 4q + 2, 4q + 3) at complex offset (q M + j) 4 of the group.
+template <typename T, int M>
+__host__ __device__ constexpr bool packed_spectra() { return sizeof(T) == 4 && M >= 8; }
+__device__ __forceinline__ void st_global_32B(void* dst, const float (&v)[8]) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+}
+
 template <typename T, int P, int MMAX>
 __global__ void __launch_bounds__(ColCfg<T, P, MMAX>::THREADS, sizeof(T) == 4 && ColCfg<T, P, MMAX>::THREADS <= 256 ? 3 : 1)
 k_fwd_cols(const cpx<T>* __restrict__ T1, int H, int nplanes, int Qh, int Qs, cpx<T>* __restrict__ F, Tw<T> tw,
@@ -319,11 +349,25 @@ k_fwd_cols(const cpx<T>* __restrict__ T1, int H, int nplanes, int Qh, int Qs, cp
     if (!active) return;
     // Column ky is stored at slot (ky % R) * M*M + ky / R: the samples that one
     // group of the pair-product transform (same P, same R) takes are contiguous.
-    cpx<T>* out = F + ((size_t)plane * Qh + kx) * P;
+    cpx<T>* out = F + ((size_t)plane * Qh + kx) * P + r * (M * M);
+    if constexpr (packed_spectra<T, M>()) {
 #pragma unroll
-    for (int k2 = 0; k2 < M; ++k2) {
-        const cpx<T> z = v[brev(k2, M)];
-        out[r * (M * M) + j + M * k2] = {z.x * out_scale, z.y * out_scale};
+        for (int q = 0; q < M / 4; ++q) {
+            float w[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const cpx<T> z = v[brev(4 * q + i, M)];
+                w[4 * (i / 2) + i % 2] = z.x * out_scale;
+                w[4 * (i / 2) + 2 + i % 2] = z.y * out_scale;
+            }
+            st_global_32B(out + 4 * (M * q + j), w);
+        }
+    } else {
+#pragma unroll
+        for (int k2 = 0; k2 < M; ++k2) {
+            const cpx<T> z = v[brev(k2, M)];
+            out[j + M * k2] = {z.x * out_scale, z.y * out_scale};
+        }
     }
 }
 
@@ -349,30 +393,139 @@ __device__ __forceinline__ void stage_table(cpx<T>* dst, const cpx<T>* __restric
 }
 
 // ---------------------------------------------------------------------------
+// Layout of Y.  A row of Y holds the L = Q/2 inputs z_k of the complex row transform,
+// z[m] = x[2m] + i x[2m + 1] = IDFT_L(z_k):
+//     z_k = E + i O,  E = y_k + conj(y_{L-k}),  O = (y_k - conj(y_{L-k})) e^{2 pi i k / Q}
+// (y_k: the column-inverted product at frequency kx = k <= L).  z_k and z_{L-k} need the
+// same two columns, so the pair-column kernel, which has them side by side, forms both: the
+// row kernels would each load two values and a twiddle per input.  y_0 and y_L are
+// real, so one column transform yields both: column 0 carries y_0 + i y_L.
+// Columns are kept in 32-byte chunks (whole sectors) that one block writes:
+//   FP32, L / 4 chunks of 4: k0, k1 and the mirrors of k1, k0 (L - k; of 0: L / 2), as
+//     two 16-byte halves (direct, mirrored), swapped in every other group of 4 chunks
+//     so that the row kernels' reads of consecutive k meet no bank conflicts;
+//       Q = 512, 1024, 2048 (Tensor-Memory row kernel): k1 = k0 + 32 with real and
+//       imaginary parts grouped, (re, re', im, im'), in the order of the packed
+//       row transform's even and odd inputs;
+//       other Q: k0 = 2c, k1 = 2c + 1 as complex values.
+//     Four rows' chunks c form a 128-byte line, lines of one row group in the order of c
+//     (Y[pair][row / 4][c][row % 4]): the pair-column kernel's lanes, which hold consecutive
+//     rows, write whole lines (8 shared-pipe wavefronts per 32 lanes instead of 32), and the
+//     row kernels gather a row's chunks (TMA, or 16-byte asynchronous copies).
+//   FP64, two-term FP32, L / 2 chunks of 2: z_c, z_{L-c}; rows contiguous.
+template <typename T>
+constexpr int kChunk = sizeof(T) == 4 ? 4 : 2;
+__host__ __device__ constexpr bool split32_rows(int Q) { return Q == 512 || Q == 1024 || Q == 2048; }
+// Rows of one pair in Y, and the element offset of chunk c of a row.
+template <typename T>
+__host__ __device__ constexpr int y_rows(int Rout) { return sizeof(T) == 4 ? (Rout + 3) / 4 * 4 : Rout; }
+template <typename T>
+__device__ __forceinline__ size_t y_chunk(int row, int c, int L) {
+    if constexpr (sizeof(T) == 4) return (size_t)(row >> 2) * (4 * L) + c * 16 + (row & 3) * 4;
+    else return (size_t)row * L + c * 2;
+}
+__device__ __forceinline__ bool halves_swapped(int c) { return (c >> 2) & 1; }
+
+// First direct column of chunk c (the second is k0 + 32 in split rows, else k0 + 1).
+template <typename T>
+__device__ __forceinline__ int chunk_k0(int c, bool split) {
+    if constexpr (sizeof(T) == 4) return split ? (c >> 5) * 64 + (c & 31) : 2 * c;
+    else return c;
+}
+__device__ __forceinline__ int mirror_k(int k, int L) { return k ? L - k : L / 2; }
+// Column (frequency kx) that slot i of chunk c transforms: the chunk's order in memory.
+template <typename T>
+__device__ __forceinline__ int chunk_col(int c, int i, int L, bool split) {
+    if constexpr (sizeof(T) == 4) {
+        const int m = halves_swapped(c) ? i ^ 2 : i;
+        const int k = chunk_k0<T>(c, split) + (m == 1 || m == 2 ? (split ? 32 : 1) : 0);
+        return m < 2 ? k : mirror_k(k, L);
+    } else {
+        return i ? mirror_k(c, L) : c;
+    }
+}
+// z_k of a row whose chunks lie back to back.
+template <typename T, int Q>
+__device__ __forceinline__ cpx<T> load_z(const cpx<T>* row, int k) {
+    constexpr int L = Q / 2;
+    const bool mir = k >= L / 2;
+    const int kk = k == L / 2 ? 0 : (mir ? L - k : k);  // the direct partner
+    if constexpr (sizeof(T) != 4) {
+        return row[2 * kk + (mir ? 1 : 0)];
+    } else {
+        constexpr bool split = split32_rows(Q);
+        const int c = split ? (kk >> 6) * 32 + (kk & 31) : kk >> 1, second = split ? (kk >> 5) & 1 : kk & 1;
+        const int half = (mir ? 1 : 0) ^ (halves_swapped(c) ? 1 : 0), e = mir ? 1 - second : second;
+        if constexpr (split) {
+            const float* f = reinterpret_cast<const float*>(row) + c * 8 + half * 4 + e;
+            return {f[0], f[2]};
+        } else {
+            return row[c * 4 + half * 2 + e];
+        }
+    }
+}
+// 32-byte global load (sm_100+), past L1: the spectra are shared through L2
+__device__ __forceinline__ void ld_global_32B(const float* src, float (&v)[8]) {
+    asm("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(src));
+}
+// Store one chunk in memory order; SPLIT groups real and imaginary parts.
+template <bool SPLIT>
+__device__ __forceinline__ void store_chunk(cpx<float>* dst, const cpx<float> (&z)[4]) {
+    float v[8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        v[4 * h] = z[2 * h].x;
+        v[4 * h + (SPLIT ? 2 : 1)] = z[2 * h].y;
+        v[4 * h + (SPLIT ? 1 : 2)] = z[2 * h + 1].x;
+        v[4 * h + 3] = z[2 * h + 1].y;
+    }
+    st_global_32B(dst, v);
+}
+template <bool SPLIT, typename T>
+__device__ __forceinline__ void store_chunk(cpx<T>* dst, const cpx<T> (&z)[2]) {
+    dst[0] = z[0];
+    dst[1] = z[1];
+}
+// The Hermitian step: z_k and z_{L-k} from y_k, y_{L-k}; t = e^{-2 pi i k / Q} (table),
+// i O = (y_k - conj(y_{L-k})) i conj(t) = d (t.y, t.x), z_{L-k} = conj(E - i O).  Holds for
+// every k, so a chunk with swapped halves only takes the mirror's twiddle.
+__device__ __forceinline__ void hermitian_step(cpx<float> yk, cpx<float> ym, cpx<float> t, cpx<float>& zk, cpx<float>& zm) {
+    const float2 k2 = make_float2(yk.x, yk.y), m2 = make_float2(ym.x, ym.y);
+    const float2 e = __ffma2_rn(m2, make_float2(1.f, -1.f), k2), d = __ffma2_rn(m2, make_float2(-1.f, 1.f), k2);
+    const cpx<float> io = cmul(cpx<float>{d.x, d.y}, cpx<float>{t.y, t.x});
+    zk = {e.x + io.x, e.y + io.y};
+    zm = {e.x - io.x, io.y - e.y};
+}
+template <typename T>
+__device__ __forceinline__ void hermitian_step(cpx<T> yk, cpx<T> ym, cpx<T> t, cpx<T>& zk, cpx<T>& zm) {
+    const cpx<T> e = {yk.x + ym.x, yk.y - ym.y}, d = {yk.x - ym.x, yk.y + ym.y};
+    const cpx<T> io = cmul(d, cpx<T>{t.y, t.x});
+    zk = {e.x + io.x, e.y + io.y};
+    zm = {e.x - io.x, io.y - e.y};
+}
+
+// ---------------------------------------------------------------------------
 // Configuration of the pair-product + inverse column kernel (k_pair_cols below):
 // TPB columns per block, one team of R x M lanes per column; the block's shared
-// memory holds one buffer (the teams' exchange, then the P x TPB output tile,
-// with the transpose scratch aliased on it) and the twiddle tables.
+// memory holds the teams' P sub-transform values each (a group's slice first serves
+// as its transpose scratch) and the twiddle tables.
 template <typename T, int P, int MMAX = max_m<T>()>
 struct PairColsCfg {
     using G = TeamGeom<T, P, MMAX>;
     static constexpr int M = G::M, R = G::R, TEAM = G::TEAM, NQ = M * M;
-    // at least 256 threads, and at least 32 bytes of adjacent kx per tile row (whole sectors)
-    static constexpr int TPB0 = TEAM >= 256 ? 1 : pow2_floor(256 / TEAM);  // a power of two (swizzle)
-    static constexpr int TPB = TPB0 * (int)sizeof(cpx<T>) >= 32 ? TPB0 : 32 / (int)sizeof(cpx<T>);
+    // at least 256 threads, and at least one whole chunk of Y columns
+    static constexpr int TPB0 = TEAM >= 256 ? 1 : pow2_floor(256 / TEAM);
+    static constexpr int TPB = TPB0 >= kChunk<T> ? TPB0 : kChunk<T>;
     static constexpr int THREADS = TPB * TEAM;
-    static constexpr int PER = R > 2 ? M / R : 1;  // points per lane of the radix-R combine (R a power of two)
-    static constexpr int PTS = (NQ + TEAM - 1) / TEAM;  // points per lane of the radix-3/6 combine
-    static constexpr int SWZ = TPB >= 16 ? 0 : (TPB == 8 ? 1 : (TPB == 4 ? 2 : 3));
-    // one buffer per block: the teams' group-transform exchange, then the P x TPB output tile
-    static constexpr size_t XBUF = (size_t)TPB * P * sizeof(cpx<T>);
-    static constexpr size_t FFT = (size_t)TPB * G::SCRATCH;
-    static constexpr size_t MAIN = (XBUF > FFT ? XBUF : FFT);
-    static constexpr size_t FFT_WIDE = (size_t)TPB * R * M * M * sizeof(cpx<T>);  // complex transposes
+    static constexpr int UPR = TPB / kChunk<T>;  // chunks per block and row
+    static constexpr size_t MAIN = (size_t)TPB * P * sizeof(cpx<T>);
     static constexpr int TW_N = R == 2 ? P / 2 : (R > 2 ? P : 0);  // combine twiddles W_P^k
     static constexpr size_t SMEM = MAIN + (size_t)(NQ + TW_N) * sizeof(cpx<T>);
-    // FP32: two blocks per SM (M = 32 needs 128 registers a thread, so 256 threads)
-    static constexpr int MIN_BLOCKS = sizeof(T) == 4 && (M < 32 ? is_pow2(R) && THREADS <= 512 : THREADS <= 256) ? 2 : 1;
+    // FP32: two blocks per SM (M = 32 needs 128 registers a thread, so 256 threads);
+    // radix 6 and 8 combines hold too many values for that
+    static constexpr int MIN_BLOCKS = sizeof(T) == 4 && (M < 32 ? R < 6 && is_pow2(R) && THREADS <= 512 : THREADS <= 256) ? 2 : 1;
 };
 
 // Pair product + inverse column transform of length P = R*M*M.  Persistent
@@ -380,15 +533,17 @@ struct PairColsCfg {
 // the items in flight at one time read the same few spectrum columns (L2
 // reuse).  Decimation in time across the R groups of a team: group r
 // transforms the M*M samples ky = R*m + r (every input is loaded and
-// multiplied once per team), the groups exchange their sub-transforms through
-// shared memory, and group r forms the outputs [r*M*M, (r+1)*M*M) by the
-// radix-R butterfly (FP32 groups of 16 or 32 lanes transpose complex values in
-// one pass through their M*M slice of the same buffer).  The exchange buffer then serves as a P x TPB tile
-// (column slots XOR-swizzled by row, conflict-free writes) whose rows leave
-// as chunks of TPB adjacent kx.  While the tile leaves, the F_a loads of the
-// block's next item are already in flight, and items at the head of a kx
-// block ask L2 for the spectrum columns two kx blocks ahead.  work_ctr must
-// be zero at launch.
+// multiplied once per team) and leaves its sub-transform in its own slice of the
+// block's buffer (which was its transpose scratch, so nothing but warp syncs comes
+// before).  After one barrier every thread takes a row residue k of a chunk's columns: it
+// joins the R groups' values by the radix-R butterfly, forms the row transform's
+// inputs from the columns and their mirrors (the layout of Y above) and stores R rows'
+// 32-byte chunks.  An item thus passes shared memory twice (transpose, combine) and takes two
+// block barriers.  While the rows leave, the F_a loads of the block's next item are
+// already in flight, and
+// items at the head of a kx block ask L2 for the spectrum columns two kx blocks ahead.
+// FP32 groups of 8 lanes and more: spectra in the order of the packed DFTs, 32 bytes per
+// load (fwd_cols).  work_ctr must be zero at launch.
 // VOL (volumes): items are (pair, depth offset dz, kx block); the product is
 // the sum over the slices z of conj(F_a,z) F_b,z+dz (the 3-D correlation's
 // depth sum, taken before the inverse transform, which is linear), and the
@@ -396,17 +551,20 @@ struct PairColsCfg {
 template <typename T, int P, bool VOL, int MMAX>
 __global__ void __launch_bounds__(PairColsCfg<T, P, MMAX>::THREADS, PairColsCfg<T, P, MMAX>::MIN_BLOCKS)
 k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA, int KB, int Qh, int HA, int HB,
-            int Rout, int Qs, int r0, int r1, cpx<T>* __restrict__ Y, Tw<T> tw, const DevStatus* __restrict__ st,
-            int conditional, int* __restrict__ work_ctr, int DA, int DB, int R2, const int* __restrict__ plist,
-            const int* __restrict__ lrange, int chunk_off, int chunk_cap, int units) {
+            int Rout, int r0, int r1, cpx<T>* __restrict__ Y, Tw<T> tw, const cpx<T>* __restrict__ twq,
+            const DevStatus* __restrict__ st, int conditional, int* __restrict__ work_ctr, int DA, int DB, int R2,
+            const int* __restrict__ plist, const int* __restrict__ lrange, int chunk_off, int chunk_cap, int units) {
+    // twq: the table of e^{-2 pi i k / Q}, Q = 2 (Qh - 1).
     // units > 1 (images only): several floating images (rotation angles) at once;
     // unit u's spectra are F_b plane b * units + u, its output rows u * R2 + (row).
     // List mode (plist non-null): only the pairs plist[lrange[0] + chunk_off + e],
     // e < min(chunk_cap, lrange[1] - lrange[0] - chunk_off), are computed, pair e's
-    // rows going to Y + e * Rout * Qs.
+    // rows going to pair slot e of Y.
     using C = PairColsCfg<T, P, MMAX>;
     if (conditional && !(st->flags & STATUS_ESCALATE)) return;
-    constexpr int M = C::M, R = C::R, TPB = C::TPB, NQ = C::NQ;
+    constexpr int M = C::M, R = C::R, TPB = C::TPB, NQ = C::NQ, CH = kChunk<T>, UPR = C::UPR;
+    const int L = Qh - 1;
+    const bool split = sizeof(T) == 4 && split32_rows(2 * L);
     const int Dz = VOL ? DA + DB - 1 : 1;
     int npairs = KA * KB, lbase = 0;
     if (plist) {
@@ -416,247 +574,236 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
     }
     auto real_pair = [&](int e) { return plist ? ::__ldg(plist + lbase + e) : e; };
     const int U = VOL ? Dz : units;  // the middle item dimension: depth offsets or units
-    const int nkxb = (Qh + TPB - 1) / TPB, n_items = npairs * nkxb * U;
+    const int nkxb = (L + TPB - 1) / TPB, n_items = npairs * nkxb * U;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ int s_item;
+    __shared__ int s_next[6];  // the next item: whether there is one, e, a, b, kx block, unit / depth offset
     cpx<T>* xbuf = reinterpret_cast<cpx<T>*>(smem_raw);
     cpx<T>* tw_sq = reinterpret_cast<cpx<T>*>(smem_raw + C::MAIN);
     cpx<T>* tw_n = tw_sq + NQ;
     // Items are handed out in order from a counter (zeroed before the launch), so
     // that the items in flight stay within a few kx blocks whatever the blocks' pace.
-    if (threadIdx.x == 0) s_item = atomicAdd(work_ctr, 1);
+    // One thread decodes them (the divisions would cost every thread more than its share
+    // of the transform's loads).
+    // volumes: kx block outermost, then the depth offset (the slices' spectra of one
+    // kx block serve every depth offset); units: the unit outermost, so that the
+    // items in flight write the rows of few maps and complete their lines in L2
+    auto decode = [&](int it) {
+        s_next[0] = it < n_items;
+        if (it >= n_items) return;
+        const int e = it % npairs, rest = it / npairs, pair = real_pair(e), a = pair / KB;
+        s_next[1] = e;
+        s_next[2] = a;
+        s_next[3] = pair - a * KB;
+        s_next[4] = VOL ? rest / U : rest % nkxb;
+        s_next[5] = VOL ? rest % U : rest / nkxb;
+    };
+    if (threadIdx.x == 0) decode(atomicAdd(work_ctr, 1));
     stage_table(tw_sq, tw.sq[ilog2c(M)], NQ);
     if (R > 1) stage_table(tw_n, tw_of<P>(tw), C::TW_N);
     __syncthreads();
-    int item = s_item;
-    if (item >= n_items) return;
+    if (!s_next[0]) return;
+    int e = s_next[1], a = s_next[2], b = s_next[3], kxb = s_next[4], dzo = s_next[5];
     const int team = threadIdx.x / C::TEAM, lt = threadIdx.x % C::TEAM, r = lt / M, j = lt % M;
+    cpx<T>* slice = xbuf + (size_t)team * P + r * NQ;  // this group's transpose scratch, then its sub-transform
+    // the frequency kx this team transforms for kx block kxb, or -1 beyond the last
+    auto column = [&](int kxb, int t) {
+        const int s = kxb * TPB + t;
+        return s < L ? chunk_col<T>(s / CH, s % CH, L, split) : -1;
+    };
     // group r: the samples ky = R*m + r, m = j + M*i, stored contiguously from slot
     // r*NQ (the forward column transform's output order).  conj(F_a) F_b, F_b
     // carrying the 1/(P Q) of the inverse.
-    cpx<T> v[M];
-    cpx<T> wo[(R > 2 && !is_pow2(R)) ? C::PTS * R : 1];  // outputs of the radix-3/6 combine
-    auto load_fa = [&](int it) {
+    constexpr bool PK = packed_spectra<T, M>();
+    constexpr int H = PK ? M / 2 : 1, NV = PK ? M / 4 : 1;  // pairs, 32-byte loads
+    cpx<T> v[PK ? 1 : M];
+    float2 re[H], im[H];  // PK: the F_a values, then the products, in pairs
+    const size_t lane_off = PK ? (size_t)r * NQ + 4 * j : (size_t)r * NQ + j;
+    auto load_fa = [&]() {
         if constexpr (VOL) return;  // volumes sum over slices in the item itself
-        const int kx = (VOL ? it / npairs / U : (it / npairs) % nkxb) * TPB + team, a = real_pair(it % npairs) / KB;
-        if (kx < Qh) {
-            const cpx<T>* ga = FA + ((size_t)a * Qh + kx) * P + r * NQ + j;
+        const int kx = column(kxb, team);
+        const cpx<T>* ga = FA + ((size_t)a * Qh + (kx < 0 ? 0 : kx)) * P + lane_off;
+        if constexpr (PK) {
 #pragma unroll
-            for (int i = 0; i < M; ++i) v[i] = __ldg(ga + M * i);
+            for (int q = 0; q < NV; ++q) {
+                float w[8];
+                ld_global_32B(reinterpret_cast<const float*>(ga + 4 * M * q), w);
+                re[2 * q] = make_float2(w[0], w[1]);
+                im[2 * q] = make_float2(w[2], w[3]);
+                re[2 * q + 1] = make_float2(w[4], w[5]);
+                im[2 * q + 1] = make_float2(w[6], w[7]);
+            }
         } else {
 #pragma unroll
-            for (int i = 0; i < M; ++i) v[i] = {T(0), T(0)};
+            for (int i = 0; i < M; ++i) v[i] = __ldg(ga + M * i);
         }
     };
-    load_fa(item);
+    // conj(a) b of pairs
+    auto mulc2 = [](float2 ar, float2 ai, float2 br, float2 bi, float2& pr, float2& pi) {
+        pr = __ffma2_rn(ai, bi, __fmul2_rn(ar, br));
+        const float2 t = __fmul2_rn(ar, bi);
+        pi = make_float2(fmaf(-ai.x, br.x, t.x), fmaf(-ai.y, br.y, t.y));
+    };
+    // (re, im) += w conj(F_a) F_b of one column, w = 1 or (ROT) i
+    auto add_product = [&](auto rotc, const cpx<T>* ga, const cpx<T>* gb) {
+        constexpr bool ROT = decltype(rotc)::value;
+        if constexpr (PK) {
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                float x[8], y[8];
+                ld_global_32B(reinterpret_cast<const float*>(ga + 4 * M * q), x);
+                ld_global_32B(reinterpret_cast<const float*>(gb + 4 * M * q), y);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float2 pr, pi;
+                    mulc2(make_float2(x[4 * h], x[4 * h + 1]), make_float2(x[4 * h + 2], x[4 * h + 3]),
+                          make_float2(y[4 * h], y[4 * h + 1]), make_float2(y[4 * h + 2], y[4 * h + 3]), pr, pi);
+                    re[2 * q + h] = ROT ? subv(re[2 * q + h], pi) : addv(re[2 * q + h], pr);
+                    im[2 * q + h] = ROT ? addv(im[2 * q + h], pr) : addv(im[2 * q + h], pi);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                const cpx<T> q = cmulc(__ldg(gb + M * i), __ldg(ga + M * i));
+                v[i] = ROT ? cpx<T>{v[i].x - q.y, v[i].y + q.x} : v[i] + q;
+            }
+        }
+    };
+    load_fa();
     while (true) {
         int next = 0;
         if (threadIdx.x == 0) next = atomicAdd(work_ctr, 1);
-        const int e = item % npairs, pair = real_pair(e);
-        // volumes: kx block outermost, then the depth offset (the slices' spectra of one
-        // kx block serve every depth offset); units: the unit outermost, so that the
-        // items in flight write the rows of few maps and complete their lines in L2
-        const int kxb = VOL ? item / npairs / U : (item / npairs) % nkxb;
-        const int dzo = VOL ? (item / npairs) % U : item / npairs / nkxb;  // VOL: depth offset index; else the unit
-        const int kx0 = kxb * TPB, kx = kx0 + team, b = pair % KB;
-        if constexpr (VOL) {
+        const int kx = column(kxb, team), pair = a * KB + b;
+        if (VOL || kx < 0) {
+            if constexpr (PK) {
 #pragma unroll
-            for (int i = 0; i < M; ++i) v[i] = {T(0), T(0)};
-            if (kx < Qh) {
-                const int a = pair / KB, dz = dzo - (DA - 1);
+                for (int i = 0; i < H; ++i) re[i] = im[i] = make_float2(0.f, 0.f);
+            } else {
+#pragma unroll
+                for (int i = 0; i < M; ++i) v[i] = {T(0), T(0)};
+            }
+        }
+        if constexpr (VOL) {
+            if (kx >= 0) {
+                const int dz = dzo - (DA - 1);
                 const int z0 = dz < 0 ? -dz : 0, z1 = DA < DB - dz ? DA : DB - dz;
                 for (int z = z0; z < z1; ++z) {
-                    const cpx<T>* ga = FA + ((size_t)(a * DA + z) * Qh + kx) * P + r * NQ + j;
-                    const cpx<T>* gb = FB + ((size_t)(b * DB + z + dz) * Qh + kx) * P + r * NQ + j;
-#pragma unroll
-                    for (int i = 0; i < M; ++i) v[i] = v[i] + cmulc(__ldg(gb + M * i), __ldg(ga + M * i));
+                    const cpx<T>* ga = FA + ((size_t)(a * DA + z) * Qh + kx) * P + lane_off;
+                    const cpx<T>* gb = FB + ((size_t)(b * DB + z + dz) * Qh + kx) * P + lane_off;
+                    add_product(std::false_type{}, ga, gb);
+                    if (kx == 0) add_product(std::true_type{}, ga + (size_t)L * P, gb + (size_t)L * P);
                 }
             }
-        } else if (kx < Qh) {
-            const cpx<T>* gb = FB + ((size_t)(b * units + dzo) * Qh + kx) * P + r * NQ + j;
+        } else if (kx >= 0) {
+            const cpx<T>* gb = FB + ((size_t)(b * units + dzo) * Qh + kx) * P + lane_off;
+            if constexpr (PK) {
 #pragma unroll
-            for (int i = 0; i < M; ++i) v[i] = cmulc(__ldg(gb + M * i), v[i]);
+                for (int q = 0; q < NV; ++q) {
+                    float y[8];
+                    ld_global_32B(reinterpret_cast<const float*>(gb + 4 * M * q), y);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        mulc2(re[2 * q + h], im[2 * q + h], make_float2(y[4 * h], y[4 * h + 1]),
+                              make_float2(y[4 * h + 2], y[4 * h + 3]), re[2 * q + h], im[2 * q + h]);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < M; ++i) v[i] = cmulc(__ldg(gb + M * i), v[i]);
+            }
+            // column 0 carries y_0 + i y_L
+            if (kx == 0) add_product(std::true_type{}, FA + ((size_t)a * Qh + L) * P + lane_off, gb + (size_t)L * P);
         }
         if (!VOL && !plist && pair < KA + KB && (int)threadIdx.x < TPB && kxb + 2 < nkxb) {
             // the items of this kx block with pair < K_A + K_B each prefetch one
             // spectrum's columns of kx block kxb + 2 into L2 (one bulk request per column)
-            const int kf = (kxb + 2) * TPB + threadIdx.x;
-            if (kf < Qh) {
+            const int kf = column(kxb + 2, threadIdx.x);
+            if (kf >= 0) {
                 const cpx<T>* src = pair < KA ? FA + ((size_t)pair * Qh + kf) * P
                                               : FB + ((size_t)((pair - KA) * units + dzo) * Qh + kf) * P;
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((unsigned)(P * sizeof(cpx<T>)))
                              : "memory");
             }
         }
-        if constexpr (sizeof(T) == 4 && M >= 16 && C::FFT_WIDE <= C::MAIN)  // scratch of M*M complex per group
-            // radix-2^2 register DFTs at R = 1 (at R = 2 both made the kernel spill, the
-            // second alone measured no faster)
-            team_fft_core<M, +1, true, true, R == 1 ? 3 : 0>(v, j, smem_raw + (size_t)(team * R + r) * (M * M * sizeof(cpx<T>)), tw_sq);
-        else
-            team_fft_core<M, +1>(v, j, smem_raw + (size_t)team * C::G::SCRATCH + r * grp_scratch_bytes<T, M>(), tw_sq);
-        if (threadIdx.x == 0) s_item = next;  // read by all after the tile barrier below
-        cpx<T>* tx = xbuf + (size_t)team * P;  // this team's R sub-transforms
-        if constexpr (R == 2) {
-            // X[k] = E_0[k] + W^k E_1[k], X[k + NQ] = E_0[k] - W^k E_1[k] (W = W_P, inverse
-            // direction, W^NQ = -1).  Lane j of both groups holds the same k = j + M k2:
-            // group 1 forms W^k E_1[k] once, the groups swap values through shared memory.
-            __syncthreads();  // every group is done with its transpose scratch (aliases xbuf)
-            if (r == 1) {
+        if constexpr (PK) {
+            team_core_pk<M, +1, true>(re, im, j, reinterpret_cast<float*>(slice), reinterpret_cast<const float4*>(tw_sq));
 #pragma unroll
-                for (int k2 = 0; k2 < M; ++k2)
-                    v[brev(k2, M)] = cmul(v[brev(k2, M)], twl<+1>(tw_n, j + M * k2));
-            }
-#pragma unroll
-            for (int k2 = 0; k2 < M; ++k2) tx[r * NQ + j + M * k2] = v[brev(k2, M)];
-            __syncthreads();
-#pragma unroll
-            for (int k2 = 0; k2 < M; ++k2) {
-                const int k = j + M * k2;
-                v[brev(k2, M)] = r == 0 ? v[brev(k2, M)] + tx[NQ + k] : tx[k] - v[brev(k2, M)];
-            }
-        } else if constexpr (R > 2 && !is_pow2(R)) {
-            // R = 3, 6: as below, with the team's lanes l = r M + j taking the points
-            // k = l + TEAM t (the outputs stay in wo[] until the exchange reads are done)
-            __syncthreads();  // every group is done with its transpose scratch (aliases xbuf)
-#pragma unroll
-            for (int k2 = 0; k2 < M; ++k2) {
-                const int k = j + M * k2;
-                const cpx<T> e = v[brev(k2, M)];
-                tx[r * NQ + k] = r ? cmul(e, twl<+1>(tw_n, r * k)) : e;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int t = 0; t < C::PTS; ++t) {
-                const int k = lt + C::TEAM * t;
-                if (C::PTS * C::TEAM == NQ || k < NQ) {
-                    cpx<T> u[R];
-#pragma unroll
-                    for (int s2 = 0; s2 < R; ++s2) u[s2] = tx[s2 * NQ + k];
-                    dft_nat<R, +1>(u);
-#pragma unroll
-                    for (int q = 0; q < R; ++q) wo[t * R + q] = u[q];
-                }
-            }
-        } else if constexpr (R > 2) {
-            // X[k + q NQ] = sum_s w_R^{sq} (W^{sk} E_s[k]) (W = W_P, inverse direction): group
-            // s twiddles its own values, the team exchanges them through shared memory, and
-            // lane (r, j) forms all R outputs of the points k = j + M (r PER + t), t < PER,
-            // with an R-point DFT in registers (outputs kept as v[t R + q]).
-            __syncthreads();  // every group is done with its transpose scratch (aliases xbuf)
-#pragma unroll
-            for (int k2 = 0; k2 < M; ++k2) {
-                const int k = j + M * k2;
-                const cpx<T> e = v[brev(k2, M)];
-                tx[r * NQ + k] = r ? cmul(e, twl<+1>(tw_n, r * k)) : e;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int t = 0; t < C::PER; ++t) {
-                const int k = j + M * (r * C::PER + t);
-                cpx<T> u[R];
-#pragma unroll
-                for (int s2 = 0; s2 < R; ++s2) u[s2] = tx[s2 * NQ + k];
-                dft_reg<R, +1>(u);
-#pragma unroll
-                for (int q = 0; q < R; ++q) v[t * R + q] = u[brev(q, R)];
-            }
-        }
-        __syncthreads();  // exchange reads done: the buffer becomes the tile
-        // tile slot (row, team) swizzled by row
-        if constexpr (R > 2 && !is_pow2(R)) {
-#pragma unroll
-            for (int t = 0; t < C::PTS; ++t) {
-                const int k = lt + C::TEAM * t;
-                if (C::PTS * C::TEAM == NQ || k < NQ) {
-#pragma unroll
-                    for (int q = 0; q < R; ++q) {
-                        const int row = k + q * NQ;
-                        xbuf[(size_t)row * TPB + (team ^ ((row >> C::SWZ) & (TPB - 1)))] = wo[t * R + q];
-                    }
-                }
+            for (int k = 0; k < H; ++k) {
+                slice[j + M * k] = {re[k].x, im[k].x};
+                slice[j + M * (k + H)] = {re[k].y, im[k].y};
             }
         } else {
+            team_fft_core<M, +1>(v, j, slice, tw_sq);
 #pragma unroll
-            for (int i = 0; i < M; ++i) {
-                int row;
-                cpx<T> val;
-                if constexpr (R > 2) {
-                    row = j + M * (r * C::PER + i / R) + (i % R) * NQ;
-                    val = v[i];
-                } else {
-                    row = r * NQ + j + M * i;
-                    val = v[brev(i, M)];
-                }
-                xbuf[(size_t)row * TPB + (team ^ ((row >> C::SWZ) & (TPB - 1)))] = val;
-            }
+            for (int k2 = 0; k2 < M; ++k2) slice[j + M * k2] = v[brev(k2, M)];
         }
+        // Rows below: this item's; then its successor's fields
+        cpx<T>* yp = Y + (size_t)e * y_rows<T>(Rout) * L;
+        const int c0 = kxb * UPR, row_off = dzo * R2;
+        if (threadIdx.x == 0) decode(next);
         __syncthreads();
-        next = s_item;
-        if (next < n_items) load_fa(next);
-        cpx<T>* yp = Y + (size_t)e * Rout * Qs;
-        if constexpr (sizeof(T) == 4 && TPB >= 2) {
-            // Each row chunk of TPB complex leaves as TPB/2 16-byte pieces written by
-            // adjacent lanes.  Logical columns 2h, 2h+1 sit in physical piece
-            // h ^ (sw >> 1), swapped when sw is odd.  Qs and kx0 are even, so a
-            // piece is either wholly inside the row (kx0 + 2h < Qs) or wholly out;
-            // for TPB <= 4 always inside (Qs is a multiple of 4).
-            constexpr int PPR = TPB / 2, ROWS = C::THREADS / PPR;
-            if constexpr (ROWS % (TPB << C::SWZ) == 0) {
-                // A thread keeps its piece h and visits rows row0 + i * ROWS; ROWS is a
-                // multiple of the swizzle period, so the swizzle is fixed per thread.
-                const int h = threadIdx.x % PPR, row0 = threadIdx.x / PPR;
-                const int sw = (row0 >> C::SWZ) & (TPB - 1);
-                const bool swap_halves = sw & 1;
-                if (TPB <= 4 || kx0 + 2 * h < Qs) {
-                    const float4* src = reinterpret_cast<const float4*>(xbuf) + row0 * PPR + (h ^ (sw >> 1));
-                    float4* dst = reinterpret_cast<float4*>(yp + kx0) + h;
-                    for (int row = row0; row < P; row += ROWS, src += ROWS * PPR) {
-                        int orow = circ_to_out(row, P, HA, HB - 1);
-                        if constexpr (VOL) {
-                            if (orow < 0) continue;
-                            orow += dzo * R2;
-                        }
-                        if (orow < r0 || orow >= r1) continue;
-                        if constexpr (!VOL) orow += dzo * R2;  // the unit's rows
-                        float4 pv = *src;
-                        if (swap_halves) pv = make_float4(pv.z, pv.w, pv.x, pv.y);
-                        dst[(size_t)orow * (Qs / 2)] = pv;
+        const bool more = s_next[0] != 0;
+        e = s_next[1], a = s_next[2], b = s_next[3], kxb = s_next[4], dzo = s_next[5];
+        if (more) load_fa();
+        // Rows k + q NQ, q < R, of chunk c: X[k + q NQ] = sum_s w_R^{sq} (W_P^{sk} E_s[k])
+        auto emit = [&](auto splitc) {
+            constexpr bool SPLIT = decltype(splitc)::value;
+            cpx<T> t[CH / 2];  // the Hermitian step's twiddles of the chunk's first columns
+            auto load_t = [&](int c) {
+#pragma unroll
+                for (int i = 0; i < CH / 2; ++i) {
+                    const int kc = chunk_col<T>(c, i, L, SPLIT);
+                    t[i] = __ldg(twq + kc);
+                }
+            };
+            if constexpr (UPR == 1) load_t(c0);
+            for (int u = threadIdx.x; u < NQ * UPR; u += C::THREADS) {
+                const int h = UPR == 1 ? 0 : u / NQ, k = UPR == 1 ? u : u % NQ, c = c0 + h;
+                if (UPR > 1) {
+                    if (c * CH >= L) break;
+                    load_t(c);
+                }
+                cpx<T> x[CH][R];
+#pragma unroll
+                for (int i = 0; i < CH; ++i) {
+                    const cpx<T>* src = xbuf + (size_t)(h * CH + i) * P + k;
+                    if constexpr (R == 1) {
+                        x[i][0] = src[0];
+                    } else if constexpr (R == 2) {
+                        const cpx<T> e0 = src[0], e1 = cmul(src[NQ], twl<+1>(tw_n, k));
+                        x[i][0] = e0 + e1;
+                        x[i][1] = e0 - e1;
+                    } else {
+                        x[i][0] = src[0];
+#pragma unroll
+                        for (int s = 1; s < R; ++s) x[i][s] = cmul(src[s * NQ], twl<+1>(tw_n, s * k));
+                        dft_nat<R, +1>(x[i]);
                     }
                 }
-            } else {
-                for (int q = threadIdx.x; q < P * PPR; q += C::THREADS) {
-                    const int row = q / PPR, h = q % PPR;
-                    int orow = circ_to_out(row, P, HA, HB - 1);
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    int orow = circ_to_out(k + q * NQ, P, HA, HB - 1);
                     if constexpr (VOL) {
                         if (orow < 0) continue;
-                        orow += dzo * R2;
+                        orow += row_off;
                     }
-                    if (orow < r0 || orow >= r1 || kx0 + 2 * h >= Qs) continue;
-                    if constexpr (!VOL) orow += dzo * R2;
-                    const int sw = (row >> C::SWZ) & (TPB - 1);
-                    float4 pv = reinterpret_cast<const float4*>(xbuf)[row * PPR + (h ^ (sw >> 1))];
-                    if (sw & 1) pv = make_float4(pv.z, pv.w, pv.x, pv.y);
-                    reinterpret_cast<float4*>(yp + (size_t)orow * Qs + kx0)[h] = pv;
+                    if (orow < r0 || orow >= r1) continue;
+                    if constexpr (!VOL) orow += row_off;  // the unit's rows
+                    cpx<T> z[CH];
+#pragma unroll
+                    for (int i = 0; i < CH / 2; ++i) hermitian_step(x[i][q], x[CH - 1 - i][q], t[i], z[i], z[CH - 1 - i]);
+                    if (c == 0) {  // columns 0 (y_0 + i y_L) and L / 2
+                        const cpx<T> g0 = x[0][q], yh = x[CH - 1][q];
+                        z[0] = {g0.x + g0.y, g0.x - g0.y};
+                        z[CH - 1] = {yh.x + yh.x, T(0) - (yh.y + yh.y)};
+                    }
+                    store_chunk<SPLIT>(yp + y_chunk<T>(orow, c, L), z);
                 }
             }
-        } else {
-            // one complex per lane, adjacent lanes on adjacent columns of a row
-            for (int q = threadIdx.x; q < P * TPB; q += C::THREADS) {
-                const int row = q / TPB, c = q % TPB;
-                int orow = circ_to_out(row, P, HA, HB - 1);
-                if constexpr (VOL) {
-                    if (orow < 0) continue;
-                    orow += dzo * R2;
-                }
-                if (orow < r0 || orow >= r1 || kx0 + c >= Qs) continue;
-                if constexpr (!VOL) orow += dzo * R2;
-                const int sw = (row >> C::SWZ) & (TPB - 1);
-                yp[(size_t)orow * Qs + kx0 + c] = xbuf[(size_t)row * TPB + (c ^ sw)];
-            }
-        }
-        __syncthreads();  // tile reads (and s_item) done before the next item reuses them
-        if (next >= n_items) break;
-        item = next;
+        };
+        if (split) emit(std::true_type{});
+        else emit(std::false_type{});
+        __syncthreads();  // the buffer's reads (and s_next's) done before the next item writes it
+        if (!more) break;
     }
 }
 
@@ -666,7 +813,7 @@ constexpr size_t pair_cols_smem() {
 }
 
 // ---------------------------------------------------------------------------
-// Inverse row transform (complex-to-real, length Q) + fused entropy epilogue.
+// Inverse row transform (L = Q/2 complex inputs z_k, Q reals) + fused entropy epilogue.
 // One block per output row (grid-stride).  Per round, NT teams transform NT
 // pairs (a-major order); each thread then owns fixed shift positions p and
 // accumulates, pair by pair, the joint term T(c), the running A-marginal of
@@ -696,11 +843,11 @@ struct RowCfg {
     static constexpr int U = HALVES * UH;
     static constexpr int REGION = G::SCRATCH;                  // >= QH floats
     static constexpr size_t TEAM_SMEM = (size_t)NT * REGION;
-    // FP32: each team's next Y row (L + 1 complex, 16-byte chunks) is copied into a
+    // FP32: each team's next Y row (L complex, 16-byte pieces) is copied into a
     // shared-memory buffer by asynchronous copies (cp.async) while the current round
     // computes; the transform then loads its inputs from shared memory
     static constexpr bool STAGE = sizeof(T) == 4;
-    static constexpr int STAGE_BYTES = STAGE ? ((L + 1) * 8 + 15) / 16 * 16 : 0;
+    static constexpr int STAGE_BYTES = STAGE ? L * 8 : 0;
     static constexpr size_t OFF_STAGE = (TEAM_SMEM + 15) / 16 * 16;
     static constexpr size_t OFF_CB = OFF_STAGE + (size_t)NT * STAGE_BYTES;  // B-marginals (shared-memory variant)
     static constexpr int MIN_BLOCKS = sizeof(T) == 4 && THREADS < 512 ? 512 / THREADS : 1;  // <= 128 registers
@@ -737,9 +884,8 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                         : cb_global + (size_t)blockIdx.x * g.KB * Q;
     const int tid = threadIdx.x, team = tid / C::TEAM, lt = tid % C::TEAM, r = lt / M, j = lt % M;
     unsigned char* region = smem_raw + (size_t)team * C::REGION;
-    const int KA = g.KA, KB = g.KB, npairs = KA * KB, Rout = g.R, Cout = g.C, Qs = g.Qs;
+    const int KA = g.KA, KB = g.KB, npairs = KA * KB, Rout = g.R, Cout = g.C;
     const size_t RC = (size_t)Rout * Cout;
-    const cpx<T>* twq_c2r = tw_of<Q>(tw);
     float res_max = 0.f;
     int row_max_n = 0;
 
@@ -747,14 +893,16 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
     const int nr = g.r1 - g.r0, ntask = g.units * nr;
     auto task_row = [&](int tk) { return (tk / nr) * g.R2 + g.r0 + tk % nr; };
     // STAGE: the team's buffer for the Y row of its current pair; the team's lanes
-    // copy a row in 16-byte chunks (the rows start on 32-byte boundaries: Qs is a
-    // multiple of 4 complex)
+    // copy a row in 16-byte pieces (the rows start on 32-byte boundaries: L is a
+    // multiple of 4)
     const cpx<T>* stage = reinterpret_cast<const cpx<T>*>(smem_raw + C::OFF_STAGE + (size_t)team * C::STAGE_BYTES);
     auto stage_issue = [&](int pair_i, int row_i) {
         if constexpr (C::STAGE) {
-            const char* src = reinterpret_cast<const char*>(Y + ((size_t)pair_i * Rout + row_i) * Qs);
+            // half c % 2 of chunk c / 2, whose rows lie 128 bytes apart (layout of Y)
+            const char* src = reinterpret_cast<const char*>(Y + (size_t)pair_i * y_rows<T>(Rout) * L + y_chunk<T>(row_i, 0, L));
             const uint32_t dst = smem_u32(stage);
-            for (int c = lt; c < C::STAGE_BYTES / 16; c += C::TEAM) cp_async16(dst + 16u * c, src + 16 * c);
+            for (int c = lt; c < C::STAGE_BYTES / 16; c += C::TEAM)
+                cp_async16(dst + 16u * c, src + 128 * (c >> 1) + 16 * (c & 1));
             cp_async_commit();
         }
     };
@@ -783,7 +931,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
             const int pair = base + team;
             const bool act = pair < npairs;
             const int ovs = (act && ov_slot) ? ov_slot[pair] : -1;
-            const cpx<T>* yr = C::STAGE ? stage : Y + ((size_t)(act ? pair : 0) * Rout + row) * Qs;
+            const cpx<T>* yr = C::STAGE ? stage : Y + ((size_t)(act ? pair : 0) * Rout + row) * L;
             if (!C::STAGE && lt == 0) {
                 // ask L2 for this team's row of the next round (or of the block's next row)
                 int np = pair + NT, nrow = row;
@@ -793,18 +941,10 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                     nrow = nt2 < ntask ? (nt2 / nr) * g.R2 + g.r0 + nt2 % nr : -1;
                 }
                 if (np < npairs && nrow >= 0)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Y + ((size_t)np * Rout + nrow) * Qs),
-                                 "r"((unsigned)(Qs * sizeof(cpx<T>))) : "memory");
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Y + ((size_t)np * Rout + nrow) * L),
+                                 "r"((unsigned)(L * sizeof(cpx<T>))) : "memory");
             }
-            // Hermitian split: z = IDFT_L(E + iO), z[m] = x[2m] + i x[2m+1]
-            auto load = [&](int k) -> cpx<T> {
-                if (!act) return {T(0), T(0)};
-                const cpx<T> yk = yr[k], ym = yr[L - k];
-                const cpx<T> e = {yk.x + ym.x, yk.y - ym.y};
-                const cpx<T> d = {yk.x - ym.x, yk.y + ym.y};
-                const cpx<T> o = cmul(d, twl<+1>(twq_c2r, k));
-                return {e.x - o.y, e.y + o.x};
-            };
+            auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q>(yr, k) : cpx<T>{T(0), T(0)}; };
             cpx<T> v[M];
             team_fft<M, R, +1>(v, r, j, load, region + r * grp_scratch_bytes<T, M>(), tw.sq[ilog2c(M)],
                                tw_of<L>(tw));
@@ -879,7 +1019,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                                     for (int uh = 0; uh < UH; ++uh) {
                                         const int u = hf * UH + uh, pl = tid + BT * uh;
                                         if (pl >= QH) continue;
-                                        S[u].marg(clog2c_fixed(CA[u]));
+                                        S[u].marg(clog2c_biased(CA[u]));
                                         N[u] += (int)CA[u];
                                         CA[u] = 0.f;
                                     }
@@ -892,7 +1032,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                                     const int u = hf * UH + uh, pl = tid + BT * uh;
                                     if (pl >= QH) continue;
                                     const float c = obt[pl];
-                                    S[u].joint(clog2c_fixed(c));
+                                    S[u].joint(clog2c_biased(c));
                                     CA[u] += c;
                                     cbb[pl] = cbv[t][uh] + c;
                                 }
@@ -907,7 +1047,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                             for (int uh = 0; uh < UH; ++uh) {
                                 const int u = hf * UH + uh, pl = tid + BT * uh;
                                 if (pl >= QH) continue;
-                                S[u].marg(clog2c_fixed(CA[u]));
+                                S[u].marg(clog2c_biased(CA[u]));
                                 N[u] += (int)CA[u];
                                 if constexpr (DBG) {
                                     const int c = circ_to_out(hf * QH + pl, Q, g.WA, g.WB - 1);
@@ -925,7 +1065,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                             const int u = hf * UH + uh, pl = tid + BT * uh;
                             if (pl >= QH) continue;
                             const float c = obt[pl];
-                            S[u].joint(clog2c_fixed(c));
+                            S[u].joint(clog2c_biased(c));
                             CA[u] += c;
                             cbb[pl] += c;
                             if constexpr (DBG) {
@@ -954,7 +1094,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
             for (int u = 0; u < U; ++u) {
                 const int pl = tid + BT * (u % UH), p = (u / UH) * QH + pl;
                 if (pl >= QH) continue;
-                S[u].marg(clog2c_fixed(cbv[u]));
+                S[u].marg(clog2c_biased(cbv[u]));
                 if (counts) {
                     const int cidx = circ_to_out(p, Q, g.WA, g.WB - 1);
                     if (cidx >= 0) counts[((size_t)npairs + KA + b) * RC + (size_t)row * Cout + cidx] = (int)cbv[u];
@@ -966,7 +1106,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
             const int pl = tid + BT * (u % UH), p = (u / UH) * QH + pl;
             if (pl >= QH) continue;
             const int cidx = circ_to_out(p, Q, g.WA, g.WB - 1);
-            S[u].marg(clog2c_fixed(CA[u]));
+            S[u].marg(clog2c_biased(CA[u]));
             N[u] += (int)CA[u];
             if (counts && cidx >= 0) counts[((size_t)npairs + cur_a[u / UH]) * RC + (size_t)row * Cout + cidx] = (int)CA[u];
             if (cidx < 0) continue;
@@ -1020,23 +1160,14 @@ k_pair_rows_counts(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, const int* __
     unsigned char* region = smem_raw + (size_t)team * C::G::SCRATCH;
     const int nrows = g.r1 - g.r0;
     const long long ntask = (long long)np * nrows;
-    const cpx<T>* twq_c2r = tw_of<Q>(tw);
     float res = 0.f;
     // a uniform trip count per block: every lane of a warp takes part in each transform's warp syncs
     for (long long t0 = (long long)blockIdx.x * NT; t0 < ntask; t0 += (long long)gridDim.x * NT) {
         const long long t = t0 + team;
         const bool act = t < ntask;
         const int e = act ? (int)(t / nrows) : 0, row = g.r0 + (act ? (int)(t % nrows) : 0);
-        const cpx<T>* yr = Y + ((size_t)e * g.R + row) * g.Qs;
-        // Hermitian split: z = IDFT_L(E + iO), z[m] = x[2m] + i x[2m+1]
-        auto load = [&](int k) -> cpx<T> {
-            if (!act) return {T(0), T(0)};
-            const cpx<T> yk = yr[k], ym = yr[L - k];
-            const cpx<T> ev = {yk.x + ym.x, yk.y - ym.y};
-            const cpx<T> d = {yk.x - ym.x, yk.y + ym.y};
-            const cpx<T> o = cmul(d, twl<+1>(twq_c2r, k));
-            return {ev.x - o.y, ev.y + o.x};
-        };
+        const cpx<T>* yr = Y + ((size_t)e * g.R + row) * L;
+        auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q>(yr, k) : cpx<T>{T(0), T(0)}; };
         cpx<T> v[M];
         team_fft<M, R, +1>(v, r, j, load, region + r * grp_scratch_bytes<T, M>(), tw.sq[ilog2c(M)],
                            tw_of<L>(tw));
@@ -1090,9 +1221,8 @@ k_pair_rows_w(const cpx<double>* __restrict__ Y, Geom g, Tw<double> tw, double* 
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int tid = threadIdx.x, team = tid / C::TEAM, lt = tid % C::TEAM, r = lt / M, j = lt % M;
     unsigned char* region = smem_raw + (size_t)team * C::REGION;
-    const int KB = g.KB, npairs = g.KA * g.KB, Rout = g.R, Cout = g.C, Qs = g.Qs;
+    const int KB = g.KB, npairs = g.KA * g.KB, Rout = g.R, Cout = g.C;
     double* cb = cbw + (size_t)blockIdx.x * KB * Q;
-    const cpx<double>* twq_c2r = tw_of<Q>(tw);
     double row_max_n = 0.0;
     for (int row = g.r0 + blockIdx.x; row < g.r1; row += gridDim.x) {
         double S[U], CA[U], N[U];
@@ -1108,16 +1238,8 @@ k_pair_rows_w(const cpx<double>* __restrict__ Y, Geom g, Tw<double> tw, double* 
         for (int base = 0; base < npairs; base += NT) {
             const int pair = base + team;
             const bool act = pair < npairs;
-            const cpx<double>* yr = Y + ((size_t)(act ? pair : 0) * Rout + row) * Qs;
-            // Hermitian split: z = IDFT_L(E + iO), z[m] = x[2m] + i x[2m+1]
-            auto load = [&](int k) -> cpx<double> {
-                if (!act) return {0.0, 0.0};
-                const cpx<double> yk = yr[k], ym = yr[L - k];
-                const cpx<double> e = {yk.x + ym.x, yk.y - ym.y};
-                const cpx<double> d = {yk.x - ym.x, yk.y + ym.y};
-                const cpx<double> o = cmul(d, twl<+1>(twq_c2r, k));
-                return {e.x - o.y, e.y + o.x};
-            };
+            const cpx<double>* yr = Y + ((size_t)(act ? pair : 0) * Rout + row) * L;
+            auto load = [&](int k) -> cpx<double> { return act ? load_z<double, Q>(yr, k) : cpx<double>{0.0, 0.0}; };
             cpx<double> v[M];
             team_fft<M, R, +1>(v, r, j, load, region + r * grp_scratch_bytes<double, M>(), tw.sq[ilog2c(M)],
                                tw_of<L>(tw));

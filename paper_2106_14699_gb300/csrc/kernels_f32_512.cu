@@ -5,7 +5,7 @@ template cudaError_t Sized<float, 512>::fwd_rows(const Geom&, const PipeArgs<flo
 template cudaError_t Sized<float, 512>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 512>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template int Sized<float, 512>::tm_cols(int);
-template cudaError_t Sized<float, 512>::tm_max_blocks(int*);
+template cudaError_t Sized<float, 512>::tm_max_blocks(int, int*);
 template cudaError_t Sized<float, 512>::pair_rows_w(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template size_t Sized<float, 512>::rows_w_smem();
 template cudaError_t Sized<float, 512>::rows_w_max_blocks(int*);

@@ -5,7 +5,7 @@ template cudaError_t Sized<df32, 16>::fwd_rows(const Geom&, const PipeArgs<df32>
 template cudaError_t Sized<df32, 16>::fwd_cols(const Geom&, const PipeArgs<df32>&, bool, cudaStream_t);
 template cudaError_t Sized<df32, 16>::pair_cols(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template int Sized<df32, 16>::tm_cols(int);
-template cudaError_t Sized<df32, 16>::tm_max_blocks(int*);
+template cudaError_t Sized<df32, 16>::tm_max_blocks(int, int*);
 template cudaError_t Sized<df32, 16>::pair_rows_w(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template size_t Sized<df32, 16>::rows_w_smem();
 template cudaError_t Sized<df32, 16>::rows_w_max_blocks(int*);
@@ -13,7 +13,7 @@ template cudaError_t Sized<df32, 32>::fwd_rows(const Geom&, const PipeArgs<df32>
 template cudaError_t Sized<df32, 32>::fwd_cols(const Geom&, const PipeArgs<df32>&, bool, cudaStream_t);
 template cudaError_t Sized<df32, 32>::pair_cols(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template int Sized<df32, 32>::tm_cols(int);
-template cudaError_t Sized<df32, 32>::tm_max_blocks(int*);
+template cudaError_t Sized<df32, 32>::tm_max_blocks(int, int*);
 template cudaError_t Sized<df32, 32>::pair_rows_w(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template size_t Sized<df32, 32>::rows_w_smem();
 template cudaError_t Sized<df32, 32>::rows_w_max_blocks(int*);
@@ -21,7 +21,7 @@ template cudaError_t Sized<df32, 64>::fwd_rows(const Geom&, const PipeArgs<df32>
 template cudaError_t Sized<df32, 64>::fwd_cols(const Geom&, const PipeArgs<df32>&, bool, cudaStream_t);
 template cudaError_t Sized<df32, 64>::pair_cols(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template int Sized<df32, 64>::tm_cols(int);
-template cudaError_t Sized<df32, 64>::tm_max_blocks(int*);
+template cudaError_t Sized<df32, 64>::tm_max_blocks(int, int*);
 template cudaError_t Sized<df32, 64>::pair_rows_w(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template size_t Sized<df32, 64>::rows_w_smem();
 template cudaError_t Sized<df32, 64>::rows_w_max_blocks(int*);
@@ -29,7 +29,7 @@ template cudaError_t Sized<df32, 128>::fwd_rows(const Geom&, const PipeArgs<df32
 template cudaError_t Sized<df32, 128>::fwd_cols(const Geom&, const PipeArgs<df32>&, bool, cudaStream_t);
 template cudaError_t Sized<df32, 128>::pair_cols(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template int Sized<df32, 128>::tm_cols(int);
-template cudaError_t Sized<df32, 128>::tm_max_blocks(int*);
+template cudaError_t Sized<df32, 128>::tm_max_blocks(int, int*);
 template cudaError_t Sized<df32, 128>::pair_rows_w(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template size_t Sized<df32, 128>::rows_w_smem();
 template cudaError_t Sized<df32, 128>::rows_w_max_blocks(int*);
@@ -37,7 +37,7 @@ template cudaError_t Sized<df32, 256>::fwd_rows(const Geom&, const PipeArgs<df32
 template cudaError_t Sized<df32, 256>::fwd_cols(const Geom&, const PipeArgs<df32>&, bool, cudaStream_t);
 template cudaError_t Sized<df32, 256>::pair_cols(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template int Sized<df32, 256>::tm_cols(int);
-template cudaError_t Sized<df32, 256>::tm_max_blocks(int*);
+template cudaError_t Sized<df32, 256>::tm_max_blocks(int, int*);
 template cudaError_t Sized<df32, 256>::pair_rows_w(const Geom&, const PipeArgs<df32>&, cudaStream_t);
 template size_t Sized<df32, 256>::rows_w_smem();
 template cudaError_t Sized<df32, 256>::rows_w_max_blocks(int*);

@@ -7,6 +7,7 @@
 
 #include "kernels.cuh"
 #include "misc.h"
+#include "pipeline.cuh"
 
 namespace cmif {
 
@@ -460,7 +461,7 @@ cudaError_t launch_fill_labels(int32_t* X, long long n, int K, unsigned seed, cu
 // the row kernels evaluate it, for the counts c0 .. c0 + n - 1.
 __global__ void k_entropy_terms(int c0, int n, long long* __restrict__ out) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        out[i] = clog2c_fixed((float)(c0 + i));
+        out[i] = clog2c_biased((float)(c0 + i)) - (long long)kTermBias * (c0 + i);
 }
 
 cudaError_t launch_entropy_terms(int c0, int n, long long* out, cudaStream_t s) {
@@ -510,6 +511,26 @@ static void host_twiddle(long long k, long long N, double* c, double* s) {
     *s = -ss;  // e^{-i t}
 }
 
+// The FP32 four-step twiddles e^{-2 pi i j k / M^2}.  M >= 8 (packed DFTs): float4 entry
+// k M + j, k < M/2, holds rows k and k + M/2 side by side, (cos, cos', sin, sin') with
+// sin the imaginary parts; smaller M: complex entry k M + j.  (16-byte alignment: the
+// 2^14 - 1 values of the power-of-two tables and the one of M = 1 come before.)
+static void fill_sq_f32(float* out, int M) {
+    for (int k = 0; k < M; ++k)
+        for (int j = 0; j < M; ++j) {
+            double c, s;
+            host_twiddle((long long)j * k, (long long)M * M, &c, &s);
+            if (M >= 8) {
+                float* q = out + 4 * ((size_t)(k % (M / 2)) * M + j) + k / (M / 2);
+                q[0] = (float)c;
+                q[2] = (float)s;
+            } else {
+                out[2 * ((size_t)k * M + j)] = (float)c;
+                out[2 * ((size_t)k * M + j) + 1] = (float)s;
+            }
+        }
+}
+
 void twiddle_table_f32(std::vector<float>& out, size_t off_n[14], size_t off_sq[6], size_t off_n3[12]) {
     out.clear();
     size_t n = 0;
@@ -525,14 +546,10 @@ void twiddle_table_f32(std::vector<float>& out, size_t off_n[14], size_t off_sq[
     }
     for (int l = 0; l < 6; ++l) {
         off_sq[l] = n;
-        const long long M = 1LL << l;
-        for (long long k1 = 0; k1 < M; ++k1)
-            for (long long j = 0; j < M; ++j, ++n) {
-                double c, s;
-                host_twiddle(j * k1, M * M, &c, &s);
-                out.push_back((float)c);
-                out.push_back((float)s);
-            }
+        const int M = 1 << l;
+        n += (size_t)M * M;
+        out.resize(2 * n);
+        fill_sq_f32(out.data() + 2 * off_sq[l], M);
     }
     for (int l = 0; l < 12; ++l) {
         off_n3[l] = n;
@@ -610,15 +627,18 @@ cudaError_t get_twiddles(int device, Tw<float>* tf, Tw<double>* td, Tw<df32>* ts
             hs[4 * i + 2] = ih;
             hs[4 * i + 3] = (float)(im[i] - (double)ih);
         }
-        const size_t bytes_d = 2 * n * sizeof(double), bytes_f = 2 * n * sizeof(float), bytes_s = 4 * n * sizeof(float);
+        for (int l = 0; l < 6; ++l) fill_sq_f32(hf.data() + 2 * off_sq[l], 1 << l);
+        // every table starts on a 256-byte boundary (the two-term values are loaded 16 bytes at a time)
+        const size_t bytes_d = (2 * n * sizeof(double) + 255) / 256 * 256, bytes_f = (2 * n * sizeof(float) + 255) / 256 * 256;
+        const size_t bytes_s = 4 * n * sizeof(float);
         int prev = -1;
         cudaGetDevice(&prev);
         cudaError_t e = cudaSetDevice(device);
         if (e != cudaSuccess) return e;
         void* buf = nullptr;
         e = cudaMalloc(&buf, bytes_d + bytes_f + bytes_s);
-        if (e == cudaSuccess) e = cudaMemcpy(buf, hd.data(), bytes_d, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d, hf.data(), bytes_f, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(buf, hd.data(), hd.size() * sizeof(double), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d, hf.data(), hf.size() * sizeof(float), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d + bytes_f, hs.data(), bytes_s, cudaMemcpyHostToDevice);
         if (prev >= 0) cudaSetDevice(prev);
         if (e != cudaSuccess) {
@@ -637,6 +657,29 @@ cudaError_t get_twiddles(int device, Tw<float>* tf, Tw<double>* td, Tw<df32>* ts
     if (td) *td = t.td;
     if (ts) *ts = t.ts;
     return cudaSuccess;
+}
+
+// Tensor map of Y for the row copies of the Tensor-Memory row kernel: 32 floats (a line of
+// four rows' chunks) x L/4 chunks x row groups x pairs; a copy takes 8 x L/4 x 1 x 1.
+cudaError_t make_row_map(CUtensorMap* map, const cpx<float>* Y, int L, int Rout, int npairs) {
+    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {  // resolved once per process; immutable afterwards
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? reinterpret_cast<Encode>(fn) : nullptr;
+    }();
+    if (!encode) return cudaErrorNotSupported;
+    const cuuint64_t groups = (cuuint64_t)y_rows<float>(Rout) / 4;
+    const cuuint64_t dims[4] = {32, (cuuint64_t)(L / 4), groups, (cuuint64_t)npairs};
+    const cuuint64_t strides[3] = {128, 32ull * L, 32ull * L * groups};  // bytes; a row group holds 4 L complex
+    const cuuint32_t box[4] = {8, (cuuint32_t)(L / 4), 1, 1}, elem[4] = {1, 1, 1, 1};
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<cpx<float>*>(Y), dims, strides, box,
+                              elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                              CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 }  // namespace cmif

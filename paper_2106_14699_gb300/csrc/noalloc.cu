@@ -110,6 +110,7 @@ extern "C" cmif_status cmif_compute_noalloc(int H_A, int W_A, int H_B, int W_B, 
     if (g.P > 4096 || g.Q > 4096) return CMIF_ERR_UNSUPPORTED;
     g.Qh = g.Q / 2 + 1;
     g.Qs = (g.Qh + 3) / 4 * 4;
+    g.Ys = g.Q / 2;
 
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess) return CMIF_ERR_CUDA;
@@ -144,7 +145,7 @@ extern "C" cmif_status cmif_compute_noalloc(int H_A, int W_A, int H_B, int W_B, 
     const size_t oT1B = off; off = up256(off + (size_t)g.KB * g.HB * g.Qs * cs);
     const size_t oFA = off; off = up256(off + (size_t)g.KA * g.Qh * g.P * cs);
     const size_t oFB = off; off = up256(off + (size_t)g.KB * g.Qh * g.P * cs);
-    const size_t oY = off; off = up256(off + (size_t)g.KA * g.KB * g.R * g.Qs * cs);
+    const size_t oY = off; off = up256(off + (size_t)g.KA * g.KB * y_rows<float>(g.R) * g.Ys * cs);
     const size_t oCtr = off; off = up256(off + sizeof(int));
     if (off > kNoAllocBytes) return CMIF_ERR_UNSUPPORTED;
 

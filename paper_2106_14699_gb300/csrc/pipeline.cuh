@@ -1,5 +1,6 @@
 // Launch sequence of one CMIF map for one precision (FP32 or FP64 transforms).
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <type_traits>
 #include "kernels.cuh"
@@ -17,7 +18,7 @@ struct PipeArgs {
     cpx<T>* T1B;  // [K_B][H_B][Qs]
     cpx<T>* FA;   // [K_A][Qh][P]    2-D half spectra, column-contiguous
     cpx<T>* FB;   // [K_B][Qh][P]
-    cpx<T>* Y;    // [K_A*K_B][R][Qs] column-inverted products, output rows only
+    cpx<T>* Y;    // [K_A*K_B][R][Ys] row-transform inputs, output rows only (layout: kernels.cuh)
     float* cb_global;  // [rows_grid][K_B][Q] when !cb_smem
     int* work_ctr;     // item counter of the pair-column kernel (zeroed before each launch)
     Tw<T> tw;
@@ -134,7 +135,7 @@ struct Sized {
     static int rows_threads();
     static cudaError_t rows_max_blocks(int KB, bool cb_smem, int* out);
     static int tm_cols(int KB);                 // 0 unless the TMEM row kernel applies (FP32, Q = 512 / 1024 / 2048)
-    static cudaError_t tm_max_blocks(int* out);
+    static cudaError_t tm_max_blocks(int tm_cols, int* out);
     static cudaError_t pair_rows_w(const Geom& g, const PipeArgs<T>& a, cudaStream_t s);  // FP64 only
     static size_t rows_w_smem();
     static cudaError_t rows_w_max_blocks(int* out);
@@ -150,6 +151,9 @@ cudaError_t launch_rows_tm_units(const Geom& g, const PipeArgs<float>& a, cudaSt
 template <typename T>
 cudaError_t run_pair_counts(const Geom& g, const PipeArgs<T>& a, cudaStream_t s);
 
+// Tensor map of Y for the Tensor-Memory row kernel's row copies (FP32; rows_tm.cuh).
+cudaError_t make_row_map(CUtensorMap* map, const cpx<float>* Y, int L, int Rout, int npairs);
+
 // Per-precision facts the host needs at plan time.
 template <typename T>
 size_t rows_smem_bytes(int Q, int KB, bool cb_smem);
@@ -159,7 +163,7 @@ template <typename T>
 cudaError_t rows_max_blocks_per_sm(int Q, int KB, bool cb_smem, int* out);
 // TMEM columns the TMEM / TMA row kernel needs for (Q, K_B), or 0 when it does not apply.
 int rows_tm_cols(int Q, int KB);
-cudaError_t rows_tm_max_blocks_per_sm(int Q, int* out);
+cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int* out);
 // The weighted (SWMI) row kernel: its occupancy (FP64).
 cudaError_t rows_w_max_blocks_per_sm(int Q, int* out);
 

@@ -50,6 +50,12 @@ static cudaError_t launch_fwd_cols(const cpx<T>* T1, int H, int K, int Qh, int Q
     return cudaGetLastError();
 }
 
+// The table of e^{-2 pi i k / N}, N = 2^l or 3 2^l.
+template <typename T>
+static const cpx<T>* tw_table(const Tw<T>& tw, int N) {
+    return N % 3 == 0 ? tw.n3[ilog2_of(N / 3)] : tw.n[ilog2_of(N)];
+}
+
 template <typename T, int P, bool VOL, int MMAX>
 static cudaError_t launch_pair_cols(const Geom& g, const PipeArgs<T>& a, cudaStream_t s) {
     using C = PairColsCfg<T, P, MMAX>;
@@ -66,15 +72,39 @@ static cudaError_t launch_pair_cols(const Geom& g, const PipeArgs<T>& a, cudaStr
         per_sm = n > 0 ? n : 1;
     }
     const long long np = a.plist ? a.chunk_cap : (long long)g.KA * g.KB;  // list mode: at most chunk_cap pairs
-    const long long items = np * ((g.Qh + C::TPB - 1) / C::TPB) * (VOL ? g.Dz : g.units);
+    const long long items = np * ((g.Ys + C::TPB - 1) / C::TPB) * (VOL ? g.Dz : g.units);
     const int bps = a.cols_bps > 0 && a.cols_bps < per_sm ? a.cols_bps : per_sm;
     const long long slots = a.num_sms > 0 ? (long long)bps * a.num_sms : items;
     const int grid = (int)(items < slots ? items : slots);
     e = cudaMemsetAsync(a.work_ctr, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
-    kern<<<grid, C::THREADS, smem, s>>>(a.FA, a.FB, g.KA, g.KB, g.Qh, g.HA, g.HB, g.R, g.Qs, g.r0, g.r1, a.Y, a.tw,
-                                        a.st, a.conditional, a.work_ctr, g.DA, g.DB, g.R2, a.plist, a.lrange,
+    kern<<<grid, C::THREADS, smem, s>>>(a.FA, a.FB, g.KA, g.KB, g.Qh, g.HA, g.HB, g.R, g.r0, g.r1, a.Y, a.tw,
+                                        tw_table(a.tw, g.Q), a.st, a.conditional, a.work_ctr, g.DA, g.DB, g.R2, a.plist, a.lrange,
                                         a.chunk_off, a.chunk_cap, VOL ? 1 : g.units);
+    return cudaGetLastError();
+}
+
+// Teams per block of the Tensor-Memory row kernel (rows_tm.cuh).
+template <int Q>
+static constexpr int kRowTeams = Q == 2048 ? 16 : 8;
+template <int Q>
+static int rows_tm_teams(int tm_cols) { return tm_cols <= 256 ? kRowTeams<Q> : 16; }
+
+template <int Q, bool NMI, int MODE, int NT>
+static cudaError_t launch_rows_tm(const Geom& g, const PipeArgs<float>& a, cudaStream_t s) {
+    using C = RowTmCfg<Q, NT>;
+    auto kern = k_pair_rows_tm<Q, NMI, MODE, NT>;
+    cudaError_t e = ensure_smem(kern, C::SMEM);
+    if (e != cudaSuccess) return e;
+    const bool ext = MODE == 2;
+    CUtensorMap ymap;
+    e = make_row_map(&ymap, a.Y, C::L, g.R, g.KA * g.KB);
+    if (e != cudaSuccess) return e;
+    kern<<<a.rows_grid, C::THREADS, C::SMEM, s>>>(ymap, g, a.tw, a.mi, a.n, a.st, a.tm_cols,
+                                                  ext && a.wait_polls > 0 ? a.wait_polls : kDefaultWaitPolls,
+                                                  ext ? a.withhold_row : -1, ext ? a.conditional : 0,
+                                                  ext ? a.ov : nullptr, ext ? a.ov_slot : nullptr,
+                                                  ext ? a.pair_res : nullptr);
     return cudaGetLastError();
 }
 
@@ -87,13 +117,9 @@ static cudaError_t launch_pair_rows_v(const Geom& g, const PipeArgs<T>& a, cudaS
             // the multi-unit kernel lives in its own translation unit (kernels_f32_rows_units.cu):
             // compiled next to the plain one, it changed the plain kernel's register allocation
             if (!ext && g.units > 1) return launch_rows_tm_units<Q, NMI>(g, a, s);
-            auto kern = ext ? k_pair_rows_tm<Q, NMI, 2> : k_pair_rows_tm<Q, NMI, 0>;
-            cudaError_t e = ensure_smem(kern, RowTmCfg<Q>::SMEM);
-            if (e != cudaSuccess) return e;
-            kern<<<a.rows_grid, RowTmCfg<Q>::THREADS, RowTmCfg<Q>::SMEM, s>>>(
-                a.Y, g, a.tw, a.mi, a.n, a.st, a.tm_cols, a.wait_polls > 0 ? a.wait_polls : kDefaultWaitPolls,
-                a.withhold_row, a.conditional, a.ov, a.ov_slot, a.pair_res);
-            return cudaGetLastError();
+            if (rows_tm_teams<Q>(a.tm_cols) != 16)
+                return ext ? launch_rows_tm<Q, NMI, 2, kRowTeams<Q>>(g, a, s) : launch_rows_tm<Q, NMI, 0, kRowTeams<Q>>(g, a, s);
+            return ext ? launch_rows_tm<Q, NMI, 2, 16>(g, a, s) : launch_rows_tm<Q, NMI, 0, 16>(g, a, s);
         }
     }
     const size_t smem = pair_rows_smem<T, Q>(g.KB, a.cb_smem);
@@ -243,7 +269,7 @@ cudaError_t Sized<T, SZ>::rows_w_max_blocks(int* out) {
 template <typename T, int SZ>
 int Sized<T, SZ>::tm_cols(int KB) {
     if constexpr (sizeof(T) == 4 && (SZ == 512 || SZ == 1024 || SZ == 2048)) {
-        const int need = tm_cols_needed(KB, RowTmCfg<SZ>::U);
+        const int need = tm_cols_needed(KB, SZ);
         return need <= 512 ? tm_alloc_cols(need) : 0;
     } else {
         (void)KB;
@@ -252,14 +278,17 @@ int Sized<T, SZ>::tm_cols(int KB) {
 }
 
 template <typename T, int SZ>
-cudaError_t Sized<T, SZ>::tm_max_blocks(int* out) {
+cudaError_t Sized<T, SZ>::tm_max_blocks(int tm_cols, int* out) {
+    *out = 0;
     if constexpr (sizeof(T) == 4 && (SZ == 512 || SZ == 1024 || SZ == 2048)) {
-        cudaError_t e = ensure_smem(k_pair_rows_tm<SZ, false, 0>, RowTmCfg<SZ>::SMEM);
-        if (e != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_pair_rows_tm<SZ, false, 0>, RowTmCfg<SZ>::THREADS,
-                                                             RowTmCfg<SZ>::SMEM);
+        // The blocks that share an SM: as many as the kernel is bounded for (registers; shared
+        // memory is less than that), within the SM's 512 TMEM columns.  (The occupancy query
+        // answers 1 for a kernel that allocates Tensor Memory.)
+        const int blocks = rows_tm_teams<SZ>(tm_cols) == 16 ? 1 : RowTmCfg<SZ, kRowTeams<SZ>>::BLOCKS;
+        *out = std::min(blocks, 512 / tm_cols);
+        return cudaSuccess;
     } else {
-        *out = 0;
+        (void)tm_cols;
         return cudaSuccess;
     }
 }

@@ -1,13 +1,14 @@
 // Inverse row transform + fused entropy epilogue, FP32, one warp per pair
-// transform (Q = 512, 1024 or 2048), with
+// transform (L = Q/2 = 256, 512 or 1024 points), with
 //   * the B-marginal accumulators C_B^b(p) held in Tensor Memory (TMEM,
 //     tcgen05.ld / tcgen05.st), one 32-bit column per (b, position) of the
 //     owning thread, and
-//   * each team's next Y row fetched into shared memory by a TMA bulk copy
-//     (cp.async.bulk + mbarrier) while the current round computes.
+//   * each team's next Y row gathered into shared memory by a TMA tensor copy
+//     (cp.async.bulk.tensor + mbarrier) while the current round computes.
 // Same arithmetic and outputs as k_pair_rows (kernels.cuh), except the debug
 // count maps: a call that asks for them runs k_pair_rows.
 #pragma once
+#include <cuda.h>
 #include "kernels.cuh"
 
 namespace cmif {
@@ -22,10 +23,13 @@ __device__ __forceinline__ void mbar_fence_init() {
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-__device__ __forceinline__ void tma_bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+// Row `row` of pair `pair` (layout of Y): the 32-byte pieces (row % 4) of the row group's
+// 128-byte lines, one per chunk.  Tensor: 32 floats x L/4 chunks x row groups x pairs, box
+// 8 x L/4 x 1 x 1; x = 8 (row % 4) is a multiple of 4 floats (16 bytes).
+__device__ __forceinline__ void tma_row_g2s(uint32_t dst, const CUtensorMap* map, int row, int pair, uint32_t bytes, uint32_t bar) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+                 ::"r"(dst), "l"(map), "r"(bar), "r"(8 * (row & 3)), "r"(0), "r"(row >> 2), "r"(pair) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t phase) {
     uint32_t done;
@@ -84,6 +88,32 @@ __device__ __forceinline__ void tmem_st<2>(uint32_t t, const uint32_t (&r)[2]) {
     "r"(r[o + 6]), "r"(r[o + 7]), "r"(r[o + 8]), "r"(r[o + 9]), "r"(r[o + 10]), "r"(r[o + 11]),           \
     "r"(r[o + 12]), "r"(r[o + 13]), "r"(r[o + 14]), "r"(r[o + 15])
 template <>
+__device__ __forceinline__ void tmem_ld<4>(uint32_t t, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(t) : "memory");
+}
+template <>
+__device__ __forceinline__ void tmem_st<4>(uint32_t t, const uint32_t (&r)[4]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                 ::"r"(t), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+#define CMIF_R8(o) "=r"(r[o]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), \
+    "=r"(r[o + 6]), "=r"(r[o + 7])
+#define CMIF_W8(o) "r"(r[o]), "r"(r[o + 1]), "r"(r[o + 2]), "r"(r[o + 3]), "r"(r[o + 4]), "r"(r[o + 5]), \
+    "r"(r[o + 6]), "r"(r[o + 7])
+template <>
+__device__ __forceinline__ void tmem_ld<8>(uint32_t t, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : CMIF_R8(0) : "r"(t) : "memory");
+}
+template <>
+__device__ __forceinline__ void tmem_st<8>(uint32_t t, const uint32_t (&r)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"r"(t), CMIF_W8(0) : "memory");
+}
+#undef CMIF_R8
+#undef CMIF_W8
+template <>
 __device__ __forceinline__ void tmem_ld<16>(uint32_t t, uint32_t (&r)[16]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
                  "%14, %15}, [%16];"
@@ -111,40 +141,127 @@ __device__ __forceinline__ void tmem_st<32>(uint32_t t, const uint32_t (&r)[32])
 #undef CMIF_W16
 
 // ---------------------------------------------------------------------------
-template <int Q>
+// The warp's transform of L = 32 PTS points (PTS = 8, 16, 32 per lane), four-step:
+// lane j holds x[j + 32 i], i < PTS; a PTS-point DFT over i gives rows k1 < PTS; twiddle
+// w_L^{j k1}; a transpose through the warp's buffer (PTS rows of 32 floats, real plane then
+// imaginary plane, blocks of 4 floats XOR-permuted by the row: conflict-free 16-byte row
+// reads); then a 32-point DFT along each row by RS = 32 / PTS lanes, lane k1 + PTS r taking
+// the outputs k2 = RS q + r: each loads the whole row, forms its radix-RS combination
+// y_r[n] = w_32^{nr} sum_s i^{sr..} x[n + PTS s] and a second PTS-point DFT.  So output q of lane l
+// is X[l + 32 q] for every PTS, and no step but the transpose leaves the registers.  All
+// DFTs are packed (fft_pk.cuh): re[m] = values 2m, 2m + 1 on entry, q and q + PTS/2 on exit.
+// tw1[k 32 + j]: w_L^{j k}, w_L^{j (k + PTS/2)}; tw2[r PTS/2 + m]: w_32^{2m r}, w_32^{(2m+1) r},
+// both as (cos, cos', sin, sin') with the forward sign.
+__device__ __forceinline__ void mul_conj2(float2& re, float2& im, float4 w) {
+    const float2 c = make_float2(w.x, w.y), s = make_float2(w.z, w.w), a = re, b = im;
+    re = __ffma2_rn(b, s, __fmul2_rn(a, c));
+    im = __fmul2_rn(b, c);
+    im = make_float2(fmaf(-a.x, s.x, im.x), fmaf(-a.y, s.y, im.y));
+}
+template <int PTS>
+__device__ __forceinline__ void warp_fft_inv(float2 (&re)[PTS / 2], float2 (&im)[PTS / 2], int lane, float* sf,
+                                             const float4* tw1, const float4* tw2) {
+    constexpr int H = PTS / 2, RS = 32 / PTS;
+    dft_pk<PTS, +1>(re, im);
+#pragma unroll
+    for (int k = 0; k < H; ++k) mul_conj2(re[k], im[k], tw1[k * 32 + lane]);
+    float* si = sf + PTS * 32;
+    __syncwarp();
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {  // rows x, x + 8, .. share a block permutation: one address
+        char* const p = reinterpret_cast<char*>(sf) + ((lane << 2) ^ (x << 4));
+#pragma unroll
+        for (int row = x; row < PTS; row += 8) {
+            *reinterpret_cast<float*>(p + row * 128) = row < H ? re[row].x : re[row - H].y;
+            *reinterpret_cast<float*>(p + row * 128 + PTS * 128) = row < H ? im[row].x : im[row - H].y;
+        }
+    }
+    __syncwarp();
+    const int k1 = lane & (PTS - 1), r = lane / PTS;
+    auto block = [&](const float* pl, int b) {
+        return *reinterpret_cast<const float4*>(pl + k1 * 32 + (((b ^ k1) & 7) << 2));
+    };
+    auto lo = [](float4 q) { return make_float2(q.x, q.y); };
+    auto hi = [](float4 q) { return make_float2(q.z, q.w); };
+    if constexpr (RS == 1) {
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const float4 p = block(sf, b), q = block(si, b);
+            re[2 * b] = lo(p); re[2 * b + 1] = hi(p);
+            im[2 * b] = lo(q); im[2 * b + 1] = hi(q);
+        }
+    } else if constexpr (RS == 2) {
+        const float sg = r ? -1.f : 1.f;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const float4 p0 = block(sf, b), p1 = block(sf, b + 4), q0 = block(si, b), q1 = block(si, b + 4);
+            re[2 * b] = fmak(lo(p1), sg, lo(p0)); re[2 * b + 1] = fmak(hi(p1), sg, hi(p0));
+            im[2 * b] = fmak(lo(q1), sg, lo(q0)); im[2 * b + 1] = fmak(hi(q1), sg, hi(q0));
+        }
+    } else {
+        static_assert(RS == 4, "8, 16 or 32 points per lane");
+        // (x0 + (-1)^r x2) + i^r (x1 + (-1)^r x3)
+        const float sg = (r & 1) ? -1.f : 1.f, cr = r == 0 ? 1.f : r == 2 ? -1.f : 0.f, ci = r == 1 ? 1.f : r == 3 ? -1.f : 0.f;
+        auto join = [&](float2 x0, float2 x1, float2 x2, float2 x3, float2 y0, float2 y1, float2 y2, float2 y3,
+                        float2& zr, float2& zi) {
+            const float2 ar = fmak(x2, sg, x0), br = fmak(x3, sg, x1), ai = fmak(y2, sg, y0), bi = fmak(y3, sg, y1);
+            zr = fmak(bi, -ci, fmak(br, cr, ar));
+            zi = fmak(br, ci, fmak(bi, cr, ai));
+        };
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const float4 p0 = block(sf, b), p1 = block(sf, b + 2), p2 = block(sf, b + 4), p3 = block(sf, b + 6);
+            const float4 q0 = block(si, b), q1 = block(si, b + 2), q2 = block(si, b + 4), q3 = block(si, b + 6);
+            join(lo(p0), lo(p1), lo(p2), lo(p3), lo(q0), lo(q1), lo(q2), lo(q3), re[2 * b], im[2 * b]);
+            join(hi(p0), hi(p1), hi(p2), hi(p3), hi(q0), hi(q1), hi(q2), hi(q3), re[2 * b + 1], im[2 * b + 1]);
+        }
+    }
+    if constexpr (RS > 1) {
+#pragma unroll
+        for (int m = 0; m < H; ++m) mul_conj2(re[m], im[m], tw2[r * H + m]);
+    }
+    __syncwarp();  // the buffer's reads are done
+    dft_pk<PTS, +1>(re, im);
+}
+
+// NT teams (warps) per block, BLOCKS blocks per SM.  Narrow rows hold few values per lane, so
+// more warps fit, and several small blocks, each with its own barriers, run one's transforms
+// (FMA pipe) beside another's entropy terms (ALU, MUFU).  Measured at K = 16 (1e11 counts/s):
+// Q = 512: 16 warps in one block 5.0, 2 blocks of 8 5.8, 4 of 8 6.2; Q = 1024: one of 16 6.5,
+// 2 of 8 7.0, 3 of 8 (spills) 4.8; Q = 2048: one of 16 7.2, 2 of 8 7.15.  NT = 16 also where two
+// blocks' B-marginals do not fit in Tensor Memory.
+template <int Q, int NT_>
 struct RowTmCfg {
-    static constexpr int L = Q / 2;
-    // Q = 512: a one-warp team needs M = 8, R = 4 (256 = 4 * 8^2).  Q <= 1024: one
-    // pass holds the whole row (the team's scratch has room for it: at 1024 the
-    // load-once radix-2 buffer), fewer barriers and TMEM round trips per round
-    static constexpr int MMAX = Q <= 512 ? 8 : 32;
+    static constexpr int L = Q / 2, PTS = L / 32, H = PTS / 2, RS = 32 / PTS;
+    // Q <= 1024: one pass holds the whole row, fewer barriers and TMEM round trips per
+    // round; at 2048 the counts of a round go to their owners in two passes
     static constexpr int HALVES = Q <= 1024 ? 1 : 2;
-    using G = TeamGeom<float, L, MMAX>;
-    static constexpr int M = G::M, R = G::R, TEAM = G::TEAM;
-    static constexpr int NT = 16, THREADS = NT * 32;
+    static constexpr int NT = NT_, THREADS = NT * 32, BLOCKS = NT == 16 ? 1 : Q == 512 ? 4 : 2;
     static constexpr int QH = Q / HALVES;        // positions per pass
-    static constexpr int UH = QH / THREADS;      // positions per thread per pass: UH t .. UH t + UH - 1 (adjacent,
-                                                 // so that the counts of one thread come in one shared load)
+    static constexpr int UH = QH / THREADS;      // positions per thread per pass: adjacent floats of the hand-over
     static constexpr int U = HALVES * UH;
-    // radix-2 teams (Q = 1024) load every input once through a buffer of 2 M^2 complex
-    static constexpr bool ONCE = R == 2;
-    static constexpr int XS = ONCE ? R * M * M * 8 : 0;
-    static constexpr int REGION = G::SCRATCH > XS ? G::SCRATCH : XS;  // FFT scratch / one pass of rounded counts
-    static constexpr int STAGE_BYTES = ((L + 1) * 8 + 15) / 16 * 16;  // one Y row (Qh complex), 16-byte multiple
+    static constexpr int REGION = QH * 4;        // one pass of a pair's rounded counts
+    static constexpr int STAGE_BYTES = L * 8;    // one Y row, then the transpose planes
     static constexpr size_t OFF_STAGE = (size_t)NT * REGION;
     static constexpr size_t OFF_BAR = OFF_STAGE + (size_t)NT * STAGE_BYTES;
     static constexpr size_t OFF_HOLD = OFF_BAR + NT * 8;
-    static constexpr int NQ = M * M;
-    static constexpr int TW_PRE = R > 1 ? (R - 1) * NQ + 1 : 0;
-    static constexpr size_t OFF_TW = OFF_HOLD + 16;                   // twiddles staged in shared memory:
-    static constexpr size_t SMEM = OFF_TW + (size_t)(NQ + L + TW_PRE) * 8;  // four-step, C2R, pre-step
-    static_assert(TEAM == 32, "one warp per transform");
-    static_assert(UH >= 1 && QH % THREADS == 0, "whole positions per thread");
-    static_assert(REGION >= QH * 4, "scratch holds one pass");
+    static constexpr size_t OFF_TW1 = OFF_HOLD + 16;                       // twiddles, as float4
+    static constexpr size_t OFF_TW2 = OFF_TW1 + (size_t)H * 32 * 16;
+    static constexpr size_t SMEM = OFF_TW2 + (RS > 1 ? (size_t)RS * H * 16 : 0);
+    static_assert(UH == 1 || UH == 2 || UH == 4, "one, two or four positions per thread and pass");
+    static_assert((size_t)NT * REGION >= (size_t)Q * 12, "the hand-over region holds a row of MI and N");
+    // Position (0 .. Q) of float f of pass hf in a pair's hand-over region: slot f / 2 of lane
+    // l = slot % 32 holds values q and q + H of the lane, real or imaginary part
+    static __device__ __forceinline__ int position(int hf, int f) {
+        const int slot = f >> 1, l = slot & 31, qc = slot >> 5;
+        const int q = hf * (H / HALVES) + (qc >> 1) + (f & 1) * H;
+        return 2 * (l + 32 * q) + (qc & 1);
+    }
 };
 
-// TMEM columns one thread needs: K_B marginals x U positions; four warps share a lane quadrant.
-__host__ __device__ constexpr int tm_cols_needed(int KB, int U) { return 4 * KB * U; }
+// TMEM columns a block needs: K_B marginals x U = Q / (32 NT) positions per thread, NT / 4
+// warps per lane quadrant.
+__host__ __device__ constexpr int tm_cols_needed(int KB, int Q) { return KB * (Q / 128); }
 __host__ __device__ constexpr int tm_alloc_cols(int need) {
     return need <= 32 ? 32 : need <= 64 ? 64 : need <= 128 ? 128 : need <= 256 ? 256 : 512;
 }
@@ -155,9 +272,9 @@ __host__ __device__ constexpr int tm_alloc_cols(int need) {
 // residuals) and the diagnostics of the bounded waits (poll limit, withheld
 // copy).  They are separate instantiations because the plain kernel sits at
 // the register limit.
-template <int Q, bool NMI, int MODE>
-__global__ void __launch_bounds__(RowTmCfg<Q>::THREADS, 1)
-k_pair_rows_tm(const cpx<float>* __restrict__ Y, Geom g, Tw<float> tw, double* __restrict__ mi_map,
+template <int Q, bool NMI, int MODE, int NTEAMS>
+__global__ void __launch_bounds__(RowTmCfg<Q, NTEAMS>::THREADS, RowTmCfg<Q, NTEAMS>::BLOCKS)
+k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, double* __restrict__ mi_map,
                int32_t* __restrict__ n_map, DevStatus* __restrict__ st,
                int tm_cols, int wait_polls, int withhold_row, int conditional, const int32_t* __restrict__ ov,
                const int* __restrict__ ov_slot, unsigned* __restrict__ pair_res) {
@@ -167,32 +284,38 @@ k_pair_rows_tm(const cpx<float>* __restrict__ Y, Geom g, Tw<float> tw, double* _
     // only when the status word asks for the re-run.  ov, ov_slot, pair_res: the
     // exact counts of second-precision pairs and the per-pair residuals, as in
     // k_pair_rows.
-    using C = RowTmCfg<Q>;
+    using C = RowTmCfg<Q, NTEAMS>;
     constexpr bool EXT = MODE == 2, MULTI = MODE >= 1;
     if (EXT && conditional && !(st->flags & STATUS_ESCALATE)) return;  // uniform, before any set-up
     if (!EXT) {
         wait_polls = kDefaultWaitPolls;
         withhold_row = -1;
     }
-    constexpr int M = C::M, R = C::R, L = C::L, NT = C::NT, U = C::U, UH = C::UH, QH = C::QH, HALVES = C::HALVES;
+    constexpr int L = C::L, NT = C::NT, U = C::U, UH = C::UH, HALVES = C::HALVES, PTS = C::PTS, H = C::H;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int tid = threadIdx.x, team = tid >> 5, lane = tid & 31, r = lane / M, j = lane % M;
-    unsigned char* region = smem_raw + (size_t)team * C::REGION;
-    const cpx<float>* stage = reinterpret_cast<const cpx<float>*>(smem_raw + C::OFF_STAGE + (size_t)team * C::STAGE_BYTES);
+    const int tid = threadIdx.x, team = tid >> 5, lane = tid & 31;
+    float2* region = reinterpret_cast<float2*>(smem_raw + (size_t)team * C::REGION);
+    float* stage = reinterpret_cast<float*>(smem_raw + C::OFF_STAGE + (size_t)team * C::STAGE_BYTES);
     const uint32_t stage_s = smem_u32(stage);
     const uint32_t bar = smem_u32(smem_raw + C::OFF_BAR + team * 8);
     uint32_t* hold = reinterpret_cast<uint32_t*>(smem_raw + C::OFF_HOLD);
-    __shared__ int s_abort;
 
-    const int KA = g.KA, KB = g.KB, npairs = KA * KB, Rout = g.R, Cout = g.C, Qs = g.Qs;
-    cpx<float>* tw_sq = reinterpret_cast<cpx<float>*>(smem_raw + C::OFF_TW);
-    cpx<float>* twq_c2r = tw_sq + C::NQ;
-    cpx<float>* tw_pre = twq_c2r + L;
-    stage_table(tw_sq, tw.sq[ilog2c(M)], C::NQ);
-    stage_table(twq_c2r, tw_of<Q>(tw), L);
-    if (R > 1) stage_table(tw_pre, tw_of<L>(tw), C::TW_PRE);
+    const int KA = g.KA, KB = g.KB, npairs = KA * KB, Rout = g.R, Cout = g.C;
+    float4* tw1 = reinterpret_cast<float4*>(smem_raw + C::OFF_TW1);
+    float4* tw2 = reinterpret_cast<float4*>(smem_raw + C::OFF_TW2);
+    for (int i = tid; i < H * 32; i += C::THREADS) {
+        const int k = i >> 5, j = i & 31;
+        const cpx<float> a = tw_of<L>(tw)[j * k], b = tw_of<L>(tw)[j * (k + H)];
+        tw1[i] = make_float4(a.x, b.x, a.y, b.y);
+    }
+    if (C::RS > 1) {
+        for (int i = tid; i < C::RS * H; i += C::THREADS) {
+            const int r = i / H, m = i % H;
+            const cpx<float> a = tw_of<32>(tw)[2 * m * r], b = tw_of<32>(tw)[(2 * m + 1) * r];
+            tw2[i] = make_float4(a.x, b.x, a.y, b.y);
+        }
+    }
 
-    if (tid == 0) s_abort = 0;
     if (lane == 0) mbar_init(bar, 1);
     if (team == 0) tmem_alloc(smem_u32(hold), (uint32_t)tm_cols);
     mbar_fence_init();
@@ -212,8 +335,7 @@ k_pair_rows_tm(const cpx<float>* __restrict__ Y, Geom g, Tw<float> tw, double* _
         if (EXT && row_i == withhold_row && pair_i == 0) return;  // diagnostics: leave this wait without its copy
         if (lane == 0) {
             fence_proxy_async_smem();
-            const cpx<float>* src = Y + ((size_t)pair_i * Rout + row_i) * Qs;
-            tma_bulk_g2s(stage_s, src, C::STAGE_BYTES, bar);
+            tma_row_g2s(stage_s, &ymap, row_i, pair_i, C::STAGE_BYTES, bar);
         }
         pending = true;
     };
@@ -227,9 +349,8 @@ k_pair_rows_tm(const cpx<float>* __restrict__ Y, Geom g, Tw<float> tw, double* _
         const int row = MULTI ? rbase + rr : rr;
         EntAcc<NMI> S[U];
         float CA[U];
-        int N[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) { S[u].zero(); CA[u] = 0.f; N[u] = 0; }
+        for (int u = 0; u < U; ++u) { S[u].zero(); CA[u] = 0.f; }
         {   // zero this thread's B-marginal columns
             uint32_t z[16];
 #pragma unroll
@@ -244,50 +365,53 @@ k_pair_rows_tm(const cpx<float>* __restrict__ Y, Geom g, Tw<float> tw, double* _
         for (int base = 0; base < npairs; base += NT) {
             const int pair = base + team;
             const bool act = pair < npairs;
+            // A team without a pair in this round leaves its buffer alone (the copy of its
+            // next row's pair may be in flight into it); its counts are never read.
+            float2 re[H], im[H];
+            int timeout = 0;
             if (act) {
                 if (mbar_wait_bounded(bar, phase, wait_polls)) {
                     phase ^= 1u;
                     pending = false;
                 } else {
                     atomicOr(&st->flags, STATUS_TIMEOUT);
-                    s_abort = 1;
+                    timeout = 1;
                 }
-            }
-            // Hermitian split: z = IDFT_L(E + iO), z[m] = x[2m] + i x[2m+1].  With
-            // t = e^{-2 pi i k/Q} from the table: E = y_k + conj(y_{L-k}),
-            // iO = (y_k - conj(y_{L-k})) * i conj(t) = d * (t.y, t.x); packed adds.
-            auto load = [&](int k) -> cpx<float> {
-                if (!act) return {0.f, 0.f};
-                const float2 yk = reinterpret_cast<const float2*>(stage)[k];
-                const float2 ym = reinterpret_cast<const float2*>(stage)[L - k];
-                const float2 e = __ffma2_rn(ym, make_float2(1.f, -1.f), yk);
-                const float2 d = __ffma2_rn(ym, make_float2(-1.f, 1.f), yk);
-                const cpx<float> t = twq_c2r[k];
-                const cpx<float> io = cmul(cpx<float>{d.x, d.y}, cpx<float>{t.y, t.x});
-                const float2 z = __fadd2_rn(e, make_float2(io.x, io.y));
-                return {z.x, z.y};
-            };
-            cpx<float> v[M];
-            if constexpr (R == 1 && M == 32 && C::STAGE_BYTES >= M * M * 8) {
-                // the staged row is consumed by the loads: its buffer takes the one-pass
-                // complex transpose (the next copy into it is issued after the transform).
-                // A team without a pair in this round must leave the buffer alone: the copy
-                // of its next row's pair may already be in flight into it.
-                if (act) {
+                // the lane's inputs z[lane + 32 i] in pairs (layout of Y, kernels.cuh): the
+                // direct halves of chunks 32 m + lane, then the mirrored halves of lane -lane
+                const float4* sg4 = reinterpret_cast<const float4*>(stage);
+                const int jj = (32 - lane) & 31;
+                const float4* dsrc = sg4 + 2 * lane + ((lane >> 2) & 1);
+                const float4* msrc = sg4 + 2 * jj + (1 ^ ((jj >> 2) & 1));
 #pragma unroll
-                    for (int i = 0; i < M; ++i) v[i] = load(j + M * i);
-                    team_fft_core<M, +1, false, true, 3>(v, j, const_cast<cpx<float>*>(stage), tw_sq);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < M; ++i) v[i] = {0.f, 0.f};
+                for (int m = 0; m < H / 2; ++m) {
+                    const float4 d = dsrc[64 * m], w = msrc[64 * (H / 2 - 1 - m)];
+                    re[m] = make_float2(d.x, d.y);
+                    im[m] = make_float2(d.z, d.w);
+                    re[H / 2 + m] = make_float2(w.x, w.y);
+                    im[H / 2 + m] = make_float2(w.z, w.w);
                 }
+                {   // column 0's mirrors come in the other order and one pair off (its own mirror is
+                    // L / 2): lane 0's even inputs are the previous pair's second values
+                    float pr = re[H - 1].y, pi = im[H - 1].y;
+#pragma unroll
+                    for (int m = H / 2; m < H; ++m) {
+                        const float2 tr = re[m], ti = im[m];
+                        re[m].x = lane == 0 ? pr : tr.x;
+                        im[m].x = lane == 0 ? pi : ti.x;
+                        re[m].y = lane == 0 ? tr.x : tr.y;
+                        im[m].y = lane == 0 ? ti.x : ti.y;
+                        pr = tr.y;
+                        pi = ti.y;
+                    }
+                }
+                warp_fft_inv<PTS>(re, im, lane, stage, tw1, tw2);
             } else {
-                team_fft<M, R, +1, false, C::ONCE, false, 3>(v, r, j, load, region + r * grp_scratch_bytes<float, M>(),
-                                                                 tw_sq, tw_pre);
+#pragma unroll
+                for (int k = 0; k < H; ++k) re[k] = im[k] = make_float2(0.f, 0.f);
             }
             // the staging buffer is free again: prefetch this team's next active item
             // (the next round of this row, else round 0 of its next row)
-            __syncwarp();
             if (act && !pending) {
                 if constexpr (MULTI) {
                     int nb = rbase, nrr = rr, npair = pair + NT;
@@ -304,17 +428,18 @@ k_pair_rows_tm(const cpx<float>* __restrict__ Y, Geom g, Tw<float> tw, double* _
                 }
             }
             float rp = 0.f;
-#pragma unroll
-            for (int k = 0; k < M; ++k) {
-                // nearest integers (the 1.5 * 2^23 shift, packed) and the residual
-                const float2 x = make_float2(v[k].x, v[k].y);
+            auto round2 = [&](float2& x) {  // nearest integers (the 1.5 * 2^23 shift) and the residual
                 const float2 c = __fadd2_rn(__fadd2_rn(x, make_float2(12582912.0f, 12582912.0f)),
                                             make_float2(-12582912.0f, -12582912.0f));
-                const float2 dv = __ffma2_rn(c, make_float2(-1.f, -1.f), x);
+                const float2 dv = subv(x, c);
                 if constexpr (EXT) rp = fmaxf(rp, fmaxf(fabsf(dv.x), fabsf(dv.y)));
                 else res_max = fmaxf(res_max, fmaxf(fabsf(dv.x), fabsf(dv.y)));
-                v[k].x = c.x;
-                v[k].y = c.y;
+                x = c;
+            };
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                round2(re[k]);
+                round2(im[k]);
             }
             const int ovs = (EXT && act && ov_slot) ? ov_slot[pair] : -1;  // loaded after the transform: fewer live registers
             if (EXT && ovs < 0) res_max = fmaxf(res_max, rp);
@@ -325,103 +450,124 @@ k_pair_rows_tm(const cpx<float>* __restrict__ Y, Geom g, Tw<float> tw, double* _
             }
             const int nt = min(NT, npairs - base);
             const int a0 = base / KB, b0 = base - a0 * KB;
-            const bool fast = (KB == NT) && (b0 == 0);  // the round is exactly (a0, b = 0..15)
 #pragma unroll
             for (int hf = 0; hf < HALVES; ++hf) {
-                __syncthreads();
-                float2* ob = reinterpret_cast<float2*>(region);
-                if (EXT && ovs >= 0) {  // exact counts of positions 2 mf, 2 mf + 1 from the second precision
+                if (aborted) continue;
+                // every thread is done with the region's previous counts; a team whose copy
+                // never came ends the block
+                if (hf == 0) {
+                    aborted = __syncthreads_or(timeout);
+                    if (aborted) continue;
+                } else {
+                    __syncthreads();
+                }
+                constexpr int HP = H / HALVES;
+                if (EXT && ovs >= 0) {  // exact counts of positions 2 z, 2 z + 1 from the second precision
                     const int32_t* ovr = ov + ((size_t)ovs * Rout + row) * Q;
 #pragma unroll
-                    for (int k2 = hf * (M / HALVES); k2 < (hf + 1) * (M / HALVES); ++k2) {
-                        const int mf = R * (j + M * k2) + r;
-                        const int2 q = *reinterpret_cast<const int2*>(ovr + 2 * mf);
-                        ob[mf - hf * (L / HALVES)] = make_float2((float)q.x, (float)q.y);
+                    for (int q = 0; q < HP; ++q) {
+                        const int z = lane + 32 * (hf * HP + q);
+                        const int2 x = *reinterpret_cast<const int2*>(ovr + 2 * z);
+                        const int2 y = *reinterpret_cast<const int2*>(ovr + 2 * (z + 32 * H));
+                        region[2 * q * 32 + lane] = make_float2((float)x.x, (float)y.x);
+                        region[(2 * q + 1) * 32 + lane] = make_float2((float)x.y, (float)y.y);
                     }
                 } else {
 #pragma unroll
-                    for (int k2 = hf * (M / HALVES); k2 < (hf + 1) * (M / HALVES); ++k2) {
-                        const int m = R * (j + M * k2) + r - hf * (L / HALVES);
-                        const cpx<float> z = v[brev(k2, M)];
-                        ob[m] = make_float2(z.x, z.y);
+                    for (int q = 0; q < HP; ++q) {
+                        region[2 * q * 32 + lane] = re[hf * HP + q];
+                        region[(2 * q + 1) * 32 + lane] = im[hf * HP + q];
                     }
                 }
                 __syncthreads();
                 const uint32_t tcol = tbase + (uint32_t)(hf * KB * UH);
-                if (fast) {
-                    // all 16 B-marginals of this pass in registers: one TMEM load / store
-                    if (a0 != cur_a[hf]) {
+                // NB pairs of one label a, labels b .. b + NB - 1: their B-marginals of this pass in
+                // registers, one TMEM load and store
+                auto accum = [&](auto nbc, int t0, int b) {
+                    constexpr int NB = decltype(nbc)::value;
+                    uint32_t cbr[NB * UH];
+                    tmem_ld<NB * UH>(tcol + (uint32_t)(b * UH), cbr);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int t = 0; t < NB; ++t) {
+                        const float* obt = reinterpret_cast<const float*>(smem_raw + (size_t)(t0 + t) * C::REGION);
+                        if constexpr (UH == 1) {
+                            const float c = obt[tid];
+                            S[hf].joint(clog2c_biased(c));
+                            CA[hf] += c;
+                            cbr[t] = __float_as_uint(__uint_as_float(cbr[t]) + c);
+                        } else {
+                            float cv[UH];
+                            if constexpr (UH == 4) {
+                                const float4 q = reinterpret_cast<const float4*>(obt)[tid];
+                                cv[0] = q.x; cv[1] = q.y; cv[2] = q.z; cv[3] = q.w;
+                            } else {
+                                const float2 q = reinterpret_cast<const float2*>(obt)[tid];
+                                cv[0] = q.x; cv[1] = q.y;
+                            }
+#pragma unroll
+                            for (int w = 0; w < UH; w += 2) {
+                                const float2 c = make_float2(cv[w], cv[w + 1]);
+                                const int u = hf * UH + w, i = t * UH + w;
+                                long long x, y;
+                                clog2c_biased2(c, x, y);
+                                S[u].joint(x);
+                                S[u + 1].joint(y);
+                                const float2 ca = __fadd2_rn(make_float2(CA[u], CA[u + 1]), c);
+                                CA[u] = ca.x;
+                                CA[u + 1] = ca.y;
+                                const float2 m = __fadd2_rn(make_float2(__uint_as_float(cbr[i]), __uint_as_float(cbr[i + 1])), c);
+                                cbr[i] = __float_as_uint(m.x);
+                                cbr[i + 1] = __float_as_uint(m.y);
+                            }
+                        }
+                    }
+                    tmem_st<NB * UH>(tcol + (uint32_t)(b * UH), cbr);
+                    tmem_wait_st();
+                };
+                int a = a0, b = b0, t = 0;
+                while (t < nt) {
+                    if (a != cur_a[hf]) {
 #pragma unroll
                         for (int uh = 0; uh < UH; ++uh) {
                             const int u = hf * UH + uh;
-                            S[u].marg(clog2c_fixed(CA[u]));
-                            N[u] += (int)CA[u];
+                            S[u].marg(clog2c_biased(CA[u]));
                             CA[u] = 0.f;
                         }
-                        cur_a[hf] = a0;
+                        cur_a[hf] = a;
                     }
-                    uint32_t cbr[16 * UH];
-                    if constexpr (UH == 2) tmem_ld<32>(tcol, cbr);
-                    else tmem_ld<16>(tcol, cbr);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int t = 0; t < 16; ++t) {
-                        const float* obt = reinterpret_cast<const float*>(smem_raw + (size_t)t * C::REGION);
-#pragma unroll
-                        for (int uh = 0; uh < UH; ++uh) {
-                            const int u = hf * UH + uh, pl = UH * tid + uh;
-                            const float c = obt[pl];
-                            S[u].joint(clog2c_fixed(c));
-                            CA[u] += c;
-                            cbr[t * UH + uh] = __float_as_uint(__uint_as_float(cbr[t * UH + uh]) + c);
-                        }
+                    const int seg = min(KB - b, nt - t);  // the rest of label a in this round
+                    int d;
+                    if (UH <= 2 && seg >= 16) {
+                        accum(std::integral_constant<int, UH <= 2 ? 16 : 8>{}, t, b);
+                        d = 16;
+                    } else if (seg >= 8) {
+                        accum(std::integral_constant<int, 8>{}, t, b);
+                        d = 8;
+                    } else {
+                        accum(std::integral_constant<int, 1>{}, t, b);
+                        d = 1;
                     }
-                    if constexpr (UH == 2) tmem_st<32>(tcol, cbr);
-                    else tmem_st<16>(tcol, cbr);
-                    tmem_wait_st();
-                } else {
-                    int a = a0, b = b0;
-                    for (int t = 0; t < nt; ++t) {
-                        if (a != cur_a[hf]) {
-#pragma unroll
-                            for (int uh = 0; uh < UH; ++uh) {
-                                const int u = hf * UH + uh;
-                                S[u].marg(clog2c_fixed(CA[u]));
-                                N[u] += (int)CA[u];
-                                CA[u] = 0.f;
-                            }
-                            cur_a[hf] = a;
-                        }
-                        uint32_t cbr[UH];
-                        tmem_ld<UH>(tcol + (uint32_t)(b * UH), cbr);
-                        tmem_wait_ld();
-                        const float* obt = reinterpret_cast<const float*>(smem_raw + (size_t)t * C::REGION);
-#pragma unroll
-                        for (int uh = 0; uh < UH; ++uh) {
-                            const int u = hf * UH + uh, pl = UH * tid + uh;
-                            const float c = obt[pl];
-                            S[u].joint(clog2c_fixed(c));
-                            CA[u] += c;
-                            cbr[uh] = __float_as_uint(__uint_as_float(cbr[uh]) + c);
-                        }
-                        tmem_st<UH>(tcol + (uint32_t)(b * UH), cbr);
-                        tmem_wait_st();
-                        if (++b == KB) { b = 0; ++a; }
-                    }
+                    t += d;
+                    b += d;
+                    if (b == KB) { b = 0; ++a; }
                 }
             }
-            __syncthreads();  // the next round's transforms overwrite the scratch read above
-            if (s_abort) { aborted = true; break; }
+            if (aborted) break;
         }
         if (aborted) break;
-        // finish the row: last A-marginal, the B-marginals, MI
+        __syncthreads();  // the last counts are read
+        // finish the row: last A-marginal, the B-marginals, then MI and N through the
+        // hand-over region (doubles, then integers), so that the map is written in order
+        double* mrow = reinterpret_cast<double*>(smem_raw);
+        int* nrow_s = reinterpret_cast<int*>(smem_raw + (size_t)Q * 8);
 #pragma unroll
         for (int hf = 0; hf < HALVES; ++hf) {
+            float n[UH];  // N = the sum of the B-marginals (exact: below 2^23)
 #pragma unroll
             for (int uh = 0; uh < UH; ++uh) {
-                const int u = hf * UH + uh;
-                S[u].marg(clog2c_fixed(CA[u]));
-                N[u] += (int)CA[u];
+                S[hf * UH + uh].marg(clog2c_biased(CA[hf * UH + uh]));
+                n[uh] = 0.f;
             }
             for (int b = 0; b < KB; ++b) {
                 uint32_t cbr[UH];
@@ -429,20 +575,28 @@ k_pair_rows_tm(const cpx<float>* __restrict__ Y, Geom g, Tw<float> tw, double* _
                 tmem_wait_ld();
 #pragma unroll
                 for (int uh = 0; uh < UH; ++uh) {
-                    const float cbv = __uint_as_float(cbr[uh]);
-                    S[hf * UH + uh].marg(clog2c_fixed(cbv));
+                    const float c = __uint_as_float(cbr[uh]);
+                    S[hf * UH + uh].marg(clog2c_biased(c));
+                    n[uh] += c;
                 }
             }
 #pragma unroll
             for (int uh = 0; uh < UH; ++uh) {
-                const int u = hf * UH + uh;
-                const int cidx = circ_to_out(hf * QH + UH * tid + uh, Q, g.WA, g.WB - 1);
-                if (cidx < 0) continue;
-                const size_t o = (size_t)row * Cout + cidx;
-                mi_map[o] = S[u].finish(N[u]);
-                if (n_map) n_map[o] = N[u];
-                if (cidx >= g.c0 && cidx < g.c1) row_max_n = max(row_max_n, N[u]);
+                const int p = C::position(hf, UH * tid + uh), ni = (int)n[uh];
+                mrow[p] = S[hf * UH + uh].finish(ni);
+                nrow_s[p] = ni;
             }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int p = tid + C::THREADS * u, cidx = circ_to_out(p, Q, g.WA, g.WB - 1);
+            if (cidx < 0) continue;
+            const size_t o = (size_t)row * Cout + cidx;
+            const int n = nrow_s[p];
+            mi_map[o] = mrow[p];
+            if (n_map) n_map[o] = n;
+            if (cidx >= g.c0 && cidx < g.c1) row_max_n = max(row_max_n, n);
         }
         __syncthreads();
         if constexpr (MULTI) {  // past the unit's last row: the next unit's first

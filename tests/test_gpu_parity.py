@@ -136,6 +136,29 @@ def test_wide_rows_tmem_partial_rounds(cm, W, Q, K):
     assert float(np.abs(g["mi"] - ref["mi"]).max()) <= MI_TOL
 
 
+# Every transform length, across rows (Q) and down columns (P): maps just over the next
+# shorter length and maps that fill it.  Column 0 (which carries two real columns), the
+# mirrored columns and the first and last chunk of each length take part.
+LENGTHS = [16, 32, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048, 3072, 4096]
+
+
+@pytest.mark.parametrize("axis", ["rows", "columns"])
+@pytest.mark.parametrize("N", LENGTHS)
+def test_every_transform_length(cm, N, axis):
+    rng = np.random.default_rng(N)
+    lo = max([n for n in LENGTHS if n < N], default=0) + 1
+    for n in (lo, N):
+        a, b = n - n // 3, n // 3 + 1  # a + b - 1 = n
+        HA, WA, HB, WB = (9, a, 6, b) if axis == "rows" else (a, 9, b, 6)
+        A, MA, B, MB = _rand(rng, HA, WA, HB, WB, 5, 4)
+        ref = oracle.cmif(A, MA, B, MB, 5, 4)
+        for prec in ("FP32", "FP64") if N & (N - 1) == 0 else ("FP32",):
+            g = run_gpu(cm, A, MA, B, MB, 5, 4, getattr(cm, prec), counts=False, gamma=0.5)
+            assert g["status"][0] == "OK", g["status"]
+            np.testing.assert_array_equal(g["n"], ref["n"])
+            assert float(np.abs(g["mi"] - ref["mi"]).max()) <= MI_TOL
+
+
 @pytest.mark.parametrize("shape,K", WIDE[:3], ids=lambda x: "x".join(map(str, x)))
 def test_wide_rows_tmem_auto(cm, shape, K, monkeypatch):
     """CMIF_AUTO at the Tensor-Memory widths: the row kernel's AUTO form (exact
