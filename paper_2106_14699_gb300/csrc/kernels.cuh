@@ -523,9 +523,18 @@ struct PairColsCfg {
     static constexpr size_t MAIN = (size_t)TPB * P * sizeof(cpx<T>);
     static constexpr int TW_N = R == 2 ? P / 2 : (R > 2 ? P : 0);  // combine twiddles W_P^k
     static constexpr size_t SMEM = MAIN + (size_t)(NQ + TW_N) * sizeof(cpx<T>);
-    // FP32: two blocks per SM (M = 32 needs 128 registers a thread, so 256 threads);
-    // radix 6 and 8 combines hold too many values for that
-    static constexpr int MIN_BLOCKS = sizeof(T) == 4 && (M < 32 ? R < 6 && is_pow2(R) && THREADS <= 512 : THREADS <= 256) ? 2 : 1;
+    // Resident blocks the registers are bounded for.  FP32, measured in ps per point with
+    // 1 / 2 / 3 / 4 blocks: P = 64 - / 3.58 / 3.10 / 3.03, 128 - / 3.31 / 2.92 / 2.76, 192 - / 3.85 /
+    // - / 2.94, 256 - / 2.80 / 2.88 / 3.20, 384 4.01 / 4.05 / 3.44 / -, 512 - / 2.82 / 2.83 / 3.01,
+    // 768 3.07 / 3.08 / 2.86 / 2.72, 1536 3.44 / 3.59: as many as hold the values of the transform
+    // and of the radix-R combine without spilling
+    static constexpr int f32_blocks() {
+        if (M == 32) return THREADS <= 256 ? 2 : 1;
+        if (R == 6) return M == 8 ? 3 : 1;
+        if (M == 16) return R == 3 ? 4 : R <= 2 ? 2 : 1;
+        return M == 8 ? 4 : 2;
+    }
+    static constexpr int MIN_BLOCKS = sizeof(T) == 4 ? f32_blocks() : 1;
 };
 
 // Pair product + inverse column transform of length P = R*M*M.  Persistent
@@ -755,10 +764,17 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
                     t[i] = __ldg(twq + kc);
                 }
             };
-            if constexpr (UPR == 1) load_t(c0);
-            for (int u = threadIdx.x; u < NQ * UPR; u += C::THREADS) {
-                const int h = UPR == 1 ? 0 : u / NQ, k = UPR == 1 ? u : u % NQ, c = c0 + h;
-                if (UPR > 1) {
+            // chunk by chunk where the threads divide its rows (twiddles loaded once per chunk),
+            // else all the block's chunks in one run
+            constexpr bool NEST = NQ % C::THREADS == 0 || UPR == 1;
+            for (int h0 = 0; h0 < (NEST ? UPR : 1); ++h0) {
+            if (NEST) {
+                if ((c0 + h0) * CH >= L) break;
+                load_t(c0 + h0);
+            }
+            for (int u = threadIdx.x; u < (NEST ? NQ : NQ * UPR); u += C::THREADS) {
+                const int h = NEST ? h0 : u / NQ, k = NEST ? u : u % NQ, c = c0 + h;
+                if (!NEST) {
                     if (c * CH >= L) break;
                     load_t(c);
                 }
@@ -798,6 +814,7 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
                     }
                     store_chunk<SPLIT>(yp + y_chunk<T>(orow, c, L), z);
                 }
+            }
             }
         };
         if (split) emit(std::true_type{});
