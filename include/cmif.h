@@ -70,9 +70,13 @@ typedef enum {
 /* Arithmetic of the FFT correlations.  Counts are exact when every pre-rounding
  * residual |c - round(c)| stays below 0.25 (checked on every call).
  *   CMIF_FP32   : FP32 transforms (fast; exact for balanced labels up to ~1024^2)
- *   CMIF_SPLIT32: two-term FP32 transforms (hi + lo floats, ~48 significant
- *                 bits from FP32 units; exact everywhere in range)
- *   CMIF_FP64   : FP64 transforms (exact everywhere in range; slow on GB300)
+ *   CMIF_SPLIT32,
+ *   CMIF_FP64   : exact counts everywhere in range.  The transforms run over the
+ *                 integers modulo 2^31 - 1 (complex residues), which gives every
+ *                 count without rounding: the residual is 0.  (Both names once
+ *                 stood for the floating-point arithmetic that reached the same
+ *                 counts; weighted maps, whose counts are real, keep FP64
+ *                 transforms.)
  *   CMIF_AUTO   : FP32 transforms with the precision chosen per label pair,
  *                 all on the device (no host round trip).  A predicate sends a
  *                 pair to the second precision up front when the estimated
@@ -83,9 +87,10 @@ typedef enum {
  *                 residual; pairs that still reach the guard are computed in
  *                 the second precision as well and the FP32 row pass runs once
  *                 more.  Only the listed pairs (at most 128 per map) pay for
- *                 the second precision.  The second precision is two-term FP32;
- *                 the environment variable CMIF_AUTO_TIER2=fp64 at plan creation
- *                 makes it FP64, CMIF_AUTO_PREDICATE=0 turns the predicate
+ *                 the second precision.  The second precision is the exact
+ *                 integer transform (the environment variable CMIF_AUTO_TIER2
+ *                 is accepted and changes nothing: every choice it named gave
+ *                 the same counts).  CMIF_AUTO_PREDICATE=0 turns the predicate
  *                 off (the guard alone then picks the pairs) and
  *                 CMIF_AUTO_PREDICATE=all sends every pair (up to the 128-pair
  *                 list) to the second precision (diagnostics). */
@@ -333,7 +338,7 @@ cmif_status cmif_get_status(cmif_plan plan, cmif_status* device_side, double* ma
  * up front, pairs_escalated = pairs sent there after their FP32 residual
  * reached the guard, residual_fp32 = the largest residual of the pairs whose
  * FP32 counts stood, residual_second = the largest residual of the
- * second-precision pairs (FP64 and two-term plans: their one residual; FP32
+ * second-precision pairs (FP64 and SPLIT32 plans: 0; FP32
  * plans: 0).  Any output pointer may be NULL. */
 cmif_status cmif_get_precision_report(cmif_plan plan, int* pairs_predicted, int* pairs_escalated,
                                       double* residual_fp32, double* residual_second);

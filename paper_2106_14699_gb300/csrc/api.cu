@@ -8,6 +8,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "cmif.h"
@@ -80,10 +81,9 @@ struct cmif_plan_s {
     cmif_precision prec = CMIF_FP32;
     unsigned flags = 0;
     Workspace<float> w32;
-    Workspace<double> w64;
-    Workspace<df32> ws32;  // two-term FP32 (split precision)
-    bool has32 = false, has64 = false;
-    cmif_precision tier2 = CMIF_SPLIT32;  // precision of AUTO's re-run
+    Workspace<double> w64;  // weighted plans
+    Workspace<m31> wm31;    // exact transforms: FP64 and two-term plans, AUTO's second precision
+    bool has32 = false, has64 = false, has_m31 = false;
     DevStatus* st = nullptr;      // status of the map being computed (reset per map)
     DevStatus* st_total = nullptr;  // status of the whole call (what cmif_get_status reports)
     PeakPart* parts = nullptr;
@@ -143,10 +143,10 @@ cmif_status choose_rows(cmif_plan p, Workspace<T>& w) {
     cudaError_t e = cudaSuccess;
     w.args.tm_cols = 0;
     const char* no_tm = std::getenv("CMIF_DISABLE_TMEM");
-    if (sizeof(T) == 4 && !(no_tm && no_tm[0] == '1')) {
+    if (std::is_same<T, float>::value && !(no_tm && no_tm[0] == '1')) {
         const int cols = rows_tm_cols(g.Q, g.KB);
         if (cols > 0) {
-            e = rows_tm_max_blocks_per_sm(g.Q, cols, &bps);
+            e = rows_tm_max_blocks_per_sm(g.Q, cols, g.KA * g.KB, &bps);
             if (e != cudaSuccess) return from_cuda(e);
             if (bps >= 1) w.args.tm_cols = cols;
         }
@@ -318,10 +318,9 @@ bool call_geom(const cmif_plan p, double gamma, Geom* out) {
 // the level-set transforms of the planes the listed pairs need, then, chunk by
 // chunk, their products, inverse column transforms and exact counts (into the
 // plan's ov buffer).  Every launch returns at once when the stage lists nothing.
-template <typename T>
-cudaError_t tier2_stage(cmif_plan p, Workspace<T>& w, const Geom& g, const int32_t* A, const uint8_t* MA,
-                        const int32_t* B, const uint8_t* MB, const int* lrange, cudaStream_t s) {
-    PipeArgs<T> b = w.args;
+cudaError_t tier2_stage(cmif_plan p, const Geom& g, const int32_t* A, const uint8_t* MA, const int32_t* B,
+                        const uint8_t* MB, const int* lrange, cudaStream_t s) {
+    PipeArgs<m31> b = p->wm31.args;
     fill_io(b, A, MA, B, MB, nullptr, nullptr, nullptr, p->st, p);
     b.prof = p->prof.enabled ? &p->prof : nullptr;
     b.prec_slot = 1;
@@ -329,7 +328,7 @@ cudaError_t tier2_stage(cmif_plan p, Workspace<T>& w, const Geom& g, const int32
     b.needA = p->esc.needA;
     b.needB = p->esc.needB;
     b.stages = STAGE_FWD_A | STAGE_FWD_B;
-    cudaError_t e = run_pipeline<T>(g, b, s);
+    cudaError_t e = run_pipeline<m31>(g, b, s);
     if (e != cudaSuccess) return e;
     b.needA = b.needB = nullptr;
     b.plist = p->esc.plist;
@@ -338,15 +337,10 @@ cudaError_t tier2_stage(cmif_plan p, Workspace<T>& w, const Geom& g, const int32
     b.chunk_cap = p->esc.chunk;
     for (int off = 0; off < p->esc.cap; off += p->esc.chunk) {
         b.chunk_off = off;
-        e = run_pair_counts<T>(g, b, s);
+        e = run_pair_counts<m31>(g, b, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
-}
-
-template <typename Fn>
-cudaError_t with_tier2(cmif_plan p, Fn&& fn) {
-    return p->tier2 == CMIF_FP64 ? fn(p->w64) : fn(p->ws32);
 }
 
 // CMIF_AUTO: FP32 transforms with per-pair precision.  The predicate picks the
@@ -382,7 +376,7 @@ cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const
     p->prof.end(s);
     // 3. second precision for the predicted pairs
     if (e == cudaSuccess)
-        e = with_tier2(p, [&](auto& w) { return tier2_stage(p, w, g, A, MA, B, MB, E.hdr + 0, s); });
+        e = tier2_stage(p, g, A, MA, B, MB, E.hdr + 0, s);
     // 4. FP32 pair stages; listed pairs take their exact counts, the others' residuals are kept per pair
     a.ov = E.ov;
     a.ov_slot = E.ov_slot;
@@ -396,7 +390,7 @@ cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const
     p->prof.end(s);
     // 6. second precision for them, 7. the FP32 row pass again (only after a breach)
     if (e == cudaSuccess)
-        e = with_tier2(p, [&](auto& w) { return tier2_stage(p, w, g, A, MA, B, MB, E.hdr + 1, s); });
+        e = tier2_stage(p, g, A, MA, B, MB, E.hdr + 1, s);
     a.stages = STAGE_ROWS;
     a.conditional = 1;
     if (e == cudaSuccess) e = run_pipeline<float>(g, a, s);
@@ -410,7 +404,7 @@ cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const
 
 // One full map into (mi, n, counts); its status in p->st (reset here) is folded
 // into p->st_total.  stages32 selects the FP32 stages (A's transforms may be
-// reused across calls); an FP64 or two-term pass always recomputes everything.
+// reused across calls); an exact pass (FP64 and two-term plans) always recomputes everything.
 cmif_status compute_map(cmif_plan p, const Geom& g, const int32_t* A, const uint8_t* MA, const int32_t* B,
                         const uint8_t* MB, double* mi, int32_t* n, int32_t* counts, cudaStream_t s,
                         unsigned stages32 = STAGE_ALL) {
@@ -425,22 +419,14 @@ cmif_status compute_map(cmif_plan p, const Geom& g, const int32_t* A, const uint
         a.prec_slot = 0;
         a.conditional = 0;
         e = run_pipeline<float>(g, a, s);
-    } else if (p->prec == CMIF_FP64) {
-        PipeArgs<double> a = p->w64.args;
-        fill_io(a, A, MA, B, MB, mi, n, counts, p->st, p);
-        a.prof = p->prof.enabled ? &p->prof : nullptr;
-        a.stages = STAGE_ALL;
-        a.prec_slot = 1;
-        a.conditional = 0;
-        e = run_pipeline<double>(g, a, s);
     } else {
-        PipeArgs<df32> a = p->ws32.args;
+        PipeArgs<m31> a = p->wm31.args;
         fill_io(a, A, MA, B, MB, mi, n, counts, p->st, p);
         a.prof = p->prof.enabled ? &p->prof : nullptr;
         a.stages = STAGE_ALL;
         a.prec_slot = 1;
         a.conditional = 0;
-        e = run_pipeline<df32>(g, a, s);
+        e = run_pipeline<m31>(g, a, s);
     }
     if (e != cudaSuccess) return from_cuda(e);
     const int slot_default = (p->prec == CMIF_FP64 || p->prec == CMIF_SPLIT32) ? 1 : 0;
@@ -475,8 +461,8 @@ cmif_status plan_init(cmif_plan p, int H_A, int W_A, int H_B, int W_B, int K_A, 
     g.R2 = H_A + H_B - 1;
     g.R = g.Dz * g.R2;
     g.C = W_A + W_B - 1;
-    // FP32 plans may take lengths 3 * 2^k (the two-term and FP64 kernels, and hence
-    // AUTO's second precision, exist for powers of two only)
+    // FP32 plans may take lengths 3 * 2^k (the exact and FP64 kernels, and hence AUTO's
+    // second precision, exist for powers of two only)
     const char* p2e = std::getenv("CMIF_POW2_ONLY");
     const bool mixed = prec == CMIF_FP32 && !(p2e && p2e[0] == '1');
     g.P = transform_size(g.R2, mixed);
@@ -525,25 +511,22 @@ cmif_status plan_init(cmif_plan p, int H_A, int W_A, int H_B, int W_B, int K_A, 
     p->prec = prec;
     p->flags = flags;
     p->use_graph = (flags & CMIF_FLAG_GRAPH) != 0;
-    const char* t2 = std::getenv("CMIF_AUTO_TIER2");  // "fp64" makes AUTO re-run in FP64 instead of split FP32
-    p->tier2 = (t2 && std::strcmp(t2, "fp64") == 0) ? CMIF_FP64 : CMIF_SPLIT32;
     cmif_status st = CMIF_OK;
     if (prec == CMIF_FP32 || prec == CMIF_AUTO) {
         st = choose_rows<float>(p, p->w32);
         p->has32 = (st == CMIF_OK);
     }
-    if (st == CMIF_OK && (prec == CMIF_FP64 || (prec == CMIF_AUTO && p->tier2 == CMIF_FP64))) {
-        st = choose_rows<double>(p, p->w64);
-        p->has64 = (st == CMIF_OK);
-        if (st == CMIF_OK && (flags & CMIF_FLAG_WEIGHTED)) {
-            int bps = 0;
-            if (rows_w_max_blocks_per_sm(g.Q, &bps) != cudaSuccess) return CMIF_ERR_CUDA;
-            if (bps < 1) return CMIF_ERR_UNSUPPORTED;
-            p->w64.rows_grid_w = std::min(g.R, bps * p->num_sms);
-        }
+    if (st == CMIF_OK && prec != CMIF_FP32) {
+        st = choose_rows<m31>(p, p->wm31);
+        p->has_m31 = (st == CMIF_OK);
     }
-    if (st == CMIF_OK && (prec == CMIF_SPLIT32 || (prec == CMIF_AUTO && p->tier2 == CMIF_SPLIT32))) {
-        st = choose_rows<df32>(p, p->ws32);
+    if (st == CMIF_OK && (flags & CMIF_FLAG_WEIGHTED)) {
+        int bps = 0;
+        if (rows_w_max_blocks_per_sm(g.Q, &bps) != cudaSuccess) return CMIF_ERR_CUDA;
+        if (bps < 1) return CMIF_ERR_UNSUPPORTED;
+        p->w64.rows_grid_w = std::min(g.R, bps * p->num_sms);
+        p->w64.args.num_sms = p->num_sms;
+        p->has64 = true;
     }
     if (st != CMIF_OK) return st;
     if (prec == CMIF_AUTO) {
@@ -551,12 +534,11 @@ cmif_status plan_init(cmif_plan p, int H_A, int W_A, int H_B, int W_B, int K_A, 
         // of listed pairs at a time (a few GB at most), and the exact counts of at
         // most `cap` listed pairs
         const int npairs = K_A * K_B;
-        const size_t per_pair = (size_t)g.R * g.Ys * (p->tier2 == CMIF_FP64 ? sizeof(cpx<double>) : sizeof(cpx<df32>));
+        const size_t per_pair = (size_t)y_rows<m31>(g.R) * g.Ys * sizeof(cpx<m31>);
         const size_t budget = 4ull << 30;
         p->esc.chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)npairs, budget / per_pair));
         p->esc.cap = std::min(npairs, 128);
-        if (p->tier2 == CMIF_FP64) p->w64.ypairs = p->esc.chunk;
-        else p->ws32.ypairs = p->esc.chunk;
+        p->wm31.ypairs = p->esc.chunk;
         // the predicate: an FFT correlation of two 0/1 planes errs by about
         // kappa u log2(PQ) sqrt(|X_a| |Y_b|) (u = 2^-24); kappa = 0.25 bounds the
         // residuals measured at 256^2 and 1024^2 with balanced labels (1024^2, K = 16:
@@ -573,15 +555,15 @@ cmif_status plan_init(cmif_plan p, int H_A, int W_A, int H_B, int W_B, int K_A, 
     const int nmi = (flags & CMIF_FLAG_NMI) ? 1 : 0;
     p->w32.args.nmi = nmi;
     p->w64.args.nmi = nmi;
-    p->ws32.args.nmi = nmi;
+    p->wm31.args.nmi = nmi;
     Tw<float> tf;
     Tw<double> td;
-    Tw<df32> ts;
-    e = get_twiddles(p->device, &tf, &td, &ts);
+    Tw<m31> tm;
+    e = get_twiddles(p->device, &tf, &td, &tm);
     if (e != cudaSuccess) return from_cuda(e);
     p->w32.args.tw = tf;
     p->w64.args.tw = td;
-    p->ws32.args.tw = ts;
+    p->wm31.args.tw = tm;
     p->nparts = 2 * p->num_sms;
     return CMIF_OK;
 }
@@ -631,12 +613,17 @@ void esc_carve(cmif_plan p, char* base) {
     E.bytes = off;
 }
 
+// The exact and the FP64 workspace: a weighted plan has both, for its weighted and its plain
+// maps, in the same memory (calls on a plan do not overlap).
+size_t exact_bytes(const cmif_plan p) {
+    return std::max(p->has64 ? workspace_bytes<double>(p->g, p->w64) : 0,
+                    p->has_m31 ? workspace_bytes<m31>(p->g, p->wm31) : 0);
+}
+
 size_t plan_bytes(cmif_plan p) {
     size_t b = small_bytes_of(p) + esc_bytes(p);
     if (p->has32) b += workspace_bytes<float>(p->gcap, p->w32);
-    if (p->has64) b += workspace_bytes<double>(p->g, p->w64);
-    if (p->ws32.rows_grid > 0) b += workspace_bytes<df32>(p->g, p->ws32);
-    return b;
+    return b + exact_bytes(p);
 }
 
 // Point the plan's buffers into base (plan_bytes long) and clear its status words.
@@ -658,12 +645,13 @@ cmif_status plan_carve(cmif_plan p, char* base) {
         carve_workspace<float>(p->gcap, p->w32, base + off);
         off += workspace_bytes<float>(p->gcap, p->w32);
     }
-    if (p->has64) { carve_workspace<double>(g, p->w64, base + off); off += workspace_bytes<double>(g, p->w64); }
-    if (p->ws32.rows_grid > 0) { carve_workspace<df32>(g, p->ws32, base + off); off += workspace_bytes<df32>(g, p->ws32); }
+    if (p->has64) carve_workspace<double>(g, p->w64, base + off);
+    if (p->has_m31) carve_workspace<m31>(g, p->wm31, base + off);
+    off += exact_bytes(p);
     if (p->prec == CMIF_AUTO) { esc_carve(p, base + off); off += p->esc.bytes; }
     p->w32.bytes = p->has32 ? workspace_bytes<float>(p->gcap, p->w32) : 0;
     p->w64.bytes = p->has64 ? workspace_bytes<double>(g, p->w64) : 0;
-    p->ws32.bytes = p->ws32.rows_grid > 0 ? workspace_bytes<df32>(g, p->ws32) : 0;
+    p->wm31.bytes = p->has_m31 ? workspace_bytes<m31>(g, p->wm31) : 0;
     if (cudaMemset(p->st, 0, 2 * align_up(sizeof(DevStatus), 256)) != cudaSuccess) return CMIF_ERR_CUDA;
     return CMIF_OK;
 }
@@ -888,7 +876,7 @@ void apply_tune(cmif_plan p, const TuneRec& r) {
 }
 
 cmif_status autotune(cmif_plan p, const char* cache_path, cmif_tuning* out) {
-    if (!p->has32) {  // FP64 / two-term plans: nothing to choose
+    if (!p->has32) {  // exact plans: nothing to choose
         if (out) *out = cmif_tuning{0, 0, 0, 0.0, 0, 0};
         return CMIF_OK;
     }

@@ -7,7 +7,7 @@ namespace cmif {
 // Device-side status word, one per plan; read back by cmif_get_status().
 struct DevStatus {
     unsigned flags;        // STATUS_* bits below
-    unsigned res_bits[2];  // max |c - round(c)| seen, as float bits: [0] FP32 pass, [1] FP64 pass
+    unsigned res_bits[2];  // max |c - round(c)| seen, as float bits: [0] FP32 pass, [1] exact pass (0)
     int max_n;             // max_chi N(chi) of the last map (for the gamma gate of Alg. 1)
     int escalations;       // CMIF_AUTO: label pairs re-run in the second precision after the FP32 guard breached
     int predicted;         // CMIF_AUTO: label pairs the precision predicate sent to the second precision up front
@@ -18,7 +18,7 @@ enum : unsigned {
     STATUS_LABEL_RANGE = 1u,  // a label under mask 1 lies outside [0, K)
     STATUS_PRECISION = 2u,    // residual guard breached in the final precision
     STATUS_TIMEOUT = 4u,      // a bounded device wait gave up
-    STATUS_ESCALATE = 8u,     // AUTO: FP32 residual breached, FP64 pass is authoritative
+    STATUS_ESCALATE = 8u,     // AUTO: FP32 residual breached, the exact counts are authoritative
 };
 
 // Problem geometry of one CMIF map.

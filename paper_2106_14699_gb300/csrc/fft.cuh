@@ -19,8 +19,9 @@
 // DIR = +1 the unnormalised inverse.
 #pragma once
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
-#include "df32.cuh"
+#include "m31.cuh"
 
 namespace cmif {
 
@@ -58,6 +59,18 @@ __device__ __forceinline__ cpx<T> rot(cpx<T> a, T c, T s) {
     if (DIR < 0) return {a.x * c + a.y * s, a.y * c - a.x * s};
     return {a.x * c - a.y * s, a.y * c + a.x * s};
 }
+
+// Residues mod p (m31.cuh): both products of a component in one 64-bit sum and one fold.
+__device__ __forceinline__ cpx<m31> cmul(cpx<m31> a, cpx<m31> b) {
+    return {m31_fold(m31_wide(a.x, b.x) + m31_wide(a.y, -b.y)), m31_fold(m31_wide(a.x, b.y) + m31_wide(a.y, b.x))};
+}
+__device__ __forceinline__ cpx<m31> cmulc(cpx<m31> a, cpx<m31> b) {
+    return {m31_fold(m31_wide(a.x, b.x) + m31_wide(a.y, b.y)), m31_fold(m31_wide(a.y, b.x) + m31_wide(a.x, -b.y))};
+}
+// x / 2
+template <typename T>
+__device__ __forceinline__ T halve(T x) { return T(0.5) * x; }
+__device__ __forceinline__ m31 halve(m31 x) { return m31_of((x.v >> 1) | ((x.v & 1) << 30)); }
 
 __host__ __device__ constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c(n >> 1); }
 __host__ __device__ constexpr int brev(int k, int M) {
@@ -99,6 +112,25 @@ __device__ __forceinline__ cpx<T> twc(cpx<T> d, int k) {
 
 // In-register M-point DFT, natural order in, bit-reversed order out:
 // after the call v[brev(k, M)] = sum_n v_in[n] e^{DIR 2 pi i n k / M}.
+// Residues: constants from the roots of unity; eighth turns are (1 +- i) 2^15, a rotation of
+// the 31 bits.
+template <int M, int DIR>
+__device__ __forceinline__ cpx<m31> twc(cpx<m31> d, int k) {
+    const int k32 = k * (32 / M);
+    if (k32 == 0) return d;
+    if (k32 == 8) return DIR < 0 ? cpx<m31>{d.y, -d.x} : cpx<m31>{-d.y, d.x};
+    if (k32 == 16) return {-d.x, -d.y};
+    if (k32 == 24) return DIR < 0 ? cpx<m31>{-d.y, d.x} : cpx<m31>{d.y, -d.x};
+    if (k32 == 4 || k32 == 12) {
+        auto rot15 = [](m31 a) { return m31_of(((a.v << 15) & kM31) | (a.v >> 16)); };
+        const m31 s = rot15(d.x + d.y), t = rot15(d.y - d.x);  // 4: (x -+ y, y +- x); 12: i times that
+        if (k32 == 4) return DIR < 0 ? cpx<m31>{s, t} : cpx<m31>{-t, s};
+        return DIR < 0 ? cpx<m31>{t, -s} : cpx<m31>{-s, -t};
+    }
+    const uint32_t c = m31_cos32(k32), sn = m31_sin32(k32);
+    return cmul(d, cpx<m31>{m31_of(c), m31_of(DIR < 0 ? kM31 - sn : sn)});
+}
+
 template <int M, int DIR, typename T>
 __device__ __forceinline__ void dft_reg(cpx<T> (&v)[M]) {
 #pragma unroll
@@ -123,7 +155,7 @@ namespace cmif {
 
 // Lanes per group for a team transform: the largest power of two M with M*M
 // dividing N (N = R M^2; for N = 2^k or 3 * 2^k), capped so that M complex
-// values fit in registers (32 for FP32, 16 for FP64).
+// values fit in registers (32 of 4-byte values, 16 of FP64).
 __host__ __device__ constexpr int team_m(int N, int mmax) {
     int M = mmax;
     while (M > 1 && (M * M > N || N % (M * M) != 0)) M >>= 1;
@@ -178,7 +210,7 @@ __device__ __forceinline__ void dft_nat(cpx<T> (&u)[R]) {
     }
 }
 template <typename T>
-__host__ __device__ constexpr int max_m() { return sizeof(T) == 4 ? 32 : 16; }  // FP32: 32; FP64 and two-term FP32: 16
+__host__ __device__ constexpr int max_m() { return sizeof(T) == 4 ? 32 : 16; }  // 4-byte values: 32; FP64: 16
 
 // Twiddle tables in device memory, filled once per device from FP64 values.
 //   n[l][k]         = e^{-2 pi i k / 2^l},           k < 2^l
@@ -208,7 +240,7 @@ __device__ __forceinline__ cpx<T> twl(const cpx<T>* __restrict__ t, int k) {
     return w;
 }
 
-// Shared-memory scratch of one group of M lanes.  FP32 transposes go through
+// Shared-memory scratch of one group of M lanes.  Transposes of 4-byte values go through
 // shared memory in two halves (real parts, then imaginary parts), so a group
 // needs M*M floats; groups narrower than a warp get M floats of padding so
 // that the groups of one warp hit disjoint banks.  FP64 transposes complex
@@ -321,7 +353,7 @@ __device__ __forceinline__ void team_core_pk(float2 (&re)[M / 2], float2 (&im)[M
 
 template <int M, int DIR, bool WIDE = false, typename T>
 __device__ __forceinline__ void team_fft_core(cpx<T> (&v)[M], int j, void* sm, const cpx<T>* __restrict__ twq) {
-    if constexpr (sizeof(T) == 4 && M >= 8) {
+    if constexpr (std::is_same<T, float>::value && M >= 8) {
         constexpr int H = M / 2;
         float2 re[H], im[H];
 #pragma unroll
@@ -340,7 +372,7 @@ __device__ __forceinline__ void team_fft_core(cpx<T> (&v)[M], int j, void* sm, c
 #pragma unroll
         for (int k1 = 1; k1 < M; ++k1) v[brev(k1, M)] = cmul(v[brev(k1, M)], twl<DIR>(twq, k1 * M + j));
         if constexpr (sizeof(T) == 4) {
-            float* sf = reinterpret_cast<float*>(sm);
+            T* sf = reinterpret_cast<T*>(sm);
             __syncwarp();
 #pragma unroll
             for (int k1 = 0; k1 < M; ++k1) sf[k1 * M + (j ^ k1)] = v[brev(k1, M)].x;

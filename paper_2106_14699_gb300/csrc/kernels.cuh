@@ -72,6 +72,23 @@ __device__ __forceinline__ void clog2c_biased2(float2 c, long long& t0, long lon
 // leaves no fraction bits).
 __device__ __forceinline__ float round_fp32(float v) { return (v + 12582912.0f) - 12582912.0f; }
 
+// (q1 + q2) * 2^-kFixBits as a double, |q2| at most a few ulp of q1 (so the sum of the two
+// 24-bit values fits 53 bits), by integer arithmetic: the same value that the double add
+// gives, but FP64 instructions run at 1/64 rate and the two conversions, the add and the
+// product took 4096 of the about 20000 cycles of a row of 4 label pairs at Q = 2048.
+__device__ __forceinline__ double double_sum_scaled(float q1, float q2) {
+    const int b = __float_as_int(q1);
+    if ((b & 0x7FFFFFFF) == 0) return 0.0;  // q1 = 0: the whole sum is 0
+    int e = (b >> 23) & 0xFF;
+    long long m = (long long)((b & 0x7FFFFF) | 0x800000) << 29;  // 2^52 <= m < 2^53, q1 = m 2^(e - 127 - 52)
+    const float q = b < 0 ? -q2 : q2;
+    m += __float2int_rn(q * __int_as_float((306 - e) << 23));     // q2 in units of m's last bit
+    if (m < (1LL << 52)) { m <<= 1; --e; }
+    if (m >= (1LL << 53)) { m >>= 1; ++e; }
+    const unsigned long long r = ((unsigned long long)(e - 127 - kFixBits + 1023) << 52) + (unsigned long long)(m - (1LL << 52));
+    return __longlong_as_double((long long)(r | ((unsigned long long)(b < 0) << 63)));
+}
+
 // MI(chi) = (S + N log2 N) / N, where S = sum_joint c log2 c - sum_A - sum_B and
 // every c log2 c term (N log2 N included) comes from clog2c_biased, so that MI is
 // exactly 0 whenever the entropies cancel exactly (e.g. a single label).
@@ -86,7 +103,7 @@ __device__ __forceinline__ double mi_finish(long long S, int N) {
     const float q1 = sh * inv;
     const float r1 = fmaf(-q1, fN, sh) + sl;
     const float q2 = r1 * inv;
-    return ((double)q1 + (double)q2) * (1.0 / (double)(1 << kFixBits));
+    return double_sum_scaled(q1, q2);
 }
 
 // NMI(chi) = (H_A + H_B) / H_AB (the normalised MI the paper cites next to
@@ -132,14 +149,16 @@ template <>
 __device__ __forceinline__ float rint_t<float>(float v) { return rintf(v); }
 template <>
 __device__ __forceinline__ double rint_t<double>(double v) { return rint(v); }
-// nearest integer to hi + lo (|hi + lo| < 2^23): round hi, then let lo move it by one
-template <>
-__device__ __forceinline__ df32 rint_t<df32>(df32 v) {
-    float r = rintf(v.hi);
-    const float d = (v.hi - r) + v.lo;  // v.hi - r is exact
-    if (d > 0.5f) r += 1.f;
-    else if (d < -0.5f) r -= 1.f;
-    return {r, 0.f};
+// A pre-rounding count -> the count as a float, and its residual; modular counts are exact.
+template <typename T>
+__device__ __forceinline__ float round_count(T v, float& res) {
+    if constexpr (std::is_same<T, m31>::value) {
+        return m31_count(v);
+    } else {
+        const T c = rint_t<T>(v);
+        res = fmaxf(res, (float)fabs(v - c));
+        return (float)c;
+    }
 }
 
 // Map a circular shift index (0..n-1) to the output map index, or -1 when the
@@ -178,8 +197,12 @@ template <typename T, int Q>
 struct FwdRowsCfg {
     using G = TeamGeom<T, Q>;
     static constexpr int M = G::M, R = G::R, TEAM = G::TEAM;
-    static constexpr int TPB = TEAM >= 256 ? 1 : 256 / TEAM;
+    // residues: small blocks, so that a launch that needs few planes (CMIF_AUTO's second
+    // precision) still fills the SMs: one label pair of 1024^2, Q = 2048: 141 us at 256 threads
+    static constexpr int TARGET = std::is_same<T, m31>::value ? 64 : 256;
+    static constexpr int TPB = TEAM >= TARGET ? 1 : TARGET / TEAM;
     static constexpr int THREADS = TPB * TEAM;
+    static constexpr int MIN_BLOCKS = sizeof(T) == 4 && THREADS <= 512 ? 512 / THREADS : 1;
     static constexpr int REGION = (int)(Q * sizeof(cpx<T>)) > G::SCRATCH ? (int)(Q * sizeof(cpx<T>)) : G::SCRATCH;
     static constexpr size_t smem(int W, bool weighted) {
         return (size_t)TPB * REGION + (((size_t)W + 15) & ~(size_t)15) + (weighted ? (size_t)W * sizeof(double) : 0);
@@ -187,7 +210,7 @@ struct FwdRowsCfg {
 };
 
 template <typename T, int Q>
-__global__ void __launch_bounds__(FwdRowsCfg<T, Q>::THREADS)
+__global__ void __launch_bounds__(FwdRowsCfg<T, Q>::THREADS, FwdRowsCfg<T, Q>::MIN_BLOCKS)
 k_fwd_rows(const int32_t* __restrict__ X, const uint8_t* __restrict__ MX, const double* __restrict__ WX, int H, int W,
            int K, int Qs, cpx<T>* __restrict__ T1, Tw<T> tw, DevStatus* __restrict__ st, int conditional,
            int* __restrict__ popc, const unsigned char* __restrict__ plane_need) {
@@ -260,18 +283,21 @@ k_fwd_rows(const int32_t* __restrict__ X, const uint8_t* __restrict__ MX, const 
         return {c == la ? one : T(0), c == lb ? one : T(0)};
     };
     cpx<T> v[M];
-    team_fft<M, R, -1>(v, r, j, load, region + r * grp_scratch_bytes<T, M>(), tw.sq[ilog2c(M)], tw_of<Q>(tw));
+    // teams of whole warps without block barriers in their transform: an unneeded one skips it
+    const bool run = active || C::TEAM < 32 || R > 2;
+    if (run) team_fft<M, R, -1>(v, r, j, load, region + r * grp_scratch_bytes<T, M>(), tw.sq[ilog2c(M)], tw_of<Q>(tw));
     __syncthreads();
+    if (run) {
 #pragma unroll
-    for (int k2 = 0; k2 < M; ++k2) sm[R * (j + M * k2) + r] = v[brev(k2, M)];
+        for (int k2 = 0; k2 < M; ++k2) sm[R * (j + M * k2) + r] = v[brev(k2, M)];
+    }
     __syncthreads();
     if (!active) return;
-    const T h = T(0.5);
     for (int k = lt; k <= Q / 2; k += C::TEAM) {
         const cpx<T> a = sm[k], b = sm[k == 0 ? 0 : Q - k];
         // F_la = (X[k] + conj X[-k]) / 2,  F_lb = (X[k] - conj X[-k]) / (2i)
-        T1[((size_t)la * H + y) * Qs + k] = {h * (a.x + b.x), h * (a.y - b.y)};
-        if (lb < K) T1[((size_t)lb * H + y) * Qs + k] = {h * (a.y + b.y), h * (b.x - a.x)};
+        T1[((size_t)la * H + y) * Qs + k] = {halve(a.x + b.x), halve(a.y - b.y)};
+        if (lb < K) T1[((size_t)lb * H + y) * Qs + k] = {halve(a.y + b.y), halve(b.x - a.x)};
     }
 }
 
@@ -296,14 +322,14 @@ struct ColCfg {
 // samples i = 4q .. 4q + 3 of lane j as 8 floats (re, re', im, im' of 4q, 4q + 1, then of
 // 4q + 2, 4q + 3) at complex offset (q M + j) 4 of the group.
 template <typename T, int M>
-__host__ __device__ constexpr bool packed_spectra() { return sizeof(T) == 4 && M >= 8; }
+__host__ __device__ constexpr bool packed_spectra() { return std::is_same<T, float>::value && M >= 8; }
 __device__ __forceinline__ void st_global_32B(void* dst, const float (&v)[8]) {
     asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]), "f"(v[1]), "f"(v[2]),
                  "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
 }
 
 template <typename T, int P, int MMAX>
-__global__ void __launch_bounds__(ColCfg<T, P, MMAX>::THREADS, sizeof(T) == 4 && ColCfg<T, P, MMAX>::THREADS <= 256 ? 3 : 1)
+__global__ void __launch_bounds__(ColCfg<T, P, MMAX>::THREADS, sizeof(T) == 4 && ColCfg<T, P, MMAX>::THREADS <= 256 ? (std::is_same<T, float>::value ? 3 : 2) : 1)
 k_fwd_cols(const cpx<T>* __restrict__ T1, int H, int nplanes, int Qh, int Qs, cpx<T>* __restrict__ F, Tw<T> tw,
            const DevStatus* __restrict__ st, int conditional, T out_scale,
            const unsigned char* __restrict__ plane_need, int slices) {
@@ -380,9 +406,9 @@ __device__ __forceinline__ cpx<double> __ldg(const cpx<double>* p) {
     const double2 v = ::__ldg(reinterpret_cast<const double2*>(p));
     return {v.x, v.y};
 }
-__device__ __forceinline__ cpx<df32> __ldg(const cpx<df32>* p) {
-    const float4 v = ::__ldg(reinterpret_cast<const float4*>(p));
-    return {df32(v.x, v.y), df32(v.z, v.w)};
+__device__ __forceinline__ cpx<m31> __ldg(const cpx<m31>* p) {
+    const uint2 v = ::__ldg(reinterpret_cast<const uint2*>(p));
+    return {m31_of(v.x), m31_of(v.y)};
 }
 
 // ---------------------------------------------------------------------------
@@ -412,7 +438,8 @@ __device__ __forceinline__ void stage_table(cpx<T>* dst, const cpx<T>* __restric
 //     (Y[pair][row / 4][c][row % 4]): the pair-column kernel's lanes, which hold consecutive
 //     rows, write whole lines (8 shared-pipe wavefronts per 32 lanes instead of 32), and the
 //     row kernels gather a row's chunks (TMA, or 16-byte asynchronous copies).
-//   FP64, two-term FP32, L / 2 chunks of 2: z_c, z_{L-c}; rows contiguous.
+//   residues mod p: as FP32 at the other Q;
+//   FP64, L / 2 chunks of 2: z_c, z_{L-c}; rows contiguous.
 template <typename T>
 constexpr int kChunk = sizeof(T) == 4 ? 4 : 2;
 __host__ __device__ constexpr bool split32_rows(int Q) { return Q == 512 || Q == 1024 || Q == 2048; }
@@ -444,23 +471,26 @@ __device__ __forceinline__ int chunk_col(int c, int i, int L, bool split) {
         return i ? mirror_k(c, L) : c;
     }
 }
-// z_k of a row whose chunks lie back to back.
-template <typename T, int Q>
+// z_k of a row whose chunks lie CS values apart: back to back (a staged row, FP64), or in Y's
+// lines of four rows.
+template <typename T>
+constexpr int kLine = sizeof(T) == 4 ? 4 * kChunk<T> : kChunk<T>;
+template <typename T, int Q, int CS = kChunk<T>>
 __device__ __forceinline__ cpx<T> load_z(const cpx<T>* row, int k) {
     constexpr int L = Q / 2;
     const bool mir = k >= L / 2;
     const int kk = k == L / 2 ? 0 : (mir ? L - k : k);  // the direct partner
     if constexpr (sizeof(T) != 4) {
-        return row[2 * kk + (mir ? 1 : 0)];
+        return row[CS * kk + (mir ? 1 : 0)];
     } else {
-        constexpr bool split = split32_rows(Q);
+        constexpr bool split = std::is_same<T, float>::value && split32_rows(Q);
         const int c = split ? (kk >> 6) * 32 + (kk & 31) : kk >> 1, second = split ? (kk >> 5) & 1 : kk & 1;
         const int half = (mir ? 1 : 0) ^ (halves_swapped(c) ? 1 : 0), e = mir ? 1 - second : second;
         if constexpr (split) {
-            const float* f = reinterpret_cast<const float*>(row) + c * 8 + half * 4 + e;
+            const float* f = reinterpret_cast<const float*>(row) + c * 2 * CS + half * 4 + e;
             return {f[0], f[2]};
         } else {
-            return row[c * 4 + half * 2 + e];
+            return row[c * CS + half * 2 + e];
         }
     }
 }
@@ -480,6 +510,16 @@ __device__ __forceinline__ void store_chunk(cpx<float>* dst, const cpx<float> (&
         v[4 * h + (SPLIT ? 2 : 1)] = z[2 * h].y;
         v[4 * h + (SPLIT ? 1 : 2)] = z[2 * h + 1].x;
         v[4 * h + 3] = z[2 * h + 1].y;
+    }
+    st_global_32B(dst, v);
+}
+template <bool SPLIT>
+__device__ __forceinline__ void store_chunk(cpx<m31>* dst, const cpx<m31> (&z)[4]) {
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        v[2 * i] = __uint_as_float(z[i].x.v);
+        v[2 * i + 1] = __uint_as_float(z[i].y.v);
     }
     st_global_32B(dst, v);
 }
@@ -573,7 +613,7 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
     if (conditional && !(st->flags & STATUS_ESCALATE)) return;
     constexpr int M = C::M, R = C::R, TPB = C::TPB, NQ = C::NQ, CH = kChunk<T>, UPR = C::UPR;
     const int L = Qh - 1;
-    const bool split = sizeof(T) == 4 && split32_rows(2 * L);
+    const bool split = std::is_same<T, float>::value && split32_rows(2 * L);
     const int Dz = VOL ? DA + DB - 1 : 1;
     int npairs = KA * KB, lbase = 0;
     if (plist) {
@@ -836,7 +876,7 @@ constexpr size_t pair_cols_smem() {
 // accumulates, pair by pair, the joint term T(c), the running A-marginal of
 // the current label a, and the B-marginal C_B^b(p) (shared or global memory).
 // The rounded counts reach the owners through the teams' scratch, in HALVES
-// passes (two for FP32, whose scratch holds half a row).
+// passes (two for 4-byte values, whose scratch holds half a row).
 template <typename T, int Q>
 struct RowCfg {
     static constexpr int L = Q / 2;
@@ -967,13 +1007,9 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                                tw_of<L>(tw));
             // round to the nearest integer; track the worst residual (the exactness guard)
             float rp = 0.f;
+            float2 cnt[M];
 #pragma unroll
-            for (int k = 0; k < M; ++k) {
-                const T cr = rint_t<T>(v[k].x), ci = rint_t<T>(v[k].y);
-                rp = fmaxf(rp, fmaxf((float)fabs(v[k].x - cr), (float)fabs(v[k].y - ci)));
-                v[k].x = cr;
-                v[k].y = ci;
-            }
+            for (int k = 0; k < M; ++k) cnt[k] = make_float2(round_count(v[k].x, rp), round_count(v[k].y, rp));
             if (ovs < 0) res_max = fmaxf(res_max, rp);
             if (pair_res) {  // per-pair residual: reduce over the team's lanes of each warp
                 constexpr int WID = C::TEAM < 32 ? C::TEAM : 32;
@@ -1002,8 +1038,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                         const int2 q = *reinterpret_cast<const int2*>(ov + ((size_t)ovs * Rout + row) * Q + 2 * mf);
                         ob[m] = make_float2((float)q.x, (float)q.y);
                     } else {
-                        const cpx<T> z = v[brev(k2, M)];
-                        ob[m] = make_float2((float)z.x, (float)z.y);
+                        ob[m] = cnt[brev(k2, M)];
                     }
                 }
                 __syncthreads();
@@ -1183,8 +1218,8 @@ k_pair_rows_counts(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, const int* __
         const long long t = t0 + team;
         const bool act = t < ntask;
         const int e = act ? (int)(t / nrows) : 0, row = g.r0 + (act ? (int)(t % nrows) : 0);
-        const cpx<T>* yr = Y + ((size_t)e * g.R + row) * L;
-        auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q>(yr, k) : cpx<T>{T(0), T(0)}; };
+        const cpx<T>* yr = Y + (size_t)e * y_rows<T>(g.R) * L + y_chunk<T>(row, 0, L);
+        auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q, kLine<T>>(yr, k) : cpx<T>{T(0), T(0)}; };
         cpx<T> v[M];
         team_fft<M, R, +1>(v, r, j, load, region + r * grp_scratch_bytes<T, M>(), tw.sq[ilog2c(M)],
                            tw_of<L>(tw));
@@ -1194,9 +1229,7 @@ k_pair_rows_counts(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, const int* __
             for (int k2 = 0; k2 < M; ++k2) {
                 const int mf = R * (j + M * k2) + r;
                 const cpx<T> z = v[brev(k2, M)];
-                const T cr = rint_t<T>(z.x), ci = rint_t<T>(z.y);
-                res = fmaxf(res, fmaxf((float)fabs(z.x - cr), (float)fabs(z.y - ci)));
-                *reinterpret_cast<int2*>(o + 2 * mf) = make_int2((int)(float)cr, (int)(float)ci);
+                *reinterpret_cast<int2*>(o + 2 * mf) = make_int2((int)round_count(z.x, res), (int)round_count(z.y, res));
             }
         }
     }

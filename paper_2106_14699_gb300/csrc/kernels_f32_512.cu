@@ -1,12 +1,9 @@
-// FP32 forward, column, pair-product and weighted-row kernels for transform size 512.
+// FP32 forward, column and pair-product kernels for transform size 512.
 #include "pipeline_impl.cuh"
 namespace cmif {
 template cudaError_t Sized<float, 512>::fwd_rows(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 512>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 512>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template int Sized<float, 512>::tm_cols(int);
-template cudaError_t Sized<float, 512>::tm_max_blocks(int, int*);
-template cudaError_t Sized<float, 512>::pair_rows_w(const Geom&, const PipeArgs<float>&, cudaStream_t);
-template size_t Sized<float, 512>::rows_w_smem();
-template cudaError_t Sized<float, 512>::rows_w_max_blocks(int*);
+template cudaError_t Sized<float, 512>::tm_max_blocks(int, int, int*);
 }

@@ -4,9 +4,6 @@ namespace cmif {
 template cudaError_t Sized<double, 1024>::fwd_rows(const Geom&, const PipeArgs<double>&, bool, cudaStream_t);
 template cudaError_t Sized<double, 1024>::fwd_cols(const Geom&, const PipeArgs<double>&, bool, cudaStream_t);
 template cudaError_t Sized<double, 1024>::pair_cols(const Geom&, const PipeArgs<double>&, cudaStream_t);
-template int Sized<double, 1024>::tm_cols(int);
-template cudaError_t Sized<double, 1024>::tm_max_blocks(int, int*);
 template cudaError_t Sized<double, 1024>::pair_rows_w(const Geom&, const PipeArgs<double>&, cudaStream_t);
-template size_t Sized<double, 1024>::rows_w_smem();
 template cudaError_t Sized<double, 1024>::rows_w_max_blocks(int*);
 }

@@ -567,13 +567,13 @@ struct DevTables {
     void* buf = nullptr;
     Tw<float> tf{};
     Tw<double> td{};
-    Tw<df32> ts{};
+    Tw<m31> tm{};
 };
 
 static std::mutex g_tw_mu;
 static DevTables g_tw[64];
 
-cudaError_t get_twiddles(int device, Tw<float>* tf, Tw<double>* td, Tw<df32>* ts) {
+cudaError_t get_twiddles(int device, Tw<float>* tf, Tw<double>* td, Tw<m31>* tm) {
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(g_tw_mu);
     DevTables& t = g_tw[device];
@@ -615,31 +615,39 @@ cudaError_t get_twiddles(int device, Tw<float>* tf, Tw<double>* td, Tw<df32>* ts
         }
         const size_t n = re.size();
         std::vector<double> hd(2 * n);
-        std::vector<float> hf(2 * n), hs(4 * n);
+        std::vector<float> hf(2 * n);
+        std::vector<uint32_t> hm(2 * n, 0);  // the roots of unity mod p (powers of two only)
         for (size_t i = 0; i < n; ++i) {
             hd[2 * i] = re[i];
             hd[2 * i + 1] = im[i];
             hf[2 * i] = (float)re[i];
             hf[2 * i + 1] = (float)im[i];
-            const float rh = (float)re[i], ih = (float)im[i];
-            hs[4 * i] = rh;
-            hs[4 * i + 1] = (float)(re[i] - (double)rh);
-            hs[4 * i + 2] = ih;
-            hs[4 * i + 3] = (float)(im[i] - (double)ih);
+        }
+        auto put = [&](size_t at, long long k, long long N) {  // e^{-2 pi i k / N}: the conjugate of w_N^k
+            const m31c w = m31_root((uint32_t)(k % N), (uint32_t)N);
+            hm[2 * at] = w.x;
+            hm[2 * at + 1] = (kM31 - w.y) % kM31;
+        };
+        for (int l = 0; l < 14; ++l)
+            for (long long k = 0; k < (1LL << l); ++k) put(off_n[l] + k, k, 1LL << l);
+        for (int l = 0; l < 6; ++l) {
+            const long long M = 1LL << l;
+            for (long long k = 0; k < M; ++k)
+                for (long long j = 0; j < M; ++j) put(off_sq[l] + k * M + j, j * k, M * M);
         }
         for (int l = 0; l < 6; ++l) fill_sq_f32(hf.data() + 2 * off_sq[l], 1 << l);
-        // every table starts on a 256-byte boundary (the two-term values are loaded 16 bytes at a time)
+        // every table starts on a 256-byte boundary
         const size_t bytes_d = (2 * n * sizeof(double) + 255) / 256 * 256, bytes_f = (2 * n * sizeof(float) + 255) / 256 * 256;
-        const size_t bytes_s = 4 * n * sizeof(float);
+        const size_t bytes_m = hm.size() * sizeof(uint32_t);
         int prev = -1;
         cudaGetDevice(&prev);
         cudaError_t e = cudaSetDevice(device);
         if (e != cudaSuccess) return e;
         void* buf = nullptr;
-        e = cudaMalloc(&buf, bytes_d + bytes_f + bytes_s);
+        e = cudaMalloc(&buf, bytes_d + bytes_f + bytes_m);
         if (e == cudaSuccess) e = cudaMemcpy(buf, hd.data(), hd.size() * sizeof(double), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d, hf.data(), hf.size() * sizeof(float), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d + bytes_f, hs.data(), bytes_s, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d + bytes_f, hm.data(), bytes_m, cudaMemcpyHostToDevice);
         if (prev >= 0) cudaSetDevice(prev);
         if (e != cudaSuccess) {
             if (buf) cudaFree(buf);
@@ -648,14 +656,14 @@ cudaError_t get_twiddles(int device, Tw<float>* tf, Tw<double>* td, Tw<df32>* ts
         t.buf = buf;
         const cpx<double>* bd = reinterpret_cast<const cpx<double>*>(buf);
         const cpx<float>* bf = reinterpret_cast<const cpx<float>*>((char*)buf + bytes_d);
-        const cpx<df32>* bs = reinterpret_cast<const cpx<df32>*>((char*)buf + bytes_d + bytes_f);
-        for (int l = 0; l < 14; ++l) { t.td.n[l] = bd + off_n[l]; t.tf.n[l] = bf + off_n[l]; t.ts.n[l] = bs + off_n[l]; }
-        for (int l = 0; l < 6; ++l) { t.td.sq[l] = bd + off_sq[l]; t.tf.sq[l] = bf + off_sq[l]; t.ts.sq[l] = bs + off_sq[l]; }
-        for (int l = 0; l < 12; ++l) { t.td.n3[l] = bd + off_n3[l]; t.tf.n3[l] = bf + off_n3[l]; t.ts.n3[l] = bs + off_n3[l]; }
+        const cpx<m31>* bm = reinterpret_cast<const cpx<m31>*>((char*)buf + bytes_d + bytes_f);
+        for (int l = 0; l < 14; ++l) { t.td.n[l] = bd + off_n[l]; t.tf.n[l] = bf + off_n[l]; t.tm.n[l] = bm + off_n[l]; }
+        for (int l = 0; l < 6; ++l) { t.td.sq[l] = bd + off_sq[l]; t.tf.sq[l] = bf + off_sq[l]; t.tm.sq[l] = bm + off_sq[l]; }
+        for (int l = 0; l < 12; ++l) { t.td.n3[l] = bd + off_n3[l]; t.tf.n3[l] = bf + off_n3[l]; t.tm.n3[l] = bm + off_n3[l]; }
     }
     if (tf) *tf = t.tf;
     if (td) *td = t.td;
-    if (ts) *ts = t.ts;
+    if (tm) *tm = t.tm;
     return cudaSuccess;
 }
 

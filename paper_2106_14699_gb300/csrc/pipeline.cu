@@ -17,8 +17,7 @@ struct ProfScope {
 template <typename T>
 cudaError_t run_pipeline(const Geom& g, const PipeArgs<T>& a, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
-    constexpr bool f32 = sizeof(T) == 4;
-    constexpr bool split = std::is_same<T, df32>::value;
+    constexpr bool f32 = std::is_same<T, float>::value, exact = std::is_same<T, m31>::value;
     const unsigned stg = a.stages ? a.stages : STAGE_ALL;
     // A's and B's forward transforms are independent: with a second stream, A's run
     // on it, forked from s before and joined back into s after B's
@@ -31,21 +30,21 @@ cudaError_t run_pipeline(const Geom& g, const PipeArgs<T>& a, cudaStream_t s) {
     }
     if (stg & STAGE_FWD_A) {
         CMIF_SIZE_SWITCH_T(T, g.Q, {
-            ProfScope ps(a.prof, f32 ? "fwd_rows_A_f32" : split ? "fwd_rows_A_s32" : "fwd_rows_A_f64", sa);
+            ProfScope ps(a.prof, f32 ? "fwd_rows_A_f32" : exact ? "fwd_rows_A_m31" : "fwd_rows_A_f64", sa);
             e = Sized<T, SZ>::fwd_rows(g, a, false, sa);
         } if (e != cudaSuccess) return e);
         CMIF_SIZE_SWITCH_T(T, g.P, {
-            ProfScope ps(a.prof, f32 ? "fwd_cols_A_f32" : split ? "fwd_cols_A_s32" : "fwd_cols_A_f64", sa);
+            ProfScope ps(a.prof, f32 ? "fwd_cols_A_f32" : exact ? "fwd_cols_A_m31" : "fwd_cols_A_f64", sa);
             e = Sized<T, SZ>::fwd_cols(g, a, false, sa);
         } if (e != cudaSuccess) return e);
     }
     if (stg & STAGE_FWD_B) {
         CMIF_SIZE_SWITCH_T(T, g.Q, {
-            ProfScope ps(a.prof, f32 ? "fwd_rows_B_f32" : split ? "fwd_rows_B_s32" : "fwd_rows_B_f64", s);
+            ProfScope ps(a.prof, f32 ? "fwd_rows_B_f32" : exact ? "fwd_rows_B_m31" : "fwd_rows_B_f64", s);
             e = Sized<T, SZ>::fwd_rows(g, a, true, s);
         } if (e != cudaSuccess) return e);
         CMIF_SIZE_SWITCH_T(T, g.P, {
-            ProfScope ps(a.prof, f32 ? "fwd_cols_B_f32" : split ? "fwd_cols_B_s32" : "fwd_cols_B_f64", s);
+            ProfScope ps(a.prof, f32 ? "fwd_cols_B_f32" : exact ? "fwd_cols_B_m31" : "fwd_cols_B_f64", s);
             e = Sized<T, SZ>::fwd_cols(g, a, true, s);
         } if (e != cudaSuccess) return e);
     }
@@ -56,19 +55,19 @@ cudaError_t run_pipeline(const Geom& g, const PipeArgs<T>& a, cudaStream_t s) {
     }
     if (stg & STAGE_COLS) {
         CMIF_SIZE_SWITCH_T(T, g.P, {
-            ProfScope ps(a.prof, f32 ? "pair_cols_f32" : split ? "pair_cols_s32" : "pair_cols_f64", s);
+            ProfScope ps(a.prof, f32 ? "pair_cols_f32" : exact ? "pair_cols_m31" : "pair_cols_f64", s);
             e = Sized<T, SZ>::pair_cols(g, a, s);
         } if (e != cudaSuccess) return e);
     }
     if (stg & STAGE_ROWS) {
-        if (a.weighted) {
+        if constexpr (std::is_same<T, double>::value) {  // weighted maps
             CMIF_SIZE_SWITCH_T(T, g.Q, {
                 ProfScope ps(a.prof, "pair_rows_weighted_f64", s);
                 e = Sized<T, SZ>::pair_rows_w(g, a, s);
             } if (e != cudaSuccess) return e);
         } else {
             CMIF_SIZE_SWITCH_T(T, g.Q, {
-                ProfScope ps(a.prof, f32 ? "pair_rows_f32" : split ? "pair_rows_s32" : "pair_rows_f64", s);
+                ProfScope ps(a.prof, f32 ? "pair_rows_f32" : "pair_rows_m31", s);
                 e = Sized<T, SZ>::pair_rows(g, a, s);
             } if (e != cudaSuccess) return e);
         }
@@ -79,19 +78,17 @@ cudaError_t run_pipeline(const Geom& g, const PipeArgs<T>& a, cudaStream_t s) {
 template <typename T>
 cudaError_t run_pair_counts(const Geom& g, const PipeArgs<T>& a, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
-    constexpr bool split = std::is_same<T, df32>::value;
     CMIF_SIZE_SWITCH(g.P, {
-        ProfScope ps(a.prof, split ? "pair_cols_list_s32" : "pair_cols_list_f64", s);
+        ProfScope ps(a.prof, "pair_cols_list_m31", s);
         e = Sized<T, SZ>::pair_cols(g, a, s);
     } if (e != cudaSuccess) return e);
     CMIF_SIZE_SWITCH(g.Q, {
-        ProfScope ps(a.prof, split ? "pair_counts_s32" : "pair_counts_f64", s);
+        ProfScope ps(a.prof, "pair_counts_m31", s);
         e = Sized<T, SZ>::pair_rows_counts(g, a, s);
     } if (e != cudaSuccess) return e);
     return cudaSuccess;
 }
-template cudaError_t run_pair_counts<double>(const Geom&, const PipeArgs<double>&, cudaStream_t);
-template cudaError_t run_pair_counts<df32>(const Geom&, const PipeArgs<df32>&, cudaStream_t);
+template cudaError_t run_pair_counts<m31>(const Geom&, const PipeArgs<m31>&, cudaStream_t);
 
 template <typename T>
 size_t rows_smem_bytes(int Q, int KB, bool cb_smem) {
@@ -137,20 +134,20 @@ cudaError_t rows_w_max_blocks_per_sm(int Q, int* out) {
     return cudaSuccess;
 }
 
-cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int* out) {
+cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int npairs, int* out) {
     *out = 0;
-    CMIF_SIZE_SWITCH_T(float, Q, return Sized<float, SZ>::tm_max_blocks(tm_cols, out));
+    CMIF_SIZE_SWITCH_T(float, Q, return Sized<float, SZ>::tm_max_blocks(tm_cols, npairs, out));
     return cudaSuccess;
 }
 
+template cudaError_t run_pipeline<double>(const Geom&, const PipeArgs<double>&, cudaStream_t);
 #define CMIF_INSTANTIATE(T)                                                             \
     template cudaError_t run_pipeline<T>(const Geom&, const PipeArgs<T>&, cudaStream_t); \
     template size_t rows_smem_bytes<T>(int, int, bool);                                  \
     template int rows_threads<T>(int);                                                   \
     template cudaError_t rows_max_blocks_per_sm<T>(int, int, bool, int*);
 CMIF_INSTANTIATE(float)
-CMIF_INSTANTIATE(double)
-CMIF_INSTANTIATE(df32)
+CMIF_INSTANTIATE(m31)
 #undef CMIF_INSTANTIATE
 
 }  // namespace cmif

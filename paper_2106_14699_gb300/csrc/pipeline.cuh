@@ -1,4 +1,5 @@
-// Launch sequence of one CMIF map for one precision (FP32 or FP64 transforms).
+// Launch sequence of one CMIF map for one arithmetic: FP32, residues mod 2^31 - 1 (m31.cuh;
+// FP64, two-term and AUTO's second-precision counts) or FP64 (weighted maps).
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -26,7 +27,7 @@ struct PipeArgs {
     int32_t* n;
     int32_t* counts;
     DevStatus* st;
-    int prec_slot;    // 0: FP32 residual slot, 1: FP64
+    int prec_slot;    // 0: FP32 residual slot, 1: exact transforms
     int conditional;  // run only when STATUS_ESCALATE is set (AUTO re-run)
     int rows_grid;    // persistent grid of the row/epilogue kernel
     int num_sms;      // SMs of the device (persistent grid of the pair-column kernel)
@@ -34,7 +35,7 @@ struct PipeArgs {
     // spatially weighted MI (FP64 plans): weight images replace the masks
     const double* WA;  // [H_A][W_A] or nullptr
     const double* WB;  // [H_B][W_B] or nullptr
-    int weighted;      // run the weighted row kernel (real counts, no rounding)
+    int weighted;      // the level sets carry the weights
     double* cbw;       // [rows_grid_w][K_B][Q] B-marginals of the weighted row kernel
     double* nw;        // weighted N map [R][C]
     int rows_grid_w;   // persistent grid of the weighted row kernel
@@ -135,9 +136,8 @@ struct Sized {
     static int rows_threads();
     static cudaError_t rows_max_blocks(int KB, bool cb_smem, int* out);
     static int tm_cols(int KB);                 // 0 unless the TMEM row kernel applies (FP32, Q = 512 / 1024 / 2048)
-    static cudaError_t tm_max_blocks(int tm_cols, int* out);
+    static cudaError_t tm_max_blocks(int tm_cols, int npairs, int* out);
     static cudaError_t pair_rows_w(const Geom& g, const PipeArgs<T>& a, cudaStream_t s);  // FP64 only
-    static size_t rows_w_smem();
     static cudaError_t rows_w_max_blocks(int* out);
 };
 
@@ -163,7 +163,7 @@ template <typename T>
 cudaError_t rows_max_blocks_per_sm(int Q, int KB, bool cb_smem, int* out);
 // TMEM columns the TMEM / TMA row kernel needs for (Q, K_B), or 0 when it does not apply.
 int rows_tm_cols(int Q, int KB);
-cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int* out);
+cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int npairs, int* out);
 // The weighted (SWMI) row kernel: its occupancy (FP64).
 cudaError_t rows_w_max_blocks_per_sm(int Q, int* out);
 

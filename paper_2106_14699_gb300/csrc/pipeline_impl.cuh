@@ -5,6 +5,7 @@
 #include "pipeline.cuh"
 #include "rows_tm.cuh"
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 namespace cmif {
@@ -84,11 +85,12 @@ static cudaError_t launch_pair_cols(const Geom& g, const PipeArgs<T>& a, cudaStr
     return cudaGetLastError();
 }
 
-// Teams per block of the Tensor-Memory row kernel (rows_tm.cuh).
-template <int Q>
-static constexpr int kRowTeams = Q == 2048 ? 16 : 8;
-template <int Q>
-static int rows_tm_teams(int tm_cols) { return tm_cols <= 256 ? kRowTeams<Q> : 16; }
+// Teams per block of the Tensor-Memory row kernel (rows_tm.cuh): blocks of 8 where two of
+// them share an SM, except long runs of pairs at Q = 2048 (16: 64 pairs 0.410 vs 0.412 ms, 256
+// pairs 1.49 vs 1.50 ms; a few pairs leave most of 16 teams idle).
+static int rows_tm_teams(int Q, int tm_cols, int npairs) {
+    return tm_cols > 256 || (Q == 2048 && npairs > 32) ? 16 : 8;
+}
 
 template <int Q, bool NMI, int MODE, int NT>
 static cudaError_t launch_rows_tm(const Geom& g, const PipeArgs<float>& a, cudaStream_t s) {
@@ -111,14 +113,14 @@ static cudaError_t launch_rows_tm(const Geom& g, const PipeArgs<float>& a, cudaS
 template <typename T, int Q, bool NMI>
 static cudaError_t launch_pair_rows_v(const Geom& g, const PipeArgs<T>& a, cudaStream_t s) {
     using C = RowCfg<T, Q>;
-    if constexpr (sizeof(T) == 4 && (Q == 512 || Q == 1024 || Q == 2048)) {
+    if constexpr (std::is_same<T, float>::value && split32_rows(Q)) {
         if (a.tm_cols > 0 && !a.counts) {  // debug count maps: the generic kernel below
             const bool ext = a.ov_slot || a.pair_res || a.conditional || a.wait_polls > 0 || a.withhold_row >= 0;
             // the multi-unit kernel lives in its own translation unit (kernels_f32_rows_units.cu):
             // compiled next to the plain one, it changed the plain kernel's register allocation
             if (!ext && g.units > 1) return launch_rows_tm_units<Q, NMI>(g, a, s);
-            if (rows_tm_teams<Q>(a.tm_cols) != 16)
-                return ext ? launch_rows_tm<Q, NMI, 2, kRowTeams<Q>>(g, a, s) : launch_rows_tm<Q, NMI, 0, kRowTeams<Q>>(g, a, s);
+            if (rows_tm_teams(Q, a.tm_cols, g.KA * g.KB) == 8)
+                return ext ? launch_rows_tm<Q, NMI, 2, 8>(g, a, s) : launch_rows_tm<Q, NMI, 0, 8>(g, a, s);
             return ext ? launch_rows_tm<Q, NMI, 2, 16>(g, a, s) : launch_rows_tm<Q, NMI, 0, 16>(g, a, s);
         }
     }
@@ -158,6 +160,13 @@ cudaError_t Sized<T, SZ>::fwd_rows(const Geom& g, const PipeArgs<T>& a, bool b_s
                                            a.conditional, a.popA, a.needA, s);
 }
 
+// 1 / n for the unnormalised transforms (residues: n a power of two, 2^31 = 1)
+template <typename T>
+static T inverse_of(double n) {
+    if constexpr (std::is_same<T, m31>::value) return m31_of(1u << (31 - (int)std::lround(std::log2(n))));
+    else return T(1.0 / n);
+}
+
 template <typename T, int SZ>
 cudaError_t Sized<T, SZ>::fwd_cols(const Geom& g, const PipeArgs<T>& a, bool b_side, cudaStream_t s) {
     // B's spectra carry the 1/(P Q) of the unnormalised inverse transform (a power of two: exact)
@@ -165,7 +174,7 @@ cudaError_t Sized<T, SZ>::fwd_cols(const Geom& g, const PipeArgs<T>& a, bool b_s
     auto go = [&](auto mm) {
         constexpr int MM = decltype(mm)::value;
         return b_side ? launch_fwd_cols<T, SZ, MM>(a.T1B, g.HB, g.KB * g.DB, g.Qh, g.Qs, a.FB, a.tw, a.st,
-                                                   a.conditional, T(1.0 / ((double)g.P * (double)g.Q)), a.needB,
+                                                   a.conditional, inverse_of<T>((double)g.P * (double)g.Q), a.needB,
                                                    g.DB, s)
                       : launch_fwd_cols<T, SZ, MM>(a.T1A, g.HA, g.KA * g.DA, g.Qh, g.Qs, a.FA, a.tw, a.st,
                                                    a.conditional, T(1), a.needA, g.DA, s);
@@ -235,40 +244,24 @@ cudaError_t Sized<T, SZ>::rows_max_blocks(int KB, bool cb_smem, int* out) {
 
 template <typename T, int SZ>
 cudaError_t Sized<T, SZ>::pair_rows_w(const Geom& g, const PipeArgs<T>& a, cudaStream_t s) {
-    if constexpr (std::is_same<T, double>::value) {
-        using C = RowWCfg<SZ>;
-        cudaError_t e = ensure_smem(k_pair_rows_w<SZ>, C::SMEM);
-        if (e != cudaSuccess) return e;
-        k_pair_rows_w<SZ><<<a.rows_grid_w, C::THREADS, C::SMEM, s>>>(a.Y, g, a.tw, a.cbw, a.mi, a.nw, a.st);
-        return cudaGetLastError();
-    } else {
-        (void)g; (void)a; (void)s;
-        return cudaErrorNotSupported;  // weighted maps need FP64 transforms
-    }
-}
-
-template <typename T, int SZ>
-size_t Sized<T, SZ>::rows_w_smem() {
-    if constexpr (std::is_same<T, double>::value) return RowWCfg<SZ>::SMEM;
-    else return 0;
+    using C = RowWCfg<SZ>;
+    cudaError_t e = ensure_smem(k_pair_rows_w<SZ>, C::SMEM);
+    if (e != cudaSuccess) return e;
+    k_pair_rows_w<SZ><<<a.rows_grid_w, C::THREADS, C::SMEM, s>>>(a.Y, g, a.tw, a.cbw, a.mi, a.nw, a.st);
+    return cudaGetLastError();
 }
 
 template <typename T, int SZ>
 cudaError_t Sized<T, SZ>::rows_w_max_blocks(int* out) {
-    if constexpr (std::is_same<T, double>::value) {
-        using C = RowWCfg<SZ>;
-        cudaError_t e = ensure_smem(k_pair_rows_w<SZ>, C::SMEM);
-        if (e != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_pair_rows_w<SZ>, C::THREADS, C::SMEM);
-    } else {
-        *out = 0;
-        return cudaSuccess;
-    }
+    using C = RowWCfg<SZ>;
+    cudaError_t e = ensure_smem(k_pair_rows_w<SZ>, C::SMEM);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_pair_rows_w<SZ>, C::THREADS, C::SMEM);
 }
 
 template <typename T, int SZ>
 int Sized<T, SZ>::tm_cols(int KB) {
-    if constexpr (sizeof(T) == 4 && (SZ == 512 || SZ == 1024 || SZ == 2048)) {
+    if constexpr (std::is_same<T, float>::value && split32_rows(SZ)) {
         const int need = tm_cols_needed(KB, SZ);
         return need <= 512 ? tm_alloc_cols(need) : 0;
     } else {
@@ -278,17 +271,18 @@ int Sized<T, SZ>::tm_cols(int KB) {
 }
 
 template <typename T, int SZ>
-cudaError_t Sized<T, SZ>::tm_max_blocks(int tm_cols, int* out) {
+cudaError_t Sized<T, SZ>::tm_max_blocks(int tm_cols, int npairs, int* out) {
     *out = 0;
-    if constexpr (sizeof(T) == 4 && (SZ == 512 || SZ == 1024 || SZ == 2048)) {
+    if constexpr (std::is_same<T, float>::value && split32_rows(SZ)) {
         // The blocks that share an SM: as many as the kernel is bounded for (registers; shared
         // memory is less than that), within the SM's 512 TMEM columns.  (The occupancy query
         // answers 1 for a kernel that allocates Tensor Memory.)
-        const int blocks = rows_tm_teams<SZ>(tm_cols) == 16 ? 1 : RowTmCfg<SZ, kRowTeams<SZ>>::BLOCKS;
+        const int blocks = rows_tm_teams(SZ, tm_cols, npairs) == 16 ? 1 : RowTmCfg<SZ, 8>::BLOCKS;
         *out = std::min(blocks, 512 / tm_cols);
         return cudaSuccess;
     } else {
         (void)tm_cols;
+        (void)npairs;
         return cudaSuccess;
     }
 }

@@ -538,12 +538,14 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                     }
                     const int seg = min(KB - b, nt - t);  // the rest of label a in this round
                     int d;
-                    if (UH <= 2 && seg >= 16) {
-                        accum(std::integral_constant<int, UH <= 2 ? 16 : 8>{}, t, b);
-                        d = 16;
-                    } else if (seg >= 8) {
-                        accum(std::integral_constant<int, 8>{}, t, b);
-                        d = 8;
+                    // UH = 4 with two passes: 4 labels at a time hold the registers (8 spill)
+                    constexpr int NMED = UH == 4 && HALVES == 2 ? 4 : 8, NBIG = UH <= 2 ? 16 : NMED;
+                    if (NBIG > NMED && seg >= NBIG) {
+                        accum(std::integral_constant<int, NBIG>{}, t, b);
+                        d = NBIG;
+                    } else if (seg >= NMED) {
+                        accum(std::integral_constant<int, NMED>{}, t, b);
+                        d = NMED;
                     } else {
                         accum(std::integral_constant<int, 1>{}, t, b);
                         d = 1;
