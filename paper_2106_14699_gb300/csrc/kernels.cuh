@@ -574,7 +574,12 @@ struct PairColsCfg {
         if (M == 16) return R == 3 ? 4 : R <= 2 ? 2 : 1;
         return M == 8 ? 4 : 2;
     }
-    static constexpr int MIN_BLOCKS = sizeof(T) == 4 ? f32_blocks() : 1;
+    // Volumes: depth offsets per item.  The depth sum of one offset reads two slice spectra
+    // per product, which bounds the kernel by L2-to-SM traffic (20 TB/s); offsets dz .. dz + NDZ - 1
+    // share A's slice and slide over B's, two loads per NDZ products.  40 x 56 x 64, K = 8 (P = 128):
+    // 664 us with one offset per item, 463 with four.
+    static constexpr int NDZ = std::is_same<T, float>::value ? (M == 8 ? 4 : M == 16 && R <= 3 ? 2 : 1) : 1;
+    static constexpr int min_blocks(bool vol) { return sizeof(T) != 4 ? 1 : vol && NDZ > 1 ? 2 : f32_blocks(); }
 };
 
 // Pair product + inverse column transform of length P = R*M*M.  Persistent
@@ -593,12 +598,12 @@ struct PairColsCfg {
 // items at the head of a kx block ask L2 for the spectrum columns two kx blocks ahead.
 // FP32 groups of 8 lanes and more: spectra in the order of the packed DFTs, 32 bytes per
 // load (fwd_cols).  work_ctr must be zero at launch.
-// VOL (volumes): items are (pair, depth offset dz, kx block); the product is
+// VOL (volumes): items are (pair, NDZ depth offsets dz, kx block); the product is
 // the sum over the slices z of conj(F_a,z) F_b,z+dz (the 3-D correlation's
 // depth sum, taken before the inverse transform, which is linear), and the
 // output row of depth offset index dzo is dzo * R2 + (the image's output row).
 template <typename T, int P, bool VOL, int MMAX>
-__global__ void __launch_bounds__(PairColsCfg<T, P, MMAX>::THREADS, PairColsCfg<T, P, MMAX>::MIN_BLOCKS)
+__global__ void __launch_bounds__(PairColsCfg<T, P, MMAX>::THREADS, PairColsCfg<T, P, MMAX>::min_blocks(VOL))
 k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA, int KB, int Qh, int HA, int HB,
             int Rout, int r0, int r1, cpx<T>* __restrict__ Y, Tw<T> tw, const cpx<T>* __restrict__ twq,
             const DevStatus* __restrict__ st, int conditional, int* __restrict__ work_ctr, int DA, int DB, int R2,
@@ -622,7 +627,8 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
         if (npairs <= 0) return;  // uniform: nothing listed for this launch
     }
     auto real_pair = [&](int e) { return plist ? ::__ldg(plist + lbase + e) : e; };
-    const int U = VOL ? Dz : units;  // the middle item dimension: depth offsets or units
+    constexpr int NDZ = VOL ? C::NDZ : 1;
+    const int U = VOL ? (Dz + NDZ - 1) / NDZ : units;  // the middle item dimension: groups of depth offsets or units
     const int nkxb = (L + TPB - 1) / TPB, n_items = npairs * nkxb * U;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_next[6];  // the next item: whether there is one, e, a, b, kx block, unit / depth offset
@@ -732,7 +738,63 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
                 for (int i = 0; i < M; ++i) v[i] = {T(0), T(0)};
             }
         }
-        if constexpr (VOL) {
+        float2 sre[NDZ > 1 ? NDZ : 1][H], sim[NDZ > 1 ? NDZ : 1][H];  // NDZ > 1: the depth sums of the item's offsets
+        if constexpr (VOL && NDZ > 1) {
+#pragma unroll
+            for (int s = 0; s < NDZ; ++s)
+#pragma unroll
+                for (int i = 0; i < H; ++i) sre[s][i] = sim[s][i] = make_float2(0.f, 0.f);
+            // offsets dz + s, s < NDZ: slice z of A with slices z + dz + s of B, which slide through
+            // a ring of NDZ (zero beyond B's slices)
+            const int dz = dzo * NDZ - (DA - 1);
+            const int za = max(0, -dz - (NDZ - 1)), zb = min(DA, DB - dz);
+            const size_t slice_stride = (size_t)Qh * P;
+            auto depth_sum = [&](auto rotc, const cpx<T>* ga, const cpx<T>* gb) {
+                constexpr bool ROT = decltype(rotc)::value;
+#pragma unroll
+                for (int q = 0; q < NV; ++q) {
+                    float ring[NDZ][8];
+                    auto load_b = [&](int s, int zz) {
+                        if (zz >= 0 && zz < DB) {
+                            ld_global_32B(reinterpret_cast<const float*>(gb + zz * slice_stride + 4 * M * q), ring[s]);
+                        } else {
+#pragma unroll
+                            for (int x = 0; x < 8; ++x) ring[s][x] = 0.f;
+                        }
+                    };
+#pragma unroll
+                    for (int s = 1; s < NDZ; ++s) load_b(s, za + dz + s - 1);
+#pragma unroll 1
+                    for (int z = za; z < zb; ++z) {
+                        float w[8];
+                        ld_global_32B(reinterpret_cast<const float*>(ga + z * slice_stride + 4 * M * q), w);
+#pragma unroll
+                        for (int s = 0; s + 1 < NDZ; ++s)
+#pragma unroll
+                            for (int x = 0; x < 8; ++x) ring[s][x] = ring[s + 1][x];
+                        load_b(NDZ - 1, z + dz + NDZ - 1);
+#pragma unroll
+                        for (int s = 0; s < NDZ; ++s)
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const int i = 2 * q + h;
+                                float2 pr, pi;
+                                mulc2(make_float2(w[4 * h], w[4 * h + 1]), make_float2(w[4 * h + 2], w[4 * h + 3]),
+                                      make_float2(ring[s][4 * h], ring[s][4 * h + 1]),
+                                      make_float2(ring[s][4 * h + 2], ring[s][4 * h + 3]), pr, pi);
+                                sre[s][i] = ROT ? subv(sre[s][i], pi) : addv(sre[s][i], pr);
+                                sim[s][i] = ROT ? addv(sim[s][i], pr) : addv(sim[s][i], pi);
+                            }
+                    }
+                }
+            };
+            if (kx >= 0) {
+                const cpx<T>* ga = FA + ((size_t)a * DA * Qh + kx) * P + lane_off;
+                const cpx<T>* gb = FB + ((size_t)b * DB * Qh + kx) * P + lane_off;
+                depth_sum(std::false_type{}, ga, gb);
+                if (kx == 0) depth_sum(std::true_type{}, ga + (size_t)L * P, gb + (size_t)L * P);
+            }
+        } else if constexpr (VOL) {
             if (kx >= 0) {
                 const int dz = dzo - (DA - 1);
                 const int z0 = dz < 0 ? -dz : 0, z1 = DA < DB - dz ? DA : DB - dz;
@@ -773,6 +835,22 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
                              : "memory");
             }
         }
+        // this item's rows below; its successor's fields once they are known
+        cpx<T>* yp = Y + (size_t)e * y_rows<T>(Rout) * L;
+        const int c0 = kxb * UPR, dz0 = dzo * NDZ;
+        bool more = false;
+#pragma unroll 1
+        for (int s = 0; s < NDZ; ++s) {
+        if (NDZ > 1) {
+            if (dz0 + s >= Dz) break;  // uniform
+#pragma unroll
+            for (int t = 0; t < NDZ; ++t)
+#pragma unroll
+                for (int i = 0; i < H; ++i) {
+                    re[i] = s == t ? sre[t % (NDZ > 1 ? NDZ : 1)][i] : re[i];
+                    im[i] = s == t ? sim[t % (NDZ > 1 ? NDZ : 1)][i] : im[i];
+                }
+        }
         if constexpr (PK) {
             team_core_pk<M, +1, true>(re, im, j, reinterpret_cast<float*>(slice), reinterpret_cast<const float4*>(tw_sq));
 #pragma unroll
@@ -785,14 +863,14 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
 #pragma unroll
             for (int k2 = 0; k2 < M; ++k2) slice[j + M * k2] = v[brev(k2, M)];
         }
-        // Rows below: this item's; then its successor's fields
-        cpx<T>* yp = Y + (size_t)e * y_rows<T>(Rout) * L;
-        const int c0 = kxb * UPR, row_off = dzo * R2;
-        if (threadIdx.x == 0) decode(next);
+        const int row_off = (dz0 + s) * R2;
+        if (s == 0 && threadIdx.x == 0) decode(next);
         __syncthreads();
-        const bool more = s_next[0] != 0;
-        e = s_next[1], a = s_next[2], b = s_next[3], kxb = s_next[4], dzo = s_next[5];
-        if (more) load_fa();
+        if (s == 0) {
+            more = s_next[0] != 0;
+            e = s_next[1], a = s_next[2], b = s_next[3], kxb = s_next[4], dzo = s_next[5];
+            if (more) load_fa();
+        }
         // Rows k + q NQ, q < R, of chunk c: X[k + q NQ] = sum_s w_R^{sq} (W_P^{sk} E_s[k])
         auto emit = [&](auto splitc) {
             constexpr bool SPLIT = decltype(splitc)::value;
@@ -859,7 +937,8 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
         };
         if (split) emit(std::true_type{});
         else emit(std::false_type{});
-        __syncthreads();  // the buffer's reads (and s_next's) done before the next item writes it
+        __syncthreads();  // the buffer's reads (and s_next's) done before it is written again
+        }
         if (!more) break;
     }
 }

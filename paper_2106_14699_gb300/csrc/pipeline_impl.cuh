@@ -73,7 +73,7 @@ static cudaError_t launch_pair_cols(const Geom& g, const PipeArgs<T>& a, cudaStr
         per_sm = n > 0 ? n : 1;
     }
     const long long np = a.plist ? a.chunk_cap : (long long)g.KA * g.KB;  // list mode: at most chunk_cap pairs
-    const long long items = np * ((g.Ys + C::TPB - 1) / C::TPB) * (VOL ? g.Dz : g.units);
+    const long long items = np * ((g.Ys + C::TPB - 1) / C::TPB) * (VOL ? (g.Dz + C::NDZ - 1) / C::NDZ : g.units);
     const int bps = a.cols_bps > 0 && a.cols_bps < per_sm ? a.cols_bps : per_sm;
     const long long slots = a.num_sms > 0 ? (long long)bps * a.num_sms : items;
     const int grid = (int)(items < slots ? items : slots);
