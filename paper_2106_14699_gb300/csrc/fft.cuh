@@ -223,6 +223,7 @@ struct Tw {
     const cpx<T>* n[14];
     const cpx<T>* sq[6];
     const cpx<T>* n3[12];
+    const double2* lg;  // FP64: the c log2 c table of weighted maps (kernels.cuh)
 };
 
 // The table of e^{-2 pi i k / N} for a transform length N = 2^l or 3 2^l.
@@ -368,7 +369,11 @@ __device__ __forceinline__ void team_fft_core(cpx<T> (&v)[M], int j, void* sm, c
             v[brev(k + H, M)] = {re[k].y, im[k].y};
         }
     } else {
-        dft_reg<M, DIR>(v);  // v[brev(k1)] = A[j][k1]
+        auto dft = [&]() {
+            if constexpr (std::is_same<T, double>::value) dft_lf<M, DIR>(v);
+            else dft_reg<M, DIR>(v);
+        };
+        dft();  // v[brev(k1)] = A[j][k1]
 #pragma unroll
         for (int k1 = 1; k1 < M; ++k1) v[brev(k1, M)] = cmul(v[brev(k1, M)], twl<DIR>(twq, k1 * M + j));
         if constexpr (sizeof(T) == 4) {
@@ -396,7 +401,7 @@ __device__ __forceinline__ void team_fft_core(cpx<T> (&v)[M], int j, void* sm, c
             for (int n2 = 0; n2 < M; ++n2) v[n2] = sc[j * M + (n2 ^ j)];
             __syncwarp();
         }
-        dft_reg<M, DIR>(v);  // v[brev(k2)] = X_r[j + M k2]
+        dft();  // v[brev(k2)] = X_r[j + M k2]
     }
 }
 

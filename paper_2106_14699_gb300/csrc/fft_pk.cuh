@@ -19,7 +19,13 @@
 
 namespace cmif {
 
+// FP64 register DFTs (weighted maps) take the same butterflies: 16 points in 148 instead of 168
+// FP64 instructions, which run at 1/64 rate.
+
 // a * k + b and a - b for scalars and for pairs (k a compile-time constant)
+__device__ __forceinline__ double fmak(double a, double k, double b) { return fma(a, k, b); }
+__device__ __forceinline__ double addv(double a, double b) { return a + b; }
+__device__ __forceinline__ double subv(double a, double b) { return a - b; }
 __device__ __forceinline__ float fmak(float a, float k, float b) { return fmaf(a, k, b); }
 __device__ __forceinline__ float2 fmak(float2 a, float k, float2 b) { return __ffma2_rn(a, make_float2(k, k), b); }
 __device__ __forceinline__ float addv(float a, float b) { return a + b; }
@@ -50,17 +56,18 @@ __device__ __forceinline__ void bfly(V& er, V& ei, V& orr, V& oi, int k) {
             oi = addv(b, x);
         }
     } else {
+        using K = typename std::conditional<std::is_same<V, double>::value, double, float>::type;
         const double c = cos32(k), s = DIR > 0 ? sin32(k) : -sin32(k);
         const V a = er, b = ei;
         if (c * c >= s * s) {
-            const float t = (float)(s / c), cf = (float)c;
+            const K t = (K)(s / c), cf = (K)c;
             const V u = fmak(oi, -t, orr), v = fmak(orr, t, oi);
             er = fmak(u, cf, a);
             ei = fmak(v, cf, b);
             orr = fmak(u, -cf, a);
             oi = fmak(v, -cf, b);
         } else {
-            const float t = (float)(c / s), sf = (float)s;
+            const K t = (K)(c / s), sf = (K)s;
             const V u = fmak(orr, -t, oi), v = fmak(oi, t, orr);
             er = fmak(u, -sf, a);
             ei = fmak(v, sf, b);
@@ -94,6 +101,27 @@ __device__ __forceinline__ void dft_pk(float2 (&re)[M / 2], float2 (&im)[M / 2])
         re[k] = a[k];
         im[k] = b[k];
     }
+}
+
+// The same network on scalars: M-point DFT of v, natural order in, bit-reversed order out
+// (v[brev(k, M)] = X[k], as dft_reg).
+template <int M, int DIR, typename T>
+__device__ __forceinline__ void dft_lf(cpx<T> (&v)[M]) {
+    T a[M], b[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        a[i] = v[brev(i, M)].x;
+        b[i] = v[brev(i, M)].y;
+    }
+#pragma unroll
+    for (int half = 1; half < M; half <<= 1)
+#pragma unroll
+        for (int s = 0; s < M; s += 2 * half)
+#pragma unroll
+            for (int k = 0; k < half; ++k)
+                bfly<DIR>(a[s + k], b[s + k], a[s + k + half], b[s + k + half], k * (16 / half));
+#pragma unroll
+    for (int k = 0; k < M; ++k) v[brev(k, M)] = {a[k], b[k]};
 }
 
 }  // namespace cmif

@@ -1335,11 +1335,34 @@ struct RowWCfg {
     static constexpr int THREADS = NT * TEAM;
     static constexpr int U = (Q + THREADS - 1) / THREADS;  // positions per thread
     static constexpr int REGION = G::SCRATCH;              // one row of Q doubles
-    static constexpr size_t SMEM = (size_t)NT * REGION;
+    static constexpr size_t OFF_LG = (size_t)NT * REGION;
+    static constexpr size_t SMEM = OFF_LG + (size_t)(1 << 9) * 16;  // + the logarithm table
     static_assert(REGION >= Q * 8, "team scratch must hold one row of counts");
 };
 
-__device__ __forceinline__ double xlog2x(double c) { return c > 0.0 ? c * log2(c) : 0.0; }
+// log2 c for c > 0, table-driven (Tang, ACM Trans. Math. Software 16(4), 1990): c = m 2^e, the top 9
+// bits of m pick r ~ 1 / m with log2(1 / r) tabulated, z = m r - 1 is exact to one rounding,
+// |z| <= 2^-9, and log2(1 + z) = (z - z^2/2 + z^3/3 - ...) / ln 2 to z^6 (the rest is below
+// 2^-64).  at most 1 ulp (|log2 c| >= 1; 2e-16 absolute below).  Nine FP64 instructions, at 1/64 rate the kernel's scarcest; the math library's log2
+// took over half of the kernel's time (200 x 256, K = 12: 3.45 ms, with the table 1.83).
+constexpr int kLgBits = 9, kLgSize = 1 << kLgBits;
+__device__ __forceinline__ double lg2_table(double c, const double2* lg) {
+    const int hi = __double2hiint(c);
+    if (hi < 0x00100000) return log2(c);  // denormal
+    const double2 t = lg[(hi >> (20 - kLgBits)) & (kLgSize - 1)];
+    const double m = __hiloint2double((hi & 0xFFFFF) | 0x3FF00000, __double2loint(c));
+    const double z = fma(m, t.x, -1.0);
+    // e as a double: 2^52 + 2^31 + e, less 2^52 + 2^31
+    const double e = __hiloint2double(0x43300000, ((hi >> 20) - 1023) ^ (int)0x80000000) - 4503601774854144.0;
+    constexpr double il = 1.4426950408889634074;  // 1 / ln 2
+    double p = fma(z, -il / 6, il / 5);
+    p = fma(z, p, -il / 4);
+    p = fma(z, p, il / 3);
+    p = fma(z, p, -il / 2);
+    p = fma(z, p, il);
+    return e + fma(z, p, t.y);
+}
+__device__ __forceinline__ double xlog2x(double c, const double2* lg) { return c > 0.0 ? c * lg2_table(c, lg) : 0.0; }
 
 template <int Q>
 __global__ void __launch_bounds__(RowWCfg<Q>::THREADS, 1)
@@ -1350,6 +1373,8 @@ k_pair_rows_w(const cpx<double>* __restrict__ Y, Geom g, Tw<double> tw, double* 
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int tid = threadIdx.x, team = tid / C::TEAM, lt = tid % C::TEAM, r = lt / M, j = lt % M;
     unsigned char* region = smem_raw + (size_t)team * C::REGION;
+    double2* lg = reinterpret_cast<double2*>(smem_raw + C::OFF_LG);
+    for (int i = tid; i < kLgSize; i += BT) lg[i] = tw.lg[i];  // visible after the first round's barriers
     const int KB = g.KB, npairs = g.KA * g.KB, Rout = g.R, Cout = g.C;
     double* cb = cbw + (size_t)blockIdx.x * KB * Q;
     double row_max_n = 0.0;
@@ -1386,7 +1411,7 @@ k_pair_rows_w(const cpx<double>* __restrict__ Y, Geom g, Tw<double> tw, double* 
                 if (a != cur_a) {  // uniform: the A-marginal of label cur_a is complete
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        S[u] -= xlog2x(CA[u]);
+                        S[u] -= xlog2x(CA[u], lg);
                         N[u] += CA[u];
                         CA[u] = 0.0;
                     }
@@ -1398,7 +1423,7 @@ k_pair_rows_w(const cpx<double>* __restrict__ Y, Geom g, Tw<double> tw, double* 
                     const int p = tid + BT * u;
                     if (p >= Q) continue;
                     const double c = fmax(obt[p], 0.0);
-                    S[u] += xlog2x(c);
+                    S[u] += xlog2x(c, lg);
                     CA[u] += c;
                     cb[(size_t)b * Q + p] += c;
                 }
@@ -1410,13 +1435,13 @@ k_pair_rows_w(const cpx<double>* __restrict__ Y, Geom g, Tw<double> tw, double* 
         for (int u = 0; u < U; ++u) {
             const int p = tid + BT * u;
             if (p >= Q) continue;
-            S[u] -= xlog2x(CA[u]);
+            S[u] -= xlog2x(CA[u], lg);
             N[u] += CA[u];
-            for (int b = 0; b < KB; ++b) S[u] -= xlog2x(cb[(size_t)b * Q + p]);
+            for (int b = 0; b < KB; ++b) S[u] -= xlog2x(cb[(size_t)b * Q + p], lg);
             const int cidx = circ_to_out(p, Q, g.WA, g.WB - 1);
             if (cidx < 0) continue;
             const size_t o = (size_t)row * Cout + cidx;
-            mi_map[o] = N[u] > 0.0 ? (S[u] + xlog2x(N[u])) / N[u] : 0.0;
+            mi_map[o] = N[u] > 0.0 ? (S[u] + xlog2x(N[u], lg)) / N[u] : 0.0;
             nw_map[o] = N[u];
             if (cidx >= g.c0 && cidx < g.c1) row_max_n = fmax(row_max_n, N[u]);
         }

@@ -638,22 +638,30 @@ cudaError_t get_twiddles(int device, Tw<float>* tf, Tw<double>* td, Tw<m31>* tm)
         for (int l = 0; l < 6; ++l) fill_sq_f32(hf.data() + 2 * off_sq[l], 1 << l);
         // every table starts on a 256-byte boundary
         const size_t bytes_d = (2 * n * sizeof(double) + 255) / 256 * 256, bytes_f = (2 * n * sizeof(float) + 255) / 256 * 256;
-        const size_t bytes_m = hm.size() * sizeof(uint32_t);
+        const size_t bytes_m = (hm.size() * sizeof(uint32_t) + 255) / 256 * 256, bytes_l = (size_t)kLgSize * sizeof(double2);
+        // r = 1 / (midpoint of the mantissas that share their top bits) and log2(1 / r)
+        std::vector<double> hl(2 * kLgSize);
+        for (int i = 0; i < kLgSize; ++i) {
+            hl[2 * i] = 1.0 / (1.0 + (i + 0.5) / kLgSize);
+            hl[2 * i + 1] = (double)-std::log2((long double)hl[2 * i]);
+        }
         int prev = -1;
         cudaGetDevice(&prev);
         cudaError_t e = cudaSetDevice(device);
         if (e != cudaSuccess) return e;
         void* buf = nullptr;
-        e = cudaMalloc(&buf, bytes_d + bytes_f + bytes_m);
+        e = cudaMalloc(&buf, bytes_d + bytes_f + bytes_m + bytes_l);
         if (e == cudaSuccess) e = cudaMemcpy(buf, hd.data(), hd.size() * sizeof(double), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d, hf.data(), hf.size() * sizeof(float), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d + bytes_f, hm.data(), bytes_m, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d + bytes_f, hm.data(), hm.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy((char*)buf + bytes_d + bytes_f + bytes_m, hl.data(), bytes_l, cudaMemcpyHostToDevice);
         if (prev >= 0) cudaSetDevice(prev);
         if (e != cudaSuccess) {
             if (buf) cudaFree(buf);
             return e;
         }
         t.buf = buf;
+        t.td.lg = reinterpret_cast<const double2*>((char*)buf + bytes_d + bytes_f + bytes_m);
         const cpx<double>* bd = reinterpret_cast<const cpx<double>*>(buf);
         const cpx<float>* bf = reinterpret_cast<const cpx<float>*>((char*)buf + bytes_d);
         const cpx<m31>* bm = reinterpret_cast<const cpx<m31>*>((char*)buf + bytes_d + bytes_f);
