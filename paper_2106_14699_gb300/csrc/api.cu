@@ -118,7 +118,7 @@ struct cmif_plan_s {
     // workspace is sized for (ucap units; g itself when ucap = 1).
     int ucap = 1;
     Geom gcap{};
-    int* maxn_u = nullptr;    // [ucap] per-unit max N of the gamma gate
+    int* maxn_u = nullptr;    // [2 ucap] per-unit max N of the gamma gate, then the peak search's block counts
     // CMIF_AUTO: per-pair precision (predicate up front, guard after the FP32 pass)
     Escal esc;
     double pred_scale = 0.0;   // kappa u log2(PQ): the predicate is pred_scale sqrt(|X_a| |Y_b|) >= pred_thr
@@ -314,6 +314,11 @@ bool call_geom(const cmif_plan p, double gamma, Geom* out) {
     return g.r0 < g.r1 && g.c0 < g.c1;
 }
 
+// Zero the map's status word and, for a call's first map, the call's total behind it.
+cudaError_t reset_status(cmif_plan p, bool first, cudaStream_t s) {
+    return cudaMemsetAsync(p->st, 0, first ? align_up(sizeof(DevStatus), 256) + sizeof(DevStatus) : sizeof(DevStatus), s);
+}
+
 // Second precision for one stage of the pair list (entries [lrange[0], lrange[1])):
 // the level-set transforms of the planes the listed pairs need, then, chunk by
 // chunk, their products, inverse column transforms and exact counts (into the
@@ -351,17 +356,19 @@ cudaError_t tier2_stage(cmif_plan p, const Geom& g, const int32_t* A, const uint
 // only after a breach).  Counts of every pair are then exact (Sec. 3.2).
 cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const uint8_t* MA, const int32_t* B,
                              const uint8_t* MB, double* mi, int32_t* n, int32_t* counts, cudaStream_t s,
-                             unsigned stages32) {
+                             unsigned stages32, bool first) {
     Escal& E = p->esc;
-    cudaError_t e = cudaMemsetAsync(p->st, 0, sizeof(DevStatus), s);
+    cudaError_t e = reset_status(p, first, s);
     PipeArgs<float> a = p->w32.args;
     fill_io(a, A, MA, B, MB, mi, n, counts, p->st, p);
     a.prof = p->prof.enabled ? &p->prof : nullptr;
     a.prec_slot = 0;
     a.conditional = 0;
     // 1. FP32 level-set transforms, with the label pixel counts of the predicate
-    if (e == cudaSuccess && (stages32 & STAGE_FWD_A)) e = cudaMemsetAsync(E.popA, 0, g.KA * sizeof(int), s);
-    if (e == cudaSuccess && (stages32 & STAGE_FWD_B)) e = cudaMemsetAsync(E.popB, 0, g.KB * sizeof(int), s);
+    if (e == cudaSuccess && (stages32 & STAGE_FWD_A))  // popB follows popA
+        e = cudaMemsetAsync(E.popA, 0, align_up(g.KA * sizeof(int), 256) + g.KB * sizeof(int), s);
+    else if (e == cudaSuccess && (stages32 & STAGE_FWD_B))
+        e = cudaMemsetAsync(E.popB, 0, g.KB * sizeof(int), s);
     if (e != cudaSuccess) return from_cuda(e);
     a.popA = (stages32 & STAGE_FWD_A) ? E.popA : nullptr;
     a.popB = (stages32 & STAGE_FWD_B) ? E.popB : nullptr;
@@ -374,8 +381,8 @@ cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const
         e = launch_select_pairs(E.popA, E.popB, g.KA, g.KB, p->pred_scale, p->pred_thr, E.cap, E.plist, E.hdr,
                                 E.ov_slot, E.pair_res, E.needA, E.needB, p->st, s);
     p->prof.end(s);
-    // 3. second precision for the predicted pairs
-    if (e == cudaSuccess)
+    // 3. second precision for the predicted pairs (none with the predicate off)
+    if (e == cudaSuccess && p->pred_thr < HUGE_VAL)
         e = tier2_stage(p, g, A, MA, B, MB, E.hdr + 0, s);
     // 4. FP32 pair stages; listed pairs take their exact counts, the others' residuals are kept per pair
     a.ov = E.ov;
@@ -396,8 +403,7 @@ cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const
     if (e == cudaSuccess) e = run_pipeline<float>(g, a, s);
     if (e != cudaSuccess) return from_cuda(e);
     p->prof.begin("finalize", s);
-    e = launch_finalize(p->st, 2, 2, s);
-    if (e == cudaSuccess) e = launch_merge_status(p->st, p->st_total, 2, s);
+    e = launch_finalize(p->st, p->st_total, 2, s);
     p->prof.end(s);
     return from_cuda(e);
 }
@@ -407,9 +413,9 @@ cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const
 // reused across calls); an exact pass (FP64 and two-term plans) always recomputes everything.
 cmif_status compute_map(cmif_plan p, const Geom& g, const int32_t* A, const uint8_t* MA, const int32_t* B,
                         const uint8_t* MB, double* mi, int32_t* n, int32_t* counts, cudaStream_t s,
-                        unsigned stages32 = STAGE_ALL) {
-    if (p->prec == CMIF_AUTO) return compute_map_auto(p, g, A, MA, B, MB, mi, n, counts, s, stages32);
-    cudaError_t e = cudaMemsetAsync(p->st, 0, sizeof(DevStatus), s);
+                        unsigned stages32, bool first) {
+    if (p->prec == CMIF_AUTO) return compute_map_auto(p, g, A, MA, B, MB, mi, n, counts, s, stages32, first);
+    cudaError_t e = reset_status(p, first, s);
     if (e != cudaSuccess) return from_cuda(e);
     if (p->prec == CMIF_FP32) {
         PipeArgs<float> a = p->w32.args;
@@ -431,8 +437,7 @@ cmif_status compute_map(cmif_plan p, const Geom& g, const int32_t* A, const uint
     if (e != cudaSuccess) return from_cuda(e);
     const int slot_default = (p->prec == CMIF_FP64 || p->prec == CMIF_SPLIT32) ? 1 : 0;
     p->prof.begin("finalize", s);
-    e = launch_finalize(p->st, slot_default, slot_default, s);
-    if (e == cudaSuccess) e = launch_merge_status(p->st, p->st_total, slot_default, s);
+    e = launch_finalize(p->st, p->st_total, slot_default, s);
     p->prof.end(s);
     return from_cuda(e);
 }
@@ -578,7 +583,7 @@ size_t small_bytes_of(const cmif_plan p) {
     off = align_up(off + u * g.HB * g.WB * sizeof(int32_t), 256);
     off = align_up(off + u * g.HB * g.WB, 256);
     off = align_up(off + (size_t)(kMaxAngles + 2) * sizeof(PeakRec), 256);
-    off = align_up(off + u * sizeof(int), 256);
+    off = align_up(off + 2 * u * sizeof(int), 256);
     return off;
 }
 
@@ -639,7 +644,7 @@ cmif_status plan_carve(cmif_plan p, char* base) {
     p->wB = (int32_t*)(base + off); off = align_up(off + u * g.HB * g.WB * sizeof(int32_t), 256);
     p->wM = (uint8_t*)(base + off); off = align_up(off + u * g.HB * g.WB, 256);
     p->peaks = base + off; off = align_up(off + (size_t)(kMaxAngles + 2) * sizeof(PeakRec), 256);
-    p->maxn_u = (int*)(base + off); off = align_up(off + u * sizeof(int), 256);
+    p->maxn_u = (int*)(base + off); off = align_up(off + 2 * u * sizeof(int), 256);
     p->small_bytes = off;
     if (p->has32) {
         carve_workspace<float>(p->gcap, p->w32, base + off);
@@ -743,8 +748,7 @@ cmif_status align_core_units(cmif_plan plan, const Geom& g, const int32_t* A, co
         e = run_pipeline<float>(gu, a, s);
         if (e != cudaSuccess) return from_cuda(e);
         plan->prof.begin("finalize", s);
-        e = launch_finalize(plan->st, 0, 0, s);
-        if (e == cudaSuccess) e = launch_merge_status(plan->st, plan->st_total, 0, s);
+        e = launch_finalize(plan->st, plan->st_total, 0, s);
         plan->prof.end(s);
         if (e != cudaSuccess) return from_cuda(e);
         plan->prof.begin("peak", s);
@@ -767,8 +771,7 @@ cmif_status align_core(cmif_plan plan, const int32_t* A, const uint8_t* M_A, con
     if (plan->ucap > 1 && plan->prec == CMIF_FP32)
         return align_core_units(plan, g, A, M_A, B, M_B, angles, n_angles, gamma, top_k, topk_dev, mi_maps, n_maps, s);
     const size_t RC = (size_t)g.R * g.C;
-    cudaError_t e = cudaMemsetAsync(plan->st_total, 0, sizeof(DevStatus), s);
-    if (e != cudaSuccess) return from_cuda(e);
+    cudaError_t e = cudaSuccess;
     PeakRec* peaks = reinterpret_cast<PeakRec*>(plan->peaks);
     for (int i = 0; i < n_angles; ++i) {
         plan->prof.begin("warp_nn", s);
@@ -783,7 +786,7 @@ cmif_status align_core(cmif_plan plan, const int32_t* A, const uint8_t* M_A, con
             if (e != cudaSuccess) return from_cuda(e);
         }
         const unsigned stages = (i == 0) ? STAGE_ALL : (STAGE_FWD_B | STAGE_PAIRS);
-        cmif_status cs = compute_map(plan, g, A, M_A, plan->wB, plan->wM, mi, nm, nullptr, s, stages);
+        cmif_status cs = compute_map(plan, g, A, M_A, plan->wB, plan->wM, mi, nm, nullptr, s, stages, i == 0);
         if (cs != CMIF_OK) return cs;
         plan->prof.begin("peak", s);
         e = launch_peak(mi, nm, g, plan->st, gamma, plan->parts, plan->nparts, i, peaks + i, s);
@@ -925,6 +928,7 @@ cmif_status autotune(cmif_plan p, const char* cache_path, cmif_tuning* out) {
             std::vector<float> ts;
             for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {
                 e = cudaEventRecord(e0, s);
+                if (e == cudaSuccess) e = cudaMemsetAsync(p->st, 0, sizeof(DevStatus), s);
                 if (e == cudaSuccess) e = run_pipeline<float>(g, a, s);
                 if (e == cudaSuccess) e = cudaEventRecord(e1, s);
                 if (e == cudaSuccess) e = cudaEventSynchronize(e1);
@@ -1058,8 +1062,7 @@ cmif_status cmif_compute(cmif_plan plan, const int32_t* A, const uint8_t* M_A, c
     Geom g;
     if (!call_geom(plan, gamma, &g)) return CMIF_ERR_INVALID_ARG;
     return run_graph(plan, s, key, [&](cudaStream_t cs) -> cmif_status {
-        cudaError_t e = cudaMemsetAsync(plan->st_total, 0, sizeof(DevStatus), cs);
-        if (e != cudaSuccess) return from_cuda(e);
+        cudaError_t e = cudaSuccess;
         if (g.r0 > 0 || g.r1 < g.R) {  // rows outside the window are not computed: zero
             const size_t RC = (size_t)g.R * g.C;
             e = cudaMemsetAsync(mi_map, 0, RC * sizeof(double), cs);
@@ -1068,7 +1071,7 @@ cmif_status cmif_compute(cmif_plan plan, const int32_t* A, const uint8_t* M_A, c
                 e = cudaMemsetAsync(counts, 0, RC * sizeof(int32_t) * ((size_t)g.KA * g.KB + g.KA + g.KB), cs);
             if (e != cudaSuccess) return from_cuda(e);
         }
-        cmif_status st = compute_map(plan, g, A, M_A, B, M_B, mi_map, nm, counts, cs);
+        cmif_status st = compute_map(plan, g, A, M_A, B, M_B, mi_map, nm, counts, cs, STAGE_ALL, true);
         if (st != CMIF_OK) return st;
         if (peak_dev) {
             plan->prof.begin("peak", cs);
@@ -1098,8 +1101,7 @@ cmif_status cmif_compute_weighted(cmif_plan plan, const int32_t* A, const double
     key_add(key, A); key_add(key, W_A); key_add(key, B); key_add(key, W_B);
     key_add(key, mi_map); key_add(key, nw); key_add(key, gamma); key_add(key, peak_dev);
     return run_graph(plan, s, key, [&](cudaStream_t cs) -> cmif_status {
-        cudaError_t e = cudaMemsetAsync(plan->st_total, 0, sizeof(DevStatus), cs);
-        if (e == cudaSuccess) e = cudaMemsetAsync(plan->st, 0, sizeof(DevStatus), cs);
+        cudaError_t e = reset_status(plan, true, cs);
         if (e == cudaSuccess && (g.r0 > 0 || g.r1 < g.R)) {  // rows outside the window are not computed: zero
             const size_t RC = (size_t)g.R * g.C;
             e = cudaMemsetAsync(mi_map, 0, RC * sizeof(double), cs);
@@ -1391,7 +1393,7 @@ cmif_status cmif_compute_batch(cmif_batch batch, cmif_peak* results_dev, int32_t
                 if (e != cudaSuccess) return from_cuda(e);
                 Geom g;
                 if (!call_geom(p, d.gamma, &g)) return CMIF_ERR_INVALID_ARG;
-                st = compute_map(p, g, d.A, d.M_A, d.B, d.M_B, p->mibuf, p->nbuf, nullptr, cs);
+                st = compute_map(p, g, d.A, d.M_A, d.B, d.M_B, p->mibuf, p->nbuf, nullptr, cs, STAGE_ALL, false);
                 if (st != CMIF_OK) return st;
                 e = launch_peak(p->mibuf, p->nbuf, g, p->st, d.gamma, p->parts, p->nparts, 0, results_dev + i, cs);
                 if (e != cudaSuccess) return from_cuda(e);

@@ -11,7 +11,8 @@ struct DevStatus {
     int max_n;             // max_chi N(chi) of the last map (for the gamma gate of Alg. 1)
     int escalations;       // CMIF_AUTO: label pairs re-run in the second precision after the FP32 guard breached
     int predicted;         // CMIF_AUTO: label pairs the precision predicate sent to the second precision up front
-    int pad[2];
+    int work;              // next item of the map's pair-column launch (zeroed with the status word)
+    unsigned peak_done;    // blocks of the peak search that have left their partial result
     unsigned long long max_nw_bits;  // weighted maps (SWMI): max N(chi) as double bits (N >= 0)
 };
 enum : unsigned {

@@ -18,6 +18,23 @@ __device__ __forceinline__ bool better(double m1, long long i1, double m2, long 
     return m1 > m2 || (m1 == m2 && i1 < i2);
 }
 
+// The best (value, index) of a block of at most 1024 threads, in thread 0.
+__device__ __forceinline__ void block_best(double& bm, long long& bi) {
+    __shared__ double sm_m[32];
+    __shared__ long long sm_i[32];
+    for (int off = 16; off > 0; off >>= 1) {
+        const double om = __shfl_xor_sync(0xffffffffu, bm, off);
+        const long long oi = __shfl_xor_sync(0xffffffffu, bi, off);
+        if (oi >= 0 && (bi < 0 || better(om, oi, bm, bi))) { bm = om; bi = oi; }
+    }
+    const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    if ((threadIdx.x & 31) == 0) { sm_m[w] = bm; sm_i[w] = bi; }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int k = 1; k < nw; ++k)
+            if (sm_i[k] >= 0 && (bi < 0 || better(sm_m[k], sm_i[k], bm, bi))) { bm = sm_m[k]; bi = sm_i[k]; }
+}
+
 // Scans the search window rows [r0, r1) x columns [c0, c1) of the (R x Cout) maps;
 // indices stay row-major map indices (ties: lowest).  NT: int32_t N (counts) or
 // double N (weighted maps, max N from max_nw_bits).
@@ -30,10 +47,14 @@ __device__ __forceinline__ int32_t n_record(double n) { return (int32_t)fmin(rin
 
 // Units (blockIdx.y): map u starts unit_rc elements further on, its max N comes
 // from maxn_u[u] and its partials from parts + u * gridDim.x.
+// Each block leaves its best in parts; the last one of a unit (done[u], zero at launch) reduces
+// them and writes record u: one launch.  R2 > 0 (volumes): the map rows are (depth offset, row)
+// pairs, depth-offset major; the record's first field then holds the depth offset dz.
 template <typename NT>
-__global__ void k_peak_partial(const double* __restrict__ mi, const NT* __restrict__ n, int Cout, int r0, int r1,
-                               int c0, int c1, const DevStatus* __restrict__ st, double gamma,
-                               PeakPart* __restrict__ parts, long long unit_rc, const int* __restrict__ maxn_u) {
+__global__ void k_peak(const double* __restrict__ mi, const NT* __restrict__ n, int Cout, int r0, int r1, int c0, int c1,
+                       const DevStatus* __restrict__ st, double gamma, PeakPart* parts, long long unit_rc,
+                       const int* __restrict__ maxn_u, unsigned* __restrict__ done, int HA, int WA, int angle_idx, int R2,
+                       int DA, void* __restrict__ peak_out) {
     mi += blockIdx.y * unit_rc;
     n += blockIdx.y * unit_rc;
     parts += (size_t)blockIdx.y * gridDim.x;
@@ -52,56 +73,31 @@ __global__ void k_peak_partial(const double* __restrict__ mi, const NT* __restri
             }
         }
     }
-    __shared__ double sm_m[32];
-    __shared__ long long sm_i[32];
-    for (int off = 16; off > 0; off >>= 1) {
-        const double om = __shfl_xor_sync(0xffffffffu, bm, off);
-        const long long oi = __shfl_xor_sync(0xffffffffu, bi, off);
-        if (oi >= 0 && (bi < 0 || better(om, oi, bm, bi))) { bm = om; bi = oi; }
-    }
-    const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    if ((threadIdx.x & 31) == 0) { sm_m[w] = bm; sm_i[w] = bi; }
-    __syncthreads();
+    block_best(bm, bi);
+    __shared__ bool last;
     if (threadIdx.x == 0) {
-        for (int k = 1; k < nw; ++k)
-            if (sm_i[k] >= 0 && (bi < 0 || better(sm_m[k], sm_i[k], bm, bi))) { bm = sm_m[k]; bi = sm_i[k]; }
         parts[blockIdx.x] = {bm, bi};
+        __threadfence();
+        last = atomicAdd(done + blockIdx.y, 1u) == gridDim.x - 1;
     }
-}
-
-// R2 > 0 (volumes): the map rows are (depth offset, row) pairs, depth-offset
-// major; the record's first field then holds the depth offset dz.
-// Units (blockIdx.x): unit u reads its partials and map and writes record u.
-template <typename NT>
-__global__ void k_peak_final(const PeakPart* __restrict__ parts, int nparts, const double* __restrict__ mi,
-                             const NT* __restrict__ n, int HA, int WA, int Cout, int angle_idx, int R2, int DA,
-                             void* __restrict__ peak_out, long long unit_rc) {
-    parts += (size_t)blockIdx.x * nparts;
-    mi += blockIdx.x * unit_rc;
-    n += blockIdx.x * unit_rc;
-    peak_out = reinterpret_cast<PeakRec*>(peak_out) + blockIdx.x;
-    angle_idx += blockIdx.x;
-    double bm = -INFINITY;
-    long long bi = -1;
-    for (int k = threadIdx.x; k < nparts; k += blockDim.x)
-        if (parts[k].idx >= 0 && (bi < 0 || better(parts[k].mi, parts[k].idx, bm, bi))) { bm = parts[k].mi; bi = parts[k].idx; }
-    __shared__ double sm_m[32];
-    __shared__ long long sm_i[32];
-    for (int off = 16; off > 0; off >>= 1) {
-        const double om = __shfl_xor_sync(0xffffffffu, bm, off);
-        const long long oi = __shfl_xor_sync(0xffffffffu, bi, off);
-        if (oi >= 0 && (bi < 0 || better(om, oi, bm, bi))) { bm = om; bi = oi; }
-    }
-    const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    if ((threadIdx.x & 31) == 0) { sm_m[w] = bm; sm_i[w] = bi; }
     __syncthreads();
+    if (!last) return;
+    // the unit's last block: every partial is written, reduce them to its record
+    __threadfence();
+    bm = -INFINITY;
+    bi = -1;
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) {
+        const double pm = __ldcg(&parts[k].mi);
+        const long long pi = __ldcg(&parts[k].idx);
+        if (pi >= 0 && (bi < 0 || better(pm, pi, bm, bi))) { bm = pm; bi = pi; }
+    }
+    __syncthreads();
+    block_best(bm, bi);
     if (threadIdx.x != 0) return;
-    for (int k = 1; k < nw; ++k)
-        if (sm_i[k] >= 0 && (bi < 0 || better(sm_m[k], sm_i[k], bm, bi))) { bm = sm_m[k]; bi = sm_i[k]; }
-    PeakRec* p = reinterpret_cast<PeakRec*>(peak_out);
+    PeakRec* p = reinterpret_cast<PeakRec*>(peak_out) + blockIdx.y;
     if (bi < 0) { *p = {-1, 0, 0, 0, 0.0}; return; }
     const long long row = bi / Cout;
-    p->angle_idx = R2 > 0 ? (int)(row / R2) - (DA - 1) : angle_idx;
+    p->angle_idx = R2 > 0 ? (int)(row / R2) - (DA - 1) : angle_idx + (int)blockIdx.y;
     p->dy = (int)(R2 > 0 ? row % R2 : row) - (HA - 1);
     p->dx = (int)(bi % Cout) - (WA - 1);
     p->n = n_record(n[bi]);  // weighted maps: N rounded to an integer
@@ -180,20 +176,21 @@ cudaError_t launch_warp_nn(const int32_t* B, const uint8_t* MB, int H, int W, do
     return cudaGetLastError();
 }
 
-// Fold one map's device status into the call's running total.
-__global__ void k_merge_status(const DevStatus* __restrict__ m, DevStatus* __restrict__ tot, int slot_default) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        if (slot_default == 2) {  // per-pair precision: FP32 pairs and second-precision pairs kept apart
-            tot->res_bits[0] = max(tot->res_bits[0], m->res_bits[0]);
-            tot->res_bits[1] = max(tot->res_bits[1], m->res_bits[1]);
-        } else {
-            tot->res_bits[0] = max(tot->res_bits[0], m->res_bits[slot_default]);  // the authoritative pass
-        }
-        tot->flags |= m->flags;
-        tot->escalations += m->escalations;
-        tot->predicted += m->predicted;
-        tot->max_n = max(tot->max_n, m->max_n);
+// Fold one map's device status into the call's running total (one thread).
+__device__ __forceinline__ void merge_status(const DevStatus* m, DevStatus* tot, int slot) {
+    if (slot == 2) {  // per-pair precision: FP32 pairs and second-precision pairs kept apart
+        tot->res_bits[0] = max(tot->res_bits[0], m->res_bits[0]);
+        tot->res_bits[1] = max(tot->res_bits[1], m->res_bits[1]);
+    } else {
+        tot->res_bits[0] = max(tot->res_bits[0], m->res_bits[slot]);  // the authoritative pass
     }
+    tot->flags |= m->flags;
+    tot->escalations += m->escalations;
+    tot->predicted += m->predicted;
+    tot->max_n = max(tot->max_n, m->max_n);
+}
+__global__ void k_merge_status(const DevStatus* __restrict__ m, DevStatus* __restrict__ tot, int slot) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) merge_status(m, tot, slot);
 }
 
 cudaError_t launch_merge_status(const DevStatus* m, DevStatus* tot, int slot_default, cudaStream_t s) {
@@ -249,11 +246,12 @@ cudaError_t launch_status_code(const DevStatus* st, int32_t* out, cudaStream_t s
 
 // Final decision on the authoritative precision's residual (slot 2: per-pair
 // precision, where both the FP32 pairs' and the second-precision pairs' count).
-__global__ void k_finalize(DevStatus* st, int slot_if_escalated, int slot_default) {
+// The map's status is then folded into the call's total (nullable).
+__global__ void k_finalize(DevStatus* st, DevStatus* tot, int slot) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
-        const int slot = (st->flags & STATUS_ESCALATE) ? slot_if_escalated : slot_default;
         const unsigned r = slot == 2 ? max(st->res_bits[0], st->res_bits[1]) : st->res_bits[slot];
         if (__uint_as_float(r) >= kResidualGuard) st->flags |= STATUS_PRECISION;
+        if (tot) merge_status(st, tot, slot);
     }
 }
 
@@ -270,28 +268,30 @@ __global__ void k_unit_max_n(const int32_t* __restrict__ n, int Cout, int r0, in
 }
 
 template <typename NT>
-static cudaError_t launch_peak_t(const double* mi, const NT* n, const Geom& g, const DevStatus* st, double gamma,
-                                 PeakPart* parts, int nparts, int angle_idx, void* peak_out, int units,
-                                 const int* maxn_u, cudaStream_t s) {
+static cudaError_t launch_peak_t(const double* mi, const NT* n, const Geom& g, DevStatus* st, double gamma,
+                                 PeakPart* parts, int nparts, int angle_idx, void* peak_out, int units, int* maxn_u,
+                                 cudaStream_t s) {
     const int HA = g.HA, WA = g.WA, Cout = g.C;
     const long long unit_rc = units > 1 ? (long long)g.R2 * Cout : 0;
-    k_peak_partial<NT><<<dim3(nparts, units), 256, 0, s>>>(mi, n, Cout, g.r0, g.r1, g.c0, g.c1, st, gamma, parts,
-                                                           unit_rc, units > 1 ? maxn_u : nullptr);
-    k_peak_final<NT><<<units, 256, 0, s>>>(parts, nparts, mi, n, HA, WA, Cout, angle_idx, g.Dz > 1 ? g.R2 : 0, g.DA,
-                                             peak_out, unit_rc);
+    // no more blocks than the window's rows need (a block takes whole rows)
+    const int blocks = std::max(1, std::min(nparts, g.r1 - g.r0));
+    k_peak<NT><<<dim3(blocks, units), 256, 0, s>>>(mi, n, Cout, g.r0, g.r1, g.c0, g.c1, st, gamma, parts, unit_rc,
+                                                   units > 1 ? maxn_u : nullptr,
+                                                   units > 1 ? reinterpret_cast<unsigned*>(maxn_u) + units : &st->peak_done,
+                                                   HA, WA, angle_idx, g.Dz > 1 ? g.R2 : 0, g.DA, peak_out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_peak(const double* mi, const int32_t* n, const Geom& g, const DevStatus* st, double gamma,
+cudaError_t launch_peak(const double* mi, const int32_t* n, const Geom& g, DevStatus* st, double gamma,
                         PeakPart* parts, int nparts, int angle_idx, void* peak_out, cudaStream_t s) {
     return launch_peak_t(mi, n, g, st, gamma, parts, nparts, angle_idx, peak_out, 1, nullptr, s);
 }
 
-cudaError_t launch_peak_units(const double* mi, const int32_t* n, const Geom& g, const DevStatus* st, double gamma,
+cudaError_t launch_peak_units(const double* mi, const int32_t* n, const Geom& g, DevStatus* st, double gamma,
                               PeakPart* parts, int nparts, int angle0, void* peaks_out, int* maxn_u,
                               cudaStream_t s) {
-    // per-unit max N first (zeroed here), then the gated argmax of every unit
-    cudaError_t e = cudaMemsetAsync(maxn_u, 0, (size_t)g.units * sizeof(int), s);
+    // per-unit max N first (zeroed here, with the units' block counts), then the gated argmax of every unit
+    cudaError_t e = cudaMemsetAsync(maxn_u, 0, 2 * (size_t)g.units * sizeof(int), s);
     if (e != cudaSuccess) return e;
     const long long unit_rc = (long long)g.R2 * g.C;
     k_unit_max_n<<<dim3(std::max(1, nparts / 2), g.units), 256, 0, s>>>(n, g.C, g.r0, g.r1, g.c0, g.c1, unit_rc,
@@ -299,13 +299,13 @@ cudaError_t launch_peak_units(const double* mi, const int32_t* n, const Geom& g,
     return launch_peak_t(mi, n, g, st, gamma, parts, nparts, angle0, peaks_out, g.units, maxn_u, s);
 }
 
-cudaError_t launch_peak_w(const double* mi, const double* nw, const Geom& g, const DevStatus* st, double gamma,
+cudaError_t launch_peak_w(const double* mi, const double* nw, const Geom& g, DevStatus* st, double gamma,
                           PeakPart* parts, int nparts, void* peak_out, cudaStream_t s) {
     return launch_peak_t(mi, nw, g, st, gamma, parts, nparts, 0, peak_out, 1, nullptr, s);
 }
 
-cudaError_t launch_finalize(DevStatus* st, int slot_if_escalated, int slot_default, cudaStream_t s) {
-    k_finalize<<<1, 32, 0, s>>>(st, slot_if_escalated, slot_default);
+cudaError_t launch_finalize(DevStatus* st, DevStatus* total, int slot, cudaStream_t s) {
+    k_finalize<<<1, 32, 0, s>>>(st, total, slot);
     return cudaGetLastError();
 }
 

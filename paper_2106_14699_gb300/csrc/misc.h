@@ -16,16 +16,16 @@ struct PeakRec {
 };
 
 // Alg. 1's gamma-gated argmax over the call's search window (g.r0..g.r1, g.c0..g.c1).
-cudaError_t launch_peak(const double* mi, const int32_t* n, const Geom& g, const DevStatus* st, double gamma,
+cudaError_t launch_peak(const double* mi, const int32_t* n, const Geom& g, DevStatus* st, double gamma,
                         PeakPart* parts, int nparts, int angle_idx, void* peak_out, cudaStream_t s);
 // Alg. 1's gated argmax of each of g.units maps (unit u: rows u * R2 .., window per unit,
 // its own max N in maxn_u[u], records peaks_out[u] with angle index angle0 + u); the
 // partials need nparts * g.units records.
-cudaError_t launch_peak_units(const double* mi, const int32_t* n, const Geom& g, const DevStatus* st, double gamma,
+cudaError_t launch_peak_units(const double* mi, const int32_t* n, const Geom& g, DevStatus* st, double gamma,
                               PeakPart* parts, int nparts, int angle0, void* peaks_out, int* maxn_u,
                               cudaStream_t s);
 // The same on a weighted map (real N, max N from the status word's max_nw_bits).
-cudaError_t launch_peak_w(const double* mi, const double* nw, const Geom& g, const DevStatus* st, double gamma,
+cudaError_t launch_peak_w(const double* mi, const double* nw, const Geom& g, DevStatus* st, double gamma,
                           PeakPart* parts, int nparts, void* peak_out, cudaStream_t s);
 // CMIF_AUTO per-pair precision: the predicate (list stage 1) and the guard check (stage 2).
 cudaError_t launch_select_pairs(const int* popA, const int* popB, int KA, int KB, double scale, double thr, int cap,
@@ -34,7 +34,8 @@ cudaError_t launch_select_pairs(const int* popA, const int* popB, int KA, int KB
 cudaError_t launch_check_pairs(const unsigned* pair_res, int KA, int KB, int cap, int* plist, int* hdr,
                                int* ov_slot, unsigned char* needA, unsigned char* needB, DevStatus* st,
                                cudaStream_t s);
-cudaError_t launch_finalize(DevStatus* st, int slot_if_escalated, int slot_default, cudaStream_t s);
+// The residual decision of one map, its status then folded into total (nullable).
+cudaError_t launch_finalize(DevStatus* st, DevStatus* total, int slot, cudaStream_t s);
 cudaError_t launch_warp_nn(const int32_t* B, const uint8_t* MB, int H, int W, double theta, int32_t* Bo, uint8_t* Mo,
                            cudaStream_t s);
 // The most units (rotation angles) one launch of the stage kernels takes.

@@ -176,7 +176,7 @@ extern "C" cmif_status cmif_compute_noalloc(int H_A, int W_A, int H_B, int W_B, 
     a.withhold_row = -1;
     e = run_pipeline<float>(g, a, s);
     if (e != cudaSuccess) return to_status(e);
-    e = launch_finalize(st, 0, 0, s);
+    e = launch_finalize(st, nullptr, 0, s);
     if (e != cudaSuccess) return to_status(e);
     if (peak_dev) {
         e = launch_peak(mi_map, nm, g, st, gamma, reinterpret_cast<PeakPart*>(b + oParts), nparts, 0, peak_dev, s);

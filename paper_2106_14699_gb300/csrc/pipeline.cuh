@@ -21,7 +21,7 @@ struct PipeArgs {
     cpx<T>* FB;   // [K_B][Qh][P]
     cpx<T>* Y;    // [K_A*K_B][R][Ys] row-transform inputs, output rows only (layout: kernels.cuh)
     float* cb_global;  // [rows_grid][K_B][Q] when !cb_smem
-    int* work_ctr;     // item counter of the pair-column kernel (zeroed before each launch)
+    int* work_ctr;     // item counter of the pair-column kernel's list launches (others: st->work)
     Tw<T> tw;
     double* mi;
     int32_t* n;

@@ -77,10 +77,16 @@ static cudaError_t launch_pair_cols(const Geom& g, const PipeArgs<T>& a, cudaStr
     const int bps = a.cols_bps > 0 && a.cols_bps < per_sm ? a.cols_bps : per_sm;
     const long long slots = a.num_sms > 0 ? (long long)bps * a.num_sms : items;
     const int grid = (int)(items < slots ? items : slots);
-    e = cudaMemsetAsync(a.work_ctr, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
+    // a map's one launch counts in its status word, which is zeroed with it; the list launches
+    // of the second precision, several per map, have a counter of their own
+    int* ctr = &a.st->work;
+    if (a.plist) {
+        ctr = a.work_ctr;
+        e = cudaMemsetAsync(ctr, 0, sizeof(int), s);
+        if (e != cudaSuccess) return e;
+    }
     kern<<<grid, C::THREADS, smem, s>>>(a.FA, a.FB, g.KA, g.KB, g.Qh, g.HA, g.HB, g.R, g.r0, g.r1, a.Y, a.tw,
-                                        tw_table(a.tw, g.Q), a.st, a.conditional, a.work_ctr, g.DA, g.DB, g.R2, a.plist, a.lrange,
+                                        tw_table(a.tw, g.Q), a.st, a.conditional, ctr, g.DA, g.DB, g.R2, a.plist, a.lrange,
                                         a.chunk_off, a.chunk_cap, VOL ? 1 : g.units);
     return cudaGetLastError();
 }

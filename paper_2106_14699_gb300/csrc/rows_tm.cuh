@@ -546,6 +546,9 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                     } else if (seg >= NMED) {
                         accum(std::integral_constant<int, NMED>{}, t, b);
                         d = NMED;
+                    } else if (seg >= 2) {
+                        accum(std::integral_constant<int, 2>{}, t, b);
+                        d = 2;
                     } else {
                         accum(std::integral_constant<int, 1>{}, t, b);
                         d = 1;
