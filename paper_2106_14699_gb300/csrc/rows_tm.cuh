@@ -329,8 +329,16 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
     // work items of this team: (row, base) in order; prefetch the first active one
     uint32_t phase = 0;
     bool pending = false;  // a copy issued for this team and not yet waited for
-    // work: the window's rows r0 + blockIdx.x + k * gridDim.x of every unit (units > 1:
-    // several maps, R2 rows apart), unit by unit
+    // work: tasks blockIdx.x + k * gridDim.x of the window's rows; several units (maps, R2
+    // rows apart) form one run of tasks, so that the last round of blocks is short once
+    // and not once per unit
+    const int nr = g.r1 - g.r0;
+    auto advance = [&](int& rr, int& base) {  // task offset rr within its unit, the unit's first row
+        while (rr >= g.r1) {
+            rr -= nr;
+            base += g.R2;
+        }
+    };
     auto issue = [&](int row_i, int pair_i) {
         if (EXT && row_i == withhold_row && pair_i == 0) return;  // diagnostics: leave this wait without its copy
         if (lane == 0) {
@@ -339,13 +347,16 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
         }
         pending = true;
     };
-    if (g.r0 + (int)blockIdx.x < g.r1 && team < npairs) issue(g.r0 + blockIdx.x, team);
+    int rr = g.r0 + (int)blockIdx.x, rbase = 0;  // row of the first unit's window; unit * R2 (multi-unit kernels)
+    if (MULTI) advance(rr, rbase);
+    if (MULTI ? rbase < g.R : rr < g.r1) {
+        if (team < npairs) issue(rbase + rr, team);
+    }
 
     float res_max = 0.f;
     int row_max_n = 0;
     bool aborted = false;
-    int rbase = 0;  // first map row of the current unit (multi-unit kernels: unit * R2, up to R)
-    for (int rr = g.r0 + blockIdx.x; rr < g.r1 && !aborted; rr += gridDim.x) {
+    while ((MULTI ? rbase < g.R : rr < g.r1) && !aborted) {
         const int row = MULTI ? rbase + rr : rr;
         EntAcc<NMI> S[U];
         float CA[U];
@@ -418,9 +429,9 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                     if (npair >= npairs) {
                         npair = team;
                         nrr = rr + gridDim.x;
-                        if (nrr >= g.r1) { nrr = g.r0 + blockIdx.x; nb += g.R2; }
+                        advance(nrr, nb);
                     }
-                    if (nb < g.R && nrr < g.r1) issue(nb + nrr, npair);
+                    if (nb < g.R) issue(nb + nrr, npair);
                 } else {
                     int nrow = row, npair = pair + NT;
                     if (npair >= npairs) { nrow = row + gridDim.x; npair = team; }
@@ -604,12 +615,8 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
             if (cidx >= g.c0 && cidx < g.c1) row_max_n = max(row_max_n, n);
         }
         __syncthreads();
-        if constexpr (MULTI) {  // past the unit's last row: the next unit's first
-            if (rr + (int)gridDim.x >= g.r1 && rbase + g.R2 < g.R) {
-                rbase += g.R2;
-                rr = g.r0 + (int)blockIdx.x - (int)gridDim.x;
-            }
-        }
+        rr += gridDim.x;
+        if (MULTI) advance(rr, rbase);
     }
     // A team may still have a copy in flight (prefetched for an item it will not run
     // after an abort): wait for it, bounded, before the block exits.
