@@ -160,6 +160,7 @@ cmif_status choose_rows(cmif_plan p, Workspace<T>& w) {
         w.cb_smem = smem_cb <= 200 * 1024;
         e = rows_max_blocks_per_sm<T>(g.Q, g.KB, w.cb_smem, &bps);
         if (e != cudaSuccess) return from_cuda(e);
+        w.args.rows_cap = bps * p->num_sms;
     }
     if (bps < 1) return CMIF_ERR_UNSUPPORTED;
     w.rows_grid = std::min(g.R, bps * p->num_sms);
@@ -314,6 +315,9 @@ bool call_geom(const cmif_plan p, double gamma, Geom* out) {
     return g.r0 < g.r1 && g.c0 < g.c1;
 }
 
+// The authoritative residual of a plan's maps: FP32, exact, or (AUTO) both.
+int status_slot(const cmif_plan p) { return p->prec == CMIF_AUTO ? 2 : p->prec == CMIF_FP32 ? 0 : 1; }
+
 // Zero the map's status word and, for a call's first map, the call's total behind it.
 cudaError_t reset_status(cmif_plan p, bool first, cudaStream_t s) {
     return cudaMemsetAsync(p->st, 0, first ? align_up(sizeof(DevStatus), 256) + sizeof(DevStatus) : sizeof(DevStatus), s);
@@ -356,7 +360,7 @@ cudaError_t tier2_stage(cmif_plan p, const Geom& g, const int32_t* A, const uint
 // only after a breach).  Counts of every pair are then exact (Sec. 3.2).
 cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const uint8_t* MA, const int32_t* B,
                              const uint8_t* MB, double* mi, int32_t* n, int32_t* counts, cudaStream_t s,
-                             unsigned stages32, bool first) {
+                             unsigned stages32, bool first, bool finalize) {
     Escal& E = p->esc;
     cudaError_t e = reset_status(p, first, s);
     PipeArgs<float> a = p->w32.args;
@@ -401,7 +405,7 @@ cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const
     a.stages = STAGE_ROWS;
     a.conditional = 1;
     if (e == cudaSuccess) e = run_pipeline<float>(g, a, s);
-    if (e != cudaSuccess) return from_cuda(e);
+    if (e != cudaSuccess || !finalize) return from_cuda(e);
     p->prof.begin("finalize", s);
     e = launch_finalize(p->st, p->st_total, 2, s);
     p->prof.end(s);
@@ -413,8 +417,8 @@ cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const
 // reused across calls); an exact pass (FP64 and two-term plans) always recomputes everything.
 cmif_status compute_map(cmif_plan p, const Geom& g, const int32_t* A, const uint8_t* MA, const int32_t* B,
                         const uint8_t* MB, double* mi, int32_t* n, int32_t* counts, cudaStream_t s,
-                        unsigned stages32, bool first) {
-    if (p->prec == CMIF_AUTO) return compute_map_auto(p, g, A, MA, B, MB, mi, n, counts, s, stages32, first);
+                        unsigned stages32, bool first, bool finalize) {
+    if (p->prec == CMIF_AUTO) return compute_map_auto(p, g, A, MA, B, MB, mi, n, counts, s, stages32, first, finalize);
     cudaError_t e = reset_status(p, first, s);
     if (e != cudaSuccess) return from_cuda(e);
     if (p->prec == CMIF_FP32) {
@@ -434,10 +438,9 @@ cmif_status compute_map(cmif_plan p, const Geom& g, const int32_t* A, const uint
         a.conditional = 0;
         e = run_pipeline<m31>(g, a, s);
     }
-    if (e != cudaSuccess) return from_cuda(e);
-    const int slot_default = (p->prec == CMIF_FP64 || p->prec == CMIF_SPLIT32) ? 1 : 0;
+    if (e != cudaSuccess || !finalize) return from_cuda(e);
     p->prof.begin("finalize", s);
-    e = launch_finalize(p->st, p->st_total, slot_default, s);
+    e = launch_finalize(p->st, p->st_total, status_slot(p), s);
     p->prof.end(s);
     return from_cuda(e);
 }
@@ -747,12 +750,9 @@ cmif_status align_core_units(cmif_plan plan, const Geom& g, const int32_t* A, co
         a.rows_grid = std::min(G * (g.r1 - g.r0), plan->w32.rows_grid);
         e = run_pipeline<float>(gu, a, s);
         if (e != cudaSuccess) return from_cuda(e);
-        plan->prof.begin("finalize", s);
-        e = launch_finalize(plan->st, plan->st_total, 0, s);
-        plan->prof.end(s);
-        if (e != cudaSuccess) return from_cuda(e);
         plan->prof.begin("peak", s);
-        e = launch_peak_units(mi, nm, gu, plan->st, gamma, plan->parts, plan->nparts, c0, peaks + c0, plan->maxn_u, s);
+        e = launch_peak_units(mi, nm, gu, plan->st, gamma, plan->parts, plan->nparts, c0, peaks + c0, plan->maxn_u,
+                              plan->st_total, 0, s);
         plan->prof.end(s);
         if (e != cudaSuccess) return from_cuda(e);
     }
@@ -786,10 +786,11 @@ cmif_status align_core(cmif_plan plan, const int32_t* A, const uint8_t* M_A, con
             if (e != cudaSuccess) return from_cuda(e);
         }
         const unsigned stages = (i == 0) ? STAGE_ALL : (STAGE_FWD_B | STAGE_PAIRS);
-        cmif_status cs = compute_map(plan, g, A, M_A, plan->wB, plan->wM, mi, nm, nullptr, s, stages, i == 0);
+        cmif_status cs = compute_map(plan, g, A, M_A, plan->wB, plan->wM, mi, nm, nullptr, s, stages, i == 0, false);
         if (cs != CMIF_OK) return cs;
         plan->prof.begin("peak", s);
-        e = launch_peak(mi, nm, g, plan->st, gamma, plan->parts, plan->nparts, i, peaks + i, s);
+        e = launch_peak(mi, nm, g, plan->st, gamma, plan->parts, plan->nparts, i, peaks + i, plan->st_total,
+                        status_slot(plan), s);
         plan->prof.end(s);
         if (e != cudaSuccess) return from_cuda(e);
     }
@@ -1071,11 +1072,12 @@ cmif_status cmif_compute(cmif_plan plan, const int32_t* A, const uint8_t* M_A, c
                 e = cudaMemsetAsync(counts, 0, RC * sizeof(int32_t) * ((size_t)g.KA * g.KB + g.KA + g.KB), cs);
             if (e != cudaSuccess) return from_cuda(e);
         }
-        cmif_status st = compute_map(plan, g, A, M_A, B, M_B, mi_map, nm, counts, cs, STAGE_ALL, true);
+        cmif_status st = compute_map(plan, g, A, M_A, B, M_B, mi_map, nm, counts, cs, STAGE_ALL, true, peak_dev == nullptr);
         if (st != CMIF_OK) return st;
         if (peak_dev) {
             plan->prof.begin("peak", cs);
-            e = launch_peak(mi_map, nm, g, plan->st, gamma, plan->parts, plan->nparts, 0, peak_dev, cs);
+            e = launch_peak(mi_map, nm, g, plan->st, gamma, plan->parts, plan->nparts, 0, peak_dev, plan->st_total,
+                            status_slot(plan), cs);
             plan->prof.end(cs);
             if (e != cudaSuccess) return from_cuda(e);
         }
@@ -1393,9 +1395,10 @@ cmif_status cmif_compute_batch(cmif_batch batch, cmif_peak* results_dev, int32_t
                 if (e != cudaSuccess) return from_cuda(e);
                 Geom g;
                 if (!call_geom(p, d.gamma, &g)) return CMIF_ERR_INVALID_ARG;
-                st = compute_map(p, g, d.A, d.M_A, d.B, d.M_B, p->mibuf, p->nbuf, nullptr, cs, STAGE_ALL, false);
+                st = compute_map(p, g, d.A, d.M_A, d.B, d.M_B, p->mibuf, p->nbuf, nullptr, cs, STAGE_ALL, false, false);
                 if (st != CMIF_OK) return st;
-                e = launch_peak(p->mibuf, p->nbuf, g, p->st, d.gamma, p->parts, p->nparts, 0, results_dev + i, cs);
+                e = launch_peak(p->mibuf, p->nbuf, g, p->st, d.gamma, p->parts, p->nparts, 0, results_dev + i, p->st_total,
+                                status_slot(p), cs);
                 if (e != cudaSuccess) return from_cuda(e);
             } else {
                 st = align_core(p, d.A, d.M_A, d.B, d.M_B, batch->angles[i].data(), d.n_angles, d.gamma, 1,

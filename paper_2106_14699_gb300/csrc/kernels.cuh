@@ -21,6 +21,7 @@
 #include <type_traits>
 #include <cstdint>
 #include "common.h"
+#include <cooperative_groups.h>
 #include "fft.cuh"
 
 namespace cmif {
@@ -128,6 +129,7 @@ struct EntAcc<false> {
     __device__ __forceinline__ void zero() { s = 0; }
     __device__ __forceinline__ void joint(long long t) { s += t; }
     __device__ __forceinline__ void marg(long long t) { s -= t; }
+    __device__ __forceinline__ void add(const EntAcc& o) { s += o.s; }
     __device__ __forceinline__ double finish(int N) const { return mi_finish(s, N); }
 };
 template <>
@@ -136,6 +138,7 @@ struct EntAcc<true> {
     __device__ __forceinline__ void zero() { j = 0; m = 0; }
     __device__ __forceinline__ void joint(long long t) { j += t; }
     __device__ __forceinline__ void marg(long long t) { m += t; }
+    __device__ __forceinline__ void add(const EntAcc& o) { j += o.j; m += o.m; }
     __device__ __forceinline__ double finish(int N) const { return nmi_finish(j, m, N); }
 };
 
@@ -956,6 +959,10 @@ constexpr size_t pair_cols_smem() {
 // the current label a, and the B-marginal C_B^b(p) (shared or global memory).
 // The rounded counts reach the owners through the teams' scratch, in HALVES
 // passes (two for 4-byte values, whose scratch holds half a row).
+// split > 1 (maps with too few rows to fill the GPU, B-marginals in shared memory): a cluster
+// of split blocks takes a row, each the pairs of its own labels a; at the end of the row the
+// blocks read each other's partial sums and B-marginals (distributed shared memory) and each
+// finishes its share of the positions.
 template <typename T, int Q>
 struct RowCfg {
     static constexpr int L = Q / 2;
@@ -1006,7 +1013,7 @@ __global__ void __launch_bounds__(RowCfg<T, Q>::THREADS, RowCfg<T, Q>::MIN_BLOCK
 k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ cb_global,
             double* __restrict__ mi_map, int32_t* __restrict__ n_map, int32_t* __restrict__ counts,
             DevStatus* __restrict__ st, int prec_slot, int conditional, const int32_t* __restrict__ ov,
-            const int* __restrict__ ov_slot, unsigned* __restrict__ pair_res) {
+            const int* __restrict__ ov_slot, unsigned* __restrict__ pair_res, int split) {
     // ov / ov_slot (nullable): a pair with ov_slot[pair] = s >= 0 takes its counts
     // from ov[s][row][position] (exact counts from the second precision) instead of
     // its own transform, and its residual is not counted.  pair_res (nullable):
@@ -1027,6 +1034,8 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
 
     // tasks: the window's rows of every unit (units > 1: several maps, R2 rows apart)
     const int nr = g.r1 - g.r0, ntask = g.units * nr;
+    const int rank = CB_SMEM ? (int)blockIdx.x % split : 0, ntb = (int)gridDim.x / split, task0 = (int)blockIdx.x / split;
+    const int alo = rank * KA / split, plo = alo * KB, phi = (rank + 1) * KA / split * KB;  // this block's pairs
     auto task_row = [&](int tk) { return (tk / nr) * g.R2 + g.r0 + tk % nr; };
     // STAGE: the team's buffer for the Y row of its current pair; the team's lanes
     // copy a row in 16-byte pieces (the rows start on 32-byte boundaries: L is a
@@ -1043,11 +1052,11 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
         }
     };
     if constexpr (C::STAGE) {
-        if ((int)blockIdx.x < ntask && team < npairs) stage_issue(team, task_row(blockIdx.x));
+        if (task0 < ntask && plo + team < phi) stage_issue(plo + team, task_row(task0));
         cp_async_wait_all();
         __syncthreads();
     }
-    for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
+    for (int task = task0; task < ntask; task += ntb) {
         const int row = task_row(task);
         EntAcc<NMI> S[U];
         float CA[U];
@@ -1062,21 +1071,21 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
             }
         int cur_a[HALVES];
 #pragma unroll
-        for (int hf = 0; hf < HALVES; ++hf) cur_a[hf] = 0;
-        for (int base = 0; base < npairs; base += NT) {
+        for (int hf = 0; hf < HALVES; ++hf) cur_a[hf] = alo;
+        for (int base = plo; base < phi; base += NT) {
             const int pair = base + team;
-            const bool act = pair < npairs;
+            const bool act = pair < phi;
             const int ovs = (act && ov_slot) ? ov_slot[pair] : -1;
             const cpx<T>* yr = C::STAGE ? stage : Y + ((size_t)(act ? pair : 0) * Rout + row) * L;
             if (!C::STAGE && lt == 0) {
                 // ask L2 for this team's row of the next round (or of the block's next row)
                 int np = pair + NT, nrow = row;
-                if (np >= npairs) {
-                    np = team;
-                    const int nt2 = task + (int)gridDim.x;
+                if (np >= phi) {
+                    np = plo + team;
+                    const int nt2 = task + ntb;
                     nrow = nt2 < ntask ? (nt2 / nr) * g.R2 + g.r0 + nt2 % nr : -1;
                 }
-                if (np < npairs && nrow >= 0)
+                if (np < phi && nrow >= 0)
                     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Y + ((size_t)np * Rout + nrow) * L),
                                  "r"((unsigned)(L * sizeof(cpx<T>))) : "memory");
             }
@@ -1097,7 +1106,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                 for (int off = WID / 2; off > 0; off >>= 1) rr = fmaxf(rr, __shfl_xor_sync(0xffffffffu, rr, off));
                 if (act && ovs < 0 && (lt % WID) == 0) atomic_max_float_pos(&pair_res[pair], rr);
             }
-            const int nt = min(NT, npairs - base);
+            const int nt = min(NT, phi - base);
             const int a0 = base / KB, b0 = base - a0 * KB;
 #pragma unroll
             for (int hf = 0; hf < HALVES; ++hf) {
@@ -1106,8 +1115,8 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                     // the staged rows are consumed: copy this team's next row (the next
                     // round of this task, else round 0 of the block's next task)
                     int np = pair + NT, ntk = task;
-                    if (np >= npairs) { np = team; ntk = task + (int)gridDim.x; }
-                    if (np < npairs && ntk < ntask) stage_issue(np, task_row(ntk));
+                    if (np >= phi) { np = plo + team; ntk = task + ntb; }
+                    if (np < phi && ntk < ntask) stage_issue(np, task_row(ntk));
                 }
                 float2* ob = reinterpret_cast<float2*>(region);
 #pragma unroll
@@ -1212,6 +1221,49 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
             }
             if constexpr (C::STAGE) cp_async_wait_all();  // the next round's rows, visible after the barrier
             __syncthreads();  // the next round's transforms overwrite the scratch read above
+        }
+        if constexpr (CB_SMEM) {
+            if (split > 1) {
+                namespace cg = cooperative_groups;
+                const cg::cluster_group cluster = cg::this_cluster();
+                EntAcc<NMI>* part_s = reinterpret_cast<EntAcc<NMI>*>(smem_raw + (C::OFF_CB + (size_t)KB * Q * sizeof(float) + 15) / 16 * 16);
+                int* part_n = reinterpret_cast<int*>(part_s + Q);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int pl = tid + BT * (u % UH), p = (u / UH) * QH + pl;
+                    if (pl >= QH) continue;
+                    S[u].marg(clog2c_biased(CA[u]));
+                    N[u] += (int)CA[u];
+                    const int cidx = circ_to_out(p, Q, g.WA, g.WB - 1);
+                    if (counts && cidx >= 0) counts[((size_t)npairs + cur_a[u / UH]) * RC + (size_t)row * Cout + cidx] = (int)CA[u];
+                    part_s[p] = S[u];
+                    part_n[p] = N[u];
+                }
+                cluster.sync();
+                for (int p = rank * Q / split + tid; p < (rank + 1) * Q / split; p += BT) {
+                    EntAcc<NMI> s;
+                    s.zero();
+                    int n = 0;
+                    for (int r2 = 0; r2 < split; ++r2) {
+                        s.add(cluster.map_shared_rank(part_s, r2)[p]);
+                        n += cluster.map_shared_rank(part_n, r2)[p];
+                    }
+                    const int cidx = circ_to_out(p, Q, g.WA, g.WB - 1);
+                    for (int b = 0; b < KB; ++b) {
+                        float c = 0.f;
+                        for (int r2 = 0; r2 < split; ++r2) c += cluster.map_shared_rank(cb, r2)[(size_t)b * Q + p];
+                        s.marg(clog2c_biased(c));
+                        if (counts && cidx >= 0) counts[((size_t)npairs + KA + b) * RC + (size_t)row * Cout + cidx] = (int)c;
+                    }
+                    if (cidx < 0) continue;
+                    const size_t o = (size_t)row * Cout + cidx;
+                    mi_map[o] = s.finish(n);
+                    if (n_map) n_map[o] = n;
+                    if (cidx >= g.c0 && cidx < g.c1) row_max_n = max(row_max_n, n);
+                }
+                cluster.sync();  // the others' reads of this block's sums are done
+                continue;
+            }
         }
         // the B-marginals: all of this thread's positions of one label loaded together
         for (int b = 0; b < KB; ++b) {

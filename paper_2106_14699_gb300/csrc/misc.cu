@@ -11,6 +11,27 @@
 
 namespace cmif {
 
+// Fold one map's device status into the call's running total (one thread).
+__device__ __forceinline__ void merge_status(const DevStatus* m, DevStatus* tot, int slot) {
+    if (slot == 2) {  // per-pair precision: FP32 pairs and second-precision pairs kept apart
+        tot->res_bits[0] = max(tot->res_bits[0], m->res_bits[0]);
+        tot->res_bits[1] = max(tot->res_bits[1], m->res_bits[1]);
+    } else {
+        tot->res_bits[0] = max(tot->res_bits[0], m->res_bits[slot]);  // the authoritative pass
+    }
+    tot->flags |= m->flags;
+    tot->escalations += m->escalations;
+    tot->predicted += m->predicted;
+    tot->max_n = max(tot->max_n, m->max_n);
+}
+// Final decision on the authoritative precision's residual (slot 2: per-pair precision, where both
+// the FP32 pairs' and the second-precision pairs' count), then the fold into the total (nullable).
+__device__ __forceinline__ void finalize_status(DevStatus* st, DevStatus* tot, int slot) {
+    const unsigned r = slot == 2 ? max(st->res_bits[0], st->res_bits[1]) : st->res_bits[slot];
+    if (__uint_as_float(r) >= kResidualGuard) st->flags |= STATUS_PRECISION;
+    if (tot) merge_status(st, tot, slot);
+}
+
 // ---------------------------------------------------------------------------
 // gamma-gated argmax (Alg. 1): N_cal = gamma * max_chi N; chi* maximises MI
 // among shifts with N >= N_cal; ties go to the lowest map index.
@@ -54,7 +75,8 @@ template <typename NT>
 __global__ void k_peak(const double* __restrict__ mi, const NT* __restrict__ n, int Cout, int r0, int r1, int c0, int c1,
                        const DevStatus* __restrict__ st, double gamma, PeakPart* parts, long long unit_rc,
                        const int* __restrict__ maxn_u, unsigned* __restrict__ done, int HA, int WA, int angle_idx, int R2,
-                       int DA, void* __restrict__ peak_out) {
+                       int DA, void* __restrict__ peak_out, DevStatus* fin, DevStatus* tot, int slot) {
+    // fin (nullable): the map's status, finalized and folded into tot by the first unit's last block
     mi += blockIdx.y * unit_rc;
     n += blockIdx.y * unit_rc;
     parts += (size_t)blockIdx.y * gridDim.x;
@@ -94,6 +116,7 @@ __global__ void k_peak(const double* __restrict__ mi, const NT* __restrict__ n, 
     __syncthreads();
     block_best(bm, bi);
     if (threadIdx.x != 0) return;
+    if (fin && blockIdx.y == 0) finalize_status(fin, tot, slot);
     PeakRec* p = reinterpret_cast<PeakRec*>(peak_out) + blockIdx.y;
     if (bi < 0) { *p = {-1, 0, 0, 0, 0.0}; return; }
     const long long row = bi / Cout;
@@ -176,19 +199,6 @@ cudaError_t launch_warp_nn(const int32_t* B, const uint8_t* MB, int H, int W, do
     return cudaGetLastError();
 }
 
-// Fold one map's device status into the call's running total (one thread).
-__device__ __forceinline__ void merge_status(const DevStatus* m, DevStatus* tot, int slot) {
-    if (slot == 2) {  // per-pair precision: FP32 pairs and second-precision pairs kept apart
-        tot->res_bits[0] = max(tot->res_bits[0], m->res_bits[0]);
-        tot->res_bits[1] = max(tot->res_bits[1], m->res_bits[1]);
-    } else {
-        tot->res_bits[0] = max(tot->res_bits[0], m->res_bits[slot]);  // the authoritative pass
-    }
-    tot->flags |= m->flags;
-    tot->escalations += m->escalations;
-    tot->predicted += m->predicted;
-    tot->max_n = max(tot->max_n, m->max_n);
-}
 __global__ void k_merge_status(const DevStatus* __restrict__ m, DevStatus* __restrict__ tot, int slot) {
     if (threadIdx.x == 0 && blockIdx.x == 0) merge_status(m, tot, slot);
 }
@@ -244,15 +254,8 @@ cudaError_t launch_status_code(const DevStatus* st, int32_t* out, cudaStream_t s
     return cudaGetLastError();
 }
 
-// Final decision on the authoritative precision's residual (slot 2: per-pair
-// precision, where both the FP32 pairs' and the second-precision pairs' count).
-// The map's status is then folded into the call's total (nullable).
 __global__ void k_finalize(DevStatus* st, DevStatus* tot, int slot) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        const unsigned r = slot == 2 ? max(st->res_bits[0], st->res_bits[1]) : st->res_bits[slot];
-        if (__uint_as_float(r) >= kResidualGuard) st->flags |= STATUS_PRECISION;
-        if (tot) merge_status(st, tot, slot);
-    }
+    if (threadIdx.x == 0 && blockIdx.x == 0) finalize_status(st, tot, slot);
 }
 
 // Max N over each unit's window (units > 1: the gamma gate of Alg. 1 is per map).
@@ -270,7 +273,7 @@ __global__ void k_unit_max_n(const int32_t* __restrict__ n, int Cout, int r0, in
 template <typename NT>
 static cudaError_t launch_peak_t(const double* mi, const NT* n, const Geom& g, DevStatus* st, double gamma,
                                  PeakPart* parts, int nparts, int angle_idx, void* peak_out, int units, int* maxn_u,
-                                 cudaStream_t s) {
+                                 DevStatus* tot, int slot, cudaStream_t s) {
     const int HA = g.HA, WA = g.WA, Cout = g.C;
     const long long unit_rc = units > 1 ? (long long)g.R2 * Cout : 0;
     // no more blocks than the window's rows need (a block takes whole rows)
@@ -278,30 +281,31 @@ static cudaError_t launch_peak_t(const double* mi, const NT* n, const Geom& g, D
     k_peak<NT><<<dim3(blocks, units), 256, 0, s>>>(mi, n, Cout, g.r0, g.r1, g.c0, g.c1, st, gamma, parts, unit_rc,
                                                    units > 1 ? maxn_u : nullptr,
                                                    units > 1 ? reinterpret_cast<unsigned*>(maxn_u) + units : &st->peak_done,
-                                                   HA, WA, angle_idx, g.Dz > 1 ? g.R2 : 0, g.DA, peak_out);
+                                                   HA, WA, angle_idx, g.Dz > 1 ? g.R2 : 0, g.DA, peak_out, slot >= 0 ? st : nullptr, tot, slot);
     return cudaGetLastError();
 }
 
 cudaError_t launch_peak(const double* mi, const int32_t* n, const Geom& g, DevStatus* st, double gamma,
-                        PeakPart* parts, int nparts, int angle_idx, void* peak_out, cudaStream_t s) {
-    return launch_peak_t(mi, n, g, st, gamma, parts, nparts, angle_idx, peak_out, 1, nullptr, s);
+                        PeakPart* parts, int nparts, int angle_idx, void* peak_out, DevStatus* tot, int slot,
+                        cudaStream_t s) {
+    return launch_peak_t(mi, n, g, st, gamma, parts, nparts, angle_idx, peak_out, 1, nullptr, tot, slot, s);
 }
 
 cudaError_t launch_peak_units(const double* mi, const int32_t* n, const Geom& g, DevStatus* st, double gamma,
-                              PeakPart* parts, int nparts, int angle0, void* peaks_out, int* maxn_u,
-                              cudaStream_t s) {
+                              PeakPart* parts, int nparts, int angle0, void* peaks_out, int* maxn_u, DevStatus* tot,
+                              int slot, cudaStream_t s) {
     // per-unit max N first (zeroed here, with the units' block counts), then the gated argmax of every unit
     cudaError_t e = cudaMemsetAsync(maxn_u, 0, 2 * (size_t)g.units * sizeof(int), s);
     if (e != cudaSuccess) return e;
     const long long unit_rc = (long long)g.R2 * g.C;
     k_unit_max_n<<<dim3(std::max(1, nparts / 2), g.units), 256, 0, s>>>(n, g.C, g.r0, g.r1, g.c0, g.c1, unit_rc,
                                                                          maxn_u);
-    return launch_peak_t(mi, n, g, st, gamma, parts, nparts, angle0, peaks_out, g.units, maxn_u, s);
+    return launch_peak_t(mi, n, g, st, gamma, parts, nparts, angle0, peaks_out, g.units, maxn_u, tot, slot, s);
 }
 
 cudaError_t launch_peak_w(const double* mi, const double* nw, const Geom& g, DevStatus* st, double gamma,
                           PeakPart* parts, int nparts, void* peak_out, cudaStream_t s) {
-    return launch_peak_t(mi, nw, g, st, gamma, parts, nparts, 0, peak_out, 1, nullptr, s);
+    return launch_peak_t(mi, nw, g, st, gamma, parts, nparts, 0, peak_out, 1, nullptr, nullptr, -1, s);
 }
 
 cudaError_t launch_finalize(DevStatus* st, DevStatus* total, int slot, cudaStream_t s) {

@@ -16,14 +16,16 @@ struct PeakRec {
 };
 
 // Alg. 1's gamma-gated argmax over the call's search window (g.r0..g.r1, g.c0..g.c1).
+// slot >= 0: the search's last block also does launch_finalize's work (st, tot, slot).
 cudaError_t launch_peak(const double* mi, const int32_t* n, const Geom& g, DevStatus* st, double gamma,
-                        PeakPart* parts, int nparts, int angle_idx, void* peak_out, cudaStream_t s);
+                        PeakPart* parts, int nparts, int angle_idx, void* peak_out, DevStatus* tot, int slot,
+                        cudaStream_t s);
 // Alg. 1's gated argmax of each of g.units maps (unit u: rows u * R2 .., window per unit,
 // its own max N in maxn_u[u], records peaks_out[u] with angle index angle0 + u); the
 // partials need nparts * g.units records.
 cudaError_t launch_peak_units(const double* mi, const int32_t* n, const Geom& g, DevStatus* st, double gamma,
-                              PeakPart* parts, int nparts, int angle0, void* peaks_out, int* maxn_u,
-                              cudaStream_t s);
+                              PeakPart* parts, int nparts, int angle0, void* peaks_out, int* maxn_u, DevStatus* tot,
+                              int slot, cudaStream_t s);
 // The same on a weighted map (real N, max N from the status word's max_nw_bits).
 cudaError_t launch_peak_w(const double* mi, const double* nw, const Geom& g, DevStatus* st, double gamma,
                           PeakPart* parts, int nparts, void* peak_out, cudaStream_t s);

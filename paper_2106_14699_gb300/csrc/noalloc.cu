@@ -168,6 +168,7 @@ extern "C" cmif_status cmif_compute_noalloc(int H_A, int W_A, int H_B, int W_B, 
     a.mi = mi_map; a.n = nm; a.counts = nullptr; a.st = st;
     a.prec_slot = 0; a.conditional = 0;
     a.rows_grid = std::min(g.R, bps * d->num_sms);
+    a.rows_cap = bps * d->num_sms;
     a.num_sms = d->num_sms;
     a.cb_smem = true;
     a.prof = nullptr;
@@ -176,10 +177,11 @@ extern "C" cmif_status cmif_compute_noalloc(int H_A, int W_A, int H_B, int W_B, 
     a.withhold_row = -1;
     e = run_pipeline<float>(g, a, s);
     if (e != cudaSuccess) return to_status(e);
-    e = launch_finalize(st, nullptr, 0, s);
-    if (e != cudaSuccess) return to_status(e);
-    if (peak_dev) {
-        e = launch_peak(mi_map, nm, g, st, gamma, reinterpret_cast<PeakPart*>(b + oParts), nparts, 0, peak_dev, s);
+    if (!peak_dev) {
+        e = launch_finalize(st, nullptr, 0, s);
+        if (e != cudaSuccess) return to_status(e);
+    } else {
+        e = launch_peak(mi_map, nm, g, st, gamma, reinterpret_cast<PeakPart*>(b + oParts), nparts, 0, peak_dev, nullptr, 0, s);
         if (e != cudaSuccess) return to_status(e);
     }
     if (status_dev) {

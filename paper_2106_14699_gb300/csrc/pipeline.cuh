@@ -30,6 +30,7 @@ struct PipeArgs {
     int prec_slot;    // 0: FP32 residual slot, 1: exact transforms
     int conditional;  // run only when STATUS_ESCALATE is set (AUTO re-run)
     int rows_grid;    // persistent grid of the row/epilogue kernel
+    int rows_cap;     // its blocks resident on the device (generic kernel; 0: rows are not split)
     int num_sms;      // SMs of the device (persistent grid of the pair-column kernel)
     int nmi;          // the map holds NMI = (H_A + H_B) / H_AB instead of MI
     // spatially weighted MI (FP64 plans): weight images replace the masks

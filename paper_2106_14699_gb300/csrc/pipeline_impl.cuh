@@ -130,19 +130,43 @@ static cudaError_t launch_pair_rows_v(const Geom& g, const PipeArgs<T>& a, cudaS
             return ext ? launch_rows_tm<Q, NMI, 2, 16>(g, a, s) : launch_rows_tm<Q, NMI, 0, 16>(g, a, s);
         }
     }
-    const size_t smem = pair_rows_smem<T, Q>(g.KB, a.cb_smem);
+    size_t smem = pair_rows_smem<T, Q>(g.KB, a.cb_smem);
     if (a.cb_smem) {
         auto kern = k_pair_rows<T, Q, true, NMI>;
+        // A map of few rows: a cluster of blocks per row, as many as the labels and the
+        // resident blocks allow (64^2, K = 8, 127 rows: 1 block per row 16.5 us)
+        const int ntask = g.units * (g.r1 - g.r0);
+        int split = 1;
+        while (split < 8 && 2 * split <= g.KA && (long long)ntask * 2 * split <= a.rows_cap) split *= 2;
+        if (split == 1) {
+            cudaError_t e = ensure_smem(kern, smem);
+            if (e != cudaSuccess) return e;
+            kern<<<a.rows_grid, C::THREADS, smem, s>>>(a.Y, g, a.tw, a.cb_global, a.mi, a.n, a.counts, a.st,
+                                                       a.prec_slot, a.conditional, a.ov, a.ov_slot, a.pair_res, 1);
+            return cudaGetLastError();
+        }
+        smem = (smem + 15) / 16 * 16 + Q * (sizeof(EntAcc<NMI>) + sizeof(int));
         cudaError_t e = ensure_smem(kern, smem);
         if (e != cudaSuccess) return e;
-        kern<<<a.rows_grid, C::THREADS, smem, s>>>(a.Y, g, a.tw, a.cb_global, a.mi, a.n, a.counts, a.st,
-                                                   a.prec_slot, a.conditional, a.ov, a.ov_slot, a.pair_res);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = split;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(ntask * split);
+        cfg.blockDim = dim3(C::THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kern, (const cpx<T>*)a.Y, g, a.tw, a.cb_global, a.mi, a.n, a.counts, a.st,
+                                  a.prec_slot, a.conditional, (const int32_t*)a.ov, a.ov_slot, a.pair_res, split);
     } else if constexpr (Q > 512) {  // Q <= 512: K_B (<= 64) x Q floats always fit in shared memory
         auto kern = k_pair_rows<T, Q, false, NMI>;
         cudaError_t e = ensure_smem(kern, smem);
         if (e != cudaSuccess) return e;
         kern<<<a.rows_grid, C::THREADS, smem, s>>>(a.Y, g, a.tw, a.cb_global, a.mi, a.n, a.counts, a.st,
-                                                   a.prec_slot, a.conditional, a.ov, a.ov_slot, a.pair_res);
+                                                   a.prec_slot, a.conditional, a.ov, a.ov_slot, a.pair_res, 1);
     } else {
         return cudaErrorInvalidValue;
     }
