@@ -140,7 +140,7 @@ cmif_status cmif_plan_create(cmif_plan* out, int H, int W, int K_A, int K_B, cmi
  *   H_A, W_A, H_B, W_B >= 1, H*W <= 2^22 per image; 1 <= K_A, K_B <= 64;
  *   the transform sizes P >= H_A+H_B-1 and Q >= W_A+W_B-1 must not exceed
  *   4096 (else CMIF_ERR_UNSUPPORTED).  They are the smallest powers of two
- *   (at least 16) or, for CMIF_FP32 plans, the smallest 3 * 2^k (96 .. 3072)
+ *   (at least 16) or, for CMIF_FP32 plans, the smallest 3 * 2^k (192 .. 3072)
  *   when that is smaller (CMIF_POW2_ONLY=1 in the environment at creation
  *   keeps powers of two).  Q keeps the power of two 512, 1024 or 2048 when the
  *   Tensor-Memory row kernel runs it (plans without count maps; faster than a

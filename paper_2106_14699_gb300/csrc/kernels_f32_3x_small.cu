@@ -1,11 +1,6 @@
-// FP32 forward, column and pair-product kernels for the transform sizes 96, 192, 384, 768 (3 * 2^k).
+// FP32 forward, column and pair-product kernels for the transform sizes 192, 384, 768 (3 * 2^k).
 #include "pipeline_impl.cuh"
 namespace cmif {
-template cudaError_t Sized<float, 96>::fwd_rows(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
-template cudaError_t Sized<float, 96>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
-template cudaError_t Sized<float, 96>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
-template int Sized<float, 96>::tm_cols(int);
-template cudaError_t Sized<float, 96>::tm_max_blocks(int, int, int*);
 template cudaError_t Sized<float, 192>::fwd_rows(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 192>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 192>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);

@@ -77,7 +77,7 @@ enum : unsigned {
 };
 
 // The transform sizes the kernels are compiled for: P, Q = 2^k (16 .. 4096) in
-// every precision, and 3 * 2^k (96 .. 3072) for FP32 transforms.
+// every precision, and 3 * 2^k (192 .. 3072) for FP32 transforms.
 template <typename T>
 constexpr bool kMixedSizes = std::is_same<T, float>::value;
 #define CMIF_MIXED_CASE(TT, V, ...)                                   \
@@ -98,7 +98,6 @@ constexpr bool kMixedSizes = std::is_same<T, float>::value;
         case 1024: { constexpr int SZ = 1024; __VA_ARGS__; } break; \
         case 2048: { constexpr int SZ = 2048; __VA_ARGS__; } break; \
         case 4096: { constexpr int SZ = 4096; __VA_ARGS__; } break; \
-        CMIF_MIXED_CASE(TT, 96, __VA_ARGS__)                          \
         CMIF_MIXED_CASE(TT, 192, __VA_ARGS__)                         \
         CMIF_MIXED_CASE(TT, 384, __VA_ARGS__)                         \
         CMIF_MIXED_CASE(TT, 768, __VA_ARGS__)                         \
