@@ -146,7 +146,10 @@ cmif_status choose_rows(cmif_plan p, Workspace<T>& w) {
     w.args.tm_cols = 0;
     const char* no_tm = std::getenv("CMIF_DISABLE_TMEM");
     if (std::is_same<T, float>::value && !(no_tm && no_tm[0] == '1')) {
-        const int cols = rows_tm_cols(g.Q, g.KB);
+        // widths whose rows are split only for the TMEM kernel: a plan that may be asked for the
+        // count maps, which the generic kernel makes, keeps to the generic one
+        const int cols = always_split(g.Q) || !(p->flags & CMIF_FLAG_DEBUG_COUNTS)
+                             ? rows_tm_cols(g.Q, g.KA, g.KB) : 0;
         if (cols > 0) {
             e = rows_tm_max_blocks_per_sm(g.Q, cols, g.KA * g.KB, &bps);
             if (e != cudaSuccess) return from_cuda(e);
@@ -173,7 +176,7 @@ cmif_status choose_rows(cmif_plan p, Workspace<T>& w) {
         w.tm_cols_avail = w.args.tm_cols;
         w.grid_tm = w.rows_grid;
         int bg = 0;
-        if (rows_smem_bytes<T>(g.Q, g.KB, true) <= 200 * 1024 &&
+        if (always_split(g.Q) && rows_smem_bytes<T>(g.Q, g.KB, true) <= 200 * 1024 &&
             rows_max_blocks_per_sm<T>(g.Q, g.KB, true, &bg) == cudaSuccess && bg >= 1)
             w.grid_gen = std::min(g.R, bg * p->num_sms);
         cudaGetLastError();
@@ -478,16 +481,20 @@ cmif_status plan_init(cmif_plan p, int H_A, int W_A, int H_B, int W_B, int K_A, 
     g.P = transform_size(g.R2, mixed);
     g.Q = transform_size(g.C, mixed);
     {
-        // The row transform prefers the widths of the Tensor-Memory row kernel (512,
-        // 1024, 2048) to a shorter 3 * 2^k: that kernel turns out counts about twice as
-        // fast as the generic one, which outweighs the 4/3 more points of the longer
-        // rows (and of the pair-column transforms over their columns).  Plans that ask
-        // for the count maps run the generic kernel and keep the shorter width.
+        // The row transform prefers 512, 1024 and 2048 to the shorter 384, 768 and 1536: the
+        // Tensor-Memory row kernel of those widths turns out counts about twice as fast as the
+        // generic one, which outweighs the 4/3 more points of the longer rows (and of the
+        // pair-column transforms over their columns).  1536 has that kernel, too, and is kept
+        // while two of its blocks fit in Tensor Memory (rows + columns, ms, 1536 against 2048:
+        // 350 x 751, 16 x 8 labels 2.17 / 2.32, 352 x 620, 16 x 24 6.01 / 6.11; one block only:
+        // 303 x 761, 24 x 24 9.15 / 8.29).  Plans that ask for the count maps run the generic
+        // kernel and keep the shorter width.
         const char* tq = std::getenv("CMIF_ROWS_POW2");  // "0": keep the shortest width
         const char* no_tm = std::getenv("CMIF_DISABLE_TMEM");
-        const int q2 = transform_size(g.C, false);
+        const int q2 = transform_size(g.C, false), cols3 = g.Q == 1536 ? rows_tm_cols(1536, K_A, K_B) : 0;
         if (mixed && q2 != g.Q && (q2 == 512 || q2 == 1024 || q2 == 2048) && !(tq && tq[0] == '0') &&
-            !(no_tm && no_tm[0] == '1') && !(flags & CMIF_FLAG_DEBUG_COUNTS) && rows_tm_cols(q2, K_B) > 0)
+            !(no_tm && no_tm[0] == '1') && !(flags & CMIF_FLAG_DEBUG_COUNTS) && rows_tm_cols(q2, K_A, K_B) > 0 &&
+            !(cols3 > 0 && cols3 <= 256))
             g.Q = q2;
     }
     if (g.P > 4096 || g.Q > 4096) return CMIF_ERR_UNSUPPORTED;
@@ -539,6 +546,8 @@ cmif_status plan_init(cmif_plan p, int H_A, int W_A, int H_B, int W_B, int K_A, 
         p->has64 = true;
     }
     if (st != CMIF_OK) return st;
+    // the layout of Y's rows follows the FP32 row kernel (some widths: always split)
+    p->g.split = p->gcap.split = always_split(g.Q) || (tm_rows(g.Q) && p->w32.args.tm_cols > 0) ? 1 : 0;
     if (prec == CMIF_AUTO) {
         // per-pair precision: the second precision holds the products of one chunk
         // of listed pairs at a time (a few GB at most), and the exact counts of at

@@ -31,6 +31,7 @@ struct Geom {
     int Qh;              // Q/2 + 1 half-spectrum columns
     int Qs;              // padded row stride (complex elements) of row-major spectra
     int Ys;              // complex values per row of Y: Q / 2
+    int split;           // FP32: Y's rows are split (real and imaginary parts grouped; kernels.cuh)
     // Search window of the call: output rows [r0, r1) are computed, and X_S is
     // rows [r0, r1) x columns [c0, c1) (max N and the peak are taken over it).
     // The whole map unless Alg. 1's padded window is on.

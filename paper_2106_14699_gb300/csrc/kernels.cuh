@@ -433,10 +433,10 @@ __device__ __forceinline__ void stage_table(cpx<T>* dst, const cpx<T>* __restric
 //   FP32, L / 4 chunks of 4: k0, k1 and the mirrors of k1, k0 (L - k; of 0: L / 2), as
 //     two 16-byte halves (direct, mirrored), swapped in every other group of 4 chunks
 //     so that the row kernels' reads of consecutive k meet no bank conflicts;
-//       Q = 512, 1024, 2048 (Tensor-Memory row kernel): k1 = k0 + 32 with real and
-//       imaginary parts grouped, (re, re', im, im'), in the order of the packed
-//       row transform's even and odd inputs;
-//       other Q: k0 = 2c, k1 = 2c + 1 as complex values.
+//       split rows (Tensor-Memory row kernel): k1 = k0 + 32 with real and imaginary parts
+//       grouped, (re, re', im, im'), in the order of the packed row transform's even and
+//       odd inputs;
+//       else: k0 = 2c, k1 = 2c + 1 as complex values.
 //     Four rows' chunks c form a 128-byte line, lines of one row group in the order of c
 //     (Y[pair][row / 4][c][row % 4]): the pair-column kernel's lanes, which hold consecutive
 //     rows, write whole lines (8 shared-pipe wavefronts per 32 lanes instead of 32), and the
@@ -445,7 +445,12 @@ __device__ __forceinline__ void stage_table(cpx<T>* dst, const cpx<T>* __restric
 //   FP64, L / 2 chunks of 2: z_c, z_{L-c}; rows contiguous.
 template <typename T>
 constexpr int kChunk = sizeof(T) == 4 ? 4 : 2;
-__host__ __device__ constexpr bool split32_rows(int Q) { return Q == 512 || Q == 1024 || Q == 2048; }
+// Row widths with a Tensor-Memory row kernel; of these, the ones whose rows are always split
+// (the others only where that kernel runs: Geom::split).
+__host__ __device__ constexpr bool tm_rows(int Q) {
+    return Q == 512 || Q == 1024 || Q == 1536 || Q == 2048 || Q == 3072 || Q == 4096;
+}
+__host__ __device__ constexpr bool always_split(int Q) { return Q == 512 || Q == 1024 || Q == 2048; }
 // Rows of one pair in Y, and the element offset of chunk c of a row.
 template <typename T>
 __host__ __device__ constexpr int y_rows(int Rout) { return sizeof(T) == 4 ? (Rout + 3) / 4 * 4 : Rout; }
@@ -478,23 +483,21 @@ __device__ __forceinline__ int chunk_col(int c, int i, int L, bool split) {
 // lines of four rows.
 template <typename T>
 constexpr int kLine = sizeof(T) == 4 ? 4 * kChunk<T> : kChunk<T>;
-template <typename T, int Q, int CS = kChunk<T>>
+template <typename T, int Q, bool SPLIT = false, int CS = kChunk<T>>
 __device__ __forceinline__ cpx<T> load_z(const cpx<T>* row, int k) {
     constexpr int L = Q / 2;
     const bool mir = k >= L / 2;
     const int kk = k == L / 2 ? 0 : (mir ? L - k : k);  // the direct partner
     if constexpr (sizeof(T) != 4) {
         return row[CS * kk + (mir ? 1 : 0)];
-    } else {
-        constexpr bool split = std::is_same<T, float>::value && split32_rows(Q);
-        const int c = split ? (kk >> 6) * 32 + (kk & 31) : kk >> 1, second = split ? (kk >> 5) & 1 : kk & 1;
+    } else if constexpr (SPLIT) {
+        const int c = (kk >> 6) * 32 + (kk & 31), second = (kk >> 5) & 1;
         const int half = (mir ? 1 : 0) ^ (halves_swapped(c) ? 1 : 0), e = mir ? 1 - second : second;
-        if constexpr (split) {
-            const float* f = reinterpret_cast<const float*>(row) + c * 2 * CS + half * 4 + e;
-            return {f[0], f[2]};
-        } else {
-            return row[c * CS + half * 2 + e];
-        }
+        const float* f = reinterpret_cast<const float*>(row) + c * 2 * CS + half * 4 + e;
+        return {f[0], f[2]};
+    } else {
+        const int c = kk >> 1, half = (mir ? 1 : 0) ^ (halves_swapped(c) ? 1 : 0), e = mir ? 1 - (kk & 1) : kk & 1;
+        return row[c * CS + half * 2 + e];
     }
 }
 // 32-byte global load (sm_100+), past L1: the spectra are shared through L2
@@ -610,7 +613,8 @@ __global__ void __launch_bounds__(PairColsCfg<T, P, MMAX>::THREADS, PairColsCfg<
 k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA, int KB, int Qh, int HA, int HB,
             int Rout, int r0, int r1, cpx<T>* __restrict__ Y, Tw<T> tw, const cpx<T>* __restrict__ twq,
             const DevStatus* __restrict__ st, int conditional, int* __restrict__ work_ctr, int DA, int DB, int R2,
-            const int* __restrict__ plist, const int* __restrict__ lrange, int chunk_off, int chunk_cap, int units) {
+            const int* __restrict__ plist, const int* __restrict__ lrange, int chunk_off, int chunk_cap, int units,
+            int split_rows) {
     // twq: the table of e^{-2 pi i k / Q}, Q = 2 (Qh - 1).
     // units > 1 (images only): several floating images (rotation angles) at once;
     // unit u's spectra are F_b plane b * units + u, its output rows u * R2 + (row).
@@ -621,7 +625,7 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
     if (conditional && !(st->flags & STATUS_ESCALATE)) return;
     constexpr int M = C::M, R = C::R, TPB = C::TPB, NQ = C::NQ, CH = kChunk<T>, UPR = C::UPR;
     const int L = Qh - 1;
-    const bool split = std::is_same<T, float>::value && split32_rows(2 * L);
+    const bool split = std::is_same<T, float>::value && split_rows;  // layout of Y's rows
     const int Dz = VOL ? DA + DB - 1 : 1;
     int npairs = KA * KB, lbase = 0;
     if (plist) {
@@ -938,8 +942,12 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
             }
             }
         };
-        if (split) emit(std::true_type{});
-        else emit(std::false_type{});
+        if constexpr (std::is_same<T, float>::value) {
+            if (split) emit(std::true_type{});
+            else emit(std::false_type{});
+        } else {
+            emit(std::false_type{});
+        }
         __syncthreads();  // the buffer's reads (and s_next's) done before it is written again
         }
         if (!more) break;
@@ -1089,10 +1097,14 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Y + ((size_t)np * Rout + nrow) * L),
                                  "r"((unsigned)(L * sizeof(cpx<T>))) : "memory");
             }
-            auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q>(yr, k) : cpx<T>{T(0), T(0)}; };
             cpx<T> v[M];
-            team_fft<M, R, +1>(v, r, j, load, region + r * grp_scratch_bytes<T, M>(), tw.sq[ilog2c(M)],
-                               tw_of<L>(tw));
+            auto transform = [&](auto splitc) {
+                constexpr bool SPLIT = decltype(splitc)::value;
+                auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q, SPLIT>(yr, k) : cpx<T>{T(0), T(0)}; };
+                team_fft<M, R, +1>(v, r, j, load, region + r * grp_scratch_bytes<T, M>(), tw.sq[ilog2c(M)], tw_of<L>(tw));
+            };
+            // (Geom::split of the other widths: the Tensor-Memory kernel only)
+            transform(std::integral_constant<bool, std::is_same<T, float>::value && always_split(Q)>{});
             // round to the nearest integer; track the worst residual (the exactness guard)
             float rp = 0.f;
             float2 cnt[M];
@@ -1350,7 +1362,7 @@ k_pair_rows_counts(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, const int* __
         const bool act = t < ntask;
         const int e = act ? (int)(t / nrows) : 0, row = g.r0 + (act ? (int)(t % nrows) : 0);
         const cpx<T>* yr = Y + (size_t)e * y_rows<T>(g.R) * L + y_chunk<T>(row, 0, L);
-        auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q, kLine<T>>(yr, k) : cpx<T>{T(0), T(0)}; };
+        auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q, false, kLine<T>>(yr, k) : cpx<T>{T(0), T(0)}; };
         cpx<T> v[M];
         team_fft<M, R, +1>(v, r, j, load, region + r * grp_scratch_bytes<T, M>(), tw.sq[ilog2c(M)],
                            tw_of<L>(tw));

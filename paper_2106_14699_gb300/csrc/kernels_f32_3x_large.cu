@@ -4,11 +4,11 @@ namespace cmif {
 template cudaError_t Sized<float, 1536>::fwd_rows(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 1536>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 1536>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
-template int Sized<float, 1536>::tm_cols(int);
+template int Sized<float, 1536>::tm_cols(int, int);
 template cudaError_t Sized<float, 1536>::tm_max_blocks(int, int, int*);
 template cudaError_t Sized<float, 3072>::fwd_rows(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 3072>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 3072>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
-template int Sized<float, 3072>::tm_cols(int);
+template int Sized<float, 3072>::tm_cols(int, int);
 template cudaError_t Sized<float, 3072>::tm_max_blocks(int, int, int*);
 }

@@ -4,8 +4,7 @@
 namespace cmif {
 template <int Q, bool NMI>
 cudaError_t launch_rows_tm_units(const Geom& g, const PipeArgs<float>& a, cudaStream_t s) {
-    return rows_tm_teams(Q, a.tm_cols, g.KA * g.KB) == 16 ? launch_rows_tm<Q, NMI, 1, 16>(g, a, s)
-                                                          : launch_rows_tm<Q, NMI, 1, 8>(g, a, s);
+    return launch_rows_tm_mode<Q, NMI, 1>(g, a, s);
 }
 template cudaError_t launch_rows_tm_units<512, false>(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template cudaError_t launch_rows_tm_units<512, true>(const Geom&, const PipeArgs<float>&, cudaStream_t);

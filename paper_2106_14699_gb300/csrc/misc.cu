@@ -680,7 +680,7 @@ cudaError_t get_twiddles(int device, Tw<float>* tf, Tw<double>* td, Tw<m31>* tm)
 }
 
 // Tensor map of Y for the row copies of the Tensor-Memory row kernel: 32 floats (a line of
-// four rows' chunks) x L/4 chunks x row groups x pairs; a copy takes 8 x L/4 x 1 x 1.
+// four rows' chunks) x L/4 chunks x row groups x pairs; a copy takes 8 x (at most 256) x 1 x 1.
 cudaError_t make_row_map(CUtensorMap* map, const cpx<float>* Y, int L, int Rout, int npairs) {
     using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -695,7 +695,7 @@ cudaError_t make_row_map(CUtensorMap* map, const cpx<float>* Y, int L, int Rout,
     const cuuint64_t groups = (cuuint64_t)y_rows<float>(Rout) / 4;
     const cuuint64_t dims[4] = {32, (cuuint64_t)(L / 4), groups, (cuuint64_t)npairs};
     const cuuint64_t strides[3] = {128, 32ull * L, 32ull * L * groups};  // bytes; a row group holds 4 L complex
-    const cuuint32_t box[4] = {8, (cuuint32_t)(L / 4), 1, 1}, elem[4] = {1, 1, 1, 1};
+    const cuuint32_t box[4] = {8, (cuuint32_t)(L / 4 <= 256 ? L / 4 : L / 8), 1, 1}, elem[4] = {1, 1, 1, 1};
     const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<cpx<float>*>(Y), dims, strides, box,
                               elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

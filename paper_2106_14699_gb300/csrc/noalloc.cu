@@ -111,6 +111,7 @@ extern "C" cmif_status cmif_compute_noalloc(int H_A, int W_A, int H_B, int W_B, 
     g.Qh = g.Q / 2 + 1;
     g.Qs = (g.Qh + 3) / 4 * 4;
     g.Ys = g.Q / 2;
+    g.split = always_split(g.Q) ? 1 : 0;
 
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess) return CMIF_ERR_CUDA;

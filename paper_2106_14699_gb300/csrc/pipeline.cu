@@ -118,10 +118,10 @@ cudaError_t rows_max_blocks_per_sm(int Q, int KB, bool cb_smem, int* out) {
     return cudaSuccess;
 }
 
-int rows_tm_cols(int Q, int KB) {
+int rows_tm_cols(int Q, int KA, int KB) {
     int out = 0;
     auto f = [&]() -> cudaError_t {
-        CMIF_SIZE_SWITCH_T(float, Q, out = Sized<float, SZ>::tm_cols(KB));
+        CMIF_SIZE_SWITCH_T(float, Q, out = Sized<float, SZ>::tm_cols(KA, KB));
         return cudaSuccess;
     };
     f();

@@ -135,7 +135,7 @@ struct Sized {
     static size_t rows_smem(int KB, bool cb_smem);
     static int rows_threads();
     static cudaError_t rows_max_blocks(int KB, bool cb_smem, int* out);
-    static int tm_cols(int KB);                 // 0 unless the TMEM row kernel applies (FP32, Q = 512 / 1024 / 2048)
+    static int tm_cols(int KA, int KB);         // 0 unless the TMEM row kernel applies (FP32, tm_rows(Q))
     static cudaError_t tm_max_blocks(int tm_cols, int npairs, int* out);
     static cudaError_t pair_rows_w(const Geom& g, const PipeArgs<T>& a, cudaStream_t s);  // FP64 only
     static cudaError_t rows_w_max_blocks(int* out);
@@ -143,7 +143,7 @@ struct Sized {
 
 template <typename T>
 cudaError_t run_pipeline(const Geom& g, const PipeArgs<T>& a, cudaStream_t s);
-// The Tensor-Memory row kernel over several units (FP32, Q = 512, 1024 or 2048).
+// The Tensor-Memory row kernel over several units (FP32, tm_rows(Q)).
 template <int Q, bool NMI>
 cudaError_t launch_rows_tm_units(const Geom& g, const PipeArgs<float>& a, cudaStream_t s);
 // List mode of the second precision: pair products and inverse column transforms of
@@ -161,8 +161,8 @@ template <typename T>
 int rows_threads(int Q);
 template <typename T>
 cudaError_t rows_max_blocks_per_sm(int Q, int KB, bool cb_smem, int* out);
-// TMEM columns the TMEM / TMA row kernel needs for (Q, K_B), or 0 when it does not apply.
-int rows_tm_cols(int Q, int KB);
+// TMEM columns the TMEM / TMA row kernel needs for (Q, min(K_A, K_B)), or 0 when it does not apply.
+int rows_tm_cols(int Q, int KA, int KB);
 cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int npairs, int* out);
 // The weighted (SWMI) row kernel: its occupancy (FP64).
 cudaError_t rows_w_max_blocks_per_sm(int Q, int* out);

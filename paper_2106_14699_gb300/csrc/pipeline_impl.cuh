@@ -87,14 +87,16 @@ static cudaError_t launch_pair_cols(const Geom& g, const PipeArgs<T>& a, cudaStr
     }
     kern<<<grid, C::THREADS, smem, s>>>(a.FA, a.FB, g.KA, g.KB, g.Qh, g.HA, g.HB, g.R, g.r0, g.r1, a.Y, a.tw,
                                         tw_table(a.tw, g.Q), a.st, a.conditional, ctr, g.DA, g.DB, g.R2, a.plist, a.lrange,
-                                        a.chunk_off, a.chunk_cap, VOL ? 1 : g.units);
+                                        a.chunk_off, a.chunk_cap, VOL ? 1 : g.units, g.split);
     return cudaGetLastError();
 }
 
-// Teams per block of the Tensor-Memory row kernel (rows_tm.cuh): blocks of 8 where two of
-// them share an SM, except long runs of pairs at Q = 2048 (16: 64 pairs 0.410 vs 0.412 ms, 256
-// pairs 1.49 vs 1.50 ms; a few pairs leave most of 16 teams idle).
+// Teams per block of the Tensor-Memory row kernel (rows_tm.cuh).  One-warp teams: blocks of 8
+// where two of them share an SM, except long runs of pairs at Q = 2048 (16: 64 pairs 0.410 vs
+// 0.412 ms, 256 pairs 1.49 vs 1.50 ms; a few pairs leave most of 16 teams idle).
 static int rows_tm_teams(int Q, int tm_cols, int npairs) {
+    if (Q == 4096) return 8;
+    if (Q % 3 == 0) return 4;
     return tm_cols > 256 || (Q == 2048 && npairs > 32) ? 16 : 8;
 }
 
@@ -116,18 +118,28 @@ static cudaError_t launch_rows_tm(const Geom& g, const PipeArgs<float>& a, cudaS
     return cudaGetLastError();
 }
 
+template <int Q, bool NMI, int MODE>
+static cudaError_t launch_rows_tm_mode(const Geom& g, const PipeArgs<float>& a, cudaStream_t s) {
+    if constexpr (Q == 4096) {
+        return launch_rows_tm<Q, NMI, MODE, 8>(g, a, s);
+    } else if constexpr (Q % 3 == 0) {
+        return launch_rows_tm<Q, NMI, MODE, 4>(g, a, s);
+    } else {
+        return rows_tm_teams(Q, a.tm_cols, g.KA * g.KB) == 8 ? launch_rows_tm<Q, NMI, MODE, 8>(g, a, s)
+                                                             : launch_rows_tm<Q, NMI, MODE, 16>(g, a, s);
+    }
+}
+
 template <typename T, int Q, bool NMI>
 static cudaError_t launch_pair_rows_v(const Geom& g, const PipeArgs<T>& a, cudaStream_t s) {
     using C = RowCfg<T, Q>;
-    if constexpr (std::is_same<T, float>::value && split32_rows(Q)) {
+    if constexpr (std::is_same<T, float>::value && tm_rows(Q)) {
         if (a.tm_cols > 0 && !a.counts) {  // debug count maps: the generic kernel below
             const bool ext = a.ov_slot || a.pair_res || a.conditional || a.wait_polls > 0 || a.withhold_row >= 0;
             // the multi-unit kernel lives in its own translation unit (kernels_f32_rows_units.cu):
             // compiled next to the plain one, it changed the plain kernel's register allocation
             if (!ext && g.units > 1) return launch_rows_tm_units<Q, NMI>(g, a, s);
-            if (rows_tm_teams(Q, a.tm_cols, g.KA * g.KB) == 8)
-                return ext ? launch_rows_tm<Q, NMI, 2, 8>(g, a, s) : launch_rows_tm<Q, NMI, 0, 8>(g, a, s);
-            return ext ? launch_rows_tm<Q, NMI, 2, 16>(g, a, s) : launch_rows_tm<Q, NMI, 0, 16>(g, a, s);
+            return ext ? launch_rows_tm_mode<Q, NMI, 2>(g, a, s) : launch_rows_tm_mode<Q, NMI, 0>(g, a, s);
         }
     }
     size_t smem = pair_rows_smem<T, Q>(g.KB, a.cb_smem);
@@ -290,11 +302,12 @@ cudaError_t Sized<T, SZ>::rows_w_max_blocks(int* out) {
 }
 
 template <typename T, int SZ>
-int Sized<T, SZ>::tm_cols(int KB) {
-    if constexpr (std::is_same<T, float>::value && split32_rows(SZ)) {
-        const int need = tm_cols_needed(KB, SZ);
+int Sized<T, SZ>::tm_cols(int KA, int KB) {
+    if constexpr (std::is_same<T, float>::value && tm_rows(SZ)) {
+        const int need = tm_cols_needed(tm_swapped(SZ, KA, KB) ? KA : KB, SZ);
         return need <= 512 ? tm_alloc_cols(need) : 0;
     } else {
+        (void)KA;
         (void)KB;
         return 0;
     }
@@ -303,11 +316,12 @@ int Sized<T, SZ>::tm_cols(int KB) {
 template <typename T, int SZ>
 cudaError_t Sized<T, SZ>::tm_max_blocks(int tm_cols, int npairs, int* out) {
     *out = 0;
-    if constexpr (std::is_same<T, float>::value && split32_rows(SZ)) {
+    if constexpr (std::is_same<T, float>::value && tm_rows(SZ)) {
         // The blocks that share an SM: as many as the kernel is bounded for (registers; shared
         // memory is less than that), within the SM's 512 TMEM columns.  (The occupancy query
         // answers 1 for a kernel that allocates Tensor Memory.)
-        const int blocks = rows_tm_teams(SZ, tm_cols, npairs) == 16 ? 1 : RowTmCfg<SZ, 8>::BLOCKS;
+        constexpr int NT = SZ % 3 == 0 ? 4 : 8;
+        const int blocks = rows_tm_teams(SZ, tm_cols, npairs) == 16 ? 1 : RowTmCfg<SZ, NT>::BLOCKS;
         *out = std::min(blocks, 512 / tm_cols);
         return cudaSuccess;
     } else {

@@ -1,5 +1,5 @@
 // Inverse row transform + fused entropy epilogue, FP32, one warp per pair
-// transform (L = Q/2 = 256, 512 or 1024 points), with
+// transform (L = Q/2 = 256, 512 or 1024 points; two or three warps for 2048, 768 and 1536), with
 //   * the B-marginal accumulators C_B^b(p) held in Tensor Memory (TMEM,
 //     tcgen05.ld / tcgen05.st), one 32-bit column per (b, position) of the
 //     owning thread, and
@@ -24,12 +24,16 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 // Row `row` of pair `pair` (layout of Y): the 32-byte pieces (row % 4) of the row group's
-// 128-byte lines, one per chunk.  Tensor: 32 floats x L/4 chunks x row groups x pairs, box
-// 8 x L/4 x 1 x 1; x = 8 (row % 4) is a multiple of 4 floats (16 bytes).
-__device__ __forceinline__ void tma_row_g2s(uint32_t dst, const CUtensorMap* map, int row, int pair, uint32_t bytes, uint32_t bar) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-                 ::"r"(dst), "l"(map), "r"(bar), "r"(8 * (row & 3)), "r"(0), "r"(row >> 2), "r"(pair) : "memory");
+// 128-byte lines, one per chunk.  Tensor: 32 floats x L/4 chunks x row groups x pairs, boxes of
+// 8 x (at most 256 chunks) x 1 x 1; x = 8 (row % 4) is a multiple of 4 floats (16 bytes).
+__host__ __device__ constexpr int row_box(int L) { return L / 4 <= 256 ? L / 4 : L / 8; }
+template <int L>
+__device__ __forceinline__ void tma_row_g2s(uint32_t dst, const CUtensorMap* map, int row, int pair, uint32_t bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)L * 8u) : "memory");
+#pragma unroll
+    for (int c = 0; c < L / 4; c += row_box(L))
+        asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+                     ::"r"(dst + 32u * c), "l"(map), "r"(bar), "r"(8 * (row & 3)), "r"(c), "r"(row >> 2), "r"(pair) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t phase) {
     uint32_t done;
@@ -224,44 +228,71 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&re)[PTS / 2], float2 (&im)
     dft_pk<PTS, +1>(re, im);
 }
 
-// NT teams (warps) per block, BLOCKS blocks per SM.  Narrow rows hold few values per lane, so
+// L = G LS: a team of G warps.  G = 2, 3 (Q = 4096, 1536, 3072): radix-G decimation in frequency as
+// the values are loaded: warp r forms y_r[m] = w_L^{mr} sum_s w_G^{sr} x[m + s LS] and transforms
+// its LS points; X[G k + r] = Y_r[k].  Against the generic kernel (which keeps a whole row's
+// counts and marginals in shared memory: one or two blocks of idle FMA pipes), rows of 300-row
+// maps, four angles, ms: Q = 3072, 8 x 8 labels 1.64 -> 1.03, 16 x 16 6.42 -> 3.84 (2.9 -> 4.9e11
+// counts/s); Q = 4096 2.74 -> 1.15, 13.6 -> 4.24; Q = 1536, 36 x 36 15.2 -> 12.8.  Every warp of a
+// team reads the whole row (G shared-memory reads of each value), which costs most at G = 3.
+// NT teams per block, BLOCKS blocks per SM.  Narrow rows hold few values per lane, so
 // more warps fit, and several small blocks, each with its own barriers, run one's transforms
 // (FMA pipe) beside another's entropy terms (ALU, MUFU).  Measured at K = 16 (1e11 counts/s):
 // Q = 512: 16 warps in one block 5.0, 2 blocks of 8 5.8, 4 of 8 6.2; Q = 1024: one of 16 6.5,
 // 2 of 8 7.0, 3 of 8 (spills) 4.8; Q = 2048: one of 16 7.2, 2 of 8 7.15.  NT = 16 also where two
-// blocks' B-marginals do not fit in Tensor Memory.
+// blocks' marginals do not fit in Tensor Memory.
 template <int Q, int NT_>
 struct RowTmCfg {
-    static constexpr int L = Q / 2, PTS = L / 32, H = PTS / 2, RS = 32 / PTS;
-    // Q <= 1024: one pass holds the whole row, fewer barriers and TMEM round trips per
-    // round; at 2048 the counts of a round go to their owners in two passes
-    static constexpr int HALVES = Q <= 1024 ? 1 : 2;
-    static constexpr int NT = NT_, THREADS = NT * 32, BLOCKS = NT == 16 ? 1 : Q == 512 ? 4 : 2;
+    static constexpr int L = Q / 2, G = Q % 3 == 0 ? 3 : Q == 4096 ? 2 : 1, LS = L / G;
+    static constexpr int PTS = LS / 32, H = PTS / 2, RS = 32 / PTS;
+    static constexpr int NT = NT_, WARPS = NT * G, THREADS = WARPS * 32;
+    static constexpr int BLOCKS = Q == 1536 ? 2 : G > 1 || NT == 16 ? 1 : Q == 512 ? 4 : 2;
+    // one pass holds the whole row: fewer barriers and TMEM round trips per round; at 2048 and
+    // 4096 the counts of a round go to their owners in two passes
+    static constexpr int HALVES = Q == 2048 || Q == 4096 ? 2 : 1;
     static constexpr int QH = Q / HALVES;        // positions per pass
     static constexpr int UH = QH / THREADS;      // positions per thread per pass: adjacent floats of the hand-over
     static constexpr int U = HALVES * UH;
-    static constexpr int REGION = QH * 4;        // one pass of a pair's rounded counts
-    static constexpr int STAGE_BYTES = L * 8;    // one Y row, then the transpose planes
+    static constexpr int REGION = QH * 4;        // one pass of a pair's rounded counts: G parts, one per warp
+    static constexpr int STAGE_BYTES = L * 8;    // one Y row, then the warps' transpose planes
     static constexpr size_t OFF_STAGE = (size_t)NT * REGION;
     static constexpr size_t OFF_BAR = OFF_STAGE + (size_t)NT * STAGE_BYTES;
-    static constexpr size_t OFF_HOLD = OFF_BAR + NT * 8;
+    static constexpr size_t OFF_HOLD = OFF_BAR + 16 * 8;
     static constexpr size_t OFF_TW1 = OFF_HOLD + 16;                       // twiddles, as float4
     static constexpr size_t OFF_TW2 = OFF_TW1 + (size_t)H * 32 * 16;
-    static constexpr size_t SMEM = OFF_TW2 + (RS > 1 ? (size_t)RS * H * 16 : 0);
-    static_assert(UH == 1 || UH == 2 || UH == 4, "one, two or four positions per thread and pass");
+    static constexpr size_t OFF_TW3 = OFF_TW2 + (RS > 1 ? (size_t)RS * H * 16 : 0);
+    static constexpr size_t SMEM = OFF_TW3 + (size_t)(G - 1) * H * 32 * 16;
+    // B-marginals per TMEM round trip: as many as the registers hold beside the second pass's counts
+    static constexpr int NMED = UH == 8 || (UH == 4 && HALVES == 2) ? 4 : 8, NBIG = UH <= 2 ? 16 : NMED;
+    static_assert(UH == 1 || UH == 2 || UH == 4 || UH == 8, "positions per thread and pass");
     static_assert((size_t)NT * REGION >= (size_t)Q * 12, "the hand-over region holds a row of MI and N");
-    // Position (0 .. Q) of float f of pass hf in a pair's hand-over region: slot f / 2 of lane
-    // l = slot % 32 holds values q and q + H of the lane, real or imaginary part
+    static_assert(PTS * 32 * 8 * G <= STAGE_BYTES, "a warp's planes fit its part of the staged row");
+    // Position (0 .. Q) of float f of pass hf in a pair's hand-over region: part r (warp); its slot
+    // f / 2 of lane l = slot % 32 holds values q and q + H of the lane, real or imaginary part
     static __device__ __forceinline__ int position(int hf, int f) {
-        const int slot = f >> 1, l = slot & 31, qc = slot >> 5;
-        const int q = hf * (H / HALVES) + (qc >> 1) + (f & 1) * H;
-        return 2 * (l + 32 * q) + (qc & 1);
+        constexpr int PART = QH / G;
+        const int r = G == 1 ? 0 : f / PART, fr = f - r * PART;
+        const int slot = fr >> 1, l = slot & 31, qc = slot >> 5;
+        const int q = hf * (H / HALVES) + (qc >> 1) + (fr & 1) * H;
+        return 2 * (G * (l + 32 * q) + r) + (qc & 1);
     }
 };
 
-// TMEM columns a block needs: K_B marginals x U = Q / (32 NT) positions per thread, NT / 4
-// warps per lane quadrant.
-__host__ __device__ constexpr int tm_cols_needed(int KB, int Q) { return KB * (Q / 128); }
+// A barrier over the G warps of one team (G = 1: the warp).
+template <int G>
+__device__ __forceinline__ void team_sync(int team) {
+    if constexpr (G == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(G * 32) : "memory");
+}
+
+// The order of the pairs: label a outside, b inside, or, for the wide rows of several-warp teams
+// with fewer labels a, the other way round (more inputs fit in Tensor Memory).  Not for the
+// one-warp teams, whose kernel is at the register limit: Q = 2048, 24 x 24 labels 3.79 ms
+// without, 3.91 ms with the choice.
+__host__ __device__ constexpr bool tm_swapped(int Q, int KA, int KB) { return (Q % 3 == 0 || Q == 4096) && KA < KB; }
+// TMEM columns a block needs: KI marginals (the inner labels) x U = Q / (32 WARPS) positions per
+// thread, WARPS / 4 warps per lane quadrant.
+__host__ __device__ constexpr int tm_cols_needed(int KI, int Q) { return KI * (Q / 128); }
 __host__ __device__ constexpr int tm_alloc_cols(int need) {
     return need <= 32 ? 32 : need <= 64 ? 64 : need <= 128 ? 128 : need <= 256 ? 256 : 512;
 }
@@ -291,21 +322,29 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
         wait_polls = kDefaultWaitPolls;
         withhold_row = -1;
     }
-    constexpr int L = C::L, NT = C::NT, U = C::U, UH = C::UH, HALVES = C::HALVES, PTS = C::PTS, H = C::H;
+    constexpr int L = C::L, NT = C::NT, U = C::U, UH = C::UH, HALVES = C::HALVES, PTS = C::PTS, H = C::H, G = C::G;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int tid = threadIdx.x, team = tid >> 5, lane = tid & 31;
-    float2* region = reinterpret_cast<float2*>(smem_raw + (size_t)team * C::REGION);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, team = warp / G, wr = warp % G;  // warp wr of the team
+    float2* region = reinterpret_cast<float2*>(smem_raw + (size_t)team * C::REGION + (size_t)wr * (C::REGION / G));
     float* stage = reinterpret_cast<float*>(smem_raw + C::OFF_STAGE + (size_t)team * C::STAGE_BYTES);
     const uint32_t stage_s = smem_u32(stage);
     const uint32_t bar = smem_u32(smem_raw + C::OFF_BAR + team * 8);
     uint32_t* hold = reinterpret_cast<uint32_t*>(smem_raw + C::OFF_HOLD);
 
-    const int KA = g.KA, KB = g.KB, npairs = KA * KB, Rout = g.R, Cout = g.C;
+    // pairs in runs of one outer label: its marginal in registers, the KI inner labels' in TMEM
+    const int npairs = g.KA * g.KB, Rout = g.R, Cout = g.C;
+    const bool swapped = tm_swapped(Q, g.KA, g.KB);
+    const int KI = swapped ? g.KA : g.KB;
+    auto pair_id = [&](int t) {  // pair t in this order -> a * K_B + b
+        if (!swapped) return t;
+        const int o = t / KI;
+        return (t - o * KI) * g.KB + o;
+    };
     float4* tw1 = reinterpret_cast<float4*>(smem_raw + C::OFF_TW1);
     float4* tw2 = reinterpret_cast<float4*>(smem_raw + C::OFF_TW2);
     for (int i = tid; i < H * 32; i += C::THREADS) {
         const int k = i >> 5, j = i & 31;
-        const cpx<float> a = tw_of<L>(tw)[j * k], b = tw_of<L>(tw)[j * (k + H)];
+        const cpx<float> a = tw_of<C::LS>(tw)[j * k], b = tw_of<C::LS>(tw)[j * (k + H)];
         tw1[i] = make_float4(a.x, b.x, a.y, b.y);
     }
     if (C::RS > 1) {
@@ -316,15 +355,23 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
         }
     }
 
-    if (lane == 0) mbar_init(bar, 1);
-    if (team == 0) tmem_alloc(smem_u32(hold), (uint32_t)tm_cols);
+    float4* tw3 = reinterpret_cast<float4*>(smem_raw + C::OFF_TW3);  // w_L^{mr} of lane j's pairs, r >= 1
+    if (G > 1) {
+        for (int i = tid; i < (G - 1) * H * 32; i += C::THREADS) {
+            const int r = i / (H * 32) + 1, m = (i >> 5) % H, n = (i & 31) + 64 * m;
+            const cpx<float> a = tw_of<L>(tw)[n * r], b = tw_of<L>(tw)[(n + 32) * r];
+            tw3[i] = make_float4(a.x, b.x, a.y, b.y);
+        }
+    }
+    if (lane == 0 && wr == 0) mbar_init(bar, 1);
+    if (warp == 0) tmem_alloc(smem_u32(hold), (uint32_t)tm_cols);
     mbar_fence_init();
     tmem_fence_before();
     __syncthreads();
     tmem_fence_after();
     const uint32_t tmem = *hold;
     // this warp's TMEM slice: lanes of quadrant (warp % 4), columns of block (warp / 4)
-    const uint32_t tbase = tmem + ((uint32_t)(32 * (team & 3)) << 16) + (uint32_t)((team >> 2) * KB * U);
+    const uint32_t tbase = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * KI * U);
 
     // work items of this team: (row, base) in order; prefetch the first active one
     uint32_t phase = 0;
@@ -341,9 +388,9 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
     };
     auto issue = [&](int row_i, int pair_i) {
         if (EXT && row_i == withhold_row && pair_i == 0) return;  // diagnostics: leave this wait without its copy
-        if (lane == 0) {
+        if (lane == 0 && wr == 0) {
             fence_proxy_async_smem();
-            tma_row_g2s(stage_s, &ymap, row_i, pair_i, C::STAGE_BYTES, bar);
+            tma_row_g2s<L>(stage_s, &ymap, row_i, pair_id(pair_i), bar);
         }
         pending = true;
     };
@@ -366,9 +413,9 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
             uint32_t z[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) z[i] = 0u;
-            for (int c0 = 0; c0 < KB * U; c0 += 16) {
-                if (c0 + 16 <= KB * U) tmem_st<16>(tbase + c0, z);
-                else for (int c = c0; c < KB * U; ++c) { uint32_t z1[1] = {0u}; tmem_st<1>(tbase + c, z1); }
+            for (int c0 = 0; c0 < KI * U; c0 += 16) {
+                if (c0 + 16 <= KI * U) tmem_st<16>(tbase + c0, z);
+                else for (int c = c0; c < KI * U; ++c) { uint32_t z1[1] = {0u}; tmem_st<1>(tbase + c, z1); }
             }
             tmem_wait_st();
         }
@@ -394,16 +441,17 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                 const int jj = (32 - lane) & 31;
                 const float4* dsrc = sg4 + 2 * lane + ((lane >> 2) & 1);
                 const float4* msrc = sg4 + 2 * jj + (1 ^ ((jj >> 2) & 1));
+                constexpr int HP = G * H / 2;  // direct pairs of the row
+                auto raw = [&](int u) { return u < HP ? dsrc[64 * u] : msrc[64 * (2 * HP - 1 - u)]; };
+                // Column 0's mirrors come in the other order and one pair off (its own mirror is
+                // L / 2): lane 0's even inputs are the previous pair's second values.
+                if constexpr (G == 1) {
 #pragma unroll
-                for (int m = 0; m < H / 2; ++m) {
-                    const float4 d = dsrc[64 * m], w = msrc[64 * (H / 2 - 1 - m)];
-                    re[m] = make_float2(d.x, d.y);
-                    im[m] = make_float2(d.z, d.w);
-                    re[H / 2 + m] = make_float2(w.x, w.y);
-                    im[H / 2 + m] = make_float2(w.z, w.w);
-                }
-                {   // column 0's mirrors come in the other order and one pair off (its own mirror is
-                    // L / 2): lane 0's even inputs are the previous pair's second values
+                    for (int m = 0; m < H; ++m) {
+                        const float4 x = raw(m);
+                        re[m] = make_float2(x.x, x.y);
+                        im[m] = make_float2(x.z, x.w);
+                    }
                     float pr = re[H - 1].y, pi = im[H - 1].y;
 #pragma unroll
                     for (int m = H / 2; m < H; ++m) {
@@ -415,8 +463,55 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                         pr = tr.y;
                         pi = ti.y;
                     }
+                } else {
+                    float2 prev[G];  // the raw pair before the next one of the row's part s
+                    auto input = [&](int s, int m) {
+                        const int u = s * H + m;
+                        float4 x = raw(u);
+                        if (u >= HP) {
+                            if (u == HP) {
+                                const float4 w = raw(2 * HP - 1);
+                                prev[s] = make_float2(w.y, w.w);
+                            } else if (m == 0) {
+                                const float4 w = raw(u - 1);
+                                prev[s] = make_float2(w.y, w.w);
+                            }
+                            const float2 next = make_float2(x.y, x.w);
+                            x = lane == 0 ? make_float4(prev[s].x, x.x, prev[s].y, x.z) : x;
+                            prev[s] = next;
+                        }
+                        return x;
+                    };
+#pragma unroll
+                    for (int m = 0; m < H; ++m) {
+                        const float4 x0 = input(0, m);
+                        if constexpr (G == 2) {
+                            const float4 x1 = input(1, m);
+                            const float sg = wr ? -1.f : 1.f;
+                            re[m] = fmak(make_float2(x1.x, x1.y), sg, make_float2(x0.x, x0.y));
+                            im[m] = fmak(make_float2(x1.z, x1.w), sg, make_float2(x0.z, x0.w));
+                        } else {
+                            // x0 + w_3^r x1 + w_3^{2r} x2: x0 + x1 + x2, or x0 - t/2 +- i (sqrt 3 / 2) d
+                            const float4 x1 = input(1, m), x2 = input(2, m);
+                            const float2 tr = addv(make_float2(x1.x, x1.y), make_float2(x2.x, x2.y));
+                            const float2 ti = addv(make_float2(x1.z, x1.w), make_float2(x2.z, x2.w));
+                            if (wr == 0) {
+                                re[m] = addv(make_float2(x0.x, x0.y), tr);
+                                im[m] = addv(make_float2(x0.z, x0.w), ti);
+                            } else {
+                                const float2 dr = subv(make_float2(x1.x, x1.y), make_float2(x2.x, x2.y));
+                                const float2 di = subv(make_float2(x1.z, x1.w), make_float2(x2.z, x2.w));
+                                const float s3 = wr == 1 ? 0.86602540378443864676f : -0.86602540378443864676f;
+                                re[m] = fmak(di, -s3, fmak(tr, -0.5f, make_float2(x0.x, x0.y)));
+                                im[m] = fmak(dr, s3, fmak(ti, -0.5f, make_float2(x0.z, x0.w)));
+                            }
+                        }
+                        if (wr > 0) mul_conj2(re[m], im[m], tw3[((wr - 1) * H + m) * 32 + lane]);
+                    }
                 }
-                warp_fft_inv<PTS>(re, im, lane, stage, tw1, tw2);
+                if (G > 1) team_sync<G>(team);  // the team's warps have read the row: it becomes their planes
+                warp_fft_inv<PTS>(re, im, lane, stage + wr * (PTS * 64), tw1, tw2);
+                if (G > 1) team_sync<G>(team);  // and their planes are read
             } else {
 #pragma unroll
                 for (int k = 0; k < H; ++k) re[k] = im[k] = make_float2(0.f, 0.f);
@@ -452,15 +547,15 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                 round2(re[k]);
                 round2(im[k]);
             }
-            const int ovs = (EXT && act && ov_slot) ? ov_slot[pair] : -1;  // loaded after the transform: fewer live registers
+            const int ovs = (EXT && act && ov_slot) ? ov_slot[pair_id(pair)] : -1;  // loaded after the transform: fewer live registers
             if (EXT && ovs < 0) res_max = fmaxf(res_max, rp);
-            if (EXT && pair_res && act && ovs < 0) {  // the warp is this pair's team
+            if (EXT && pair_res && act && ovs < 0) {
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) rp = fmaxf(rp, __shfl_xor_sync(0xffffffffu, rp, off));
-                if (lane == 0) atomic_max_float_pos(&pair_res[pair], rp);
+                if (lane == 0) atomic_max_float_pos(&pair_res[pair_id(pair)], rp);
             }
             const int nt = min(NT, npairs - base);
-            const int a0 = base / KB, b0 = base - a0 * KB;
+            const int a0 = base / KI, b0 = base - a0 * KI;  // outer and inner label of the round's first pair
 #pragma unroll
             for (int hf = 0; hf < HALVES; ++hf) {
                 if (aborted) continue;
@@ -478,8 +573,8 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
 #pragma unroll
                     for (int q = 0; q < HP; ++q) {
                         const int z = lane + 32 * (hf * HP + q);
-                        const int2 x = *reinterpret_cast<const int2*>(ovr + 2 * z);
-                        const int2 y = *reinterpret_cast<const int2*>(ovr + 2 * (z + 32 * H));
+                        const int2 x = *reinterpret_cast<const int2*>(ovr + 2 * (G * z + wr));
+                        const int2 y = *reinterpret_cast<const int2*>(ovr + 2 * (G * (z + 32 * H) + wr));
                         region[2 * q * 32 + lane] = make_float2((float)x.x, (float)y.x);
                         region[(2 * q + 1) * 32 + lane] = make_float2((float)x.y, (float)y.y);
                     }
@@ -491,7 +586,7 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                     }
                 }
                 __syncthreads();
-                const uint32_t tcol = tbase + (uint32_t)(hf * KB * UH);
+                const uint32_t tcol = tbase + (uint32_t)(hf * KI * UH);
                 // NB pairs of one label a, labels b .. b + NB - 1: their B-marginals of this pass in
                 // registers, one TMEM load and store
                 auto accum = [&](auto nbc, int t0, int b) {
@@ -509,9 +604,12 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                             cbr[t] = __float_as_uint(__uint_as_float(cbr[t]) + c);
                         } else {
                             float cv[UH];
-                            if constexpr (UH == 4) {
-                                const float4 q = reinterpret_cast<const float4*>(obt)[tid];
-                                cv[0] = q.x; cv[1] = q.y; cv[2] = q.z; cv[3] = q.w;
+                            if constexpr (UH >= 4) {
+#pragma unroll
+                                for (int w = 0; w < UH / 4; ++w) {
+                                    const float4 q = reinterpret_cast<const float4*>(obt)[UH / 4 * tid + w];
+                                    cv[4 * w] = q.x; cv[4 * w + 1] = q.y; cv[4 * w + 2] = q.z; cv[4 * w + 3] = q.w;
+                                }
                             } else {
                                 const float2 q = reinterpret_cast<const float2*>(obt)[tid];
                                 cv[0] = q.x; cv[1] = q.y;
@@ -547,10 +645,9 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                         }
                         cur_a[hf] = a;
                     }
-                    const int seg = min(KB - b, nt - t);  // the rest of label a in this round
+                    const int seg = min(KI - b, nt - t);  // the rest of the outer label's run in this round
                     int d;
-                    // UH = 4 with two passes: 4 labels at a time hold the registers (8 spill)
-                    constexpr int NMED = UH == 4 && HALVES == 2 ? 4 : 8, NBIG = UH <= 2 ? 16 : NMED;
+                    constexpr int NMED = C::NMED, NBIG = C::NBIG;
                     if (NBIG > NMED && seg >= NBIG) {
                         accum(std::integral_constant<int, NBIG>{}, t, b);
                         d = NBIG;
@@ -566,28 +663,28 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
                     }
                     t += d;
                     b += d;
-                    if (b == KB) { b = 0; ++a; }
+                    if (b == KI) { b = 0; ++a; }
                 }
             }
             if (aborted) break;
         }
         if (aborted) break;
         __syncthreads();  // the last counts are read
-        // finish the row: last A-marginal, the B-marginals, then MI and N through the
+        // finish the row: the last outer label's marginal, the inner labels', then MI and N through the
         // hand-over region (doubles, then integers), so that the map is written in order
         double* mrow = reinterpret_cast<double*>(smem_raw);
         int* nrow_s = reinterpret_cast<int*>(smem_raw + (size_t)Q * 8);
 #pragma unroll
         for (int hf = 0; hf < HALVES; ++hf) {
-            float n[UH];  // N = the sum of the B-marginals (exact: below 2^23)
+            float n[UH];  // N = the sum of the inner labels' marginals (exact: below 2^23)
 #pragma unroll
             for (int uh = 0; uh < UH; ++uh) {
                 S[hf * UH + uh].marg(clog2c_biased(CA[hf * UH + uh]));
                 n[uh] = 0.f;
             }
-            for (int b = 0; b < KB; ++b) {
+            for (int b = 0; b < KI; ++b) {
                 uint32_t cbr[UH];
-                tmem_ld<UH>(tbase + (uint32_t)(hf * KB * UH + b * UH), cbr);
+                tmem_ld<UH>(tbase + (uint32_t)(hf * KI * UH + b * UH), cbr);
                 tmem_wait_ld();
 #pragma unroll
                 for (int uh = 0; uh < UH; ++uh) {
@@ -633,7 +730,7 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
     tmem_fence_before();
     __syncthreads();
     tmem_fence_after();
-    if (team == 0) tmem_dealloc(tmem, (uint32_t)tm_cols);
+    if (warp == 0) tmem_dealloc(tmem, (uint32_t)tm_cols);
 }
 
 }  // namespace cmif

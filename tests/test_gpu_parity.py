@@ -136,6 +136,35 @@ def test_wide_rows_tmem_partial_rounds(cm, W, Q, K):
     assert float(np.abs(g["mi"] - ref["mi"]).max()) <= MI_TOL
 
 
+@pytest.mark.parametrize("K", [(3, 7), (9, 3), (22, 22)], ids=lambda x: "x".join(map(str, x)))
+@pytest.mark.parametrize("W", [1240, 1490, 2600, 3000, 3200, 4090])
+def test_wide_rows_tmem_team_of_warps(cm, W, K):
+    """Widths 1536, 3072 and 4096, whose rows take two or three warps: fewer labels a than b
+    (the order of the pairs is swapped) and more, last rounds that are not full, more rows than
+    resident blocks, both ends of each width; 22 x 22 is past two blocks' Tensor Memory at 1536
+    and past one block's at 3072 and 4096.  N and MI over the whole map against the oracle,
+    one map and two angles at once."""
+    rng = np.random.default_rng(W + K[0])
+    A, MA, B, MB = _rand(rng, 170, W - 6, 160, 7, *K)
+    if K[0] > 9:
+        A, MA, B, MB = A[:20], MA[:20], B[:12], MB[:12]
+    ref = oracle.cmif(A, MA, B, MB, *K)
+    g = run_gpu(cm, A, MA, B, MB, *K, cm.FP32, counts=False, gamma=0.5)
+    assert g["status"][0] == "OK", g["status"]
+    np.testing.assert_array_equal(g["n"], ref["n"])
+    assert float(np.abs(g["mi"] - ref["mi"]).max()) <= MI_TOL
+    t = [torch.tensor(np.ascontiguousarray(x), device="cuda") for x in (A, MA, B, MB)]
+    if K[0] == 3:  # two units per launch
+        found = []
+        for batch in (False, True):
+            p = cm.Plan(*A.shape, *B.shape, *K, cm.FP32, batch_angles=batch)
+            rec = torch.zeros(240, dtype=torch.uint8, device="cuda")
+            p.align_rotations(*t, [0.0, 3.0], 0.5, 1, rec)
+            found.append(rec.cpu().numpy().tobytes())
+            p.close()
+        assert found[0] == found[1]
+
+
 # Every transform length, across rows (Q) and down columns (P): maps just over the next
 # shorter length and maps that fill it.  Column 0 (which carries two real columns), the
 # mirrored columns and the first and last chunk of each length take part.
