@@ -405,9 +405,14 @@ __device__ __forceinline__ void team_fft_core(cpx<T> (&v)[M], int j, void* sm, c
     }
 }
 
-template <int M, int R, int DIR, typename T, typename Load>
+// loaded(sync): called once this lane's loads are done; sync: those of the whole block are.
+struct NothingOnceLoaded {
+    __device__ __forceinline__ void operator()(bool) const {}
+};
+template <int M, int R, int DIR, typename T, typename Load, typename Loaded = NothingOnceLoaded>
 __device__ __forceinline__ void team_fft(cpx<T> (&v)[M], int r, int j, Load&& load, void* sm,
-                                         const cpx<T>* __restrict__ twq, const cpx<T>* __restrict__ twn) {
+                                         const cpx<T>* __restrict__ twq, const cpx<T>* __restrict__ twn,
+                                         Loaded loaded = Loaded()) {
     constexpr int NQ = M * M;
     if constexpr (R > 2 && !is_pow2(R)) {
         // Radix-R decimation in frequency (R = 3, 6) with every input loaded once: the
@@ -431,6 +436,7 @@ __device__ __forceinline__ void team_fft(cpx<T> (&v)[M], int r, int j, Load&& lo
             }
         }
         __syncthreads();
+        loaded(true);
 #pragma unroll
         for (int i = 0; i < M; ++i) v[i] = xs[r * NQ + j + M * i];
         __syncthreads();
@@ -459,6 +465,7 @@ __device__ __forceinline__ void team_fft(cpx<T> (&v)[M], int r, int j, Load&& lo
             }
         }
         __syncthreads();
+        loaded(true);
 #pragma unroll
         for (int i = 0; i < M; ++i) v[i] = xs[r * NQ + j + M * i];
         __syncthreads();  // the groups' transposes below reuse this buffer
@@ -475,6 +482,7 @@ __device__ __forceinline__ void team_fft(cpx<T> (&v)[M], int r, int j, Load&& lo
                 v[i] = (r == 0) ? acc : cmul(acc, twl<DIR>(twn, m * r));
             }
         }
+        loaded(false);
     }
     team_fft_core<M, DIR>(v, j, sm, twq);
 }

@@ -305,10 +305,15 @@ k_fwd_rows(const int32_t* __restrict__ X, const uint8_t* __restrict__ MX, const 
 }
 
 // ---------------------------------------------------------------------------
-// Forward column transforms.  Block = (TPB adjacent kx columns, plane).  The
-// block first stages its H x TPB input tile in shared memory with coalesced
+// Forward column transforms.  Item = (TPB adjacent kx columns, plane).  The
+// block first stages the item's H x TPB input tile in shared memory with coalesced
 // 16-byte loads (column slots XOR-swizzled by row, so that the teams' column
-// reads are conflict-free), then each team transforms one column.
+// reads meet few bank conflicts), then each team transforms one column.  FP32: persistent
+// blocks; the next item's tile is copied asynchronously (cp.async) into the same buffer from the
+// moment the columns are in registers, behind the transform and its stores: with one item per
+// block, waiting for the tile (4.1 of 12 cycles per issue) and for the block's other warps (3.7)
+// bounded the kernel.  16 labels, us: 1024 x 1024 223 -> 193, 512 x 512 43 -> 38, 32 labels of
+// 834 x 834 416 -> 364; P = 768, 331 x 1203, 12 labels 112 -> 77.
 template <typename T, int P, int MMAX = max_m<T>()>
 struct ColCfg {
     using G = TeamGeom<T, P, MMAX>;
@@ -319,6 +324,11 @@ struct ColCfg {
     static constexpr size_t SCR = (size_t)TPB * G::SCRATCH;
     static constexpr size_t TILE_MAX = (size_t)P * TPB * sizeof(cpx<T>);  // H <= P rows
     static constexpr size_t smem(int H) { return SCR + (size_t)H * TPB * sizeof(cpx<T>); }
+    static constexpr bool PIPE = std::is_same<T, float>::value && TPB >= 2;
+    // Resident blocks the registers are bounded for (FP32): without spills.  M = 32: two blocks 193 us, three
+    // with spills 221 (16 labels, 1024 x 1024).
+    static constexpr int f32_blocks() { return M == 32 ? 2 : M == 16 ? (THREADS < 256 ? 4 : 3) : M == 8 ? (THREADS < 256 ? 6 : 4) : 3; }
+    static constexpr int MIN_BLOCKS = sizeof(T) == 4 && THREADS <= 256 ? (std::is_same<T, float>::value ? f32_blocks() : 2) : 1;
 };
 
 // FP32 groups of 8 lanes and more keep the spectra in the order the packed DFTs take them:
@@ -332,7 +342,7 @@ __device__ __forceinline__ void st_global_32B(void* dst, const float (&v)[8]) {
 }
 
 template <typename T, int P, int MMAX>
-__global__ void __launch_bounds__(ColCfg<T, P, MMAX>::THREADS, sizeof(T) == 4 && ColCfg<T, P, MMAX>::THREADS <= 256 ? (std::is_same<T, float>::value ? 3 : 2) : 1)
+__global__ void __launch_bounds__(ColCfg<T, P, MMAX>::THREADS, ColCfg<T, P, MMAX>::MIN_BLOCKS)
 k_fwd_cols(const cpx<T>* __restrict__ T1, int H, int nplanes, int Qh, int Qs, cpx<T>* __restrict__ F, Tw<T> tw,
            const DevStatus* __restrict__ st, int conditional, T out_scale,
            const unsigned char* __restrict__ plane_need, int slices) {
@@ -340,63 +350,98 @@ k_fwd_cols(const cpx<T>* __restrict__ T1, int H, int nplanes, int Qh, int Qs, cp
     // transformed; plane p belongs to label p / slices (volumes: slices = depth).
     using C = ColCfg<T, P, MMAX>;
     if (conditional && !(st->flags & STATUS_ESCALATE)) return;
-    if (plane_need && plane_need[blockIdx.y / slices] != 1) return;
     constexpr int M = C::M, R = C::R, TPB = C::TPB;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     cpx<T>* tile = reinterpret_cast<cpx<T>*>(smem_raw + C::SCR);
     const int team = threadIdx.x / C::TEAM, lt = threadIdx.x % C::TEAM, r = lt / M, j = lt % M;
-    const int kx0 = blockIdx.x * TPB, kx = kx0 + team, plane = blockIdx.y;
-    const cpx<T>* src = T1 + (size_t)plane * H * Qs + kx0;
-    if constexpr (sizeof(T) == 4 && TPB >= 2) {
-        // 16-byte pieces (two columns each); Qs and kx0 are even, so a piece is
-        // wholly inside the row or wholly beyond Qs (never read: zeros)
-        constexpr int PPR = TPB / 2;
-        for (int q = threadIdx.x; q < H * PPR; q += C::THREADS) {
-            const int y = q / PPR, h = q % PPR;
-            float4 pv = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (kx0 + 2 * h < Qs) pv = __ldg(reinterpret_cast<const float4*>(src + (size_t)y * Qs) + h);
-            const int sw = (y >> C::SWZ) & (TPB - 1);
-            if (sw & 1) pv = make_float4(pv.z, pv.w, pv.x, pv.y);
-            reinterpret_cast<float4*>(tile)[y * PPR + (h ^ (sw >> 1))] = pv;
-        }
-    } else {
-        for (int q = threadIdx.x; q < H * TPB; q += C::THREADS) {
-            const int y = q / TPB, c = q % TPB;
-            const int sw = (y >> C::SWZ) & (TPB - 1);
-            tile[y * TPB + (c ^ sw)] = kx0 + c < Qs ? src[(size_t)y * Qs + c] : cpx<T>{T(0), T(0)};
-        }
-    }
-    __syncthreads();
-    const bool active = kx < Qh;
-    auto load = [&](int y) -> cpx<T> {
-        if (!active || y >= H) return {T(0), T(0)};
-        return tile[y * TPB + (team ^ ((y >> C::SWZ) & (TPB - 1)))];
+    const int nkxb = (Qh + TPB - 1) / TPB, n_items = nkxb * nplanes;
+    auto needed = [&](int it) {  // the next item from `it` on whose plane is needed
+        if (plane_need)
+            while (it < n_items && plane_need[it / nkxb / slices] != 1) it += gridDim.x;
+        return it;
     };
-    cpx<T> v[M];
-    team_fft<M, R, -1>(v, r, j, load, smem_raw + (size_t)team * C::G::SCRATCH + r * grp_scratch_bytes<T, M>(),
-                       tw.sq[ilog2c(M)], tw_of<P>(tw));
-    if (!active) return;
-    // Column ky is stored at slot (ky % R) * M*M + ky / R: the samples that one
-    // group of the pair-product transform (same P, same R) takes are contiguous.
-    cpx<T>* out = F + ((size_t)plane * Qh + kx) * P + r * (M * M);
-    if constexpr (packed_spectra<T, M>()) {
-#pragma unroll
-        for (int q = 0; q < M / 4; ++q) {
-            float w[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const cpx<T> z = v[brev(4 * q + i, M)];
-                w[4 * (i / 2) + i % 2] = z.x * out_scale;
-                w[4 * (i / 2) + 2 + i % 2] = z.y * out_scale;
+    // Slot of (row y, column c) in the tile: 16-byte pieces of two columns XOR-permuted by the row
+    // (without the asynchronous copies, the two columns of a piece, too).
+    auto slot = [&](int y, int c) {
+        const int sw = (y >> C::SWZ) & (TPB - 1);
+        return y * TPB + (c ^ (C::PIPE ? sw & ~1 : sw));
+    };
+    auto stage = [&](int it) {
+        const int plane = it / nkxb, kx0 = (it - plane * nkxb) * TPB;
+        const cpx<T>* src = T1 + (size_t)plane * H * Qs + kx0;
+        if constexpr (sizeof(T) == 4 && TPB >= 2) {
+            // 16-byte pieces (two columns each); Qs and kx0 are even, so a piece is
+            // wholly inside the row or wholly beyond Qs (never read: zeros)
+            constexpr int PPR = TPB / 2;
+            for (int q = threadIdx.x; q < H * PPR; q += C::THREADS) {
+                const int y = q / PPR, h = q % PPR;
+                const bool in = kx0 + 2 * h < Qs;
+                if constexpr (C::PIPE) {
+                    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(tile + slot(y, 2 * h));
+                    const cpx<T>* from = in ? src + (size_t)y * Qs + 2 * h : T1;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(from), "r"(in ? 16 : 0) : "memory");
+                } else {
+                    float4 pv = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (in) pv = __ldg(reinterpret_cast<const float4*>(src + (size_t)y * Qs) + h);
+                    const int sw = (y >> C::SWZ) & (TPB - 1);
+                    if (sw & 1) pv = make_float4(pv.z, pv.w, pv.x, pv.y);
+                    reinterpret_cast<float4*>(tile)[y * PPR + (h ^ (sw >> 1))] = pv;
+                }
             }
-            st_global_32B(out + 4 * (M * q + j), w);
+        } else {
+            for (int q = threadIdx.x; q < H * TPB; q += C::THREADS) {
+                const int y = q / TPB, c = q % TPB;
+                tile[slot(y, c)] = kx0 + c < Qs ? src[(size_t)y * Qs + c] : cpx<T>{T(0), T(0)};
+            }
         }
-    } else {
+    };
+    int it = needed(blockIdx.x);
+    if (it >= n_items) return;
+    stage(it);
+    while (true) {
+        if constexpr (C::PIPE) asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        const int plane = it / nkxb, kx = (it - plane * nkxb) * TPB + team;
+        const bool active = kx < Qh;
+        const int next = C::PIPE ? needed(it + gridDim.x) : n_items;
+        auto load = [&](int y) -> cpx<T> {
+            if (!active || y >= H) return {T(0), T(0)};
+            return tile[slot(y, team)];
+        };
+        auto loaded = [&](bool sync) {  // the tile's values are in registers
+            if (!C::PIPE || next >= n_items) return;
+            if (!sync) __syncthreads();
+            stage(next);
+        };
+        cpx<T> v[M];
+        team_fft<M, R, -1>(v, r, j, load, smem_raw + (size_t)team * C::G::SCRATCH + r * grp_scratch_bytes<T, M>(),
+                           tw.sq[ilog2c(M)], tw_of<P>(tw), loaded);
+        // Column ky is stored at slot (ky % R) * M*M + ky / R: the samples that one
+        // group of the pair-product transform (same P, same R) takes are contiguous.
+        cpx<T>* out = F + ((size_t)plane * Qh + kx) * P + r * (M * M);
+        if (active) {
+            if constexpr (packed_spectra<T, M>()) {
 #pragma unroll
-        for (int k2 = 0; k2 < M; ++k2) {
-            const cpx<T> z = v[brev(k2, M)];
-            out[j + M * k2] = {z.x * out_scale, z.y * out_scale};
+                for (int q = 0; q < M / 4; ++q) {
+                    float w[8];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const cpx<T> z = v[brev(4 * q + i, M)];
+                        w[4 * (i / 2) + i % 2] = z.x * out_scale;
+                        w[4 * (i / 2) + 2 + i % 2] = z.y * out_scale;
+                    }
+                    st_global_32B(out + 4 * (M * q + j), w);
+                }
+            } else {
+#pragma unroll
+                for (int k2 = 0; k2 < M; ++k2) {
+                    const cpx<T> z = v[brev(k2, M)];
+                    out[j + M * k2] = {z.x * out_scale, z.y * out_scale};
+                }
+            }
         }
+        it = next;
+        if (it >= n_items) break;
     }
 }
 

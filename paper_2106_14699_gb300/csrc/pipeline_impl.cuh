@@ -41,13 +41,25 @@ static cudaError_t launch_fwd_rows(const int32_t* X, const uint8_t* MX, const do
 template <typename T, int P, int MMAX>
 static cudaError_t launch_fwd_cols(const cpx<T>* T1, int H, int K, int Qh, int Qs, cpx<T>* F, const Tw<T>& tw,
                                    const DevStatus* st, int conditional, T out_scale, const unsigned char* need,
-                                   int slices, cudaStream_t s) {
+                                   int slices, int num_sms, cudaStream_t s) {
     using C = ColCfg<T, P, MMAX>;
     auto kern = k_fwd_cols<T, P, MMAX>;
     cudaError_t e = ensure_smem(kern, C::smem(P));
     if (e != cudaSuccess) return e;
-    dim3 grid((Qh + C::TPB - 1) / C::TPB, K);
-    kern<<<grid, C::THREADS, C::smem(H), s>>>(T1, H, K, Qh, Qs, F, tw, st, conditional, out_scale, need, slices);
+    const long long items = (long long)((Qh + C::TPB - 1) / C::TPB) * K;
+    long long slots = items;
+    if (C::PIPE && num_sms > 0) {  // persistent: every resident block slot
+        static int by_regs = -1;
+        if (by_regs < 0) {
+            int n = 0;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, C::THREADS, 0);
+            if (e != cudaSuccess) return e;
+            by_regs = n > 0 ? n : 1;
+        }
+        const int by_smem = (int)(228 * 1024 / (C::smem(H) + 1024));
+        slots = (long long)std::max(1, std::min(by_regs, by_smem)) * num_sms;
+    }
+    kern<<<(int)std::min(items, slots), C::THREADS, C::smem(H), s>>>(T1, H, K, Qh, Qs, F, tw, st, conditional, out_scale, need, slices);
     return cudaGetLastError();
 }
 
@@ -217,9 +229,9 @@ cudaError_t Sized<T, SZ>::fwd_cols(const Geom& g, const PipeArgs<T>& a, bool b_s
         constexpr int MM = decltype(mm)::value;
         return b_side ? launch_fwd_cols<T, SZ, MM>(a.T1B, g.HB, g.KB * g.DB, g.Qh, g.Qs, a.FB, a.tw, a.st,
                                                    a.conditional, inverse_of<T>((double)g.P * (double)g.Q), a.needB,
-                                                   g.DB, s)
+                                                   g.DB, a.num_sms, s)
                       : launch_fwd_cols<T, SZ, MM>(a.T1A, g.HA, g.KA * g.DA, g.Qh, g.Qs, a.FA, a.tw, a.st,
-                                                   a.conditional, T(1), a.needA, g.DA, s);
+                                                   a.conditional, T(1), a.needA, g.DA, a.num_sms, s);
     };
     if constexpr (kHasColVariant<T, SZ>) {
         if (a.col_m == 16) return go(std::integral_constant<int, 16>{});

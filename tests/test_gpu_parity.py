@@ -188,6 +188,21 @@ def test_every_transform_length(cm, N, axis):
             assert float(np.abs(g["mi"] - ref["mi"]).max()) <= MI_TOL
 
 
+@pytest.mark.parametrize("P", [16, 32, 64, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048, 3072, 4096])
+def test_forward_columns_many_items(cm, P):
+    """More column tiles than resident blocks: each block stages its next tile while it
+    transforms the present one.  A height that is odd and leaves rows to pad, a last tile
+    that is not full."""
+    rng = np.random.default_rng(P)
+    H, W, K = P - 3, 1490 if P < 3000 else 1010, (24, 3)
+    A, MA, B, MB = _rand(rng, H, W, 2, 5, *K)
+    ref = oracle.cmif(A, MA, B, MB, *K)
+    g = run_gpu(cm, A, MA, B, MB, *K, cm.FP32, counts=False, gamma=0.5)
+    assert g["status"][0] == "OK", g["status"]
+    np.testing.assert_array_equal(g["n"], ref["n"])
+    assert float(np.abs(g["mi"] - ref["mi"]).max()) <= MI_TOL
+
+
 @pytest.mark.parametrize("shape,K", WIDE[:3], ids=lambda x: "x".join(map(str, x)))
 def test_wide_rows_tmem_auto(cm, shape, K, monkeypatch):
     """CMIF_AUTO at the Tensor-Memory widths: the row kernel's AUTO form (exact
