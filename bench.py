@@ -36,13 +36,12 @@ WORKLOAD = "single-1024x1024-K16"
 GAMMA = 0.5
 L2_FLUSH_BYTES = 256 << 20  # > 129 MB L2
 
-# DRAM bytes per launch of the pair kernels, from ncu captures of the same
-# kernel instantiations on smaller cases (1024 x 256 and 256 x 1024 pairs) scaled
-# by the units processed (2047/511 output rows; 1025/257 kx columns).  Set to
-# None when a kernel changes after its capture.
+# DRAM bytes per launch of the pair kernels, from an ncu capture of the same kernels on a
+# smaller case (512 x 512, K = 16) scaled by the volume of Y (2047 x 1024 / (1023 x 512)).
+# Set to None when a kernel changes after its capture.
 NCU_TRAFFIC = {
-    "pair_rows_f32": 4.36e9,  # (1.076 GB read + 0.013 GB written) at 511 rows x 2047/511
-    "pair_cols_f32": 5.03e9,  # 0.202 GB read x 1025/257 + 1.067 GB written x 1028/260
+    "pair_rows_f32": 4.46e9,  # 1.100 GB read + 0.015 GB written, x 4.00
+    "pair_cols_f32": 4.62e9,  # 0.135 GB read + 1.019 GB written, x 4.00
 }
 
 
