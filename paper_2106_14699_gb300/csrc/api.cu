@@ -64,8 +64,9 @@ int pow2_at_least(int v, int lo) {
 
 // Transform length for n outputs: the smallest power of two >= max(n, 16), or,
 // for FP32 transforms, the smallest 3 * 2^k (192 .. 3072) if that is smaller.  (96 = 6 * 4^2 has
-// groups of 4 lanes and no packed DFTs: 10.8 ps per column point against 3.6 at 128, rows 1.2e11
-// counts/s against 2.9e11.)
+// groups of 4 lanes and no packed DFTs: down columns 10.8 ps per point against 3.6 at 128; across
+// rows, four angles of 700 x 40, 16 x 16 labels: rows 540 us against 385 at 128, columns 262
+// against 348.)
 int transform_size(int n, bool mixed) {
     int best = pow2_at_least(n, 16);
     if (mixed)

@@ -646,7 +646,7 @@ struct PairColsCfg {
 // 32-byte chunks.  An item thus passes shared memory twice (transpose, combine) and takes two
 // block barriers.  While the rows leave, the F_a loads of the block's next item are
 // already in flight, and
-// items at the head of a kx block ask L2 for the spectrum columns two kx blocks ahead.
+// items at the head of a kx block ask L2 for the spectrum columns of a later one.
 // FP32 groups of 8 lanes and more: spectra in the order of the packed DFTs, 32 bytes per
 // load (fwd_cols).  work_ctr must be zero at launch.
 // VOL (volumes): items are (pair, NDZ depth offsets dz, kx block); the product is
@@ -682,6 +682,10 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
     constexpr int NDZ = VOL ? C::NDZ : 1;
     const int U = VOL ? (Dz + NDZ - 1) / NDZ : units;  // the middle item dimension: groups of depth offsets or units
     const int nkxb = (L + TPB - 1) / TPB, n_items = npairs * nkxb * U;
+    // L2 prefetch distance in kx blocks: the one beyond those that the blocks in flight cover
+    // (columns, us, against a fixed 2: rotations of 300 x 300, 8 x 8 labels 2940 -> 2844, four of 134
+    // x 343 208 -> 184; 16 x 16 labels: the same)
+    const int ahead = max(2, 1 + (int)gridDim.x / npairs);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_next[6];  // the next item: whether there is one, e, a, b, kx block, unit / depth offset
     cpx<T>* xbuf = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -876,13 +880,19 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
             // column 0 carries y_0 + i y_L
             if (kx == 0) add_product(std::true_type{}, FA + ((size_t)a * Qh + L) * P + lane_off, gb + (size_t)L * P);
         }
-        if (!VOL && !plist && pair < KA + KB && (int)threadIdx.x < TPB && kxb + 2 < nkxb) {
+        if (!VOL && !plist && pair < KA + KB && (int)threadIdx.x < TPB) {
             // the items of this kx block with pair < K_A + K_B each prefetch one
-            // spectrum's columns of kx block kxb + 2 into L2 (one bulk request per column)
-            const int kf = column(kxb + 2, threadIdx.x);
+            // spectrum's columns of kx block kxb + ahead into L2 (one bulk request per column),
+            // or of the next unit's first ones
+            int kp = kxb + ahead, up = dzo;
+            if (kp >= nkxb) {
+                kp -= nkxb;
+                ++up;
+            }
+            const int kf = up < U && kp < nkxb ? column(kp, threadIdx.x) : -1;
             if (kf >= 0) {
                 const cpx<T>* src = pair < KA ? FA + ((size_t)pair * Qh + kf) * P
-                                              : FB + ((size_t)((pair - KA) * units + dzo) * Qh + kf) * P;
+                                              : FB + ((size_t)((pair - KA) * units + up) * Qh + kf) * P;
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((unsigned)(P * sizeof(cpx<T>)))
                              : "memory");
             }
