@@ -712,8 +712,10 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
     stage_table(tw_sq, tw.sq[ilog2c(M)], NQ);
     if (R > 1) stage_table(tw_n, tw_of<P>(tw), C::TW_N);
     __syncthreads();
-    if (!s_next[0]) return;
+    bool more = s_next[0] != 0;
     int e = s_next[1], a = s_next[2], b = s_next[3], kxb = s_next[4], dzo = s_next[5];
+    __syncthreads();  // s_next is read by every thread before thread 0 decodes the next item into it
+    if (!more) return;
     const int team = threadIdx.x / C::TEAM, lt = threadIdx.x % C::TEAM, r = lt / M, j = lt % M;
     cpx<T>* slice = xbuf + (size_t)team * P + r * NQ;  // this group's transpose scratch, then its sub-transform
     // the frequency kx this team transforms for kx block kxb, or -1 beyond the last
@@ -900,7 +902,6 @@ k_pair_cols(const cpx<T>* __restrict__ FA, const cpx<T>* __restrict__ FB, int KA
         // this item's rows below; its successor's fields once they are known
         cpx<T>* yp = Y + (size_t)e * y_rows<T>(Rout) * L;
         const int c0 = kxb * UPR, dz0 = dzo * NDZ;
-        bool more = false;
 #pragma unroll 1
         for (int s = 0; s < NDZ; ++s) {
         if (NDZ > 1) {

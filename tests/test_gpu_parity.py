@@ -203,6 +203,30 @@ def test_forward_columns_many_items(cm, P):
     assert float(np.abs(g["mi"] - ref["mi"]).max()) <= MI_TOL
 
 
+@pytest.mark.parametrize("prec", ["FP32", "FP64"])
+@pytest.mark.parametrize("N,K", [(20, 16), (60, 16), (120, 12), (250, 8)])
+def test_pair_columns_items_in_turn(cm, prec, N, K):
+    """Each pair-column block takes several items and every warp of it must see the same one:
+    the maps of many calls are the oracle's, bit for bit the same."""
+    rng = np.random.default_rng(N)
+    A, MA, B, MB = _rand(rng, N, N, N - 7, N + 3, K, K)
+    t = [torch.tensor(np.ascontiguousarray(x), device="cuda") for x in (A, MA, B, MB)]
+    plan = cm.Plan(*A.shape, *B.shape, K, K, getattr(cm, prec))
+    mi = torch.zeros((plan.R, plan.C), dtype=torch.float64, device="cuda")
+    n = torch.zeros((plan.R, plan.C), dtype=torch.int32, device="cuda")
+    plan.compute(*t, mi, n)
+    mi0, n0, same = mi.clone(), n.clone(), []
+    for _ in range(100):
+        mi.fill_(-1.0)
+        plan.compute(*t, mi, n)
+        same.append((mi == mi0).all() & (n == n0).all())
+    assert plan.status()[0] == "OK" and bool(torch.stack(same).all())
+    plan.close()
+    ref = oracle.cmif(A, MA, B, MB, K, K)
+    np.testing.assert_array_equal(n0.cpu().numpy(), ref["n"])
+    assert float(np.abs(mi0.cpu().numpy() - ref["mi"]).max()) <= MI_TOL
+
+
 @pytest.mark.parametrize("shape,K", WIDE[:3], ids=lambda x: "x".join(map(str, x)))
 def test_wide_rows_tmem_auto(cm, shape, K, monkeypatch):
     """CMIF_AUTO at the Tensor-Memory widths: the row kernel's AUTO form (exact
