@@ -378,12 +378,12 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
     bool pending = false;  // a copy issued for this team and not yet waited for
     // work: tasks blockIdx.x + k * gridDim.x of the window's rows; several units (maps, R2
     // rows apart) form one run of tasks, so that the last round of blocks is short once
-    // and not once per unit
-    const int nr = g.r1 - g.r0;
+    // and not once per unit.  One unit is the whole map: a volume's R = Dz R2 rows.
+    const int nr = g.r1 - g.r0, unit_rows = g.units > 1 ? g.R2 : Rout;
     auto advance = [&](int& rr, int& base) {  // task offset rr within its unit, the unit's first row
         while (rr >= g.r1) {
             rr -= nr;
-            base += g.R2;
+            base += unit_rows;
         }
     };
     auto issue = [&](int row_i, int pair_i) {
@@ -394,7 +394,7 @@ k_pair_rows_tm(const __grid_constant__ CUtensorMap ymap, Geom g, Tw<float> tw, d
         }
         pending = true;
     };
-    int rr = g.r0 + (int)blockIdx.x, rbase = 0;  // row of the first unit's window; unit * R2 (multi-unit kernels)
+    int rr = g.r0 + (int)blockIdx.x, rbase = 0;  // row of the first unit's window; unit * unit_rows (multi-unit kernels)
     if (MULTI) advance(rr, rbase);
     if (MULTI ? rbase < g.R : rr < g.r1) {
         if (team < npairs) issue(rbase + rr, team);

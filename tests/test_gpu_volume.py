@@ -133,3 +133,31 @@ def test_volume_auto_every_pair_listed(cm, monkeypatch):
     ref = oracle.cmif3(A, None, B, MB, 3, 3)
     np.testing.assert_array_equal(n, ref["n"])
     assert float(np.abs(mi - ref["mi"]).max()) <= MI_TOL
+
+
+@pytest.mark.parametrize("prec,W", [("AUTO", 200), ("AUTO", 400), ("AUTO", 800), ("AUTO", 1500),
+                                    ("FP32", 400), ("FP32", 700), ("FP32", 1400), ("FP32", 1900)])
+def test_volume_wide_rows(cm, prec, W):
+    """Volumes whose rows (W + 70 shifts) take the Tensor-Memory row kernel: every output row
+    once and nothing behind the maps.  AUTO, and FP32 with an explicit poll limit, run its form
+    that walks several maps per launch; a volume is one map of D_z R_2 rows."""
+    rng = np.random.default_rng(W)
+    A = rng.integers(0, 3, (2, 3, W)).astype(np.int32)
+    A[:, :2, : W // 3] = 1
+    B = rng.integers(0, 4, (3, 2, 71)).astype(np.int32)
+    MB = (rng.random(B.shape) > 0.2).astype(np.uint8)
+    ref = oracle.cmif3(A, None, B, MB, 3, 4)
+    R, C = ref["n"].shape
+    for polls in (0, 1 << 24) if prec == "FP32" else (0,):
+        plan = cm.VolumePlan(*A.shape, *B.shape, 3, 4, getattr(cm, prec))
+        assert (plan.R, plan.C) == (R, C)
+        mi = torch.full((4 * R, C), -7.0, dtype=torch.float64, device="cuda:0")  # 3 R guard rows
+        n = torch.full((4 * R, C), -7, dtype=torch.int32, device="cuda:0")
+        plan.set_wait_test(polls, -1)
+        plan.compute(_dev(A), None, _dev(B), _dev(MB), mi, n, None, 0.5)
+        st = plan.status()
+        plan.close()
+        assert st[0] == "OK", st
+        assert bool((mi[R:] == -7.0).all()) and bool((n[R:] == -7).all())
+        np.testing.assert_array_equal(n[:R].cpu().numpy(), ref["n"])
+        assert float(np.abs(mi[:R].cpu().numpy() - ref["mi"]).max()) <= MI_TOL
