@@ -132,6 +132,7 @@ namespace {
 
 cmif_status from_cuda(cudaError_t e) {
     if (e == cudaSuccess) return CMIF_OK;
+    cudaGetLastError();  // reported here: the next call's launch checks do not see it again
     if (e == cudaErrorMemoryAllocation) return CMIF_ERR_OOM;
     return CMIF_ERR_CUDA;
 }

@@ -80,6 +80,7 @@ __global__ void k_status_code(const DevStatus* st, int32_t* out) {
 
 cmif_status to_status(cudaError_t e) {
     if (e == cudaSuccess) return CMIF_OK;
+    cudaGetLastError();  // reported here: the next call's launch checks do not see it again
     return CMIF_ERR_CUDA;
 }
 

@@ -14,6 +14,9 @@ namespace cmif {
 template <typename T, int SZ>
 constexpr bool kHasColVariant = std::is_same<T, float>::value && SZ >= 1024 && is_pow2(SZ);
 
+// Shared memory of an SM (each block takes 1 KB more than it asks for) and the most one block may have.
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemPerBlock = 227 * 1024;
+
 // Opt the kernel in to `bytes` of dynamic shared memory.  Without the attribute,
 // static plus dynamic shared memory must stay within 48 KB, so a kernel with a
 // little static memory (a work index, an abort flag) fails to launch just below
@@ -56,7 +59,7 @@ static cudaError_t launch_fwd_cols(const cpx<T>* T1, int H, int K, int Qh, int Q
             if (e != cudaSuccess) return e;
             by_regs = n > 0 ? n : 1;
         }
-        const int by_smem = (int)(228 * 1024 / (C::smem(H) + 1024));
+        const int by_smem = (int)(kSmemPerSm / (C::smem(H) + 1024));
         slots = (long long)std::max(1, std::min(by_regs, by_smem)) * num_sms;
     }
     kern<<<(int)std::min(items, slots), C::THREADS, C::smem(H), s>>>(T1, H, K, Qh, Qs, F, tw, st, conditional, out_scale, need, slices);
@@ -158,10 +161,15 @@ static cudaError_t launch_pair_rows_v(const Geom& g, const PipeArgs<T>& a, cudaS
     if (a.cb_smem) {
         auto kern = k_pair_rows<T, Q, true, NMI>;
         // A map of few rows: a cluster of blocks per row, as many as the labels and the
-        // resident blocks allow (64^2, K = 8, 127 rows: 1 block per row 16.5 us)
+        // resident blocks allow (64^2, K = 8, 127 rows: 1 block per row 16.5 us).  The blocks
+        // of a cluster also hold a row of partial sums: where those do not fit (or leave fewer
+        // blocks per SM), one block (or fewer) per row, as without.
         const int ntask = g.units * (g.r1 - g.r0);
+        const size_t smem_split = (smem + 15) / 16 * 16 + Q * (sizeof(EntAcc<NMI>) + sizeof(int));
+        const long long fit = smem_split <= kSmemPerBlock ? (long long)(kSmemPerSm / (smem_split + 1024)) * a.num_sms : 0;
+        const long long cap = std::min<long long>(a.rows_cap, fit);
         int split = 1;
-        while (split < 8 && 2 * split <= g.KA && (long long)ntask * 2 * split <= a.rows_cap) split *= 2;
+        while (split < 8 && 2 * split <= g.KA && (long long)ntask * 2 * split <= cap) split *= 2;
         if (split == 1) {
             cudaError_t e = ensure_smem(kern, smem);
             if (e != cudaSuccess) return e;
@@ -169,7 +177,7 @@ static cudaError_t launch_pair_rows_v(const Geom& g, const PipeArgs<T>& a, cudaS
                                                        a.prec_slot, a.conditional, a.ov, a.ov_slot, a.pair_res, 1);
             return cudaGetLastError();
         }
-        smem = (smem + 15) / 16 * 16 + Q * (sizeof(EntAcc<NMI>) + sizeof(int));
+        smem = smem_split;
         cudaError_t e = ensure_smem(kern, smem);
         if (e != cudaSuccess) return e;
         cudaLaunchAttribute attr[1];

@@ -42,7 +42,7 @@ def _check(got, ref):
 @pytest.mark.parametrize("shape,K,prec", [
     ((150, 200), 8, "FP32"),     # TMEM row kernel (Q = 512)
     ((96, 520), 8, "FP32"),      # TMEM row kernel (Q = 2048)
-    ((40, 1100), 6, "FP32"),     # generic FP32 row kernel (Q = 3072)
+    ((40, 1100), 6, "FP32"),     # TMEM row kernel, teams of three warps (Q = 3072)
     ((70, 66), 6, "FP64"),
     ((70, 66), 6, "SPLIT32"),
 ])
@@ -82,3 +82,48 @@ def test_nmi_single256_full_map(cm):
     assert plan.status()[0] == "OK"
     _check(m.cpu().numpy(), oracle.nmi(A, MA, B, MB, 16, 16))
     plan.close()
+
+
+@pytest.mark.parametrize("W,KB", [(1100, 8), (1100, 7), (1100, 6), (1100, 5), (700, 17), (700, 16)])
+def test_few_rows_near_the_shared_memory_limit(cm, W, KB):
+    """Maps of few, wide rows with count maps (generic row kernel, Q = 3072 and 1536): a cluster
+    of blocks per row where its partial sums fit beside the B-marginals (MI: up to 7 labels at
+    3072; NMI: up to 5, and up to 16 at 1536), else one block per row.  MI, NMI, N and every
+    count against the oracle."""
+    rng = np.random.default_rng(W + KB)
+    A = rng.integers(0, 4, (30, W)).astype(np.int32)
+    B = rng.integers(0, KB, (30, W - 3)).astype(np.int32)
+    MB = (rng.random(B.shape) > 0.1).astype(np.uint8)
+    ref = oracle.cmif(A, None, B, MB, 4, KB, counts=True, marginals=True)
+    R, C = ref["mi"].shape
+    for nmi in (False, True):
+        plan = cm.Plan(*A.shape, *B.shape, 4, KB, cm.FP32, nmi=nmi, debug_counts=True)
+        m = torch.empty((R, C), dtype=torch.float64, device="cuda:0")
+        n = torch.empty((R, C), dtype=torch.int32, device="cuda:0")
+        counts = torch.empty((4 * KB + 4 + KB, R, C), dtype=torch.int32, device="cuda:0")
+        plan.compute(_dev(A), None, _dev(B), _dev(MB), m, n, counts)
+        assert plan.status()[0] == "OK"
+        plan.close()
+        assert np.array_equal(n.cpu().numpy(), ref["n"])
+        got = counts.cpu().numpy()
+        assert np.array_equal(got, np.concatenate([ref["joint"], ref["marg_a"], ref["marg_b"]]))
+        if nmi:
+            _check(m.cpu().numpy(), oracle.nmi(A, None, B, MB, 4, KB))
+        else:
+            assert float(np.abs(m.cpu().numpy() - ref["mi"]).max()) <= MI_TOL
+
+
+@pytest.mark.parametrize("prec", ["FP64", "SPLIT32"])
+def test_few_rows_exact_nmi(cm, prec):
+    """The same limit of the exact plans: NMI at Q = 2048 with one label b, whose row takes
+    200 KB without a cluster's partial sums."""
+    rng = np.random.default_rng(9)
+    A = rng.integers(0, 3, (20, 620)).astype(np.int32)
+    B = np.zeros((25, 600), np.int32)
+    MB = (rng.random(B.shape) > 0.3).astype(np.uint8)
+    plan = cm.Plan(*A.shape, *B.shape, 3, 1, getattr(cm, prec), nmi=True)
+    m = torch.empty((plan.R, plan.C), dtype=torch.float64, device="cuda:0")
+    plan.compute(_dev(A), None, _dev(B), _dev(MB), m)
+    assert plan.status()[0] == "OK"
+    plan.close()
+    _check(m.cpu().numpy(), oracle.nmi(A, None, B, MB, 3, 1))
