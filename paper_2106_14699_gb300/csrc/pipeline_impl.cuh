@@ -162,14 +162,14 @@ static cudaError_t launch_pair_rows_v(const Geom& g, const PipeArgs<T>& a, cudaS
         auto kern = k_pair_rows<T, Q, true, NMI>;
         // A map of few rows: a cluster of blocks per row, as many as the labels and the
         // resident blocks allow (64^2, K = 8, 127 rows: 1 block per row 16.5 us).  The blocks
-        // of a cluster also hold a row of partial sums: where those do not fit (or leave fewer
-        // blocks per SM), one block (or fewer) per row, as without.
+        // of a cluster also hold a row of partial sums: where those do not fit, one block per
+        // row.  (Where they leave fewer blocks per SM the split stays: 37 rows of 32 x 32
+        // labels at Q = 512, exact, 8 blocks per row 164 us, 4 190 us.)
         const int ntask = g.units * (g.r1 - g.r0);
         const size_t smem_split = (smem + 15) / 16 * 16 + Q * (sizeof(EntAcc<NMI>) + sizeof(int));
-        const long long fit = smem_split <= kSmemPerBlock ? (long long)(kSmemPerSm / (smem_split + 1024)) * a.num_sms : 0;
-        const long long cap = std::min<long long>(a.rows_cap, fit);
         int split = 1;
-        while (split < 8 && 2 * split <= g.KA && (long long)ntask * 2 * split <= cap) split *= 2;
+        if (smem_split <= kSmemPerBlock)
+            while (split < 8 && 2 * split <= g.KA && (long long)ntask * 2 * split <= a.rows_cap) split *= 2;
         if (split == 1) {
             cudaError_t e = ensure_smem(kern, smem);
             if (e != cudaSuccess) return e;

@@ -10,6 +10,7 @@ import pytest
 
 import oracle
 import synth
+from tolerances import MI_TOL
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
