@@ -730,7 +730,7 @@ cmif_status align_core_units(cmif_plan plan, const Geom& g, const int32_t* A, co
                              void* topk_dev, double* mi_maps, int32_t* n_maps, cudaStream_t s) {
     const size_t RC = (size_t)g.R * g.C;
     PeakRec* peaks = reinterpret_cast<PeakRec*>(plan->peaks);
-    cudaError_t e = cudaMemsetAsync(plan->st_total, 0, sizeof(DevStatus), s);
+    cudaError_t e = reset_status(plan, true, s);  // A's transforms and the first chunk share a status word
     if (e != cudaSuccess) return from_cuda(e);
     PipeArgs<float> a = plan->w32.args;
     fill_io(a, A, M_A, nullptr, nullptr, nullptr, nullptr, nullptr, plan->st, plan);
@@ -756,7 +756,7 @@ cmif_status align_core_units(cmif_plan plan, const Geom& g, const int32_t* A, co
         plan->prof.begin("warp_nn", s);
         e = launch_warp_nn_multi(B, M_B, g.HB, g.WB, angles + c0, G, plan->wB, plan->wM, s);
         plan->prof.end(s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(plan->st, 0, sizeof(DevStatus), s);
+        if (e == cudaSuccess && c0 > 0) e = reset_status(plan, false, s);
         if (e != cudaSuccess) return from_cuda(e);
         fill_io(a, A, M_A, plan->wB, plan->wM, mi, nm, nullptr, plan->st, plan);
         a.stages = STAGE_FWD_B | STAGE_PAIRS;

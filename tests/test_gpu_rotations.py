@@ -191,3 +191,32 @@ def test_batched_angles_vs_oracle(cm):
     for (ga, gdy, gdx, gnn, gmi), (ra, ridx, rmi, rn) in zip(got, top):
         assert abs(gmi - rmi) <= MI_TOL
     plan.close()
+
+
+@pytest.mark.parametrize("where", ["A", "B"])
+@pytest.mark.parametrize("batched", [False, True])
+def test_label_out_of_range_over_angles(cm, where, batched, monkeypatch):
+    """One pixel under mask 1 whose label is K: the status of the whole call says so, with one
+    angle or two (of five) per launch and through a batch, and the next call's is OK again.  (B:
+    the pixel stays in the picture at every angle.)"""
+    monkeypatch.setenv("CMIF_ANGLE_BATCH", "2")
+    rng = np.random.default_rng(8)
+    X = {k: rng.integers(0, 5, (40, 44)).astype(np.int32) for k in "AB"}
+    good = {k: _dev(v) for k, v in X.items()}
+    X[where][20, 22] = 5
+    bad = {k: _dev(v) for k, v in X.items()}
+    angles = [0.0, 0.3, 0.9, 2.0, 3.1]
+    plan = cm.Plan(40, 44, 40, 44, 5, 5, cm.FP32, batch_angles=batched)
+    topk = torch.empty(24 * 2, dtype=torch.uint8, device="cuda:0")
+    for x, want in ((bad, "LABEL_RANGE"), (good, "OK"), (bad, "LABEL_RANGE")):
+        plan.align_rotations(x["A"], None, x["B"], None, angles, 0.5, 2, topk)
+        assert plan.status()[0] == want
+    plan.close()
+    pairs = [dict(A=x["A"], M_A=None, B=x["B"], M_B=None, K_A=5, K_B=5, angles=angles, gamma=0.5) for x in (good, bad, good)]
+    batch = cm.Batch(pairs, cm.FP32, batch_angles=batched)
+    res = torch.empty(24 * 3, dtype=torch.uint8, device="cuda:0")
+    stat = torch.full((3,), -1, dtype=torch.int32, device="cuda:0")
+    batch.run(res, stat)
+    torch.cuda.synchronize()
+    assert stat.cpu().tolist() == [0, 2, 0] and batch.status()[0] == "LABEL_RANGE"
+    batch.close()
