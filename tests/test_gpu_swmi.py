@@ -84,3 +84,20 @@ def test_swmi_unit_weights_equal_mi_and_window(cm):
     assert float(np.abs(miw[r0:r1] - ref["mi"][r0:r1]).max()) <= MI_TOL
     assert not miw[:r0].any() and not miw[r1:].any()
     assert (pkw[1], pkw[2]) == (3, -4)
+
+
+@pytest.mark.parametrize("axis", ["rows", "columns"])
+@pytest.mark.parametrize("N", [129, 500, 1000, 1100, 2050, 4096])
+def test_swmi_long_transforms(cm, axis, N):
+    """Every weighted transform length from 256 to 4096, across rows and down columns."""
+    rng = np.random.default_rng(N)
+    a, b = N - N // 3, N // 3 + 1  # a + b - 1 = N
+    shape_a, shape_b = ((2, a), (3, b)) if axis == "rows" else ((a, 2), (b, 3))
+    A, B = (rng.integers(0, 3, s).astype(np.int32) for s in (shape_a, shape_b))
+    WA = rng.random(shape_a) * (rng.random(shape_a) > 0.1)
+    WB = rng.gamma(2.0, 1.0, shape_b)
+    mi, nw, pk, st = _run(cm, A, WA, B, WB, 3, 3, 0.4)
+    assert st[0] == "OK", st
+    ref = oracle.swmi(A, WA, B, WB, 3, 3)
+    assert float(np.abs(mi - ref["mi"]).max()) <= MI_TOL
+    assert np.allclose(nw, ref["nw"], rtol=1e-9, atol=1e-9)

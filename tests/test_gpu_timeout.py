@@ -57,3 +57,26 @@ def test_row_kernel_wait_times_out_then_recovers(cm):
     np.testing.assert_array_equal(got_n[dys + H - 1, dxs + W - 1], ref["n"])
     assert np.abs(got_mi[dys + H - 1, dxs + W - 1] - ref["mi"]).max() <= MI_TOL
     plan.close()
+
+
+@pytest.mark.parametrize("W", [1400, 2000])
+def test_wait_of_a_team_of_warps_times_out_then_recovers(cm, W):
+    """The same at the widths 3072 and 4096, where several warps wait for a row's copy."""
+    rng = np.random.default_rng(W)
+    A = rng.integers(0, 4, (30, W)).astype(np.int32)
+    B = rng.integers(0, 4, (20, W + 9)).astype(np.int32)
+    dA, dB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    plan = cm.Plan(*A.shape, *B.shape, 4, 4, cm.FP32)
+    mi = torch.zeros((plan.R, plan.C), dtype=torch.float64, device="cuda:0")
+    n = torch.zeros((plan.R, plan.C), dtype=torch.int32, device="cuda:0")
+    plan.set_wait_test(1 << 12, 20)
+    plan.compute(dA, None, dB, None, mi, n, None, 0.5)
+    assert plan.status()[0] == "TIMEOUT"
+    assert int(n[20].abs().sum()) == 0
+    plan.set_wait_test(0, -1)
+    plan.compute(dA, None, dB, None, mi, n, None, 0.5)
+    assert plan.status()[0] == "OK"
+    plan.close()
+    ref = oracle.cmif(A, None, B, None, 4, 4)
+    np.testing.assert_array_equal(n.cpu().numpy(), ref["n"])
+    assert float(np.abs(mi.cpu().numpy() - ref["mi"]).max()) <= MI_TOL

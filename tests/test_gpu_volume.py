@@ -161,3 +161,21 @@ def test_volume_wide_rows(cm, prec, W):
         assert bool((mi[R:] == -7.0).all()) and bool((n[R:] == -7).all())
         np.testing.assert_array_equal(n[:R].cpu().numpy(), ref["n"])
         assert float(np.abs(mi[:R].cpu().numpy() - ref["mi"]).max()) <= MI_TOL
+
+
+@pytest.mark.parametrize("HA,HB", [(70, 50), (100, 80), (130, 120), (190, 150), (300, 140), (400, 201), (700, 301)])
+def test_volume_tall(cm, HA, HB):
+    """Column lengths 128, 192, 256, 384, 512, 768 and 1024 of a volume (an item sums four, four,
+    two, four, two, two and one depth offsets), six depth offsets, which four does not divide;
+    FP32 and, at the power of two, the exact transforms."""
+    rng = np.random.default_rng(HA)
+    A = rng.integers(0, 3, (3, HA, 4)).astype(np.int32)
+    A[:, : HA // 2] = 1
+    B = rng.integers(0, 3, (4, HB, 3)).astype(np.int32)
+    MB = (rng.random(B.shape) > 0.2).astype(np.uint8)
+    ref = oracle.cmif3(A, None, B, MB, 3, 3)
+    for prec in (cm.FP32, cm.FP64):
+        mi, n, pk, st = _run(cm, A, None, B, MB, 3, prec)
+        assert st[0] == "OK", st
+        np.testing.assert_array_equal(n, ref["n"])
+        assert float(np.abs(mi - ref["mi"]).max()) <= MI_TOL
