@@ -23,8 +23,6 @@ namespace {
 
 template <typename T>
 struct Workspace {
-    void* base = nullptr;
-    size_t bytes = 0;
     PipeArgs<T> args{};  // pointer part filled at create time
     int rows_grid = 0;
     bool cb_smem = true;
@@ -238,20 +236,6 @@ void carve_workspace(const Geom& g, Workspace<T>& w, char* base) {
         w.args.cbw = (double*)(base + off); off = align_up(off + (size_t)w.rows_grid_w * g.KB * g.Q * sizeof(double), 256);
         w.args.nw = (double*)(base + off);
     }
-}
-
-template <typename T>
-cmif_status alloc_workspace(cmif_plan p, Workspace<T>& w) {
-    cmif_status st = choose_rows<T>(p, w);
-    if (st != CMIF_OK) return st;
-    const size_t bytes = workspace_bytes<T>(p->g, w);
-    void* base = nullptr;
-    cudaError_t e = cudaMalloc(&base, bytes);
-    if (e != cudaSuccess) { cudaGetLastError(); return CMIF_ERR_OOM; }
-    w.base = base;
-    w.bytes = bytes;
-    carve_workspace<T>(p->g, w, (char*)base);
-    return CMIF_OK;
 }
 
 void free_plan(cmif_plan p) {
@@ -670,9 +654,6 @@ cmif_status plan_carve(cmif_plan p, char* base) {
     if (p->has_m31) carve_workspace<m31>(g, p->wm31, base + off);
     off += exact_bytes(p);
     if (p->prec == CMIF_AUTO) { esc_carve(p, base + off); off += p->esc.bytes; }
-    p->w32.bytes = p->has32 ? workspace_bytes<float>(p->gcap, p->w32) : 0;
-    p->w64.bytes = p->has64 ? workspace_bytes<double>(g, p->w64) : 0;
-    p->wm31.bytes = p->has_m31 ? workspace_bytes<m31>(g, p->wm31) : 0;
     if (cudaMemset(p->st, 0, 2 * align_up(sizeof(DevStatus), 256)) != cudaSuccess) return CMIF_ERR_CUDA;
     return CMIF_OK;
 }

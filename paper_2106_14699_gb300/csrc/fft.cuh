@@ -352,7 +352,7 @@ __device__ __forceinline__ void team_core_pk(float2 (&re)[M / 2], float2 (&im)[M
     dft_pk<M, DIR>(re, im);
 }
 
-template <int M, int DIR, bool WIDE = false, typename T>
+template <int M, int DIR, typename T>
 __device__ __forceinline__ void team_fft_core(cpx<T> (&v)[M], int j, void* sm, const cpx<T>* __restrict__ twq) {
     if constexpr (std::is_same<T, float>::value && M >= 8) {
         constexpr int H = M / 2;
@@ -362,7 +362,7 @@ __device__ __forceinline__ void team_fft_core(cpx<T> (&v)[M], int j, void* sm, c
             re[m] = make_float2(v[2 * m].x, v[2 * m + 1].x);
             im[m] = make_float2(v[2 * m].y, v[2 * m + 1].y);
         }
-        team_core_pk<M, DIR, WIDE>(re, im, j, reinterpret_cast<float*>(sm), reinterpret_cast<const float4*>(twq));
+        team_core_pk<M, DIR, false>(re, im, j, reinterpret_cast<float*>(sm), reinterpret_cast<const float4*>(twq));
 #pragma unroll
         for (int k = 0; k < H; ++k) {
             v[brev(k, M)] = {re[k].x, im[k].x};

@@ -69,10 +69,6 @@ __device__ __forceinline__ void clog2c_biased2(float2 c, long long& t0, long lon
     t1 = (long long)(__float_as_int(b.y) - 0x4B000000) * (long long)(x1 - m1 + __float_as_int(t.y));
 }
 
-// Nearest integer of |v| < 2^22 with two FP32 adds (the 1.5 * 2^23 shift
-// leaves no fraction bits).
-__device__ __forceinline__ float round_fp32(float v) { return (v + 12582912.0f) - 12582912.0f; }
-
 // (q1 + q2) * 2^-kFixBits as a double, |q2| at most a few ulp of q1 (so the sum of the two
 // 24-bit values fits 53 bits), by integer arithmetic: the same value that the double add
 // gives, but FP64 instructions run at 1/64 rate and the two conversions, the add and the
@@ -146,21 +142,15 @@ __device__ __forceinline__ void atomic_max_float_pos(unsigned* addr, float v) {
     atomicMax(addr, __float_as_uint(v));  // v >= 0: float order = unsigned order
 }
 
-template <typename T>
-__device__ __forceinline__ T rint_t(T v);
-template <>
-__device__ __forceinline__ float rint_t<float>(float v) { return rintf(v); }
-template <>
-__device__ __forceinline__ double rint_t<double>(double v) { return rint(v); }
 // A pre-rounding count -> the count as a float, and its residual; modular counts are exact.
 template <typename T>
 __device__ __forceinline__ float round_count(T v, float& res) {
     if constexpr (std::is_same<T, m31>::value) {
         return m31_count(v);
     } else {
-        const T c = rint_t<T>(v);
-        res = fmaxf(res, (float)fabs(v - c));
-        return (float)c;
+        const float c = rintf(v);
+        res = fmaxf(res, fabsf(v - c));
+        return c;
     }
 }
 
@@ -1022,42 +1012,42 @@ constexpr size_t pair_cols_smem() {
 // accumulates, pair by pair, the joint term T(c), the running A-marginal of
 // the current label a, and the B-marginal C_B^b(p) (shared or global memory).
 // The rounded counts reach the owners through the teams' scratch, in HALVES
-// passes (two for 4-byte values, whose scratch holds half a row).
+// passes: the scratch holds half a row.
 // split > 1 (maps with too few rows to fill the GPU, B-marginals in shared memory): a cluster
 // of split blocks takes a row, each the pairs of its own labels a; at the end of the row the
 // blocks read each other's partial sums and B-marginals (distributed shared memory) and each
 // finishes its share of the positions.
 template <typename T, int Q>
 struct RowCfg {
+    static_assert(sizeof(T) == 4, "FP32 values or residues (weighted maps: RowWCfg)");
     static constexpr int L = Q / 2;
     using G = TeamGeom<T, L>;
     static constexpr int M = G::M, R = G::R, TEAM = G::TEAM;
-    // FP32: one thread per position of a pass (Q / 2), between one warp and 512
+    // one thread per position of a pass (Q / 2), between one warp and 512
     // threads, so that no thread idles in the epilogue; smaller blocks share an SM.
-    static constexpr int BT_TARGET = sizeof(T) == 4 ? (Q / 2 >= 512 ? 512 : (Q / 2 >= 32 ? Q / 2 : 32)) : 256;
-    // FP32: as many teams as the target allows, fewer when that lets the threads divide
+    static constexpr int BT_TARGET = Q / 2 >= 512 ? 512 : (Q / 2 >= 32 ? Q / 2 : 32);
+    // as many teams as the target allows, fewer when that lets the threads divide
     // a pass's positions exactly (no idle lanes in the epilogue) at no more than a
     // quarter fewer teams (3072: 4 teams of 96 lanes, 1536: 8 of 48)
     static constexpr int NT0 = TEAM >= BT_TARGET ? 1 : BT_TARGET / TEAM;
     static constexpr int nt_exact(int nt) {
-        return nt <= 1 ? 1 : ((Q / (sizeof(T) == 4 ? 2 : 1)) % (nt * TEAM) == 0 ? nt : nt_exact(nt - 1));
+        return nt <= 1 ? 1 : ((Q / 2) % (nt * TEAM) == 0 ? nt : nt_exact(nt - 1));
     }
-    static constexpr int NT = (sizeof(T) == 4 && nt_exact(NT0) * 4 >= NT0 * 3) ? nt_exact(NT0) : NT0;
+    static constexpr int NT = nt_exact(NT0) * 4 >= NT0 * 3 ? nt_exact(NT0) : NT0;
     static constexpr int THREADS = NT * TEAM;
-    static constexpr int HALVES = sizeof(T) == 4 ? 2 : 1;
+    static constexpr int HALVES = 2;
     static constexpr int QH = Q / HALVES;                      // positions per pass
     static constexpr int UH = (QH + THREADS - 1) / THREADS;    // positions per thread per pass
     static constexpr int U = HALVES * UH;
     static constexpr int REGION = G::SCRATCH;                  // >= QH floats
     static constexpr size_t TEAM_SMEM = (size_t)NT * REGION;
-    // FP32: each team's next Y row (L complex, 16-byte pieces) is copied into a
+    // each team's next Y row (L complex, 16-byte pieces) is copied into a
     // shared-memory buffer by asynchronous copies (cp.async) while the current round
     // computes; the transform then loads its inputs from shared memory
-    static constexpr bool STAGE = sizeof(T) == 4;
-    static constexpr int STAGE_BYTES = STAGE ? L * 8 : 0;
+    static constexpr int STAGE_BYTES = L * 8;
     static constexpr size_t OFF_STAGE = (TEAM_SMEM + 15) / 16 * 16;
     static constexpr size_t OFF_CB = OFF_STAGE + (size_t)NT * STAGE_BYTES;  // B-marginals (shared-memory variant)
-    static constexpr int MIN_BLOCKS = sizeof(T) == 4 && THREADS < 512 ? 512 / THREADS : 1;  // <= 128 registers
+    static constexpr int MIN_BLOCKS = THREADS < 512 ? 512 / THREADS : 1;  // <= 128 registers
     static_assert(REGION >= QH * 4, "team scratch must hold one pass of rounded counts");
 };
 
@@ -1101,25 +1091,21 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
     const int rank = CB_SMEM ? (int)blockIdx.x % split : 0, ntb = (int)gridDim.x / split, task0 = (int)blockIdx.x / split;
     const int alo = rank * KA / split, plo = alo * KB, phi = (rank + 1) * KA / split * KB;  // this block's pairs
     auto task_row = [&](int tk) { return (tk / nr) * g.R2 + g.r0 + tk % nr; };
-    // STAGE: the team's buffer for the Y row of its current pair; the team's lanes
+    // stage: the team's buffer for the Y row of its current pair; the team's lanes
     // copy a row in 16-byte pieces (the rows start on 32-byte boundaries: L is a
     // multiple of 4)
     const cpx<T>* stage = reinterpret_cast<const cpx<T>*>(smem_raw + C::OFF_STAGE + (size_t)team * C::STAGE_BYTES);
     auto stage_issue = [&](int pair_i, int row_i) {
-        if constexpr (C::STAGE) {
-            // half c % 2 of chunk c / 2, whose rows lie 128 bytes apart (layout of Y)
-            const char* src = reinterpret_cast<const char*>(Y + (size_t)pair_i * y_rows<T>(Rout) * L + y_chunk<T>(row_i, 0, L));
-            const uint32_t dst = smem_u32(stage);
-            for (int c = lt; c < C::STAGE_BYTES / 16; c += C::TEAM)
-                cp_async16(dst + 16u * c, src + 128 * (c >> 1) + 16 * (c & 1));
-            cp_async_commit();
-        }
+        // half c % 2 of chunk c / 2, whose rows lie 128 bytes apart (layout of Y)
+        const char* src = reinterpret_cast<const char*>(Y + (size_t)pair_i * y_rows<T>(Rout) * L + y_chunk<T>(row_i, 0, L));
+        const uint32_t dst = smem_u32(stage);
+        for (int c = lt; c < C::STAGE_BYTES / 16; c += C::TEAM)
+            cp_async16(dst + 16u * c, src + 128 * (c >> 1) + 16 * (c & 1));
+        cp_async_commit();
     };
-    if constexpr (C::STAGE) {
-        if (task0 < ntask && plo + team < phi) stage_issue(plo + team, task_row(task0));
-        cp_async_wait_all();
-        __syncthreads();
-    }
+    if (task0 < ntask && plo + team < phi) stage_issue(plo + team, task_row(task0));
+    cp_async_wait_all();
+    __syncthreads();
     for (int task = task0; task < ntask; task += ntb) {
         const int row = task_row(task);
         EntAcc<NMI> S[U];
@@ -1140,23 +1126,10 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
             const int pair = base + team;
             const bool act = pair < phi;
             const int ovs = (act && ov_slot) ? ov_slot[pair] : -1;
-            const cpx<T>* yr = C::STAGE ? stage : Y + ((size_t)(act ? pair : 0) * Rout + row) * L;
-            if (!C::STAGE && lt == 0) {
-                // ask L2 for this team's row of the next round (or of the block's next row)
-                int np = pair + NT, nrow = row;
-                if (np >= phi) {
-                    np = plo + team;
-                    const int nt2 = task + ntb;
-                    nrow = nt2 < ntask ? (nt2 / nr) * g.R2 + g.r0 + nt2 % nr : -1;
-                }
-                if (np < phi && nrow >= 0)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Y + ((size_t)np * Rout + nrow) * L),
-                                 "r"((unsigned)(L * sizeof(cpx<T>))) : "memory");
-            }
             cpx<T> v[M];
             auto transform = [&](auto splitc) {
                 constexpr bool SPLIT = decltype(splitc)::value;
-                auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q, SPLIT>(yr, k) : cpx<T>{T(0), T(0)}; };
+                auto load = [&](int k) -> cpx<T> { return act ? load_z<T, Q, SPLIT>(stage, k) : cpx<T>{T(0), T(0)}; };
                 team_fft<M, R, +1>(v, r, j, load, region + r * grp_scratch_bytes<T, M>(), tw.sq[ilog2c(M)], tw_of<L>(tw));
             };
             // (Geom::split of the other widths: the Tensor-Memory kernel only)
@@ -1179,7 +1152,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
 #pragma unroll
             for (int hf = 0; hf < HALVES; ++hf) {
                 __syncthreads();  // all scratch reads (FFT or previous pass) done
-                if (C::STAGE && hf == 0) {
+                if (hf == 0) {
                     // the staged rows are consumed: copy this team's next row (the next
                     // round of this task, else round 0 of the block's next task)
                     int np = pair + NT, ntk = task;
@@ -1287,7 +1260,7 @@ k_pair_rows(const cpx<T>* __restrict__ Y, Geom g, Tw<T> tw, float* __restrict__ 
                 if (counts) accumulate(std::true_type{});
                 else accumulate(std::false_type{});
             }
-            if constexpr (C::STAGE) cp_async_wait_all();  // the next round's rows, visible after the barrier
+            cp_async_wait_all();  // the next round's rows, visible after the barrier
             __syncthreads();  // the next round's transforms overwrite the scratch read above
         }
         if constexpr (CB_SMEM) {

@@ -3,14 +3,11 @@
 namespace cmif {
 template cudaError_t Sized<float, 192>::pair_rows(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template size_t Sized<float, 192>::rows_smem(int, bool);
-template int Sized<float, 192>::rows_threads();
 template cudaError_t Sized<float, 192>::rows_max_blocks(int, bool, int*);
 template cudaError_t Sized<float, 384>::pair_rows(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template size_t Sized<float, 384>::rows_smem(int, bool);
-template int Sized<float, 384>::rows_threads();
 template cudaError_t Sized<float, 384>::rows_max_blocks(int, bool, int*);
 template cudaError_t Sized<float, 768>::pair_rows(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template size_t Sized<float, 768>::rows_smem(int, bool);
-template int Sized<float, 768>::rows_threads();
 template cudaError_t Sized<float, 768>::rows_max_blocks(int, bool, int*);
 }

@@ -4,6 +4,5 @@ namespace cmif {
 template cudaError_t Sized<m31, 1024>::pair_rows(const Geom&, const PipeArgs<m31>&, cudaStream_t);
 template cudaError_t Sized<m31, 1024>::pair_rows_counts(const Geom&, const PipeArgs<m31>&, cudaStream_t);
 template size_t Sized<m31, 1024>::rows_smem(int, bool);
-template int Sized<m31, 1024>::rows_threads();
 template cudaError_t Sized<m31, 1024>::rows_max_blocks(int, bool, int*);
 }

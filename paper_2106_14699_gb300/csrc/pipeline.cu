@@ -102,17 +102,6 @@ size_t rows_smem_bytes(int Q, int KB, bool cb_smem) {
 }
 
 template <typename T>
-int rows_threads(int Q) {
-    int out = 0;
-    auto f = [&]() -> cudaError_t {
-        CMIF_SIZE_SWITCH_T(T, Q, out = Sized<T, SZ>::rows_threads());
-        return cudaSuccess;
-    };
-    f();
-    return out;
-}
-
-template <typename T>
 cudaError_t rows_max_blocks_per_sm(int Q, int KB, bool cb_smem, int* out) {
     CMIF_SIZE_SWITCH_T(T, Q, return Sized<T, SZ>::rows_max_blocks(KB, cb_smem, out));
     return cudaSuccess;
@@ -144,7 +133,6 @@ template cudaError_t run_pipeline<double>(const Geom&, const PipeArgs<double>&, 
 #define CMIF_INSTANTIATE(T)                                                             \
     template cudaError_t run_pipeline<T>(const Geom&, const PipeArgs<T>&, cudaStream_t); \
     template size_t rows_smem_bytes<T>(int, int, bool);                                  \
-    template int rows_threads<T>(int);                                                   \
     template cudaError_t rows_max_blocks_per_sm<T>(int, int, bool, int*);
 CMIF_INSTANTIATE(float)
 CMIF_INSTANTIATE(m31)

@@ -133,7 +133,6 @@ struct Sized {
     static cudaError_t pair_rows(const Geom& g, const PipeArgs<T>& a, cudaStream_t s);              // Q = SZ
     static cudaError_t pair_rows_counts(const Geom& g, const PipeArgs<T>& a, cudaStream_t s);       // Q = SZ, list mode
     static size_t rows_smem(int KB, bool cb_smem);
-    static int rows_threads();
     static cudaError_t rows_max_blocks(int KB, bool cb_smem, int* out);
     static int tm_cols(int KA, int KB);         // 0 unless the TMEM row kernel applies (FP32, tm_rows(Q))
     static cudaError_t tm_max_blocks(int tm_cols, int npairs, int* out);
@@ -157,8 +156,6 @@ cudaError_t make_row_map(CUtensorMap* map, const cpx<float>* Y, int L, int Rout,
 // Per-precision facts the host needs at plan time.
 template <typename T>
 size_t rows_smem_bytes(int Q, int KB, bool cb_smem);
-template <typename T>
-int rows_threads(int Q);
 template <typename T>
 cudaError_t rows_max_blocks_per_sm(int Q, int KB, bool cb_smem, int* out);
 // TMEM columns the TMEM / TMA row kernel needs for (Q, min(K_A, K_B)), or 0 when it does not apply.

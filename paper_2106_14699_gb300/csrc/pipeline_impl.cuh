@@ -281,11 +281,6 @@ size_t Sized<T, SZ>::rows_smem(int KB, bool cb_smem) {
 }
 
 template <typename T, int SZ>
-int Sized<T, SZ>::rows_threads() {
-    return RowCfg<T, SZ>::THREADS;
-}
-
-template <typename T, int SZ>
 cudaError_t Sized<T, SZ>::rows_max_blocks(int KB, bool cb_smem, int* out) {
     const size_t smem = pair_rows_smem<T, SZ>(KB, cb_smem);
     if (cb_smem) {
