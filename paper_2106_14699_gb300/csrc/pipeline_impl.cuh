@@ -5,6 +5,7 @@
 #include "pipeline.cuh"
 #include "rows_tm.cuh"
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <type_traits>
 
@@ -25,6 +26,18 @@ template <typename K>
 static cudaError_t ensure_smem(K kernel, size_t bytes) {
     if (bytes <= 32 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// Blocks of a kernel that share an SM, asked for once (any host thread; all find the same number).
+template <typename K>
+static cudaError_t blocks_per_sm(std::atomic<int>& known, K kernel, int threads, size_t smem, int* out) {
+    *out = known.load(std::memory_order_relaxed);
+    if (*out > 0) return cudaSuccess;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel, threads, smem);
+    if (e != cudaSuccess) return e;
+    *out = std::max(1, *out);
+    known.store(*out, std::memory_order_relaxed);
+    return cudaSuccess;
 }
 
 template <typename T, int Q>
@@ -52,13 +65,10 @@ static cudaError_t launch_fwd_cols(const cpx<T>* T1, int H, int K, int Qh, int Q
     const long long items = (long long)((Qh + C::TPB - 1) / C::TPB) * K;
     long long slots = items;
     if (C::PIPE && num_sms > 0) {  // persistent: every resident block slot
-        static int by_regs = -1;
-        if (by_regs < 0) {
-            int n = 0;
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, C::THREADS, 0);
-            if (e != cudaSuccess) return e;
-            by_regs = n > 0 ? n : 1;
-        }
+        static std::atomic<int> known{0};
+        int by_regs = 0;
+        e = blocks_per_sm(known, kern, C::THREADS, 0, &by_regs);
+        if (e != cudaSuccess) return e;
         const int by_smem = (int)(kSmemPerSm / (C::smem(H) + 1024));
         slots = (long long)std::max(1, std::min(by_regs, by_smem)) * num_sms;
     }
@@ -80,13 +90,10 @@ static cudaError_t launch_pair_cols(const Geom& g, const PipeArgs<T>& a, cudaStr
     cudaError_t e = ensure_smem(kern, smem);
     if (e != cudaSuccess) return e;
     // persistent grid: every resident block slot of the device, at most one per item
-    static int per_sm = -1;
-    if (per_sm < 0) {
-        int n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, C::THREADS, smem);
-        if (e != cudaSuccess) return e;
-        per_sm = n > 0 ? n : 1;
-    }
+    static std::atomic<int> known{0};
+    int per_sm = 0;
+    e = blocks_per_sm(known, kern, C::THREADS, smem, &per_sm);
+    if (e != cudaSuccess) return e;
     const long long np = a.plist ? a.chunk_cap : (long long)g.KA * g.KB;  // list mode: at most chunk_cap pairs
     const long long items = np * ((g.Ys + C::TPB - 1) / C::TPB) * (VOL ? (g.Dz + C::NDZ - 1) / C::NDZ : g.units);
     const int bps = a.cols_bps > 0 && a.cols_bps < per_sm ? a.cols_bps : per_sm;

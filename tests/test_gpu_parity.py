@@ -560,3 +560,34 @@ def test_mixed_radix_equals_power_of_two(cm, monkeypatch):
     ref = oracle.cmif_at(A, None, B, None, K, K, dys, dxs)
     np.testing.assert_array_equal(outs[0]["n"][dys + H - 1, dxs + H - 1], ref["n"])
     assert float(np.abs(outs[0]["mi"][dys + H - 1, dxs + H - 1] - ref["mi"]).max()) <= MI_TOL
+
+
+def test_plans_on_several_threads(cm):
+    """Host threads that make the first launches of some column lengths at the same time, each
+    with its own plan and stream: every map is the one the plan gives alone."""
+    import threading
+    sizes = [(20, 30), (45, 60), (70, 90), (120, 100)]
+    rng = np.random.default_rng(4)
+    jobs = []
+    for H, W in sizes:
+        t = [torch.tensor(rng.integers(0, 6, (H, W)).astype(np.int32), device="cuda") for _ in range(2)]
+        jobs += [(t, prec, torch.cuda.Stream(), []) for prec in (cm.FP32, cm.FP64)]
+
+    def work(t, prec, stream, out):
+        plan = cm.Plan(*t[0].shape, *t[1].shape, 6, 6, prec)
+        mi = torch.zeros((plan.R, plan.C), dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        for _ in range(5):
+            plan.compute(t[0], None, t[1], None, mi, stream=stream.cuda_stream)
+        assert plan.status()[0] == "OK"
+        out.append(mi.cpu().numpy())
+        plan.close()
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    for j in jobs:
+        work(*j)
+        assert len(j[3]) == 2 and np.array_equal(*j[3])
