@@ -151,7 +151,7 @@ cmif_status choose_rows(cmif_plan p, Workspace<T>& w) {
         const int cols = always_split(g.Q) || !(p->flags & CMIF_FLAG_DEBUG_COUNTS)
                              ? rows_tm_cols(g.Q, g.KA, g.KB) : 0;
         if (cols > 0) {
-            e = rows_tm_max_blocks_per_sm(g.Q, cols, g.KA * g.KB, &bps);
+            e = rows_tm_max_blocks_per_sm(g.Q, cols, &bps);
             if (e != cudaSuccess) return from_cuda(e);
             if (bps >= 1) w.args.tm_cols = cols;
         }

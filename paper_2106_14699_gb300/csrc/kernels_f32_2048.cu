@@ -5,5 +5,5 @@ template cudaError_t Sized<float, 2048>::fwd_rows(const Geom&, const PipeArgs<fl
 template cudaError_t Sized<float, 2048>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 2048>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template int Sized<float, 2048>::tm_cols(int, int);
-template cudaError_t Sized<float, 2048>::tm_max_blocks(int, int, int*);
+template cudaError_t Sized<float, 2048>::tm_max_blocks(int, int*);
 }

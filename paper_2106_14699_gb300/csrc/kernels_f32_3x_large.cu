@@ -5,10 +5,10 @@ template cudaError_t Sized<float, 1536>::fwd_rows(const Geom&, const PipeArgs<fl
 template cudaError_t Sized<float, 1536>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 1536>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template int Sized<float, 1536>::tm_cols(int, int);
-template cudaError_t Sized<float, 1536>::tm_max_blocks(int, int, int*);
+template cudaError_t Sized<float, 1536>::tm_max_blocks(int, int*);
 template cudaError_t Sized<float, 3072>::fwd_rows(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 3072>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 3072>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template int Sized<float, 3072>::tm_cols(int, int);
-template cudaError_t Sized<float, 3072>::tm_max_blocks(int, int, int*);
+template cudaError_t Sized<float, 3072>::tm_max_blocks(int, int*);
 }

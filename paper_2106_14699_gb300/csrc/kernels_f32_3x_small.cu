@@ -5,15 +5,15 @@ template cudaError_t Sized<float, 192>::fwd_rows(const Geom&, const PipeArgs<flo
 template cudaError_t Sized<float, 192>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 192>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template int Sized<float, 192>::tm_cols(int, int);
-template cudaError_t Sized<float, 192>::tm_max_blocks(int, int, int*);
+template cudaError_t Sized<float, 192>::tm_max_blocks(int, int*);
 template cudaError_t Sized<float, 384>::fwd_rows(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 384>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 384>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template int Sized<float, 384>::tm_cols(int, int);
-template cudaError_t Sized<float, 384>::tm_max_blocks(int, int, int*);
+template cudaError_t Sized<float, 384>::tm_max_blocks(int, int*);
 template cudaError_t Sized<float, 768>::fwd_rows(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 768>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 768>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template int Sized<float, 768>::tm_cols(int, int);
-template cudaError_t Sized<float, 768>::tm_max_blocks(int, int, int*);
+template cudaError_t Sized<float, 768>::tm_max_blocks(int, int*);
 }

@@ -5,5 +5,5 @@ template cudaError_t Sized<float, 512>::fwd_rows(const Geom&, const PipeArgs<flo
 template cudaError_t Sized<float, 512>::fwd_cols(const Geom&, const PipeArgs<float>&, bool, cudaStream_t);
 template cudaError_t Sized<float, 512>::pair_cols(const Geom&, const PipeArgs<float>&, cudaStream_t);
 template int Sized<float, 512>::tm_cols(int, int);
-template cudaError_t Sized<float, 512>::tm_max_blocks(int, int, int*);
+template cudaError_t Sized<float, 512>::tm_max_blocks(int, int*);
 }

@@ -123,9 +123,9 @@ cudaError_t rows_w_max_blocks_per_sm(int Q, int* out) {
     return cudaSuccess;
 }
 
-cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int npairs, int* out) {
+cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int* out) {
     *out = 0;
-    CMIF_SIZE_SWITCH_T(float, Q, return Sized<float, SZ>::tm_max_blocks(tm_cols, npairs, out));
+    CMIF_SIZE_SWITCH_T(float, Q, return Sized<float, SZ>::tm_max_blocks(tm_cols, out));
     return cudaSuccess;
 }
 

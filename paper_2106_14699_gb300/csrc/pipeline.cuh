@@ -135,7 +135,7 @@ struct Sized {
     static size_t rows_smem(int KB, bool cb_smem);
     static cudaError_t rows_max_blocks(int KB, bool cb_smem, int* out);
     static int tm_cols(int KA, int KB);         // 0 unless the TMEM row kernel applies (FP32, tm_rows(Q))
-    static cudaError_t tm_max_blocks(int tm_cols, int npairs, int* out);
+    static cudaError_t tm_max_blocks(int tm_cols, int* out);
     static cudaError_t pair_rows_w(const Geom& g, const PipeArgs<T>& a, cudaStream_t s);  // FP64 only
     static cudaError_t rows_w_max_blocks(int* out);
 };
@@ -160,7 +160,7 @@ template <typename T>
 cudaError_t rows_max_blocks_per_sm(int Q, int KB, bool cb_smem, int* out);
 // TMEM columns the TMEM / TMA row kernel needs for (Q, min(K_A, K_B)), or 0 when it does not apply.
 int rows_tm_cols(int Q, int KA, int KB);
-cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int npairs, int* out);
+cudaError_t rows_tm_max_blocks_per_sm(int Q, int tm_cols, int* out);
 // The weighted (SWMI) row kernel: its occupancy (FP64).
 cudaError_t rows_w_max_blocks_per_sm(int Q, int* out);
 

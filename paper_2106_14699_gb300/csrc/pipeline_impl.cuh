@@ -113,13 +113,18 @@ static cudaError_t launch_pair_cols(const Geom& g, const PipeArgs<T>& a, cudaStr
     return cudaGetLastError();
 }
 
-// Teams per block of the Tensor-Memory row kernel (rows_tm.cuh).  One-warp teams: blocks of 8
-// where two of them share an SM, except long runs of pairs at Q = 2048 (16: 64 pairs 0.410 vs
-// 0.412 ms, 256 pairs 1.49 vs 1.50 ms; a few pairs leave most of 16 teams idle).
-static int rows_tm_teams(int Q, int tm_cols, int npairs) {
-    if (Q == 4096) return 8;
-    if (Q % 3 == 0) return 4;
-    return tm_cols > 256 || (Q == 2048 && npairs > 32) ? 16 : 8;
+// Teams per block of the one-warp Tensor-Memory row kernel (rows_tm.cuh): blocks of 8 where two
+// of them share an SM.  At Q = 2048 a block of 16 is the better one for more than 32 pairs when
+// every row has an SM of its own, and the slower one beyond.  Time with 16 over time with 8, MI,
+// outputs of 151 rows / 155 rows / 999 rows: 7 x 7 labels 0.97 / 1.18 / 1.27, 8 x 8 0.86 / 1.03 /
+// 1.08, 11 x 11 0.90 / 1.09 / 1.14, 16 x 16 0.85 / 1.01 / 1.04 (2047 rows 1.01: 1.524 against
+// 1.509 ms); AUTO and several angles per launch alike.  NMI, whose blocks of 8 spill, has no such
+// line (151 / 999 rows: 8 x 8 0.84 / 1.06, 16 x 16 0.79 / 1.00) and takes 16 beyond 32 pairs.
+template <int Q, bool NMI>
+static int rows_tm_teams(const Geom& g, const PipeArgs<float>& a) {
+    const int rows = g.units * (g.r1 - g.r0);
+    if (a.tm_cols > 256) return 16;
+    return Q == 2048 && g.KA * g.KB > 32 && (NMI || rows <= a.num_sms) ? 16 : 8;
 }
 
 template <int Q, bool NMI, int MODE, int NT>
@@ -132,11 +137,12 @@ static cudaError_t launch_rows_tm(const Geom& g, const PipeArgs<float>& a, cudaS
     CUtensorMap ymap;
     e = make_row_map(&ymap, a.Y, C::L, g.R, g.KA * g.KB);
     if (e != cudaSuccess) return e;
-    kern<<<a.rows_grid, C::THREADS, C::SMEM, s>>>(ymap, g, a.tw, a.mi, a.n, a.st, a.tm_cols,
-                                                  ext && a.wait_polls > 0 ? a.wait_polls : kDefaultWaitPolls,
-                                                  ext ? a.withhold_row : -1, ext ? a.conditional : 0,
-                                                  ext ? a.ov : nullptr, ext ? a.ov_slot : nullptr,
-                                                  ext ? a.pair_res : nullptr);
+    const int grid = std::min(a.rows_grid, C::BLOCKS * a.num_sms);
+    kern<<<grid, C::THREADS, C::SMEM, s>>>(ymap, g, a.tw, a.mi, a.n, a.st, a.tm_cols,
+                                           ext && a.wait_polls > 0 ? a.wait_polls : kDefaultWaitPolls,
+                                           ext ? a.withhold_row : -1, ext ? a.conditional : 0,
+                                           ext ? a.ov : nullptr, ext ? a.ov_slot : nullptr,
+                                           ext ? a.pair_res : nullptr);
     return cudaGetLastError();
 }
 
@@ -147,8 +153,8 @@ static cudaError_t launch_rows_tm_mode(const Geom& g, const PipeArgs<float>& a, 
     } else if constexpr (Q % 3 == 0) {
         return launch_rows_tm<Q, NMI, MODE, 4>(g, a, s);
     } else {
-        return rows_tm_teams(Q, a.tm_cols, g.KA * g.KB) == 8 ? launch_rows_tm<Q, NMI, MODE, 8>(g, a, s)
-                                                             : launch_rows_tm<Q, NMI, MODE, 16>(g, a, s);
+        return rows_tm_teams<Q, NMI>(g, a) == 8 ? launch_rows_tm<Q, NMI, MODE, 8>(g, a, s)
+                                                : launch_rows_tm<Q, NMI, MODE, 16>(g, a, s);
     }
 }
 
@@ -336,19 +342,17 @@ int Sized<T, SZ>::tm_cols(int KA, int KB) {
 }
 
 template <typename T, int SZ>
-cudaError_t Sized<T, SZ>::tm_max_blocks(int tm_cols, int npairs, int* out) {
+cudaError_t Sized<T, SZ>::tm_max_blocks(int tm_cols, int* out) {
     *out = 0;
     if constexpr (std::is_same<T, float>::value && tm_rows(SZ)) {
         // The blocks that share an SM: as many as the kernel is bounded for (registers; shared
         // memory is less than that), within the SM's 512 TMEM columns.  (The occupancy query
         // answers 1 for a kernel that allocates Tensor Memory.)
         constexpr int NT = SZ % 3 == 0 ? 4 : 8;
-        const int blocks = rows_tm_teams(SZ, tm_cols, npairs) == 16 ? 1 : RowTmCfg<SZ, NT>::BLOCKS;
-        *out = std::min(blocks, 512 / tm_cols);
+        *out = std::min(RowTmCfg<SZ, NT>::BLOCKS, 512 / tm_cols);
         return cudaSuccess;
     } else {
         (void)tm_cols;
-        (void)npairs;
         return cudaSuccess;
     }
 }

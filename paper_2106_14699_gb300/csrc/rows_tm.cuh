@@ -239,8 +239,8 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&re)[PTS / 2], float2 (&im)
 // more warps fit, and several small blocks, each with its own barriers, run one's transforms
 // (FMA pipe) beside another's entropy terms (ALU, MUFU).  Measured at K = 16 (1e11 counts/s):
 // Q = 512: 16 warps in one block 5.0, 2 blocks of 8 5.8, 4 of 8 6.2; Q = 1024: one of 16 6.5,
-// 2 of 8 7.0, 3 of 8 (spills) 4.8; Q = 2048: one of 16 7.2, 2 of 8 7.15.  NT = 16 also where two
-// blocks' marginals do not fit in Tensor Memory.
+// 2 of 8 7.0, 3 of 8 (spills) 4.8; Q = 2048: one of 16 7.0, 2 of 8 7.1 (1024 x 1024; few rows:
+// rows_tm_teams).  NT = 16 also where two blocks' marginals do not fit in Tensor Memory.
 template <int Q, int NT_>
 struct RowTmCfg {
     static constexpr int L = Q / 2, G = Q % 3 == 0 ? 3 : Q == 4096 ? 2 : 1, LS = L / G;

@@ -136,6 +136,37 @@ def test_wide_rows_tmem_partial_rounds(cm, W, Q, K):
     assert float(np.abs(g["mi"] - ref["mi"]).max()) <= MI_TOL
 
 
+@pytest.mark.parametrize("nmi", [False, True])
+@pytest.mark.parametrize("H", [30, 70, 170])
+@pytest.mark.parametrize("K", [(5, 8), (7, 7), (3, 16)], ids=lambda x: "x".join(map(str, x)))
+def test_wide_rows_tmem_teams(cm, K, H, nmi):
+    """Q = 2048 on both sides of the lines between blocks of 8 and of 16 teams (more than 32
+    pairs; as many rows as SMs, for one map and for two angles at once), AUTO too: the same maps
+    from all of them, N and MI against the oracle."""
+    rng = np.random.default_rng(H + K[1])
+    A, MA, B, MB = _rand(rng, H, 1500, H + 3, 60, *K)
+    ref = (oracle.nmi if nmi else oracle.cmif)(A, MA, B, MB, *K)
+    want = ref["nmi"] if nmi else ref["mi"]
+    tol = 5e-6 / np.maximum(ref["h_ab"], 1e-300) if nmi else MI_TOL
+    t = [torch.tensor(np.ascontiguousarray(x), device="cuda") for x in (A, MA, B, MB)]
+    maps = []
+    for prec, batch in ((cm.FP32, False), (cm.AUTO, False), (cm.FP32, True)):
+        p = cm.Plan(*A.shape, *B.shape, *K, prec, nmi=nmi, batch_angles=batch)
+        mi = torch.zeros((2, p.R, p.C), dtype=torch.float64, device="cuda")
+        n = torch.zeros((2, p.R, p.C), dtype=torch.int32, device="cuda")
+        if batch:
+            rec = torch.zeros(48, dtype=torch.uint8, device="cuda")
+            p.align_rotations(*t, [0.0, 0.0], 0.5, 2, rec, mi, n_maps=n)
+            assert bool((mi[0] == mi[1]).all()) and bool((n[0] == n[1]).all())
+        else:
+            p.compute(*t, mi[0], n[0])
+        assert p.status()[0] == "OK"
+        p.close()
+        np.testing.assert_array_equal(n[0].cpu().numpy(), ref["n"])
+        maps.append(mi[0].cpu().numpy())
+        assert np.all(np.abs(maps[-1] - want) <= tol) and np.array_equal(maps[-1], maps[0])
+
+
 @pytest.mark.parametrize("K", [(3, 7), (9, 3), (22, 22)], ids=lambda x: "x".join(map(str, x)))
 @pytest.mark.parametrize("W", [1240, 1490, 2600, 3000, 3200, 4090])
 def test_wide_rows_tmem_team_of_warps(cm, W, K):
