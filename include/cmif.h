@@ -99,7 +99,10 @@ typedef enum { CMIF_FP32 = 0, CMIF_SPLIT32 = 1, CMIF_FP64 = 2, CMIF_AUTO = 3 } c
 /* Plan flags. */
 #define CMIF_FLAG_DEBUG_COUNTS 1u /* allow a non-NULL counts output in cmif_compute */
 #define CMIF_FLAG_GRAPH 2u        /* capture each call's launches in a CUDA graph once and replay it while the
-                                     call's arguments (pointers, gamma, angles) are unchanged */
+                                     call's arguments (pointers, gamma, angles) are unchanged.  Other arguments
+                                     are captured anew, which takes longer than a call without a graph (64 x 64,
+                                     8 x 8 labels, each call waited for: replayed 48 us, captured 105, no graph
+                                     63): for callers that keep their buffers */
 #define CMIF_FLAG_WINDOW 4u       /* Alg. 1's padded search window (Sec. 3.6, Alg. 1's ZERO-PAD step: A and M_A zero-padded
                                      by p_i = ceil(|X_B|_i (1 - gamma)) along each axis).  X_S becomes the shifts
                                      that keep B's domain inside padded A's: chi_i in [|X_B|_i - |X_A|_i - p_i, p_i]
@@ -398,7 +401,7 @@ typedef struct {
  * that JSON-lines file and read back by later processes, keyed on the
  * transform sizes, label counts, depths, precision, SM count and device name.
  * Results do not depend on the choice (the same counts and MI).  Synchronous;
- * uses a temporary device buffer for the synthetic labels.  FP64 and two-term
+ * uses a temporary device buffer for the synthetic labels.  FP64 and SPLIT32
  * plans have nothing to choose (out reports zeros).  out may be NULL. */
 cmif_status cmif_plan_autotune(cmif_plan plan, const char* cache_path, cmif_tuning* out);
 

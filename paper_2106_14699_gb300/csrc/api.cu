@@ -83,7 +83,7 @@ struct cmif_plan_s {
     unsigned flags = 0;
     Workspace<float> w32;
     Workspace<double> w64;  // weighted plans
-    Workspace<m31> wm31;    // exact transforms: FP64 and two-term plans, AUTO's second precision
+    Workspace<m31> wm31;    // exact transforms: FP64 and SPLIT32 plans, AUTO's second precision
     bool has32 = false, has64 = false, has_m31 = false;
     DevStatus* st = nullptr;      // status of the map being computed (reset per map)
     DevStatus* st_total = nullptr;  // status of the whole call (what cmif_get_status reports)
@@ -136,7 +136,7 @@ cmif_status from_cuda(cudaError_t e) {
 }
 
 // Row-kernel choice for precision T: the TMEM / TMA variant where it applies
-// (FP32, Q = 512, 1024 or 2048), else B-marginals in shared memory when they fit,
+// (FP32, tm_rows(Q), the marginals within Tensor Memory), else B-marginals in shared memory when they fit,
 // else in global memory.  Fills tm_cols, cb_smem and rows_grid.
 template <typename T>
 cmif_status choose_rows(cmif_plan p, Workspace<T>& w) {
@@ -405,7 +405,7 @@ cmif_status compute_map_auto(cmif_plan p, const Geom& g, const int32_t* A, const
 
 // One full map into (mi, n, counts); its status in p->st (reset here) is folded
 // into p->st_total.  stages32 selects the FP32 stages (A's transforms may be
-// reused across calls); an exact pass (FP64 and two-term plans) always recomputes everything.
+// reused across calls); an exact pass (FP64 and SPLIT32 plans) always recomputes everything.
 cmif_status compute_map(cmif_plan p, const Geom& g, const int32_t* A, const uint8_t* MA, const int32_t* B,
                         const uint8_t* MB, double* mi, int32_t* n, int32_t* counts, cudaStream_t s,
                         unsigned stages32, bool first, bool finalize) {

@@ -27,7 +27,7 @@ struct Geom {
     int HA, WA, HB, WB;  // image sizes
     int KA, KB;          // label counts
     int R, C;            // output map rows / cols: H_A+H_B-1, W_A+W_B-1
-    int P, Q;            // transform sizes (powers of two >= R, C)
+    int P, Q;            // transform sizes >= R2, C (2^k; FP32 also 3 * 2^k)
     int Qh;              // Q/2 + 1 half-spectrum columns
     int Qs;              // padded row stride (complex elements) of row-major spectra
     int Ys;              // complex values per row of Y: Q / 2

@@ -615,10 +615,10 @@ struct PairColsCfg {
         if (M == 16) return R == 3 ? 4 : R <= 2 ? 2 : 1;
         return M == 8 ? 4 : 2;
     }
-    // Volumes: depth offsets per item.  The depth sum of one offset reads two slice spectra
-    // per product, which bounds the kernel by L2-to-SM traffic (20 TB/s); offsets dz .. dz + NDZ - 1
-    // share A's slice and slide over B's, two loads per NDZ products.  40 x 56 x 64, K = 8 (P = 128):
-    // 664 us with one offset per item, 463 with four.
+    // Volumes: depth offsets per item.  The depth sum of one offset loads two slice spectra
+    // per product; offsets dz .. dz + NDZ - 1 share A's slice and slide over B's, two loads per
+    // NDZ products.  40 x 56 x 64, K = 8 (P = 128): 664 us with one offset per item, 463 with four,
+    // still waiting for those loads most of all (2.9 cycles per issue; L2 32 %, FMA pipe 45 %).
     static constexpr int NDZ = std::is_same<T, float>::value ? (M == 8 ? 4 : M == 16 && R <= 3 ? 2 : 1) : 1;
     static constexpr int min_blocks(bool vol) { return sizeof(T) != 4 ? 1 : vol && NDZ > 1 ? 2 : f32_blocks(); }
 };

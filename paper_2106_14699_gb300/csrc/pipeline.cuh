@@ -1,5 +1,5 @@
 // Launch sequence of one CMIF map for one arithmetic: FP32, residues mod 2^31 - 1 (m31.cuh;
-// FP64, two-term and AUTO's second-precision counts) or FP64 (weighted maps).
+// FP64, SPLIT32 and AUTO's second-precision counts) or FP64 (weighted maps).
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>

@@ -378,8 +378,8 @@ def test_auto_per_pair_precision_unbalanced_labels(cm, mode, monkeypatch):
     """A dominant label (98% of 1024^2 pixels) makes the FP32 correlation of the
     pair (0, 0) inexact.  CMIF_AUTO computes that pair in the second precision:
     chosen up front by the predicate, or, with the predicate off, after the FP32
-    guard breached (two-term FP32, or FP64 on request).  Only the listed pairs pay
-    for it: N exact and MI within tolerance at sampled shifts, and the AUTO map
+    guard breached (guard-fp64: with CMIF_AUTO_TIER2 set, which is accepted and changes
+    nothing).  Only the listed pairs pay for it: N exact and MI within tolerance at sampled shifts, and the AUTO map
     costs the FP32 map plus well under the second-precision map it replaced (one
     pair of four listed: about a quarter of it)."""
     if mode != "predicate":

@@ -1,5 +1,5 @@
 """The three transform precisions side by side at the benchmark size
-(1024^2, K = 16): FP32, two-term FP32 (split) and FP64.  For each: time of one
+(1024^2, K = 16): FP32, SPLIT32 and FP64 (both exact integer transforms).  For each: time of one
 map, max pre-rounding residual, count mismatches and MI error against the
 oracle on sampled shifts (all K_A*K_B + K_A + K_B counts there), and count
 mismatches of the whole map against the FP64 map."""

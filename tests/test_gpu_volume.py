@@ -122,7 +122,7 @@ def test_volume_host_entry_auto_and_nmi(cm):
 def test_volume_auto_every_pair_listed(cm, monkeypatch):
     """Volume plan with CMIF_AUTO and every pair sent to the second precision
     (CMIF_AUTO_PREDICATE=all): the listed pairs' depth-summed products and exact
-    counts come from the two-term transforms; N and MI equal the oracle's."""
+    counts come from the exact integer transforms; N and MI equal the oracle's."""
     monkeypatch.setenv("CMIF_AUTO_PREDICATE", "all")
     rng = np.random.default_rng(41)
     A = rng.integers(0, 3, (4, 9, 10)).astype(np.int32)
