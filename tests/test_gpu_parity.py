@@ -85,11 +85,10 @@ def test_ragged_random(cm, prec_name, shape):
     check_exact(cm, A, MA, B, MB, shape[4], shape[5], getattr(cm, prec_name), gamma=0.3)
 
 
-# Wide maps (Q = 1024 / 2048) run the row kernel that keeps the B-marginals in
-# Tensor Memory and prefetches Y rows with TMA: K_B = 16 takes its fast path,
-# other K_B the general one.  Also check it against the shared-memory kernel.
-# Row widths C = W_A + W_B - 1 whose transform width Q is 512, 1024 or 2048 (the
-# smallest 2^k or 3 * 2^k >= C), the widths of the Tensor-Memory row kernel.
+# Wide maps run the row kernel that keeps the B-marginals in Tensor Memory and
+# copies Y rows with TMA.  Also check it against the shared-memory kernel.  Row
+# widths C = W_A + W_B - 1 whose transform width Q is 512, 1024 or 2048 (the
+# smallest 2^k or 3 * 2^k >= C), where one warp transforms a row.
 WIDE = [((20, 450, 30, 500), (16, 16)), ((16, 300, 12, 480), (5, 7)), ((20, 200, 30, 250), (16, 16)),
         ((9, 900, 11, 800), (16, 16)), ((12, 880, 10, 900), (24, 3)), ((16, 240, 12, 260), (5, 7))]
 
@@ -101,9 +100,8 @@ def _transform_width(c):
 @pytest.mark.parametrize("shape,K", WIDE, ids=lambda x: "x".join(map(str, x)))
 def test_wide_rows_tmem_path(cm, shape, K, monkeypatch):
     """Q = 512, 1024 and 2048 with no count maps requested run the Tensor-Memory row
-    kernel (TMA-staged rows, B-marginals in TMEM; at Q = 1024 the load-once radix-2
-    step, at Q = 512 radix-4 teams and one pass per row): N and MI against the
-    oracle over the whole map.  The generic kernel
+    kernel (TMA-staged rows, B-marginals in TMEM; 8, 16 or 32 points per lane): N and
+    MI against the oracle over the whole map.  The generic kernel
     (CMIF_DISABLE_TMEM=1, with count maps, every count against the oracle) gives
     the same N and bit-identical MI."""
     HA, WA, HB, WB = shape
@@ -196,8 +194,8 @@ def test_wide_rows_tmem_team_of_warps(cm, W, K):
         assert found[0] == found[1]
 
 
-# Every transform length, across rows (Q) and down columns (P): maps just over the next
-# shorter length and maps that fill it.  Column 0 (which carries two real columns), the
+# Every transform length, across rows (Q) and down columns (P), and 96, whose outputs take
+# 128: maps just over the next shorter length and maps that fill it.  Column 0 (which carries two real columns), the
 # mirrored columns and the first and last chunk of each length take part.
 LENGTHS = [16, 32, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048, 3072, 4096]
 
